@@ -19,6 +19,7 @@
 
 #include "cp.h"
 #include "cp_internal.cuh"
+#include "cp_spec.cuh"
 
 using namespace cpk;
 
@@ -119,6 +120,24 @@ struct cp_plan_s {
     void* d_W16 = nullptr;             // pre-swizzled W' tiles (tensor form)
     float* d_coef = nullptr;           // [n_curves * n_max]
     float* d_wrho = nullptr;           // tensor form: per sample, row sum of the 16-bit operand's rounding error
+
+    // direct-form curves on the uniform grid through the pair spectrum (cp_spec.cu)
+    bool spec = false;
+    int64_t spec_m0 = 0, spec_mq = 1;  // frequencies (m0 + mq k) delta
+    double spec_delta = 0;
+    int spec_chunk = 0;                // curves per chunk
+    int spec_chunks = 0;               // chunks of all waves
+    int spec_seg = 0;                  // cells per spreading item
+    int spec_min_logq = 0, spec_max_logq = 0;
+    int64_t spec_p_ld = 0;
+    int spec_fc_min = kFcMax;
+    SpecCurve* d_sc = nullptr;
+    float* d_scoef = nullptr;
+    uint64_t* d_sxs = nullptr;
+    float *d_sys = nullptr, *d_sP = nullptr, *d_srow = nullptr;
+    float2 *d_sx = nullptr, *d_tw = nullptr;
+    unsigned int* d_svmax = nullptr;
+    int32_t *d_scand = nullptr, *d_sfb = nullptr;
 
     // device buffers
     void* dblock = nullptr;              // one allocation for everything below
@@ -598,6 +617,92 @@ cp_status enqueue_pair(cp_plan_t p, int stage, int w, float* out, cudaStream_t s
     return CP_OK;
 }
 
+// The uniform grid of a wave of direct-form curves through the pair spectrum:
+// chunk by chunk the spectrum and the harmonic sums, then the pair sum at the
+// few frequencies that can be the largest, then (normally none) the curves whose
+// whole grid the pair sum evaluates.
+cp_status enqueue_spec(cp_plan_t p, int w, float* out, cudaStream_t s, int* ev_idx)
+{
+    const Wave& wv = p->waves[w];
+    if (ev_idx) {
+        CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx)], s, rec_flags(p)));
+        p->ev_cls[*ev_idx] = 0;
+    }
+    int chunk0 = 0;      // chunks of the waves before this one
+    for (int v = 0; v < w; v++)
+        if (p->waves[v].cls == 0)
+            chunk0 += (p->waves[v].slot_end - p->waves[v].slot_begin + p->spec_chunk - 1) / p->spec_chunk;
+    unsigned long long* q0 = queue_word(p, kQueuesPerWave * (int)p->waves.size());
+    int* fb_count = reinterpret_cast<int*>(q0 + p->spec_chunks + w);
+    SpecArgs a{};
+    a.cp = p->d_cp;
+    a.sc = p->d_sc;
+    a.coef = p->d_scoef;
+    a.order = p->d_order;
+    a.times = p->host_inputs ? p->d_times : p->times;
+    a.yp = p->d_yp;
+    a.xs = p->d_sxs;
+    a.ys = p->d_sys;
+    a.delta = p->spec_delta;
+    a.m0 = p->spec_m0;
+    a.mq = p->spec_mq;
+    a.n_freq = p->grid.n_freq;
+    a.np2max = p->np2max;
+    a.seg = p->spec_seg;
+    a.x = p->d_sx;
+    a.x_ld = (int64_t)1 << p->spec_max_logq;
+    a.P = p->d_sP;
+    a.p_ld = p->spec_p_ld;
+    a.rows = out ? out : p->d_srow;
+    a.row_ld = p->grid.n_freq;
+    a.rows_by_curve = out ? 1 : 0;
+    a.vmax = p->d_svmax;
+    a.cand = p->d_scand;
+    a.fb_slots = p->d_sfb;
+    a.fb_count = fb_count;
+    a.tw = p->d_tw;
+    a.ex = exclusion_of(p);
+    a.slot_begin = wv.slot_begin;
+    a.slot_end = wv.slot_end;
+    CP_CUDA(launch_spec_prep(a, s));
+    for (int b = wv.slot_begin, k = chunk0; b < wv.slot_end; b += p->spec_chunk, k++) {
+        a.slot_begin = b;
+        a.slot_end = std::min(b + p->spec_chunk, wv.slot_end);
+        a.queue = q0 + k;
+        CP_CUDA(launch_spec_chunk(a, p->n_sm, p->max_n, p->spec_min_logq <= kSpecOneLogQ,
+                                  p->spec_max_logq > kSpecOneLogQ, s));
+    }
+    PairArgs l = pair_args(p, kStageFull, w, out);
+    PairArgs f = l;
+    l.stage = kStageList;
+    l.queue = queue_word(p, kQueuesPerWave * w + kStageList);
+    l.trials = p->d_scand;
+    l.n_trials = kSpecCand;
+    l.trial_stat = nullptr;
+    l.candidates = 1;
+    l.upc = (kSpecCand + p->spec_fc_min - 1) / p->spec_fc_min;
+    l.unit_begin = 0;
+    l.unit_end = l.upc * (wv.slot_end - wv.slot_begin);
+    CP_CUDA(launch_pair_direct(l, p->pair_grid, p->pair_smem, s));
+    f.upc = (p->grid.n_freq + p->spec_fc_min - 1) / p->spec_fc_min;
+    f.fb_count = fb_count;
+    f.fb_slots = p->d_sfb;
+    f.unit_begin = 0;
+    CP_CUDA(launch_pair_direct(f, p->pair_grid, p->pair_smem, s));
+    if (ev_idx) {
+        CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx) + 1], s, rec_flags(p)));
+        (*ev_idx)++;
+    }
+    return CP_OK;
+}
+
+// The uniform grid of a wave.
+cp_status enqueue_full(cp_plan_t p, int w, float* out, cudaStream_t s, int* ev_idx)
+{
+    if (p->spec && p->waves[w].cls == 0) return enqueue_spec(p, w, out, s, ev_idx);
+    return enqueue_pair(p, kStageFull, w, out, s, ev_idx);
+}
+
 cp_status enqueue_search(cp_plan_t p, cudaStream_t s)
 {
     cp_status st;
@@ -640,7 +745,7 @@ cp_status enqueue_search(cp_plan_t p, cudaStream_t s)
         if (p->bands) {
             if ((st = enqueue_pair(p, kStageList, w, nullptr, s, &ev)) != CP_OK) return st;
         } else if (!p->grid.hierarchical) {
-            if ((st = enqueue_pair(p, kStageFull, w, nullptr, s, &ev)) != CP_OK) return st;
+            if ((st = enqueue_full(p, w, nullptr, s, &ev)) != CP_OK) return st;
         } else {
             if ((st = enqueue_pair(p, kStageCoarse, w, nullptr, s, &ev)) != CP_OK) return st;
             TopkArgs t{};
@@ -666,6 +771,8 @@ cp_status enqueue_search(cp_plan_t p, cudaStream_t s)
     f.top_k = p->grid.top_k;
     f.trials = p->d_trials;
     f.n_trials = p->n_trials;
+    f.cand = p->d_scand;
+    f.n_cand = kSpecCand;
     f.fine_half = p->J;
     f.f_min = p->grid.f_min;
     f.df = p->grid.df;
@@ -789,6 +896,82 @@ void cp_destroy(cp_plan_t p)
     cudaSetDevice(prev);
     cudaGetLastError();
     delete p;
+}
+
+// Whether the uniform grid of the direct-form curves goes through the pair
+// spectrum, and its workspace.  The frequencies must be multiples of one
+// spacing, df / q, and the spectrum must pay: the pair sum takes
+// N (N - 1) / 2 exponentials per frequency, the spectrum a few operations per
+// pair, the transform and nh products per frequency, and a few more launches.
+static void plan_spec(cp_plan_t p, const float* st_per_curve)
+{
+    const cp_freq_grid& g = p->grid;
+    int64_t mq = 0, m0 = 0;
+    for (int64_t q : {1, 2, 3, 4, 5, 6, 8, 10}) {
+        const double r = g.f_min / g.df * (double)q, k = std::nearbyint(r);
+        if (k < 1e9 && std::fabs(r - k) <= 1e-15 * k + 1e-13) {
+            mq = q;
+            m0 = (int64_t)k;
+            break;
+        }
+    }
+    if (!mq) return;
+    const int64_t top = m0 + mq * (g.n_freq - 1);
+    double t_pair = 0, t_spec = 0;
+    int lo = kSpecMaxLogQ + 1, hi = 0, nh_hi = 0, fc_min = kFcMax;
+    const int usual_nh = spec_harmonics(0.4);
+    float last_st = -1.f;
+    int nh = 0;
+    for (int64_t c = 0; c < p->n_curves; c++) {
+        if (p->cls[c]) continue;
+        // sigma_t of the rule lies in [0.1, 0.6]: workspace for the smallest, cost at a usual one
+        const float st = p->opt.sigma_t_mode == CP_SIGMA_T_FIXED ? p->opt.sigma_t
+                         : p->opt.sigma_t_mode == CP_SIGMA_T_PER_CURVE ? st_per_curve[c] : 0.1f;
+        if (st != last_st) nh = spec_harmonics(last_st = st);
+        const double n = (double)(p->offsets[c + 1] - p->offsets[c]), pairs = 0.5 * n * (n - 1);
+        // pair sum: per unit of fc frequencies about 4 us for its trig table and sums and 6 us (at 16
+        // frequencies) for every 16 tiles, one unit per SM at a time (measured at N = 150 and 650)
+        const double whole = std::ceil((double)g.n_freq / p->fc[c]) *
+                             (4e-6 + 6e-6 * p->fc[c] / kFcMax * std::ceil(tiles_of((int)n) / 16.0)) / p->n_sm;
+        fc_min = std::min(fc_min, p->fc[c]);
+        t_pair += whole;
+        if (!nh) {
+            t_spec += whole;
+            continue;
+        }
+        int lq = spec_logq((int64_t)nh * top + 1);
+        if (!lq) lq = kSpecMaxLogQ;          // a curve that needs more is evaluated by the pair sum
+        const int usual = p->opt.sigma_t_mode == CP_SIGMA_T_RULE ? usual_nh : nh;
+        const int ul = spec_logq((int64_t)usual * top + 1);
+        t_spec += ul ? pairs * 8e-12 + std::ldexp(1.4e-11, ul) + (double)g.n_freq * usual * 6e-12 : whole;
+        lo = std::min(lo, spec_logq(top + 1) ? spec_logq(top + 1) : lq);
+        hi = std::max(hi, lq);
+        nh_hi = std::max(nh_hi, nh);
+    }
+    if (!nh_hi || t_spec + 60e-6 >= t_pair) return;
+    const int64_t p_ld = std::min<int64_t>((int64_t)nh_hi * top + 1, (int64_t)(std::ldexp(2.0, hi) / kSpecOver)) + 1;
+    const size_t per = (sizeof(float2) << hi) + (size_t)p_ld * sizeof(float) + (size_t)g.n_freq * sizeof(float);
+    int64_t largest = 0, in_wave = 0;
+    for (const Wave& w : p->waves)
+        if (w.cls == 0) largest = std::max<int64_t>(largest, w.slot_end - w.slot_begin);
+    in_wave = std::min<int64_t>({largest, (int64_t)std::max<size_t>(1, ((size_t)1 << 30) / per), (int64_t)kSpecMaxChunk});
+    p->spec = true;
+    p->spec_mq = mq;
+    p->spec_m0 = m0;
+    p->spec_delta = g.df / (double)mq;
+    p->spec_min_logq = lo;
+    p->spec_max_logq = hi;
+    p->spec_p_ld = p_ld;
+    p->spec_chunk = (int)in_wave;
+    p->spec_fc_min = fc_min;
+    for (const Wave& w : p->waves)
+        if (w.cls == 0) p->spec_chunks += (w.slot_end - w.slot_begin + p->spec_chunk - 1) / p->spec_chunk;
+    // cells per spreading item: about four items per SM for a chunk, between 512 and 8192
+    const double cells = std::ldexp(2.0, std::min(hi, spec_logq(14 * top + 1) ? spec_logq(14 * top + 1) : hi)) * 0.5 *
+                         (double)p->spec_chunk;
+    int seg = 512;
+    while (seg < 8192 && cells / (double)(2 * seg) > 4.0 * (double)p->n_sm) seg *= 2;
+    p->spec_seg = seg;
 }
 
 static cp_status plan_impl(const double* times, const float* mags, const float* errs,
@@ -1068,9 +1251,11 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         close_wave(sb, (int)n_curves);
     }
 
+    plan_spec(p, opt.sigma_t_per_curve);
+
     // device allocation (one block)
     const int64_t np = p->n_points, nc = n_curves;
-    const int nq = kQueuesPerWave * (int)p->waves.size();
+    const int nq = kQueuesPerWave * (int)p->waves.size() + (p->spec ? p->spec_chunks + (int)p->waves.size() : 0);
     p->n_u64 = 1 + nc + nq;
     struct Part { void** dst; size_t bytes; };
     const bool hier = g.hierarchical == CP_SEARCH_COARSE_FINE;
@@ -1104,6 +1289,17 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         {(void**)&p->d_W16, (size_t)max_tiles16 * tile16_bytes},
         {(void**)&p->d_coef, p->tensor ? (size_t)nc * kCoefStride * sizeof(float) : 0},
         {(void**)&p->d_wrho, p->tensor ? np * sizeof(float) : 0},
+        {(void**)&p->d_sc, p->spec ? (size_t)nc * sizeof(SpecCurve) : 0},
+        {(void**)&p->d_scoef, p->spec ? (size_t)nc * kSpecMaxHarm * sizeof(float) : 0},
+        {(void**)&p->d_sxs, p->spec ? np * sizeof(uint64_t) : 0},
+        {(void**)&p->d_sys, p->spec ? np * sizeof(float) : 0},
+        {(void**)&p->d_sx, p->spec ? ((size_t)p->spec_chunk << p->spec_max_logq) * sizeof(float2) : 0},
+        {(void**)&p->d_sP, p->spec ? (size_t)p->spec_chunk * p->spec_p_ld * sizeof(float) : 0},
+        {(void**)&p->d_srow, p->spec ? (size_t)p->spec_chunk * g.n_freq * sizeof(float) : 0},
+        {(void**)&p->d_tw, p->spec ? (size_t)kSpecTwiddles * sizeof(float2) : 0},
+        {(void**)&p->d_svmax, p->spec ? (size_t)nc * sizeof(unsigned int) : 0},
+        {(void**)&p->d_scand, p->spec ? (size_t)nc * kSpecCand * sizeof(int32_t) : 0},
+        {(void**)&p->d_sfb, p->spec ? (size_t)nc * sizeof(int32_t) : 0},
         {(void**)&p->d_coarse, hier ? (size_t)nc * p->kc * sizeof(float) : 0},
         {(void**)&p->d_peaks, hier ? (size_t)nc * g.top_k * sizeof(int32_t) : 0},
         {(void**)&p->d_npeaks, hier ? nc * sizeof(int32_t) : 0},
@@ -1183,6 +1379,11 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     }
     p->opt.sigma_t_per_curve = nullptr;
 
+    if (p->spec) {
+        CP_CUDA(spec_prepare(p->np2max, p->max_n, p->spec_seg));
+        CP_CUDA(launch_spec_twiddle(p->d_tw, p->stream));
+    }
+
     // launch geometry of the persistent pair kernel
     CP_CUDA(prepare_kernels(p->np2max, p->pair_smem));
     if (bnd) {
@@ -1215,6 +1416,12 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     p->launches_per_search =
         2 /* zero, stats */ + (p->tensor ? 1 : 0) /* harmonic coefficients */ + (bnd ? 2 : 0) /* bands, window */ +
         (int64_t)p->waves.size() * (hier ? 4 : 2) + 1 /* finalize */;
+    if (p->spec && !hier && !bnd)
+        for (const Wave& w : p->waves)
+            if (w.cls == 0)
+                p->launches_per_search += 2 + (int64_t)((w.slot_end - w.slot_begin + p->spec_chunk - 1) / p->spec_chunk) *
+                                                  (3 + (p->spec_min_logq <= kSpecOneLogQ ? 1 : 0) +
+                                                   (p->spec_max_logq > kSpecOneLogQ ? 2 : 0));
     return CP_OK;
 }
 
@@ -1286,7 +1493,7 @@ static cp_status periodogram_impl(cp_plan_t p, float* out)
     if ((st = enqueue_inputs(p, p->stream)) == CP_OK && (st = enqueue_stats(p, p->stream)) == CP_OK) {
         for (int w = 0; w < (int)p->waves.size() && st == CP_OK; w++) {
             st = enqueue_wave_w(p, w, p->stream);
-            if (st == CP_OK) st = enqueue_pair(p, kStageFull, w, out, p->stream, nullptr);
+            if (st == CP_OK) st = enqueue_full(p, w, out, p->stream, nullptr);
         }
     }
     if (st == CP_OK)

@@ -50,6 +50,9 @@ struct CurveParams {
                       // (tensor form: its harmonic count's truncation target; else 0)
     float dwsum;      // tensor form: sum over all (i, j) of the 16-bit operand's rounding
                       // error of w_ij (the row sums per sample are in StatsArgs::wrho)
+    int32_t by_list;  // full grid through the pair spectrum (cp_spec.cu): the best key holds a
+                      // position in the curve's candidate list, not a grid index
+    int32_t reserved;
 };
 
 // sigma_t = 0.1 + 0.5 exp(-12 S^2), S the Bowley skewness of the magnitudes
@@ -163,6 +166,11 @@ struct PairArgs {
     const int32_t* trials;       // list stage: [n_curves * n_trials] grid indices, -1 = none
     int32_t n_trials;
     float* trial_stat;           // list stage: nCKP per trial (may be null)
+    int32_t candidates;          // list stage: the list is a pair-spectrum candidate list (entries
+                                 // from its start, -1 after the last; values also go to `out`)
+    int64_t upc;                 // > 0: upc units per curve (candidate lists, whole curves of fb_slots)
+    const int* fb_count;         // full stage: only the slots fb_slots[0 .. *fb_count) (else null)
+    const int32_t* fb_slots;
     Exclusion ex;                // spurious-period windows (Section 6.1)
 };
 
@@ -220,6 +228,8 @@ struct FinalArgs {
     double f_min, df, coarse_df, fine_df;
     const int32_t* trials;        // bands method: best key index -> grid index
     int32_t n_trials;
+    const int32_t* cand;          // pair spectrum: list position -> grid index, n_cand per curve
+    int32_t n_cand;
     int64_t* best_idx;
     double* best_freq;
     float* best_stat;

@@ -417,6 +417,10 @@ __device__ __forceinline__ void pair_item(const ulonglong2* SC, const f2* NS, in
     }
 }
 
+// SEL: a launch over chosen frequencies (candidate lists) or chosen curves
+// (fb_slots) of the pair-spectrum path; its own instantiation, so that the
+// units of a plain launch carry none of it.
+template <bool SEL>
 __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs a)
 {
     constexpr int NW = kPairThreads / 32;
@@ -431,19 +435,27 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
         if (tid == 0) s_unit = (long long)atomicAdd(a.queue, 1ull) + a.unit_begin;
         __syncthreads();
         const long long u = s_unit;
-        if (u >= a.unit_end) break;
+        if (u >= (SEL && a.fb_count ? (long long)*a.fb_count * a.upc : a.unit_end)) break;
 
-        int lo = a.slot_begin, hi = a.slot_end - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (a.unit_start[mid] <= u) lo = mid; else hi = mid - 1;
+        int slot;
+        long long chunk;
+        if (SEL) {
+            const int64_t q = u / a.upc;
+            chunk = u - q * a.upc;
+            slot = a.fb_count ? a.fb_slots[q] : a.slot_begin + (int)q;
+        } else {
+            int lo = a.slot_begin, hi = a.slot_end - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (a.unit_start[mid] <= u) lo = mid; else hi = mid - 1;
+            }
+            slot = lo;
+            chunk = u - a.unit_start[slot];
         }
-        const int slot = lo;
         const int c = a.order[slot];
         const CurveParams& P = a.cp[c];
-        const int n = P.n, fc = P.fc, nfp = fc >> 1;
+        const int n = P.n, fc = P.fc;
         const int npad = (n + kTile - 1) & ~(kTile - 1);
-        const long long chunk = u - a.unit_start[slot];
         const int64_t off = P.off;
 
         // frequencies of this unit: phase(i, kk) = base_i + mult0 * step_i + kk * step_i
@@ -466,8 +478,16 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
         } else {
             kfirst = chunk * fc;
             count = (int)min((long long)fc, a.n_freq - kfirst);
+            if (SEL && count <= 0) continue;   // fewer units than the launch gives a curve
         }
         const int32_t* tl = a.trials + (int64_t)c * a.n_trials;   // list stage only
+        if (SEL && a.candidates) {
+            int have = 0;
+            while (have < count && tl[kfirst + have] >= 0) have++;
+            if (have == 0) continue;
+            count = have;
+        }
+        const int nfp = SEL ? (count + 1) >> 1 : fc >> 1;   // frequency pairs of the unit
 
         // trig table: SC[fp][i] = {(s_f, s_f'), (c_f, c_f')} * sqrt(beta), NS[fp][i] = -(s_f, s_f')
         // (sin form), or the sines and cosines of the doubled angle * sqrt(beta / 2) (cos form)
@@ -592,6 +612,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
                 } else if (a.stage == kStageList) {
                     const bool valid = tl[kk] >= 0;
                     if (a.trial_stat) a.trial_stat[(int64_t)c * a.n_trials + kk] = valid ? v : __int_as_float(0x7fc00000);
+                    if (SEL && a.candidates && a.out) a.out[(int64_t)c * a.out_ld + tl[kk]] = v;
                     if (valid && !excluded_k(a.ex.full_k, a.ex.n, tl[kk])) key = make_key(v, (uint32_t)kk);
                 } else {
                     const double fpk = grid_freq(a.f_min, (double)peak_mult, a.coarse_df);
@@ -683,7 +704,8 @@ __global__ void k_finalize(const FinalArgs a)
         const double fpk = __dadd_rn(a.f_min, __dmul_rn((double)a.peaks[(int64_t)c * a.top_k + p], a.coarse_df));
         f = __dadd_rn(fpk, __dmul_rn((double)j, a.fine_df));
     } else {
-        f = __dadd_rn(a.f_min, __dmul_rn((double)idx, a.df));
+        if (a.cp[c].by_list) kout = (uint32_t)a.cand[(int64_t)c * a.n_cand + idx];   // list position -> grid index
+        f = __dadd_rn(a.f_min, __dmul_rn((double)kout, a.df));
     }
     a.best_idx[c] = (int64_t)kout;
     a.best_freq[c] = f;
@@ -732,7 +754,8 @@ cudaError_t launch_build_w(const BuildWArgs& a, cudaStream_t s)
 
 cudaError_t launch_pair_direct(const PairArgs& a, int grid, size_t smem, cudaStream_t s)
 {
-    k_pair_direct<<<grid, kPairThreads, smem, s>>>(a);
+    if (a.upc > 0) k_pair_direct<true><<<grid, kPairThreads, smem, s>>>(a);
+    else k_pair_direct<false><<<grid, kPairThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -776,14 +799,16 @@ cudaError_t prepare_kernels(int np2max, size_t pair_smem)
 {
     cudaError_t e = raise_dyn_smem((const void*)k_stats, stats_smem_bytes(np2max));
     if (e != cudaSuccess) return e;
-    return raise_dyn_smem((const void*)k_pair_direct, pair_smem);
+    e = raise_dyn_smem((const void*)k_pair_direct<true>, pair_smem);
+    if (e != cudaSuccess) return e;
+    return raise_dyn_smem((const void*)k_pair_direct<false>, pair_smem);
 }
 
 cudaError_t pair_direct_occupancy(int* blocks_per_sm, size_t smem)
 {
-    cudaError_t e = raise_dyn_smem((const void*)k_pair_direct, smem);
+    cudaError_t e = raise_dyn_smem((const void*)k_pair_direct<false>, smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_pair_direct, kPairThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_pair_direct<false>, kPairThreads, smem);
 }
 
 cudaError_t launch_zero_u64(unsigned long long* p, int64_t n, cudaStream_t s)

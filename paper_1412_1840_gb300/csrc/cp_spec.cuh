@@ -1,0 +1,80 @@
+// cp_spec.cuh -- the pair-spectrum evaluation of the direct form (cp_spec.cu):
+// types and launchers shared with the host API.
+//
+// The periodic kernel is even and periodic in the phase, so (Eq. (taylor)
+// regrouped by harmonic) the pair sum of Eq. (HP) is
+//   S(f) = N (1 - ip) (1 - a_0) + 2 sum_{n=1}^{nh} a_n P(n f),
+//   P(nu) = sum_{i<j} w_ij cos(2 pi nu (t_i - t_j)),
+// and P does not depend on the trial frequency: one cosine transform of the
+// pairs' time differences serves every frequency of the grid.
+#pragma once
+#include "cp_internal.cuh"
+
+namespace cpk {
+
+constexpr int kSpecMaxHarm = 64;       // harmonics kept per curve
+constexpr int kSpecMinLogQ = 8;        // complex transform length 2^logq
+constexpr int kSpecMaxLogQ = 22;
+constexpr int kSpecOneLogQ = 13;       // up to this length one CTA transforms a curve
+constexpr int kSpecCand = 64;          // frequencies per curve evaluated again by the pair sum
+constexpr int kSpecMaxChunk = 64;      // curves per chunk
+constexpr double kSpecTail = 2e-8;     // harmonics left out: at most this much of the kernel's peak
+constexpr double kSpecOver = 1.1;      // transform length over the highest frequency needed, at least
+
+// What the device decides for one curve (its sigma_t and span are known there).
+struct SpecCurve {
+    double cells_per_day;   // 2 H / L: grid cells per day of time difference
+    int64_t H;              // cells of the half period, 2 Q
+    int32_t nh;             // harmonics
+    int32_t logq;           // Q = 2^logq
+    int32_t support;        // cells that can be non-zero, a multiple of 4 (H: all)
+    int32_t n_out;          // pair-spectrum values needed
+    float one_minus_a0;
+    float pad;
+};
+
+struct SpecArgs {
+    CurveParams* cp;
+    SpecCurve* sc;                // [n_curves]
+    float* coef;                  // [n_curves * kSpecMaxHarm] a_1..
+    const int32_t* order;
+    const double* times;
+    const float* yp;              // scaled magnitudes, caller's order
+    uint64_t* xs;                 // sorted times in cells, 32.32 fixed point
+    float* ys;                    // scaled magnitudes in time order
+    double delta;                 // spacing of the pair spectrum (1/day): frequencies are (m0 + mq k) delta
+    int64_t m0, mq;
+    int64_t n_freq;
+    int slot_begin, slot_end;     // curves of this launch
+    int np2max;
+    int seg;                      // cells per spreading item
+    float2* x;                    // chunk workspace: transform data, x_ld per curve
+    int64_t x_ld;
+    float* P;                     // pair spectrum, p_ld per curve
+    int64_t p_ld;
+    float* rows;                  // periodogram rows: row index = caller's curve, or slot - slot_begin
+    int64_t row_ld;
+    int rows_by_curve;
+    unsigned int* vmax;           // [n_curves] largest admissible value (orderable bits)
+    int32_t* cand;                // [n_curves * kSpecCand] grid indices, -1 = none
+    int32_t* fb_slots;            // slots whose candidates do not fit
+    int* fb_count;
+    unsigned long long* queue;    // spreading items
+    const float2* tw;             // exp(-2 pi i k / 8192), k < 8192
+    Exclusion ex;
+};
+
+constexpr int kSpecTwiddles = 8192;
+cudaError_t launch_spec_twiddle(float2* tw, cudaStream_t s);   // fills kSpecTwiddles entries
+cudaError_t spec_prepare(int np2max, int max_n, int seg);
+size_t spec_spread_smem(int max_n, int seg);
+cudaError_t launch_spec_prep(const SpecArgs& a, cudaStream_t s);
+// spread, transform, harmonic sums, candidates of one chunk (slot_end - slot_begin <= kSpecMaxChunk)
+cudaError_t launch_spec_chunk(const SpecArgs& a, int n_sm, int max_n, bool one_pass, bool two_pass, cudaStream_t s);
+
+// Host: harmonics needed at sigma_t for a truncation tail of kSpecTail (0: more than kSpecMaxHarm).
+int spec_harmonics(double sigma_t);
+// Host: log2 of the complex transform length for n_out values (0: too long).
+int spec_logq(int64_t n_out);
+
+}  // namespace cpk
