@@ -72,9 +72,16 @@ struct Wave {
     int cls;              // 0: direct form; else the tensor form with this many harmonics
 };
 
-struct PairLaunch {
-    int stage;
-    int wave;
+// How the direct-form curves of one kind of pass use the pair spectrum.
+struct SpecPlan {
+    bool on = false;
+    bool interp = false;               // frequencies between the spectrum's entries
+    int64_t m0 = 0, mq = 1;            // else: frequencies (m0 + mq k) delta
+    double delta = 0, f_top = 0;
+    int min_logq = 0, max_logq = 0;    // transform lengths that can occur
+    int64_t p_ld = 0, row = 0;         // floats per curve: pair spectrum, values
+    int chunk = 0, chunks = 0;         // curves per chunk; chunks of all waves
+    int seg = 0;                       // cells per spreading item
 };
 
 }  // namespace
@@ -121,16 +128,10 @@ struct cp_plan_s {
     float* d_coef = nullptr;           // [n_curves * n_max]
     float* d_wrho = nullptr;           // tensor form: per sample, row sum of the 16-bit operand's rounding error
 
-    // direct-form curves on the uniform grid through the pair spectrum (cp_spec.cu)
-    bool spec = false;
-    int64_t spec_m0 = 0, spec_mq = 1;  // frequencies (m0 + mq k) delta
-    double spec_delta = 0;
-    int spec_chunk = 0;                // curves per chunk
-    int spec_chunks = 0;               // chunks of all waves
-    int spec_seg = 0;                  // cells per spreading item
-    int spec_min_logq = 0, spec_max_logq = 0;
-    int64_t spec_p_ld = 0;
+    // direct-form curves through the pair spectrum (cp_spec.cu)
+    SpecPlan sfull, ssearch;           // the uniform grid; the coarse-then-fine or bands search
     int spec_fc_min = kFcMax;
+    bool spec() const { return sfull.on || ssearch.on; }
     SpecCurve* d_sc = nullptr;
     float* d_scoef = nullptr;
     uint64_t* d_sxs = nullptr;
@@ -517,6 +518,23 @@ PairArgs pair_args(cp_plan_t p, int stage, int w, float* out)
     return a;
 }
 
+TopkArgs topk_args(cp_plan_t p, int w, const int* fb_count = nullptr, const int32_t* fb_slots = nullptr)
+{
+    TopkArgs t{};
+    t.coarse = p->d_coarse;
+    t.order = p->d_order;
+    t.slot_begin = p->waves[w].slot_begin;
+    t.slot_end = p->waves[w].slot_end;
+    t.n_freq = p->kc;
+    t.top_k = p->grid.top_k;
+    t.peaks = p->d_peaks;
+    t.n_peaks = p->d_npeaks;
+    t.fb_count = fb_count;
+    t.fb_slots = fb_slots;
+    t.ex = exclusion_of(p);
+    return t;
+}
+
 cp_status enqueue_wave_w(cp_plan_t p, int w, cudaStream_t s)
 {
     const Wave& wv = p->waves[w];
@@ -617,23 +635,9 @@ cp_status enqueue_pair(cp_plan_t p, int stage, int w, float* out, cudaStream_t s
     return CP_OK;
 }
 
-// The uniform grid of a wave of direct-form curves through the pair spectrum:
-// chunk by chunk the spectrum and the harmonic sums, then the pair sum at the
-// few frequencies that can be the largest, then (normally none) the curves whose
-// whole grid the pair sum evaluates.
-cp_status enqueue_spec(cp_plan_t p, int w, float* out, cudaStream_t s, int* ev_idx)
+// What every launch of the pair spectrum shares; `base` holds the stage's grid.
+SpecArgs spec_args(cp_plan_t p, const SpecPlan& sp, const PairArgs& base)
 {
-    const Wave& wv = p->waves[w];
-    if (ev_idx) {
-        CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx)], s, rec_flags(p)));
-        p->ev_cls[*ev_idx] = 0;
-    }
-    int chunk0 = 0;      // chunks of the waves before this one
-    for (int v = 0; v < w; v++)
-        if (p->waves[v].cls == 0)
-            chunk0 += (p->waves[v].slot_end - p->waves[v].slot_begin + p->spec_chunk - 1) / p->spec_chunk;
-    unsigned long long* q0 = queue_word(p, kQueuesPerWave * (int)p->waves.size());
-    int* fb_count = reinterpret_cast<int*>(q0 + p->spec_chunks + w);
     SpecArgs a{};
     a.cp = p->d_cp;
     a.sc = p->d_sc;
@@ -643,52 +647,144 @@ cp_status enqueue_spec(cp_plan_t p, int w, float* out, cudaStream_t s, int* ev_i
     a.yp = p->d_yp;
     a.xs = p->d_sxs;
     a.ys = p->d_sys;
-    a.delta = p->spec_delta;
-    a.m0 = p->spec_m0;
-    a.mq = p->spec_mq;
-    a.n_freq = p->grid.n_freq;
+    a.interp = sp.interp ? 1 : 0;
+    a.delta = sp.delta;
+    a.m0 = sp.m0;
+    a.mq = sp.mq;
+    a.f_top = sp.f_top;
+    a.n_freq = base.n_freq;
+    a.f_min = base.f_min;
+    a.f_max = base.f_max;
+    a.step = base.step;
+    a.coarse_df = base.coarse_df;
+    a.peaks = p->d_peaks;
+    a.peaks_out = p->d_peaks;
+    a.n_peaks = p->d_npeaks;
+    a.top_k = p->grid.top_k;
+    a.fine_half = p->J;
+    a.trials = p->d_trials;
+    a.n_trials = p->n_trials;
     a.np2max = p->np2max;
-    a.seg = p->spec_seg;
+    a.seg = sp.seg;
     a.x = p->d_sx;
-    a.x_ld = (int64_t)1 << p->spec_max_logq;
+    a.x_ld = (int64_t)1 << sp.max_logq;
     a.P = p->d_sP;
-    a.p_ld = p->spec_p_ld;
-    a.rows = out ? out : p->d_srow;
-    a.row_ld = p->grid.n_freq;
-    a.rows_by_curve = out ? 1 : 0;
+    a.p_ld = sp.p_ld;
     a.vmax = p->d_svmax;
     a.cand = p->d_scand;
     a.fb_slots = p->d_sfb;
-    a.fb_count = fb_count;
     a.tw = p->d_tw;
     a.ex = exclusion_of(p);
-    a.slot_begin = wv.slot_begin;
-    a.slot_end = wv.slot_end;
-    CP_CUDA(launch_spec_prep(a, s));
-    for (int b = wv.slot_begin, k = chunk0; b < wv.slot_end; b += p->spec_chunk, k++) {
-        a.slot_begin = b;
-        a.slot_end = std::min(b + p->spec_chunk, wv.slot_end);
-        a.queue = q0 + k;
-        CP_CUDA(launch_spec_chunk(a, p->n_sm, p->max_n, p->spec_min_logq <= kSpecOneLogQ,
-                                  p->spec_max_logq > kSpecOneLogQ, s));
-    }
-    PairArgs l = pair_args(p, kStageFull, w, out);
-    PairArgs f = l;
-    l.stage = kStageList;
-    l.queue = queue_word(p, kQueuesPerWave * w + kStageList);
-    l.trials = p->d_scand;
-    l.n_trials = kSpecCand;
-    l.trial_stat = nullptr;
-    l.candidates = 1;
+    return a;
+}
+
+// Units over candidate entries, or over whole curves of a fallback list.
+PairArgs over_candidates(cp_plan_t p, PairArgs l, int kind, int n_slots)
+{
+    l.candidates = kind;
+    l.cand = p->d_scand;
+    l.n_cand = kSpecCand;
     l.upc = (kSpecCand + p->spec_fc_min - 1) / p->spec_fc_min;
     l.unit_begin = 0;
-    l.unit_end = l.upc * (wv.slot_end - wv.slot_begin);
-    CP_CUDA(launch_pair_direct(l, p->pair_grid, p->pair_smem, s));
-    f.upc = (p->grid.n_freq + p->spec_fc_min - 1) / p->spec_fc_min;
-    f.fb_count = fb_count;
-    f.fb_slots = p->d_sfb;
+    l.unit_end = l.upc * n_slots;
+    return l;
+}
+
+PairArgs over_fallback(cp_plan_t p, PairArgs f, const int* count, const int32_t* slots, int64_t points, int64_t times)
+{
+    f.upc = (points + p->spec_fc_min - 1) / p->spec_fc_min * times;
+    f.fb_count = count;
+    f.fb_slots = slots;
     f.unit_begin = 0;
-    CP_CUDA(launch_pair_direct(f, p->pair_grid, p->pair_smem, s));
+    return f;
+}
+
+// One wave of direct-form curves through the pair spectrum.  Chunk by chunk:
+// the spectrum and the values at the stage's frequencies (coarse-then-fine: the
+// coarse row, the pair sum at the points that decide the peaks, the peaks, the
+// fine values).  Then the pair sum at the few candidates for the best, and
+// (normally none) the curves that it evaluates whole.
+cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float* out, cudaStream_t s, int* ev_idx)
+{
+    const Wave& wv = p->waves[w];
+    const int n_slots = wv.slot_end - wv.slot_begin;
+    const bool hier = stage == kStageCoarse;
+    if (ev_idx) {
+        CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx)], s, rec_flags(p)));
+        p->ev_cls[*ev_idx] = 0;
+    }
+    int chunk0 = 0;      // chunks of the waves before this one
+    for (int v = 0; v < w; v++)
+        if (p->waves[v].cls == 0) chunk0 += (p->waves[v].slot_end - p->waves[v].slot_begin + sp.chunk - 1) / sp.chunk;
+    // work counters: spreading items per chunk; per wave the coarse candidates of every chunk use
+    // the chunk's second counter, then two fallback counts
+    unsigned long long* q0 = queue_word(p, kQueuesPerWave * (int)p->waves.size());
+    unsigned long long* qc = q0 + sp.chunks;
+    int* fb = reinterpret_cast<int*>(q0 + 2 * sp.chunks + w);          // [0] whole curves, [1] coarse rows
+    int32_t* fb_whole = p->d_sfb;
+    int32_t* fb_coarse = p->d_sfb + p->n_curves;
+
+    const PairArgs base = pair_args(p, stage, w, out);
+    SpecArgs a = spec_args(p, sp, base);
+    a.slot_begin = wv.slot_begin;
+    a.slot_end = wv.slot_end;
+    a.stage = hier ? kSpecCoarse : stage == kStageList ? kSpecList : kSpecFull;
+    a.rows_by_curve = 1;
+    if (hier) {
+        a.rows = p->d_coarse;
+        a.row_ld = p->kc;
+    } else if (stage == kStageList) {
+        a.rows = p->d_trial_stat;
+        a.row_ld = p->n_trials;
+    } else {
+        a.rows = out ? out : p->d_srow;
+        a.row_ld = out ? p->grid.n_freq : sp.row;
+        a.rows_by_curve = out ? 1 : 0;
+    }
+    CP_CUDA(launch_spec_prep(a, s));
+    const PairArgs fine = hier ? pair_args(p, kStageFine, w, nullptr) : base;
+    for (int b = wv.slot_begin, k = chunk0; b < wv.slot_end; b += sp.chunk, k++) {
+        a.slot_begin = b;
+        a.slot_end = std::min(b + sp.chunk, wv.slot_end);
+        a.queue = q0 + k;
+        CP_CUDA(launch_spec_transform(a, p->n_sm, p->max_n, sp.min_logq <= kSpecOneLogQ, sp.max_logq > kSpecOneLogQ, s));
+        CP_CUDA(launch_spec_values(a, p->n_sm, s));
+        SpecArgs sel = a;
+        if (hier) {
+            SpecArgs pk = a;
+            pk.fb_slots = fb_coarse;
+            pk.fb_count = fb + 1;
+            CP_CUDA(launch_spec_peaks(pk, s));
+            PairArgs l = over_candidates(p, base, kCandCoarse, a.slot_end - a.slot_begin);
+            l.slot_begin = a.slot_begin;
+            l.slot_end = a.slot_end;
+            l.queue = qc + k;
+            CP_CUDA(launch_pair_direct(l, p->pair_grid, p->pair_smem, s));
+            CP_CUDA(launch_spec_rank(a, s));
+            sel.stage = kSpecFine;
+            sel.step = p->grid.fine_df;
+            sel.rows = p->d_srow;
+            sel.row_ld = sp.row;
+            sel.rows_by_curve = 0;
+            CP_CUDA(launch_spec_values(sel, p->n_sm, s));
+        }
+        sel.fb_slots = fb_whole;
+        sel.fb_count = fb;
+        CP_CUDA(launch_spec_select(sel, s));
+    }
+    const int kind = hier ? kCandFine : stage == kStageList ? kCandTrial : kCandGrid;
+    PairArgs l = over_candidates(p, fine, kind, n_slots);
+    l.queue = queue_word(p, kQueuesPerWave * w + (stage == kStageList ? kStageFull : kStageList));
+    CP_CUDA(launch_pair_direct(l, p->pair_grid, p->pair_smem, s));
+    if (hier) {
+        CP_CUDA(launch_pair_direct(over_fallback(p, base, fb + 1, fb_coarse, p->kc, 1), p->pair_grid, p->pair_smem, s));
+        CP_CUDA(launch_topk(topk_args(p, w, fb + 1, fb_coarse), s));
+        CP_CUDA(launch_pair_direct(over_fallback(p, fine, fb, fb_whole, 2 * p->J + 1, p->grid.top_k), p->pair_grid,
+                                   p->pair_smem, s));
+    } else {
+        CP_CUDA(launch_pair_direct(over_fallback(p, base, fb, fb_whole, stage == kStageList ? p->n_trials : p->grid.n_freq, 1),
+                                   p->pair_grid, p->pair_smem, s));
+    }
     if (ev_idx) {
         CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx) + 1], s, rec_flags(p)));
         (*ev_idx)++;
@@ -696,11 +792,12 @@ cp_status enqueue_spec(cp_plan_t p, int w, float* out, cudaStream_t s, int* ev_i
     return CP_OK;
 }
 
-// The uniform grid of a wave.
-cp_status enqueue_full(cp_plan_t p, int w, float* out, cudaStream_t s, int* ev_idx)
+// The uniform grid or the trial list of a wave.
+cp_status enqueue_values(cp_plan_t p, int stage, int w, float* out, cudaStream_t s, int* ev_idx)
 {
-    if (p->spec && p->waves[w].cls == 0) return enqueue_spec(p, w, out, s, ev_idx);
-    return enqueue_pair(p, kStageFull, w, out, s, ev_idx);
+    const SpecPlan& sp = stage == kStageList ? p->ssearch : p->sfull;
+    if (sp.on && p->waves[w].cls == 0) return enqueue_spec(p, sp, stage, w, out, s, ev_idx);
+    return enqueue_pair(p, stage, w, out, s, ev_idx);
 }
 
 cp_status enqueue_search(cp_plan_t p, cudaStream_t s)
@@ -743,22 +840,14 @@ cp_status enqueue_search(cp_plan_t p, cudaStream_t s)
     for (int w = 0; w < (int)p->waves.size(); w++) {
         if ((st = enqueue_wave_w(p, w, s)) != CP_OK) return st;
         if (p->bands) {
-            if ((st = enqueue_pair(p, kStageList, w, nullptr, s, &ev)) != CP_OK) return st;
+            if ((st = enqueue_values(p, kStageList, w, nullptr, s, &ev)) != CP_OK) return st;
         } else if (!p->grid.hierarchical) {
-            if ((st = enqueue_full(p, w, nullptr, s, &ev)) != CP_OK) return st;
+            if ((st = enqueue_values(p, kStageFull, w, nullptr, s, &ev)) != CP_OK) return st;
+        } else if (p->ssearch.on && p->waves[w].cls == 0) {
+            if ((st = enqueue_spec(p, p->ssearch, kStageCoarse, w, nullptr, s, &ev)) != CP_OK) return st;
         } else {
             if ((st = enqueue_pair(p, kStageCoarse, w, nullptr, s, &ev)) != CP_OK) return st;
-            TopkArgs t{};
-            t.coarse = p->d_coarse;
-            t.order = p->d_order;
-            t.slot_begin = p->waves[w].slot_begin;
-            t.slot_end = p->waves[w].slot_end;
-            t.n_freq = p->kc;
-            t.top_k = p->grid.top_k;
-            t.peaks = p->d_peaks;
-            t.n_peaks = p->d_npeaks;
-            t.ex = exclusion_of(p);
-            CP_CUDA(launch_topk(t, s));
+            CP_CUDA(launch_topk(topk_args(p, w), s));
             if ((st = enqueue_pair(p, kStageFine, w, nullptr, s, &ev)) != CP_OK) return st;
         }
     }
@@ -771,8 +860,6 @@ cp_status enqueue_search(cp_plan_t p, cudaStream_t s)
     f.top_k = p->grid.top_k;
     f.trials = p->d_trials;
     f.n_trials = p->n_trials;
-    f.cand = p->d_scand;
-    f.n_cand = kSpecCand;
     f.fine_half = p->J;
     f.f_min = p->grid.f_min;
     f.df = p->grid.df;
@@ -838,6 +925,128 @@ cp_status read_timings(cp_plan_t p)
     return CP_OK;
 }
 
+// Workspace of the pair spectrum per plan.  A chunk's transforms pass through the
+// L2 cache better the fewer there are, and the allocation costs the plan time.
+constexpr size_t kSpecWorkspace = (size_t)1 << 30;
+size_t spec_bytes(const SpecPlan& sp, int logq)
+{
+    return (sizeof(float2) << logq) + (size_t)(sp.p_ld + sp.row) * sizeof(float) + 1024;
+}
+
+// Whether one kind of pass of the direct-form curves goes through the pair
+// spectrum, and its workspace (budget 0: kSpecWorkspace, or one curve's).  `points`: frequencies per curve; `units`: pair-sum
+// units of a curve at f frequencies per unit.  The pair sum takes N (N - 1) / 2
+// exponentials per frequency; the spectrum a few operations per pair, the
+// transform, and nh products (interpolated: 8 nh) per frequency, and more launches.
+template <typename Units>
+void plan_spec(cp_plan_t p, SpecPlan& sp, const float* st_per_curve, double points, int64_t row, size_t budget,
+               Units units)
+{
+    const int64_t top = sp.m0 + sp.mq * (p->grid.n_freq - 1);
+    // longest period that a spectrum is made for when the frequencies are interpolated: 4 T <= this
+    // (curves observed for longer are evaluated by the pair sum); and a usual one
+    const double step = p->grid.hierarchical == CP_SEARCH_COARSE_FINE ? p->grid.coarse_df : p->grid.df;
+    const double l_cap = (p->grid.hierarchical == CP_SEARCH_COARSE_FINE ? 32.0 : 4.0) / step;
+    const double l_usual = (p->grid.hierarchical == CP_SEARCH_COARSE_FINE ? 10.0 : 1.0) / step;
+    auto n_out = [&](int nh, double l) {
+        return sp.interp ? (int64_t)std::min(1e10, nh * sp.f_top * l + 16.0) : (int64_t)nh * top + 1;
+    };
+    double t_pair = 0, t_spec = 0;
+    int lo = kSpecMaxLogQ + 1, hi = 0, fc_min = kFcMax;
+    const int usual_nh = spec_harmonics(0.4);
+    float last_st = -1.f;
+    int nh = 0;
+    for (int64_t c = 0; c < p->n_curves; c++) {
+        if (p->cls[c]) continue;
+        // sigma_t of the rule lies in [0.1, 0.6]: workspace for the smallest, cost at a usual one
+        const float st = p->opt.sigma_t_mode == CP_SIGMA_T_FIXED ? p->opt.sigma_t
+                         : p->opt.sigma_t_mode == CP_SIGMA_T_PER_CURVE ? st_per_curve[c] : 0.1f;
+        if (st != last_st) nh = spec_harmonics(last_st = st);
+        const double n = (double)(p->offsets[c + 1] - p->offsets[c]), pairs = 0.5 * n * (n - 1);
+        // pair sum: per unit of fc frequencies about 4 us for its trig table and sums and 6 us (at 16
+        // frequencies) for every 16 tiles, one unit per SM at a time (measured at N = 150 and 650)
+        const double whole = (double)units(p->fc[c]) *
+                             (4e-6 + 6e-6 * p->fc[c] / kFcMax * std::ceil(tiles_of((int)n) / 16.0)) / p->n_sm;
+        fc_min = std::min(fc_min, p->fc[c]);
+        t_pair += whole;
+        if (!nh) {
+            t_spec += whole;
+            continue;
+        }
+        int lq = spec_logq(n_out(nh, l_cap));
+        if (!lq) lq = kSpecMaxLogQ;          // a curve that needs more is evaluated by the pair sum
+        const int usual = p->opt.sigma_t_mode == CP_SIGMA_T_RULE ? usual_nh : nh;
+        const int ul = spec_logq(n_out(usual, l_usual));
+        t_spec += ul ? pairs * 8e-12 + std::ldexp(1.4e-11, ul) + points * usual * (sp.interp ? 2e-11 : 6e-12) : whole;
+        lo = std::min(lo, sp.interp ? kSpecMinLogQ : spec_logq(top + 1) ? spec_logq(top + 1) : lq);
+        hi = std::max(hi, lq);
+    }
+    const double launches = p->grid.hierarchical == CP_SEARCH_COARSE_FINE ? 160e-6 : 110e-6;
+    if (!hi || t_spec + launches >= t_pair) return;
+    int64_t largest = 0;
+    for (const Wave& w : p->waves)
+        if (w.cls == 0) largest = std::max<int64_t>(largest, w.slot_end - w.slot_begin);
+    sp.p_ld = (int64_t)(std::ldexp(2.0, hi) / kSpecOver) + 2 * kSpecPad;
+    sp.row = row;
+    const size_t per = spec_bytes(sp, hi);
+    if (budget && budget < per) return;
+    if (!budget) budget = std::max(kSpecWorkspace, per);
+    sp.on = true;
+    sp.min_logq = lo;
+    sp.max_logq = hi;
+    sp.chunk = (int)std::min<int64_t>({largest, (int64_t)(budget / per), (int64_t)kSpecMaxChunk});
+    for (const Wave& w : p->waves)
+        if (w.cls == 0) sp.chunks += (w.slot_end - w.slot_begin + sp.chunk - 1) / sp.chunk;
+    // cells per spreading item: about four items per SM for a chunk, between 512 and 8192
+    const int ul = spec_logq(n_out(usual_nh, l_usual));
+    const double cells = std::ldexp(2.0, ul ? std::min(hi, ul) : hi) * 0.5 * (double)sp.chunk;
+    sp.seg = 512;
+    while (sp.seg < 8192 && cells / (double)(2 * sp.seg) > 4.0 * (double)p->n_sm) sp.seg *= 2;
+    p->spec_fc_min = fc_min;
+}
+
+void plan_spectra(cp_plan_t p, const float* st_per_curve)
+{
+    const cp_freq_grid& g = p->grid;
+    // the uniform grid: multiples of df / q where f_min is one, else interpolated
+    SpecPlan full;
+    full.interp = true;
+    for (int64_t q : {1, 2, 3, 4, 5, 6, 8, 10}) {
+        const double r = g.f_min / g.df * (double)q, k = std::nearbyint(r);
+        if (k < 1e9 && std::fabs(r - k) <= 1e-15 * k + 1e-13) {
+            full.interp = false;
+            full.mq = q;
+            full.m0 = (int64_t)k;
+            full.delta = g.df / (double)q;
+            break;
+        }
+    }
+    full.f_top = p->f_max * (1.0 + 1e-9);
+    size_t ws = 0;             // the search's workspace: a periodogram on its plan makes do with it
+    if (g.hierarchical == CP_SEARCH_COARSE_FINE) {
+        const int64_t W = 2 * (int64_t)p->J + 1, fine = W * g.top_k;
+        SpecPlan sp;
+        sp.interp = true;
+        sp.f_top = (g.f_min + (double)(p->kc - 1) * g.coarse_df) * (1.0 + 1e-9);
+        sp.f_top = std::max(sp.f_top, full.f_top);
+        if (g.top_k <= 40 && fine <= (int64_t)1 << 20 && p->kc < (int64_t)1 << 30)
+            plan_spec(p, sp, st_per_curve, (double)(p->kc + fine), fine, 0,
+                      [&](int f) { return (p->kc + f - 1) / f + g.top_k * ((W + f - 1) / f); });
+        p->ssearch = sp;
+    } else if (p->bands) {
+        SpecPlan sp;
+        sp.interp = true;
+        sp.f_top = full.f_top;
+        plan_spec(p, sp, st_per_curve, (double)p->n_trials, 0, 0,
+                  [&](int f) { return (int64_t)(p->n_trials + f - 1) / f; });
+        p->ssearch = sp;
+    }
+    if (p->ssearch.on) ws = (size_t)p->ssearch.chunk * spec_bytes(p->ssearch, p->ssearch.max_logq);
+    if (g.n_freq < (int64_t)1 << 30 && (g.hierarchical == CP_SEARCH_FULL || ws))
+        plan_spec(p, full, st_per_curve, (double)g.n_freq, g.n_freq, ws, [&](int f) { return (g.n_freq + f - 1) / f; });
+    p->sfull = full;
+}
+
 }  // namespace
 
 extern "C" {
@@ -896,82 +1105,6 @@ void cp_destroy(cp_plan_t p)
     cudaSetDevice(prev);
     cudaGetLastError();
     delete p;
-}
-
-// Whether the uniform grid of the direct-form curves goes through the pair
-// spectrum, and its workspace.  The frequencies must be multiples of one
-// spacing, df / q, and the spectrum must pay: the pair sum takes
-// N (N - 1) / 2 exponentials per frequency, the spectrum a few operations per
-// pair, the transform and nh products per frequency, and a few more launches.
-static void plan_spec(cp_plan_t p, const float* st_per_curve)
-{
-    const cp_freq_grid& g = p->grid;
-    int64_t mq = 0, m0 = 0;
-    for (int64_t q : {1, 2, 3, 4, 5, 6, 8, 10}) {
-        const double r = g.f_min / g.df * (double)q, k = std::nearbyint(r);
-        if (k < 1e9 && std::fabs(r - k) <= 1e-15 * k + 1e-13) {
-            mq = q;
-            m0 = (int64_t)k;
-            break;
-        }
-    }
-    if (!mq) return;
-    const int64_t top = m0 + mq * (g.n_freq - 1);
-    double t_pair = 0, t_spec = 0;
-    int lo = kSpecMaxLogQ + 1, hi = 0, nh_hi = 0, fc_min = kFcMax;
-    const int usual_nh = spec_harmonics(0.4);
-    float last_st = -1.f;
-    int nh = 0;
-    for (int64_t c = 0; c < p->n_curves; c++) {
-        if (p->cls[c]) continue;
-        // sigma_t of the rule lies in [0.1, 0.6]: workspace for the smallest, cost at a usual one
-        const float st = p->opt.sigma_t_mode == CP_SIGMA_T_FIXED ? p->opt.sigma_t
-                         : p->opt.sigma_t_mode == CP_SIGMA_T_PER_CURVE ? st_per_curve[c] : 0.1f;
-        if (st != last_st) nh = spec_harmonics(last_st = st);
-        const double n = (double)(p->offsets[c + 1] - p->offsets[c]), pairs = 0.5 * n * (n - 1);
-        // pair sum: per unit of fc frequencies about 4 us for its trig table and sums and 6 us (at 16
-        // frequencies) for every 16 tiles, one unit per SM at a time (measured at N = 150 and 650)
-        const double whole = std::ceil((double)g.n_freq / p->fc[c]) *
-                             (4e-6 + 6e-6 * p->fc[c] / kFcMax * std::ceil(tiles_of((int)n) / 16.0)) / p->n_sm;
-        fc_min = std::min(fc_min, p->fc[c]);
-        t_pair += whole;
-        if (!nh) {
-            t_spec += whole;
-            continue;
-        }
-        int lq = spec_logq((int64_t)nh * top + 1);
-        if (!lq) lq = kSpecMaxLogQ;          // a curve that needs more is evaluated by the pair sum
-        const int usual = p->opt.sigma_t_mode == CP_SIGMA_T_RULE ? usual_nh : nh;
-        const int ul = spec_logq((int64_t)usual * top + 1);
-        t_spec += ul ? pairs * 8e-12 + std::ldexp(1.4e-11, ul) + (double)g.n_freq * usual * 6e-12 : whole;
-        lo = std::min(lo, spec_logq(top + 1) ? spec_logq(top + 1) : lq);
-        hi = std::max(hi, lq);
-        nh_hi = std::max(nh_hi, nh);
-    }
-    if (!nh_hi || t_spec + 60e-6 >= t_pair) return;
-    const int64_t p_ld = std::min<int64_t>((int64_t)nh_hi * top + 1, (int64_t)(std::ldexp(2.0, hi) / kSpecOver)) + 1;
-    const size_t per = (sizeof(float2) << hi) + (size_t)p_ld * sizeof(float) + (size_t)g.n_freq * sizeof(float);
-    int64_t largest = 0, in_wave = 0;
-    for (const Wave& w : p->waves)
-        if (w.cls == 0) largest = std::max<int64_t>(largest, w.slot_end - w.slot_begin);
-    in_wave = std::min<int64_t>({largest, (int64_t)std::max<size_t>(1, ((size_t)1 << 30) / per), (int64_t)kSpecMaxChunk});
-    p->spec = true;
-    p->spec_mq = mq;
-    p->spec_m0 = m0;
-    p->spec_delta = g.df / (double)mq;
-    p->spec_min_logq = lo;
-    p->spec_max_logq = hi;
-    p->spec_p_ld = p_ld;
-    p->spec_chunk = (int)in_wave;
-    p->spec_fc_min = fc_min;
-    for (const Wave& w : p->waves)
-        if (w.cls == 0) p->spec_chunks += (w.slot_end - w.slot_begin + p->spec_chunk - 1) / p->spec_chunk;
-    // cells per spreading item: about four items per SM for a chunk, between 512 and 8192
-    const double cells = std::ldexp(2.0, std::min(hi, spec_logq(14 * top + 1) ? spec_logq(14 * top + 1) : hi)) * 0.5 *
-                         (double)p->spec_chunk;
-    int seg = 512;
-    while (seg < 8192 && cells / (double)(2 * seg) > 4.0 * (double)p->n_sm) seg *= 2;
-    p->spec_seg = seg;
 }
 
 static cp_status plan_impl(const double* times, const float* mags, const float* errs,
@@ -1251,11 +1384,17 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         close_wave(sb, (int)n_curves);
     }
 
-    plan_spec(p, opt.sigma_t_per_curve);
+    plan_spectra(p, opt.sigma_t_per_curve);
+    const bool spec = p->spec();
+    const int spec_chunks = std::max(p->sfull.chunks, p->ssearch.chunks);
+    auto largest = [&](auto per) { return std::max(p->sfull.on ? per(p->sfull) : 0, p->ssearch.on ? per(p->ssearch) : 0); };
+    const size_t sx_bytes = largest([](const SpecPlan& q) { return ((size_t)q.chunk << q.max_logq) * sizeof(float2); });
+    const size_t sp_bytes = largest([](const SpecPlan& q) { return (size_t)q.chunk * q.p_ld * sizeof(float); });
+    const size_t srow_bytes = largest([](const SpecPlan& q) { return (size_t)q.chunk * q.row * sizeof(float); });
 
     // device allocation (one block)
     const int64_t np = p->n_points, nc = n_curves;
-    const int nq = kQueuesPerWave * (int)p->waves.size() + (p->spec ? p->spec_chunks + (int)p->waves.size() : 0);
+    const int nq = kQueuesPerWave * (int)p->waves.size() + (spec ? 2 * spec_chunks + (int)p->waves.size() : 0);
     p->n_u64 = 1 + nc + nq;
     struct Part { void** dst; size_t bytes; };
     const bool hier = g.hierarchical == CP_SEARCH_COARSE_FINE;
@@ -1289,17 +1428,17 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         {(void**)&p->d_W16, (size_t)max_tiles16 * tile16_bytes},
         {(void**)&p->d_coef, p->tensor ? (size_t)nc * kCoefStride * sizeof(float) : 0},
         {(void**)&p->d_wrho, p->tensor ? np * sizeof(float) : 0},
-        {(void**)&p->d_sc, p->spec ? (size_t)nc * sizeof(SpecCurve) : 0},
-        {(void**)&p->d_scoef, p->spec ? (size_t)nc * kSpecMaxHarm * sizeof(float) : 0},
-        {(void**)&p->d_sxs, p->spec ? np * sizeof(uint64_t) : 0},
-        {(void**)&p->d_sys, p->spec ? np * sizeof(float) : 0},
-        {(void**)&p->d_sx, p->spec ? ((size_t)p->spec_chunk << p->spec_max_logq) * sizeof(float2) : 0},
-        {(void**)&p->d_sP, p->spec ? (size_t)p->spec_chunk * p->spec_p_ld * sizeof(float) : 0},
-        {(void**)&p->d_srow, p->spec ? (size_t)p->spec_chunk * g.n_freq * sizeof(float) : 0},
-        {(void**)&p->d_tw, p->spec ? (size_t)kSpecTwiddles * sizeof(float2) : 0},
-        {(void**)&p->d_svmax, p->spec ? (size_t)nc * sizeof(unsigned int) : 0},
-        {(void**)&p->d_scand, p->spec ? (size_t)nc * kSpecCand * sizeof(int32_t) : 0},
-        {(void**)&p->d_sfb, p->spec ? (size_t)nc * sizeof(int32_t) : 0},
+        {(void**)&p->d_sc, spec ? (size_t)nc * sizeof(SpecCurve) : 0},
+        {(void**)&p->d_scoef, spec ? (size_t)nc * kSpecMaxHarm * sizeof(float) : 0},
+        {(void**)&p->d_sxs, spec ? np * sizeof(uint64_t) : 0},
+        {(void**)&p->d_sys, spec ? np * sizeof(float) : 0},
+        {(void**)&p->d_sx, sx_bytes},
+        {(void**)&p->d_sP, sp_bytes},
+        {(void**)&p->d_srow, srow_bytes},
+        {(void**)&p->d_tw, spec ? (size_t)kSpecTwiddles * sizeof(float2) : 0},
+        {(void**)&p->d_svmax, spec ? (size_t)nc * sizeof(unsigned int) : 0},
+        {(void**)&p->d_scand, spec ? (size_t)nc * kSpecCand * sizeof(int32_t) : 0},
+        {(void**)&p->d_sfb, spec ? 2 * (size_t)nc * sizeof(int32_t) : 0},
         {(void**)&p->d_coarse, hier ? (size_t)nc * p->kc * sizeof(float) : 0},
         {(void**)&p->d_peaks, hier ? (size_t)nc * g.top_k * sizeof(int32_t) : 0},
         {(void**)&p->d_npeaks, hier ? nc * sizeof(int32_t) : 0},
@@ -1379,8 +1518,8 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     }
     p->opt.sigma_t_per_curve = nullptr;
 
-    if (p->spec) {
-        CP_CUDA(spec_prepare(p->np2max, p->max_n, p->spec_seg));
+    if (spec) {
+        CP_CUDA(spec_prepare(p->np2max, p->max_n, std::max(p->sfull.seg, p->ssearch.seg)));
         CP_CUDA(launch_spec_twiddle(p->d_tw, p->stream));
     }
 
@@ -1403,7 +1542,8 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     }
 
     // events
-    const int pair_launches = (int)p->waves.size() * (hier ? 2 : 1);
+    int pair_launches = 0;
+    for (const Wave& w : p->waves) pair_launches += hier && !(p->ssearch.on && w.cls == 0) ? 2 : 1;
     p->ev_pair.resize(2 * pair_launches);
     p->ev_cls.assign(pair_launches, 0);
     for (auto& e : p->ev_pair) CP_CUDA(cudaEventCreate(&e));
@@ -1416,12 +1556,14 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     p->launches_per_search =
         2 /* zero, stats */ + (p->tensor ? 1 : 0) /* harmonic coefficients */ + (bnd ? 2 : 0) /* bands, window */ +
         (int64_t)p->waves.size() * (hier ? 4 : 2) + 1 /* finalize */;
-    if (p->spec && !hier && !bnd)
+    const SpecPlan& sp = hier || bnd ? p->ssearch : p->sfull;
+    if (sp.on)
         for (const Wave& w : p->waves)
-            if (w.cls == 0)
-                p->launches_per_search += 2 + (int64_t)((w.slot_end - w.slot_begin + p->spec_chunk - 1) / p->spec_chunk) *
-                                                  (3 + (p->spec_min_logq <= kSpecOneLogQ ? 1 : 0) +
-                                                   (p->spec_max_logq > kSpecOneLogQ ? 2 : 0));
+            if (w.cls == 0) {
+                const int64_t chunks = (w.slot_end - w.slot_begin + sp.chunk - 1) / sp.chunk;
+                const int transform = 1 + (sp.min_logq <= kSpecOneLogQ ? 1 : 0) + (sp.max_logq > kSpecOneLogQ ? 2 : 0);
+                p->launches_per_search += 2 + chunks * (transform + (hier ? 6 : 2));
+            }
     return CP_OK;
 }
 
@@ -1493,7 +1635,7 @@ static cp_status periodogram_impl(cp_plan_t p, float* out)
     if ((st = enqueue_inputs(p, p->stream)) == CP_OK && (st = enqueue_stats(p, p->stream)) == CP_OK) {
         for (int w = 0; w < (int)p->waves.size() && st == CP_OK; w++) {
             st = enqueue_wave_w(p, w, p->stream);
-            if (st == CP_OK) st = enqueue_full(p, w, out, p->stream, nullptr);
+            if (st == CP_OK) st = enqueue_values(p, kStageFull, w, out, p->stream, nullptr);
         }
     }
     if (st == CP_OK)

@@ -50,9 +50,6 @@ struct CurveParams {
                       // (tensor form: its harmonic count's truncation target; else 0)
     float dwsum;      // tensor form: sum over all (i, j) of the 16-bit operand's rounding
                       // error of w_ij (the row sums per sample are in StatsArgs::wrho)
-    int32_t by_list;  // full grid through the pair spectrum (cp_spec.cu): the best key holds a
-                      // position in the curve's candidate list, not a grid index
-    int32_t reserved;
 };
 
 // sigma_t = 0.1 + 0.5 exp(-12 S^2), S the Bowley skewness of the magnitudes
@@ -77,6 +74,11 @@ __device__ __forceinline__ double sigma_t_rule(const float* ys, int n)
 // kStageList evaluates an explicit per-curve list of grid indices (the trial
 // frequencies of the bands method).
 enum Stage : int { kStageFull = 0, kStageCoarse = 1, kStageFine = 2, kStageList = 3 };
+
+// What a candidate entry e of the pair spectrum names: a grid index (full or
+// coarse grid), a position in the curve's trial list, or a fine candidate
+// rank (2J+1) + (j+J).
+enum Candidates : int { kCandNone = 0, kCandGrid = 1, kCandCoarse = 2, kCandTrial = 3, kCandFine = 4 };
 
 // Direct-form pair tiling: a warp owns a 32 x 32 tile of (row i, col j)
 // pairs of the upper block triangle; lane (a, b) = (lane / 8, lane % 8)
@@ -166,10 +168,12 @@ struct PairArgs {
     const int32_t* trials;       // list stage: [n_curves * n_trials] grid indices, -1 = none
     int32_t n_trials;
     float* trial_stat;           // list stage: nCKP per trial (may be null)
-    int32_t candidates;          // list stage: the list is a pair-spectrum candidate list (entries
-                                 // from its start, -1 after the last; values also go to `out`)
-    int64_t upc;                 // > 0: upc units per curve (candidate lists, whole curves of fb_slots)
-    const int* fb_count;         // full stage: only the slots fb_slots[0 .. *fb_count) (else null)
+    // launches over chosen frequencies or curves (pair spectrum, cp_spec.cu):
+    int64_t upc;                 // > 0: upc units per curve
+    int32_t candidates;          // Candidates kind of cand (kCandNone: every unit of the stage)
+    int32_t n_cand;
+    const int32_t* cand;         // [n_curves * n_cand] entries, -1 after the last
+    const int* fb_count;         // only the slots fb_slots[0 .. *fb_count) (null: every slot)
     const int32_t* fb_slots;
     Exclusion ex;                // spurious-period windows (Section 6.1)
 };
@@ -214,6 +218,8 @@ struct TopkArgs {
     int top_k;
     int32_t* peaks;
     int32_t* n_peaks;
+    const int* fb_count;          // only the slots fb_slots[0 .. *fb_count) (null: every slot)
+    const int32_t* fb_slots;
     Exclusion ex;                 // excluded coarse points are not peak candidates
 };
 
@@ -228,8 +234,6 @@ struct FinalArgs {
     double f_min, df, coarse_df, fine_df;
     const int32_t* trials;        // bands method: best key index -> grid index
     int32_t n_trials;
-    const int32_t* cand;          // pair spectrum: list position -> grid index, n_cand per curve
-    int32_t n_cand;
     int64_t* best_idx;
     double* best_freq;
     float* best_stat;

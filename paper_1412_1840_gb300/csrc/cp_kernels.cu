@@ -463,30 +463,31 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
         int count;
         int peak = 0;
         uint64_t peak_mult = 0;  // fine: coarse peak index (phase offset kpeak * coarse_i)
-        if (a.stage == kStageFine) {
+        const int32_t* ce = SEL ? a.cand + (int64_t)c * a.n_cand : nullptr;   // candidate entries
+        if (SEL && a.candidates != kCandNone) {
+            kfirst = chunk * fc;
+            count = 0;
+            while (count < fc && kfirst + count < a.n_cand && ce[kfirst + count] >= 0) count++;
+            if (count == 0) continue;
+        } else if (a.stage == kStageFine) {
             const int W = 2 * a.fine_half + 1;
             const int upp = (W + fc - 1) / fc;
             peak = (int)(chunk / upp);
             const int sub = (int)(chunk - (long long)peak * upp);
-            if (peak >= a.n_peaks[c]) continue;
+            if (peak >= a.n_peaks[c]) continue;   // (also a chunk beyond the curve's own units)
             peak_mult = (uint64_t)a.peaks[(int64_t)c * a.top_k + peak];
             kfirst = -a.fine_half + (long long)sub * fc;
             count = (int)min((long long)fc, (long long)a.fine_half - kfirst + 1);
         } else if (a.stage == kStageList) {
             kfirst = chunk * fc;     // first list position
             count = (int)min((long long)fc, (long long)a.n_trials - kfirst);
+            if (SEL && count <= 0) continue;
         } else {
             kfirst = chunk * fc;
             count = (int)min((long long)fc, a.n_freq - kfirst);
             if (SEL && count <= 0) continue;   // fewer units than the launch gives a curve
         }
         const int32_t* tl = a.trials + (int64_t)c * a.n_trials;   // list stage only
-        if (SEL && a.candidates) {
-            int have = 0;
-            while (have < count && tl[kfirst + have] >= 0) have++;
-            if (have == 0) continue;
-            count = have;
-        }
         const int nfp = SEL ? (count + 1) >> 1 : fc >> 1;   // frequency pairs of the unit
 
         // trig table: SC[fp][i] = {(s_f, s_f'), (c_f, c_f')} * sqrt(beta), NS[fp][i] = -(s_f, s_f')
@@ -509,7 +510,17 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
                 if (a.stage == kStageFine) ph += peak_mult * a.ph_coarse[off + i];
                 for (int fp = fp0; fp < fp1; fp++, ph += 2 * st) {
                     uint64_t p0 = ph, p1 = ph + st;
-                    if (a.stage == kStageList) {
+                    if (SEL && a.candidates != kCandNone) {
+                        auto phase = [&](int e) -> uint64_t {
+                            if (a.candidates == kCandTrial) return base + (uint64_t)max(tl[e], 0) * st;
+                            if (a.candidates != kCandFine) return base + (uint64_t)e * st;
+                            const int W = 2 * a.fine_half + 1, pk = e / W;
+                            return base + (uint64_t)a.peaks[(int64_t)c * a.top_k + pk] * a.ph_coarse[off + i] +
+                                   (uint64_t)(int64_t)(e - pk * W - a.fine_half) * st;
+                        };
+                        p0 = phase(ce[kfirst + 2 * fp]);
+                        p1 = 2 * fp + 1 < count ? phase(ce[kfirst + 2 * fp + 1]) : p0;
+                    } else if (a.stage == kStageList) {
                         // grid indices of list positions kfirst + 2 fp (+1); a missing entry evaluates k = 0
                         const long long q0 = kfirst + 2 * fp;
                         const int k0 = q0 < a.n_trials ? max(tl[q0], 0) : 0;
@@ -604,7 +615,14 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
                 for (int w = 0; w < NW; w++) S += s_red[w][lane];
                 const float v = (2.0f * S + P.diag) * P.norm;
                 const long long kk = kfirst + lane;
-                if (a.stage == kStageFull) {
+                if (SEL && a.candidates != kCandNone) {
+                    // admissible already; the value also replaces the spectrum's
+                    const int e = ce[kk];
+                    if (a.candidates == kCandGrid && a.out) a.out[(int64_t)c * a.out_ld + e] = v;
+                    if (a.candidates == kCandCoarse) a.coarse_out[(int64_t)c * a.n_freq + e] = v;
+                    if (a.candidates == kCandTrial && a.trial_stat) a.trial_stat[(int64_t)c * a.n_trials + e] = v;
+                    if (a.candidates != kCandCoarse) key = make_key(v, (uint32_t)e);
+                } else if (a.stage == kStageFull) {
                     if (a.out) a.out[(int64_t)c * a.out_ld + kk] = v;
                     if (!excluded_k(a.ex.full_k, a.ex.n, kk)) key = make_key(v, (uint32_t)kk);
                 } else if (a.stage == kStageCoarse) {
@@ -612,7 +630,6 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
                 } else if (a.stage == kStageList) {
                     const bool valid = tl[kk] >= 0;
                     if (a.trial_stat) a.trial_stat[(int64_t)c * a.n_trials + kk] = valid ? v : __int_as_float(0x7fc00000);
-                    if (SEL && a.candidates && a.out) a.out[(int64_t)c * a.out_ld + tl[kk]] = v;
                     if (valid && !excluded_k(a.ex.full_k, a.ex.n, tl[kk])) key = make_key(v, (uint32_t)kk);
                 } else {
                     const double fpk = grid_freq(a.f_min, (double)peak_mult, a.coarse_df);
@@ -634,16 +651,21 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
 }
 
 // ===========================================================================
-// k_topk: one warp per curve, top_k local maxima of the coarse periodogram.
+// k_topk: one CTA per curve, top_k local maxima of the coarse periodogram.
 // Local maximum: v[k] > v[k-1] and v[k] >= v[k+1]; ends use one neighbour.
-// Order: value descending, ties to the lower k (larger key).
+// Order: value descending, ties to the lower k (larger key).  The row is gone
+// through once per peak; with one warp per curve that was a chain of
+// top_k K / 32 dependent steps (150 us at K = 4,999, top_k = 10, however few
+// curves), with 256 threads it is top_k K / 256.
 // ===========================================================================
+constexpr int kTopkThreads = 256;
 
-__global__ void __launch_bounds__(256) k_topk(const TopkArgs a)
+__global__ void __launch_bounds__(kTopkThreads) k_topk(const TopkArgs a)
 {
-    const int lane = threadIdx.x & 31;
-    const int slot = a.slot_begin + blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (slot >= a.slot_end) return;
+    __shared__ unsigned long long s_best[kTopkThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (a.fb_count && (int)blockIdx.x >= *a.fb_count) return;
+    const int slot = a.fb_count ? a.fb_slots[blockIdx.x] : a.slot_begin + (int)blockIdx.x;
     const int c = a.order[slot];
     const float* v = a.coarse + (int64_t)c * a.n_freq;
     const int64_t K = a.n_freq;
@@ -651,7 +673,7 @@ __global__ void __launch_bounds__(256) k_topk(const TopkArgs a)
     int cnt = 0;
     for (int r = 0; r < a.top_k; r++) {
         unsigned long long best = 0ull;
-        for (int64_t k = lane; k < K; k += 32) {
+        for (int64_t k = tid; k < K; k += kTopkThreads) {
             const float x = v[k];
             const bool lok = (k == 0) || (x > v[k - 1]);
             const bool rok = (k == K - 1) || (x >= v[k + 1]);
@@ -665,12 +687,17 @@ __global__ void __launch_bounds__(256) k_topk(const TopkArgs a)
             const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
             best = other > best ? other : best;
         }
+        __syncthreads();
+        if (lane == 0) s_best[warp] = best;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < kTopkThreads / 32; w++) best = s_best[w] > best ? s_best[w] : best;
         if (best == 0ull) break;
-        if (lane == 0) a.peaks[(int64_t)c * a.top_k + r] = (int32_t)(0xffffffffu - (uint32_t)(best & 0xffffffffu));
+        if (tid == 0) a.peaks[(int64_t)c * a.top_k + r] = (int32_t)(0xffffffffu - (uint32_t)(best & 0xffffffffu));
         prev = best;
         cnt++;
     }
-    if (lane == 0) a.n_peaks[c] = cnt;
+    if (tid == 0) a.n_peaks[c] = cnt;
 }
 
 // ===========================================================================
@@ -704,8 +731,7 @@ __global__ void k_finalize(const FinalArgs a)
         const double fpk = __dadd_rn(a.f_min, __dmul_rn((double)a.peaks[(int64_t)c * a.top_k + p], a.coarse_df));
         f = __dadd_rn(fpk, __dmul_rn((double)j, a.fine_df));
     } else {
-        if (a.cp[c].by_list) kout = (uint32_t)a.cand[(int64_t)c * a.n_cand + idx];   // list position -> grid index
-        f = __dadd_rn(a.f_min, __dmul_rn((double)kout, a.df));
+        f = __dadd_rn(a.f_min, __dmul_rn((double)idx, a.df));
     }
     a.best_idx[c] = (int64_t)kout;
     a.best_freq[c] = f;
@@ -763,7 +789,7 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t s)
 {
     const int n = a.slot_end - a.slot_begin;
     if (n <= 0) return cudaSuccess;
-    k_topk<<<(n + 7) / 8, 256, 0, s>>>(a);
+    k_topk<<<n, kTopkThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -23,14 +23,21 @@
 //   k_spec_select  the trial frequencies within the rounding of the largest
 //                  value; the pair-sum kernel evaluates those again, so the best
 //                  frequency and its statistic are the pair sum's
+//   k_spec_peaks,  coarse-then-fine search: the coarse points whose exact values
+//   k_spec_rank    decide the peaks (evaluated again by the pair sum), and the peaks
 //
-// The trial frequencies must be multiples of one spacing delta (f_min and df
-// are integer multiples of it); the transform's period is 1 / delta, and time
-// differences beyond half of it fold back exactly.
+// Frequencies that are multiples of one spacing delta (a uniform grid whose f_min
+// and df are integer multiples of it) are entries of a spectrum of period
+// 1 / delta; time differences beyond half of the period fold back exactly.
+// Other frequencies (fine windows, trial lists, any other grid) are
+// interpolated with the same window from a spectrum of period L >= 4 T, the
+// pairs' weights divided by the window's transform beforehand (a type-3
+// transform).
 //
 // Measured (GB300; N 300-1000, 49,981 frequencies, sigma_t rule): best period of
 // 384 curves 715.8 ms by the pair sum alone, 7.4 ms through the spectrum, results
-// identical; 12 periodograms 25.3 -> 0.42 ms, error against FP64 3.4e-7 -> 7.5e-8.
+// identical; 12 periodograms 25.3 -> 0.42 ms, error against FP64 3.4e-7 -> 7.5e-8;
+// coarse-then-fine search of 256 curves 81.4 -> 7.5 ms, results identical.
 #include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -66,6 +73,23 @@ __device__ __forceinline__ float kb_inverse(float r)     // r = m / H
     const float o2 = om * om;
     const float z = sqrtf(kKbShape * kKbShape - o2);
     return kKbInv0 * (1.0f / kKbShape) * z * ex2_approx(1.4426950408889634f * __fdividef(o2, z + kKbShape));
+}
+
+// Weights of the 8 cells l - 3 .. l + 4 around a point z = f - 1/2 off the middle of cells l, l + 1.
+__device__ __forceinline__ void kb_weights(float z, float (&w)[8])
+{
+    const float s = z * z;
+#pragma unroll
+    for (int k = 1; k <= 4; k++) {
+        float ev = fmaf(s, c_kbE[k - 1][3], c_kbE[k - 1][2]);
+        ev = fmaf(s, ev, c_kbE[k - 1][1]);
+        ev = fmaf(s, ev, c_kbE[k - 1][0]);
+        float od = fmaf(s, c_kbO[k - 1][3], c_kbO[k - 1][2]);
+        od = fmaf(s, od, c_kbO[k - 1][1]);
+        od = fmaf(s, od, c_kbO[k - 1][0]);
+        w[3 + k] = fmaf(z, od, ev);
+        w[4 - k] = fmaf(-z, od, ev);
+    }
 }
 
 // ===========================================================================
@@ -182,24 +206,37 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
         S.nh = 0;
         S.logq = 0;
         S.H = 0;
+        S.L = 0.0;
         S.support = 0;
         S.n_out = 0;
         S.cells_per_day = 0.0;
         S.one_minus_a0 = 0.f;
-        S.pad = 0.f;
+        S.whole = 0;
         if (nh <= kSpecMaxHarm) {
             S.one_minus_a0 = (float)(1.0 - s_a[0] * s_inv);
-            const int64_t n_out = (int64_t)nh * (a.m0 + a.mq * (a.n_freq - 1)) + 1;
-            const int lq = spec_logq_of(n_out);
+            int lq;
+            double n_out;
+            if (a.interp) {
+                // period at least 4 T, stretched to fill the transform
+                const double top = fmax((double)nh * a.f_top, 1e-9);
+                const double need = fmin(4.0 * s_T * top + 8.0, 1e9);
+                lq = spec_logq_of((int64_t)need);
+                S.L = ((double)((int64_t)2 << lq) / kSpecOver - 8.0) / top;
+                n_out = floor(top * S.L) + 7.0;
+            } else {
+                n_out = (double)((int64_t)nh * (a.m0 + a.mq * (a.n_freq - 1)) + 1);
+                lq = spec_logq_of((int64_t)n_out);
+                S.L = 1.0 / a.delta;
+            }
             S.logq = lq;
             S.H = (int64_t)2 << lq;
-            S.n_out = (int32_t)n_out;
-            S.cells_per_day = 2.0 * (double)S.H * a.delta;
+            S.cells_per_day = a.interp ? 2.0 * (double)S.H / S.L : 2.0 * (double)S.H * a.delta;
             const double cells = s_T * S.cells_per_day;
             // a curve that the workspace was not sized for, or spread over many periods: the pair sum
-            if (n_out <= a.p_ld && ((int64_t)1 << lq) <= a.x_ld && cells < 64.0 * (double)S.H) {
+            if (n_out + kSpecPad <= (double)a.p_ld && ((int64_t)1 << lq) <= a.x_ld && cells < 64.0 * (double)S.H) {
                 const double sup = ceil(cells) + 6.0;
                 S.nh = nh;
+                S.n_out = (int32_t)n_out;
                 S.support = sup >= (double)S.H ? (int32_t)S.H : min((int32_t)S.H, ((int32_t)sup + 3) & ~3);
             }
         }
@@ -224,6 +261,7 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
 // borrow (rare) goes to the high word.
 // ===========================================================================
 constexpr int kSpreadThreads = 512;
+constexpr float kQuanta = 268435456.0f;          // 2^28 per unit of weight
 
 __device__ __forceinline__ int lower_bound_x(const uint64_t* x, int lo, int hi, uint64_t v)
 {
@@ -266,6 +304,9 @@ __device__ __forceinline__ int item_curve(const int* pre, int nc, int item)
     return lo;
 }
 
+// INTERP: the weights are divided by the interpolation window's transform at the
+// pair's time difference (all differences lie below half of the half period).
+template <bool INTERP>
 __global__ void __launch_bounds__(kSpreadThreads) k_spec_spread(const SpecArgs a, int max_n)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -312,6 +353,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spec_spread(const SpecArgs a
         }
         __syncthreads();
         const float iph = P.ip_hi, ipl = P.ip_lo;
+        const float inv_h = 1.0f / (float)H;
         const uint64_t span = X[n - 1];
         // folded interval of the differences that touch the segment (window half-width 4, half-cell centres)
         const int flo = A - 5 > 0 ? A - 5 : 0, fhi = B + 5 < H ? B + 5 : H;
@@ -366,29 +408,21 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spec_spread(const SpecArgs a
                 const uint64_t u = ((r & 1) ? fold - d : d - fold) - 0x80000000ull;    // cells from the first centre
                 const int l = (int)((int64_t)u >> 32);
                 const float z = (float)(uint32_t)u * 2.3283064365386963e-10f - 0.5f;
-                const float w = ((gauss_g(Y[i], Y[j]) - iph) - ipl) * 268435456.0f;    // 2^28 quanta
-                const float s = z * z, wz = w * z;
-                const int l0 = l - A;
+                float w = ((gauss_g(Y[i], Y[j]) - iph) - ipl) * kQuanta;
+                if (INTERP) w *= kb_inverse(((float)l + (z + 1.0f)) * inv_h);
+                float q[8];
+                kb_weights(z, q);
+                const int l0 = l - 3 - A;
 #pragma unroll
-                for (int k = 1; k <= 4; k++) {
-                    float ev = fmaf(s, c_kbE[k - 1][3], c_kbE[k - 1][2]);
-                    ev = fmaf(s, ev, c_kbE[k - 1][1]);
-                    ev = fmaf(s, ev, c_kbE[k - 1][0]);
-                    float od = fmaf(s, c_kbO[k - 1][3], c_kbO[k - 1][2]);
-                    od = fmaf(s, od, c_kbO[k - 1][1]);
-                    od = fmaf(s, od, c_kbO[k - 1][0]);
-                    const float q = w * ev;
-#pragma unroll
-                    for (int h = 0; h < 2; h++) {
-                        const int v = __float2int_rn(h ? fmaf(-wz, od, q) : fmaf(wz, od, q));
-                        int t = l0 + (h ? 1 - k : k);                   // cell relative to A
-                        if (t + A < 0) t = -1 - (t + A) - A;            // folds at 0 and at half the period
-                        else if (t + A >= H) t = 2 * H - 1 - (t + A) - A;
-                        if ((unsigned)t < (unsigned)(B - A)) {
-                            const uint32_t old = atomicAdd(&cl[t], (uint32_t)v);
-                            const int up = (v >> 31) + (old + (uint32_t)v < old ? 1 : 0);
-                            if (up) atomicAdd(&ch[t], up);
-                        }
+                for (int k = 0; k < 8; k++) {
+                    const int v = __float2int_rn(w * q[k]);
+                    int t = l0 + k;                                  // cell relative to A
+                    if (t + A < 0) t = -1 - (t + A) - A;             // folds at 0 and at half the period
+                    else if (t + A >= H) t = 2 * H - 1 - (t + A) - A;
+                    if ((unsigned)t < (unsigned)(B - A)) {
+                        const uint32_t old = atomicAdd(&cl[t], (uint32_t)v);
+                        const int up = (v >> 31) + (old + (uint32_t)v < old ? 1 : 0);
+                        if (up) atomicAdd(&ch[t], up);
                     }
                 }
             }
@@ -404,7 +438,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spec_spread(const SpecArgs a
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const long long v = ((long long)ch[4 * b + q] << 32) + (long long)cl[4 * b + q] - 0x80000000ll;
-                g[q] = (float)v * 3.7252902984619141e-09f;      // 2^-28
+                g[q] = (float)v * (1.0f / kQuanta);
             }
             const int bb = (A >> 2) + b;
             x[bb] = make_float2(g[0], g[2]);
@@ -630,7 +664,11 @@ __device__ __forceinline__ void spec_emit(const SpecCurve& S, float* P, int m, f
     const float2 cq = make_float2(h * (cm.x - cm.y), -h * (cm.x + cm.y));
     const float2 v2 = cmul(cq, make_float2(d.x, -d.y));
     const int m1 = m, m2 = Q - m, m3 = H - m, m4 = Q + m;
-    if (m1 < S.n_out) P[m1] = v1.x * kb_inverse((float)m1 * inv_h);
+    if (m1 < S.n_out) {
+        const float p = v1.x * kb_inverse((float)m1 * inv_h);
+        P[m1] = p;
+        if (m1 <= 4) P[-m1] = p;                          // the interpolation reads across 0
+    }
     if (m2 < S.n_out) P[m2] = v2.x * kb_inverse((float)m2 * inv_h);
     if (m3 < S.n_out) P[m3] = -v1.y * kb_inverse((float)m3 * inv_h);
     if (m4 < S.n_out) P[m4] = -v2.y * kb_inverse((float)m4 * inv_h);
@@ -689,7 +727,7 @@ __global__ void __launch_bounds__(kFftThreads) k_spec_fft2(const SpecArgs a)
         const int ci = item_curve(s_pre, nc, item);
         const SpecCurve S = a.sc[a.order[a.slot_begin + ci]];
         const float2* x = a.x + (int64_t)ci * a.x_ld;
-        float* P = a.P + (int64_t)ci * a.p_ld;
+        float* P = a.P + (int64_t)ci * a.p_ld + kSpecPad;
         const int blk = item - s_pre[ci];
         switch (S.logq >> 1) {
         case 7: fft2_item<7>(a, S, x, P, blk, sm); break;
@@ -740,7 +778,7 @@ __global__ void __launch_bounds__(kFftThreads) k_spec_fft_one(const SpecArgs a)
     const SpecCurve S = a.sc[a.order[a.slot_begin + ci]];
     if (!S.nh || S.logq > kSpecOneLogQ) return;
     const float2* x = a.x + (int64_t)ci * a.x_ld;
-    float* P = a.P + (int64_t)ci * a.p_ld;
+    float* P = a.P + (int64_t)ci * a.p_ld + kSpecPad;
     switch (S.logq) {
     case 8: fft_one<8>(a, S, x, P, sm); break;
     case 9: fft_one<9>(a, S, x, P, sm); break;
@@ -773,7 +811,7 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_sum(const SpecArgs a)
         const CurveParams& P = a.cp[c];
         if (tid < S.nh) s_a[tid] = a.coef[(int64_t)c * kSpecMaxHarm + tid];
         __syncthreads();
-        const float* Ps = a.P + (int64_t)ci * a.p_ld;
+        const float* Ps = a.P + (int64_t)ci * a.p_ld + kSpecPad;
         const int64_t k0 = (int64_t)(item - s_pre[ci]) * (kSumThreads * kSumPer) + tid;
         int m[kSumPer];
         float s[kSumPer];
@@ -819,15 +857,122 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_sum(const SpecArgs a)
 }
 
 // ===========================================================================
-// k_spec_select: the admissible trial frequencies whose value lies within the
-// rounding of the largest, in ascending order.  The margin, 1e-5 of the largest
-// value plus 1e-6 of the scale of a noise curve, is several times the error of
-// the pair sum and of the spectrum together (both below 2e-6 of the peak), so
-// the pair sum's own best frequency is among them.  A curve with more than
-// kSpecCand such frequencies (a constant curve) is evaluated whole by the pair
-// sum.
+// k_spec_interp: the same at any frequencies (a uniform grid, fine windows, the
+// trial list), each harmonic interpolated from 8 pair-spectrum values.  The
+// position n f L is an integer multiple of the fixed-point f L (32.32).
+// ===========================================================================
+__device__ __forceinline__ int spec_count(const SpecArgs& a, int c)
+{
+    return a.stage == kSpecFine ? a.n_peaks[c] * (2 * a.fine_half + 1) : a.stage == kSpecList ? a.n_trials : (int)a.n_freq;
+}
+
+__global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
+{
+    __shared__ int s_pre[kSpecMaxChunk + 1];
+    __shared__ float s_a[kSpecMaxHarm];
+    __shared__ unsigned int s_key[kSumThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nc = a.slot_end - a.slot_begin;
+    item_prefix(s_pre, nc, [&](int i) {
+        const int c = a.order[a.slot_begin + i];
+        return a.sc[c].nh && !a.sc[c].whole ? (spec_count(a, c) + kSumThreads - 1) / kSumThreads : 0;
+    });
+    for (int item = blockIdx.x; item < s_pre[nc]; item += gridDim.x) {
+        const int ci = item_curve(s_pre, nc, item);
+        const int c = a.order[a.slot_begin + ci];
+        const SpecCurve S = a.sc[c];
+        const CurveParams& P = a.cp[c];
+        if (tid < S.nh) s_a[tid] = a.coef[(int64_t)c * kSpecMaxHarm + tid];
+        __syncthreads();
+        const float* Ps = a.P + (int64_t)ci * a.p_ld + kSpecPad;
+        const int q = (item - s_pre[ci]) * kSumThreads + tid;
+        unsigned int key = 0u;
+        if (q < spec_count(a, c)) {
+            double f;
+            bool ok = true, live = true;          // admissible as the best; evaluated at all
+            if (a.stage == kSpecFine) {
+                const int W = 2 * a.fine_half + 1, pk = q / W;
+                const double fpk = grid_freq(a.f_min, (double)a.peaks[(int64_t)c * a.top_k + pk], a.coarse_df);
+                f = grid_freq(fpk, (double)(q - pk * W - a.fine_half), a.step);
+                live = f >= a.f_min && f <= a.f_max;
+                ok = live && !excluded_f(a.ex, f);
+            } else if (a.stage == kSpecList) {
+                const int k = a.trials[(int64_t)c * a.n_trials + q];
+                live = k >= 0;
+                ok = live && !excluded_k(a.ex.full_k, a.ex.n, k);
+                f = grid_freq(a.f_min, (double)max(k, 0), a.step);
+            } else {
+                f = grid_freq(a.f_min, (double)q, a.step);
+                ok = a.stage == kSpecFull && !excluded_k(a.ex.full_k, a.ex.n, q);
+            }
+            float v = 0.f;
+            if (live) {
+                const uint64_t step = (uint64_t)__double2ll_rn(f * S.L * 4294967296.0);
+                uint64_t pos = 0;
+                float s = 0.f;
+#pragma unroll 2
+                for (int h = 0; h < S.nh; h++) {
+                    pos += step;
+                    float w[8];
+                    kb_weights((float)(uint32_t)pos * 2.3283064365386963e-10f - 0.5f, w);
+                    const float* p = Ps + ((int)(pos >> 32) - 3);
+                    float t = 0.f;
+#pragma unroll
+                    for (int k = 0; k < 8; k++) t = fmaf(w[k], p[k], t);
+                    s = fmaf(s_a[h], t, s);
+                }
+                v = fmaf(2.0f, s, P.diag * S.one_minus_a0) * P.norm;
+            }
+            if (a.stage == kSpecFine && !ok) v = -INFINITY;
+            if (a.stage == kSpecList && !live) v = __int_as_float(0x7fc00000);
+            a.rows[(a.rows_by_curve ? (int64_t)c : (int64_t)ci) * a.row_ld + q] = v;
+            if (ok) key = orderable(v);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
+        if (lane == 0) s_key[warp] = key;
+        __syncthreads();
+        if (tid == 0) {
+#pragma unroll
+            for (int w = 1; w < kSumThreads / 32; w++) key = max(key, s_key[w]);
+            if (key) atomicMax(a.vmax + c, key);
+        }
+        __syncthreads();
+    }
+}
+
+// Margin below which two values of a curve are not told apart by the spectrum:
+// 1e-5 of the largest value plus 1e-6 of the scale of a noise curve, several
+// times the error of the pair sum and of the spectrum together (both below 2e-6
+// of the peak).
+__device__ __forceinline__ float spec_margin(float vmax, const CurveParams& P)
+{
+    return 1e-5f * fabsf(vmax) + 1e-6f * P.norm * (float)P.n;
+}
+
+// ===========================================================================
+// k_spec_select: the admissible entries (grid points, fine candidates, list
+// positions) within the margin of the largest value, in ascending order: the pair
+// sum's own best is among them.  A curve with more than kSpecCand of them (a
+// constant curve), or without a spectrum, is evaluated whole by the pair sum.
 // ===========================================================================
 constexpr int kSelThreads = 256;
+
+// Writes the n entries of s_k (distinct, any order) in ascending order, -1 after them.
+__device__ __forceinline__ void write_sorted(const int32_t* s_k, int n, int32_t* out)
+{
+    const int tid = threadIdx.x;
+    if (tid < kSpecCand) {
+        if (tid >= n) {
+            out[tid] = -1;
+        } else {
+            const int32_t k = s_k[tid];
+            int rank = 0;
+            for (int q = 0; q < n; q++) rank += s_k[q] < k;
+            out[rank] = k;
+        }
+    }
+}
 
 __global__ void __launch_bounds__(kSelThreads) k_spec_select(const SpecArgs a)
 {
@@ -835,42 +980,169 @@ __global__ void __launch_bounds__(kSelThreads) k_spec_select(const SpecArgs a)
     __shared__ int32_t s_k[kSpecCand];
     const int ci = blockIdx.x, tid = threadIdx.x;
     const int c = a.order[a.slot_begin + ci];
-    CurveParams* P = a.cp + c;
+    const CurveParams& P = a.cp[c];
     int32_t* out = a.cand + (int64_t)c * kSpecCand;
     if (tid == 0) s_n = 0;
     __syncthreads();
-    const bool spec = a.sc[c].nh != 0;
+    const bool spec = a.sc[c].nh != 0 && !a.sc[c].whole;
     const unsigned int top = a.vmax[c];
     if (spec && top) {
         const float v0 = from_orderable(top);
-        const float thr = v0 - (1e-5f * fabsf(v0) + 1e-6f * P->norm * (float)P->n);
+        const float thr = v0 - spec_margin(v0, P);
         const float* row = a.rows + (a.rows_by_curve ? (int64_t)c : (int64_t)ci) * a.row_ld;
-        for (int64_t k = tid; k < a.n_freq; k += kSelThreads) {
-            if (row[k] >= thr && !excluded_k(a.ex.full_k, a.ex.n, k)) {
+        const int count = spec_count(a, c);
+        for (int k = tid; k < count; k += kSelThreads) {
+            if (row[k] >= thr) {
+                const int g = a.stage == kSpecList ? a.trials[(int64_t)c * a.n_trials + k] : k;
+                if (a.stage != kSpecFine && excluded_k(a.ex.full_k, a.ex.n, g)) continue;
                 const int pos = atomicAdd(&s_n, 1);
-                if (pos < kSpecCand) s_k[pos] = (int32_t)k;
+                if (pos < kSpecCand) s_k[pos] = k;
             }
         }
     }
     __syncthreads();
     const int n = s_n;
     const bool whole = !spec || n > kSpecCand || (top && n == 0);
-    if (tid < kSpecCand) {
-        if (whole || tid >= n) {
-            out[tid] = -1;
+    write_sorted(s_k, whole ? 0 : n, out);
+    if (tid == 0 && whole) a.fb_slots[atomicAdd(a.fb_count, 1)] = a.slot_begin + ci;
+}
+
+// ===========================================================================
+// k_spec_peaks: the coarse points whose exact values decide the top_k peaks.
+// With m the margin: T = the top_k-th largest value that is a local maximum by
+// more than m (radix select on the value bits); every point that may be a local
+// maximum within m and lies above T - m, and any neighbour within m of it.  The
+// pair sum evaluates them again, and k_spec_rank ranks them from exact values;
+// every other comparison is decided by more than the margin.
+// ===========================================================================
+constexpr int kPeakRaw = 256;
+
+__global__ void __launch_bounds__(kSelThreads) k_spec_peaks(const SpecArgs a)
+{
+    __shared__ unsigned int s_hist[256], s_prefix, s_need;
+    __shared__ float s_max[kSelThreads / 32];
+    __shared__ int s_n, s_m;
+    __shared__ int32_t s_raw[kPeakRaw], s_k[kSpecCand];
+    const int ci = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c = a.order[a.slot_begin + ci];
+    const CurveParams& P = a.cp[c];
+    int32_t* out = a.cand + (int64_t)c * kSpecCand;
+    const int K = (int)a.n_freq;
+    const float* v = a.rows + (int64_t)c * a.row_ld;
+    if (a.sc[c].nh == 0) {
+        if (tid < kSpecCand) out[tid] = -1;
+        if (tid == 0) {
+            a.n_peaks[c] = 0;
+            a.fb_slots[atomicAdd(a.fb_count, 1)] = a.slot_begin + ci;
         }
-        __syncwarp();
-        if (!whole && tid < n) {
-            const int32_t k = s_k[tid];
-            int rank = 0;
-            for (int q = 0; q < n; q++) rank += s_k[q] < k;
-            out[rank] = k;
-        }
+        return;
     }
+    float vm = 0.f;
+    for (int k = tid; k < K; k += kSelThreads) vm = fmaxf(vm, fabsf(v[k]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) vm = fmaxf(vm, __shfl_xor_sync(0xffffffffu, vm, o));
+    if (lane == 0) s_max[warp] = vm;
     if (tid == 0) {
-        P->by_list = whole ? 0 : 1;
-        if (whole) a.fb_slots[atomicAdd(a.fb_count, 1)] = a.slot_begin + ci;
+        s_n = 0;
+        s_m = 0;
+        s_prefix = 0u;
+        s_need = (unsigned)a.top_k;
     }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kSelThreads / 32; w++) vm = fmaxf(vm, s_max[w]);
+    const float m = spec_margin(vm, P);
+    auto sure = [&](int k) {
+        const float x = v[k];
+        return (k == 0 || x > v[k - 1] + m) && (k == K - 1 || x > v[k + 1] + m) && !excluded_k(a.ex.coarse_k, a.ex.n, k);
+    };
+    // the value of the top_k-th sure maximum (none so far down: every possible maximum counts)
+    bool enough = true;
+    for (int pass = 0; pass < 4 && enough; pass++) {
+        const int shift = 24 - 8 * pass;
+        for (int i = tid; i < 256; i += kSelThreads) s_hist[i] = 0u;
+        __syncthreads();
+        const unsigned int prefix = s_prefix, need = s_need;
+        for (int k = tid; k < K; k += kSelThreads) {
+            const unsigned int u = orderable(v[k]);
+            if ((pass == 0 || (u >> (shift + 8)) == prefix) && sure(k)) atomicAdd(&s_hist[(u >> shift) & 255u], 1u);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            unsigned int cum = 0;
+            int d = 255;
+            for (; d >= 0; d--) {
+                if (cum + s_hist[d] >= need) break;
+                cum += s_hist[d];
+            }
+            if (d < 0) s_need = 0u;                      // fewer than top_k (first pass only)
+            else {
+                s_prefix = (prefix << 8) | (unsigned)d;
+                s_need = need - cum;
+            }
+        }
+        __syncthreads();
+        enough = s_need != 0u;
+    }
+    const float floor_v = enough ? from_orderable(s_prefix) - m : -INFINITY;
+    for (int k = tid; k < K; k += kSelThreads) {
+        const float x = v[k];
+        if (!(x >= floor_v) || excluded_k(a.ex.coarse_k, a.ex.n, k)) continue;
+        const float l = k > 0 ? v[k - 1] : -INFINITY, h = k < K - 1 ? v[k + 1] : -INFINITY;
+        if (x >= l - m && x >= h - m) {
+            const int add = 1 + (x - l <= m ? 1 : 0) + (x - h <= m ? 1 : 0);
+            int pos = atomicAdd(&s_n, add);
+            if (pos + add <= kPeakRaw) {
+                s_raw[pos++] = k;
+                if (x - l <= m) s_raw[pos++] = k - 1;
+                if (x - h <= m) s_raw[pos++] = k + 1;
+            }
+        }
+    }
+    __syncthreads();
+    const int raw = s_n;
+    if (raw <= kPeakRaw && tid < raw) {                  // distinct entries: the first of equal ones stays
+        const int32_t k = s_raw[tid];
+        bool first = true;
+        for (int q = 0; q < tid; q++) first = first && s_raw[q] != k;
+        if (first) {
+            const int pos = atomicAdd(&s_m, 1);
+            if (pos < kSpecCand) s_k[pos] = k;
+        }
+    }
+    __syncthreads();
+    const bool whole = raw > kPeakRaw || s_m > kSpecCand || !(vm < INFINITY);
+    write_sorted(s_k, whole ? 0 : s_m, out);
+    if (tid == 0 && whole) {
+        a.sc[c].whole = 1;
+        a.fb_slots[atomicAdd(a.fb_count, 1)] = a.slot_begin + ci;
+    }
+}
+
+// k_spec_rank: the peaks of a curve from its candidates' exact values (the rule
+// and order of k_topk).  One CTA of kSpecCand threads per curve.
+__global__ void __launch_bounds__(kSpecCand) k_spec_rank(const SpecArgs a)
+{
+    __shared__ unsigned long long s_key[kSpecCand];
+    const int tid = threadIdx.x;
+    const int c = a.order[a.slot_begin + blockIdx.x];
+    const float* v = a.rows + (int64_t)c * a.row_ld;
+    const int K = (int)a.n_freq;
+    const int k = a.cand[(int64_t)c * kSpecCand + tid];
+    unsigned long long key = 0ull;
+    if (k >= 0) {
+        const float x = v[k];
+        if ((k == 0 || x > v[k - 1]) && (k == K - 1 || x >= v[k + 1]) && !excluded_k(a.ex.coarse_k, a.ex.n, k))
+            key = make_key(x, (uint32_t)k);
+    }
+    s_key[tid] = key;
+    const int found = __syncthreads_count(key != 0ull);
+    if (key) {
+        int rank = 0;
+        for (int q = 0; q < kSpecCand; q++) rank += s_key[q] > key;
+        if (rank < a.top_k) a.peaks_out[(int64_t)c * a.top_k + rank] = k;
+    }
+    if (tid == 0) a.n_peaks[c] = min(found, a.top_k);
 }
 
 // ---------------------------------------------------------------------------
@@ -899,7 +1171,8 @@ size_t spec_spread_smem(int max_n, int seg)
 cudaError_t spec_prepare(int np2max, int max_n, int seg)
 {
     cudaError_t e = raise_dyn_smem((const void*)k_spec_prep, prep_smem(np2max));
-    if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_spread, spec_spread_smem(max_n, seg));
+    if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_spread<false>, spec_spread_smem(max_n, seg));
+    if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_spread<true>, spec_spread_smem(max_n, seg));
     if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_fft1, fft_smem());
     if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_fft2, fft_smem());
     if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_fft_one, fft_smem());
@@ -914,12 +1187,14 @@ cudaError_t launch_spec_prep(const SpecArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_spec_chunk(const SpecArgs& a, int n_sm, int max_n, bool one_pass, bool two_pass, cudaStream_t s)
+cudaError_t launch_spec_transform(const SpecArgs& a, int n_sm, int max_n, bool one_pass, bool two_pass, cudaStream_t s)
 {
     const int n = a.slot_end - a.slot_begin;
     if (n <= 0) return cudaSuccess;
     if (n > kSpecMaxChunk) return cudaErrorInvalidValue;
-    k_spec_spread<<<2 * n_sm, kSpreadThreads, spec_spread_smem(max_n, a.seg), s>>>(a, max_n);
+    const size_t smem = spec_spread_smem(max_n, a.seg);
+    if (a.interp) k_spec_spread<true><<<2 * n_sm, kSpreadThreads, smem, s>>>(a, max_n);
+    else k_spec_spread<false><<<2 * n_sm, kSpreadThreads, smem, s>>>(a, max_n);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && two_pass) {
         k_spec_fft1<<<2 * n_sm, kFftThreads, fft_smem(), s>>>(a);
@@ -933,11 +1208,31 @@ cudaError_t launch_spec_chunk(const SpecArgs& a, int n_sm, int max_n, bool one_p
         k_spec_fft_one<<<n, kFftThreads, fft_smem(), s>>>(a);
         e = cudaGetLastError();
     }
-    if (e != cudaSuccess) return e;
-    k_spec_sum<<<8 * n_sm, kSumThreads, 0, s>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_spec_select<<<n, kSelThreads, 0, s>>>(a);
+    return e;
+}
+
+cudaError_t launch_spec_values(const SpecArgs& a, int n_sm, cudaStream_t s)
+{
+    if (a.interp) k_spec_interp<<<8 * n_sm, kSumThreads, 0, s>>>(a);
+    else k_spec_sum<<<8 * n_sm, kSumThreads, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_spec_select(const SpecArgs& a, cudaStream_t s)
+{
+    k_spec_select<<<a.slot_end - a.slot_begin, kSelThreads, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_spec_peaks(const SpecArgs& a, cudaStream_t s)
+{
+    k_spec_peaks<<<a.slot_end - a.slot_begin, kSelThreads, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_spec_rank(const SpecArgs& a, cudaStream_t s)
+{
+    k_spec_rank<<<a.slot_end - a.slot_begin, kSpecCand, 0, s>>>(a);
     return cudaGetLastError();
 }
 

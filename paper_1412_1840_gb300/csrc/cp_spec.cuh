@@ -21,16 +21,22 @@ constexpr int kSpecMaxChunk = 64;      // curves per chunk
 constexpr double kSpecTail = 2e-8;     // harmonics left out: at most this much of the kernel's peak
 constexpr double kSpecOver = 1.1;      // transform length over the highest frequency needed, at least
 
+constexpr int kSpecPad = 8;            // pair-spectrum values kept before index 0 (P(-nu) = P(nu))
+
+// Which frequencies a launch evaluates.
+enum SpecStage : int { kSpecFull = 0, kSpecCoarse = 1, kSpecFine = 2, kSpecList = 3 };
+
 // What the device decides for one curve (its sigma_t and span are known there).
 struct SpecCurve {
     double cells_per_day;   // 2 H / L: grid cells per day of time difference
+    double L;               // transform period in days: the pair spectrum's spacing is 1 / L
     int64_t H;              // cells of the half period, 2 Q
-    int32_t nh;             // harmonics
+    int32_t nh;             // harmonics (0: the pair sum evaluates the curve)
     int32_t logq;           // Q = 2^logq
     int32_t support;        // cells that can be non-zero, a multiple of 4 (H: all)
     int32_t n_out;          // pair-spectrum values needed
     float one_minus_a0;
-    float pad;
+    int32_t whole;          // set when a curve's candidates do not fit its list
 };
 
 struct SpecArgs {
@@ -42,25 +48,37 @@ struct SpecArgs {
     const float* yp;              // scaled magnitudes, caller's order
     uint64_t* xs;                 // sorted times in cells, 32.32 fixed point
     float* ys;                    // scaled magnitudes in time order
-    double delta;                 // spacing of the pair spectrum (1/day): frequencies are (m0 + mq k) delta
+    int stage;                    // SpecStage
+    int interp;                   // 0: frequencies (m0 + mq k) delta are entries of the pair spectrum
+                                  // 1: any frequency up to f_top, by interpolation
+    double delta;
     int64_t m0, mq;
-    int64_t n_freq;
+    double f_top;
+    int64_t n_freq;               // points of the row (full, coarse), of the grid (list)
+    double f_min, f_max, step;    // uniform grid of the stage (fine: step of the window)
+    double coarse_df;
+    const int32_t* peaks;         // coarse peaks (peaks_out: where k_spec_rank writes them)
+    int32_t* peaks_out;
+    int32_t* n_peaks;
+    int32_t top_k, fine_half;
+    const int32_t* trials;
+    int32_t n_trials;
     int slot_begin, slot_end;     // curves of this launch
     int np2max;
     int seg;                      // cells per spreading item
     float2* x;                    // chunk workspace: transform data, x_ld per curve
     int64_t x_ld;
-    float* P;                     // pair spectrum, p_ld per curve
+    float* P;                     // pair spectrum, p_ld per curve (index 0 at kSpecPad)
     int64_t p_ld;
-    float* rows;                  // periodogram rows: row index = caller's curve, or slot - slot_begin
+    float* rows;                  // values: row index = caller's curve, or slot - slot_begin
     int64_t row_ld;
     int rows_by_curve;
     unsigned int* vmax;           // [n_curves] largest admissible value (orderable bits)
-    int32_t* cand;                // [n_curves * kSpecCand] grid indices, -1 = none
-    int32_t* fb_slots;            // slots whose candidates do not fit
+    int32_t* cand;                // [n_curves * kSpecCand] candidate entries, -1 after the last
+    int32_t* fb_slots;            // slots that the pair sum evaluates whole
     int* fb_count;
     unsigned long long* queue;    // spreading items
-    const float2* tw;             // exp(-2 pi i k / 8192), k < 8192
+    const float2* tw;             // twiddle factors, see launch_spec_twiddle
     Exclusion ex;
 };
 
@@ -69,8 +87,12 @@ cudaError_t launch_spec_twiddle(float2* tw, cudaStream_t s);   // fills kSpecTwi
 cudaError_t spec_prepare(int np2max, int max_n, int seg);
 size_t spec_spread_smem(int max_n, int seg);
 cudaError_t launch_spec_prep(const SpecArgs& a, cudaStream_t s);
-// spread, transform, harmonic sums, candidates of one chunk (slot_end - slot_begin <= kSpecMaxChunk)
-cudaError_t launch_spec_chunk(const SpecArgs& a, int n_sm, int max_n, bool one_pass, bool two_pass, cudaStream_t s);
+// pair spectrum of one chunk (slot_end - slot_begin <= kSpecMaxChunk)
+cudaError_t launch_spec_transform(const SpecArgs& a, int n_sm, int max_n, bool one_pass, bool two_pass, cudaStream_t s);
+cudaError_t launch_spec_values(const SpecArgs& a, int n_sm, cudaStream_t s);   // the stage's values and their largest
+cudaError_t launch_spec_select(const SpecArgs& a, cudaStream_t s);             // candidates for the best
+cudaError_t launch_spec_peaks(const SpecArgs& a, cudaStream_t s);              // coarse points whose exact values matter
+cudaError_t launch_spec_rank(const SpecArgs& a, cudaStream_t s);               // the coarse peaks, from exact values
 
 // Host: harmonics needed at sigma_t for a truncation tail of kSpecTail (0: more than kSpecMaxHarm).
 int spec_harmonics(double sigma_t);

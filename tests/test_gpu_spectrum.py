@@ -2,9 +2,10 @@
 FP64 oracle at the direct form's bar (1e-5 of the curve's peak), at the edges of
 its ranges: one- and two-pass transforms, time differences beyond half of the
 transform's period (df T > 1/2), grids that start at 0, between or off the
-multiples of df, equal and unordered times, sigma_t at both ends, curves that
-the pair sum evaluates whole.  The best frequency is the pair sum's own: it
-equals cp_best_period_noalloc's (pair sum at every frequency) bit for bit."""
+multiples of df (interpolated), equal and unordered times, sigma_t at both ends,
+curves that the pair sum evaluates whole.  The best frequency, of the uniform
+grid and of the coarse-then-fine search, is the pair sum's own: it equals
+cp_best_period_noalloc's (pair sum at every frequency) bit for bit."""
 import numpy as np
 import pytest
 
@@ -55,12 +56,16 @@ def run(b, g, **kw):
 
 CASES = [
     # curves, N, span, f_min, df, K, sigma_t
-    (96, 60, 90, 40.0, 0.0, 4e-3, 1200, 0.5),        # one pass, grid from 0
-    (24, 100, 300, 1500.0, 0.01, 1e-3, 2001, 0.3),   # differences folded: df T = 1.5
-    (8, 150, 400, 1500.0, 0.01, 1e-3, 3000, 0.1),    # smallest sigma_t, two passes
-    (8, 150, 400, 900.0, 5e-4, 1e-3, 3001, 0.62),    # f_min = df / 2
+    (192, 60, 90, 40.0, 0.0, 4e-3, 2400, 0.5),        # one pass, grid from 0
+    (48, 100, 300, 1500.0, 0.01, 1e-3, 2001, 0.3),   # differences folded: df T = 1.5
+    (12, 150, 400, 1500.0, 0.01, 1e-3, 4000, 0.1),    # smallest sigma_t, two passes
+    (12, 150, 400, 900.0, 5e-4, 1e-3, 4001, 0.62),    # f_min = df / 2
     (6, 300, 420, 5000.0, 0.0025, 2e-4, 9001, 1.5),  # two harmonics or so, f_min = 12.5 df
     (3, 1500, 2100, 2500.0, 0.002, 1e-4, 700, 0.25),
+    # off the multiples of df: interpolated
+    (64, 60, 130, 700.0, 0.00143, 1e-3, 3500, 0.5),
+    (6, 200, 400, 1733.0, 1.0 / 1733.0, 1e-4, 6000, 0.1),
+    (6, 300, 400, 5000.0, 0.0123457, 1e-3, 5000, 0.3),   # longer than the spectra are made for
 ]
 
 
@@ -82,19 +87,45 @@ def test_spectrum_matches_oracle(case, form):
     np.testing.assert_array_equal(best["best_stat"], rows.max(axis=1))
 
 
-@pytest.mark.parametrize("integer", [False, True])
-def test_best_frequency_is_the_pair_sums(integer):
-    b = batch(40, 60, 400, 1500.0, seed=12, integer=integer)
-    g = synth.Grid(0.01, 1e-3, 2000)
-    _, best, _, info = run(b, g, sigma_t=0.3)
-    assert info["launches_per_search"] > PLAIN
+def via_noalloc(b, g, sigma_t):
     dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (b.times, b.mags, b.errs)]
     n = b.n_curves
     out = (torch.zeros(n, dtype=torch.int64, device="cuda"), torch.zeros(n, dtype=torch.float64, device="cuda"),
            torch.zeros(n, dtype=torch.float32, device="cuda"), torch.zeros(n, dtype=torch.uint8, device="cuda"))
-    cp.cp_best_period_noalloc(*dev, b.offsets, cp.grid_from(g), 0.3, *out)
-    for got, name in zip(out, ("best_idx", "best_freq", "best_stat", "is_periodic")):
-        np.testing.assert_array_equal(got.cpu().numpy().astype(best[name].dtype), best[name])
+    cp.cp_best_period_noalloc(*dev, b.offsets, cp.grid_from(g), sigma_t, *out)
+    return dict(zip(("best_idx", "best_freq", "best_stat", "is_periodic"), (o.cpu().numpy() for o in out)))
+
+
+def same(got, want):
+    for k in want:
+        np.testing.assert_array_equal(got[k].astype(want[k].dtype), want[k], err_msg=k)
+
+
+@pytest.mark.parametrize("f_min", [0.01, 0.00977])
+@pytest.mark.parametrize("integer", [False, True])
+def test_best_frequency_is_the_pair_sums(integer, f_min):
+    b = batch(40, 60, 400, 1500.0, seed=12, integer=integer)
+    g = synth.Grid(f_min, 1e-3, 2000)
+    _, best, _, info = run(b, g, sigma_t=0.3)
+    assert info["launches_per_search"] > PLAIN
+    same(best, via_noalloc(b, g, 0.3))
+
+
+# coarse_df T from 0.5 to 4, one peak to 40 (the most that goes through the spectrum), windows that
+# overlap and that leave the band
+@pytest.mark.parametrize("span,coarse_df,top_k,half,sigma_t", [(500.0, 1e-3, 10, 2e-3, 0.45), (2500.0, 1e-3, 1, 2e-3, 0.3),
+                                                               (2500.0, 1.6e-3, 40, 1e-3, 0.25), (1733.0, 7e-4, 5, 5e-3, 0.12)])
+@pytest.mark.parametrize("integer", [False, True])
+def test_coarse_fine_is_the_pair_sums(span, coarse_df, top_k, half, sigma_t, integer):
+    b = batch(64, 150, 300, span, seed=14, integer=integer)
+    g = synth.Grid(0.0041, 1e-4, 14501, hierarchical=True, coarse_df=coarse_df, top_k=top_k, fine_df=1.3e-5,
+                   fine_halfwidth=half)
+    dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (b.times, b.mags, b.errs)]
+    with cp.Plan(*dev, b.offsets, cp.grid_from(g), sigma_t=sigma_t) as p:
+        best = p.best_period()
+        assert p.info()["launches_per_search"] > 7
+        same(p.best_period(), best)
+    same(best, via_noalloc(b, g, sigma_t))
 
 
 def test_curves_outside_the_spectrums_range():
