@@ -80,8 +80,9 @@ struct SpecPlan {
     double delta = 0, f_top = 0;
     int min_logq = 0, max_logq = 0;    // transform lengths that can occur
     int64_t p_ld = 0, row = 0;         // floats per curve: pair spectrum, values
+    int64_t points = 0;                // most values of one launch per curve
     int chunk = 0, chunks = 0;         // curves per chunk; chunks of all waves
-    int seg = 0;                       // cells per spreading item
+    int seg_items = 1;                 // spreading items per curve wanted
 };
 
 }  // namespace
@@ -131,13 +132,16 @@ struct cp_plan_s {
     // direct-form curves through the pair spectrum (cp_spec.cu)
     SpecPlan sfull, ssearch;           // the uniform grid; the coarse-then-fine or bands search
     int spec_fc_min = kFcMax;
+    int spec_seg_max = 0;
+    bool keep_w = true;                // some pass of the direct-form curves reads W tiles
     bool spec() const { return sfull.on || ssearch.on; }
     SpecCurve* d_sc = nullptr;
     float* d_scoef = nullptr;
     uint64_t* d_sxs = nullptr;
     float *d_sys = nullptr, *d_sP = nullptr, *d_srow = nullptr;
+    void* d_spart = nullptr;
     float2 *d_sx = nullptr, *d_tw = nullptr;
-    unsigned int* d_svmax = nullptr;
+    unsigned int *d_svmax = nullptr, *d_svblk = nullptr;
     int32_t *d_scand = nullptr, *d_sfb = nullptr;
 
     // device buffers
@@ -535,7 +539,7 @@ TopkArgs topk_args(cp_plan_t p, int w, const int* fb_count = nullptr, const int3
     return t;
 }
 
-cp_status enqueue_wave_w(cp_plan_t p, int w, cudaStream_t s)
+cp_status enqueue_wave_w(cp_plan_t p, int w, bool spectrum, cudaStream_t s)
 {
     const Wave& wv = p->waves[w];
     if (wv.cls != 0) {
@@ -554,6 +558,7 @@ cp_status enqueue_wave_w(cp_plan_t p, int w, cudaStream_t s)
         CP_CUDA(launch_build_w16(b, s));
         return CP_OK;
     }
+    if (spectrum) return CP_OK;      // the pass takes w from the magnitudes
     BuildWArgs b{};
     b.cp = p->d_cp;
     b.order = p->d_order;
@@ -665,12 +670,15 @@ SpecArgs spec_args(cp_plan_t p, const SpecPlan& sp, const PairArgs& base)
     a.trials = p->d_trials;
     a.n_trials = p->n_trials;
     a.np2max = p->np2max;
-    a.seg = sp.seg;
+    a.seg_max = p->spec_seg_max;
+    a.seg_items = sp.seg_items;
     a.x = p->d_sx;
     a.x_ld = (int64_t)1 << sp.max_logq;
     a.P = p->d_sP;
     a.p_ld = sp.p_ld;
     a.vmax = p->d_svmax;
+    a.vblk = p->d_svblk;
+    a.vb_ld = (sp.points + kSpecBlock - 1) / kSpecBlock;
     a.cand = p->d_scand;
     a.fb_slots = p->d_sfb;
     a.tw = p->d_tw;
@@ -678,18 +686,7 @@ SpecArgs spec_args(cp_plan_t p, const SpecPlan& sp, const PairArgs& base)
     return a;
 }
 
-// Units over candidate entries, or over whole curves of a fallback list.
-PairArgs over_candidates(cp_plan_t p, PairArgs l, int kind, int n_slots)
-{
-    l.candidates = kind;
-    l.cand = p->d_scand;
-    l.n_cand = kSpecCand;
-    l.upc = (kSpecCand + p->spec_fc_min - 1) / p->spec_fc_min;
-    l.unit_begin = 0;
-    l.unit_end = l.upc * n_slots;
-    return l;
-}
-
+// Units over whole curves of a fallback list.
 PairArgs over_fallback(cp_plan_t p, PairArgs f, const int* count, const int32_t* slots, int64_t points, int64_t times)
 {
     f.upc = (points + p->spec_fc_min - 1) / p->spec_fc_min * times;
@@ -707,7 +704,6 @@ PairArgs over_fallback(cp_plan_t p, PairArgs f, const int* count, const int32_t*
 cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float* out, cudaStream_t s, int* ev_idx)
 {
     const Wave& wv = p->waves[w];
-    const int n_slots = wv.slot_end - wv.slot_begin;
     const bool hier = stage == kStageCoarse;
     if (ev_idx) {
         CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx)], s, rec_flags(p)));
@@ -716,11 +712,9 @@ cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float*
     int chunk0 = 0;      // chunks of the waves before this one
     for (int v = 0; v < w; v++)
         if (p->waves[v].cls == 0) chunk0 += (p->waves[v].slot_end - p->waves[v].slot_begin + sp.chunk - 1) / sp.chunk;
-    // work counters: spreading items per chunk; per wave the coarse candidates of every chunk use
-    // the chunk's second counter, then two fallback counts
+    // work counters: spreading items per chunk, then two fallback counts per wave
     unsigned long long* q0 = queue_word(p, kQueuesPerWave * (int)p->waves.size());
-    unsigned long long* qc = q0 + sp.chunks;
-    int* fb = reinterpret_cast<int*>(q0 + 2 * sp.chunks + w);          // [0] whole curves, [1] coarse rows
+    int* fb = reinterpret_cast<int*>(q0 + sp.chunks + w);              // [0] whole curves, [1] coarse rows
     int32_t* fb_whole = p->d_sfb;
     int32_t* fb_coarse = p->d_sfb + p->n_curves;
 
@@ -743,6 +737,16 @@ cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float*
     }
     CP_CUDA(launch_spec_prep(a, s));
     const PairArgs fine = hier ? pair_args(p, kStageFine, w, nullptr) : base;
+    cp_status st = CP_OK;
+    auto confirm = [&](PairArgs l, int kind) {
+        l.candidates = kind;
+        l.cand = p->d_scand;
+        l.n_cand = kSpecCand;
+        l.slot_begin = a.slot_begin;
+        l.slot_end = a.slot_end;
+        CP_CUDA(launch_confirm(l, p->d_spart, (int64_t)(confirm_bytes(p->max_n) / sizeof(f2)), p->n_sm, p->max_n, s));
+        return CP_OK;
+    };
     for (int b = wv.slot_begin, k = chunk0; b < wv.slot_end; b += sp.chunk, k++) {
         a.slot_begin = b;
         a.slot_end = std::min(b + sp.chunk, wv.slot_end);
@@ -755,11 +759,7 @@ cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float*
             pk.fb_slots = fb_coarse;
             pk.fb_count = fb + 1;
             CP_CUDA(launch_spec_peaks(pk, s));
-            PairArgs l = over_candidates(p, base, kCandCoarse, a.slot_end - a.slot_begin);
-            l.slot_begin = a.slot_begin;
-            l.slot_end = a.slot_end;
-            l.queue = qc + k;
-            CP_CUDA(launch_pair_direct(l, p->pair_grid, p->pair_smem, s));
+            if ((st = confirm(base, kCandCoarse)) != CP_OK) return st;
             CP_CUDA(launch_spec_rank(a, s));
             sel.stage = kSpecFine;
             sel.step = p->grid.fine_df;
@@ -771,19 +771,16 @@ cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float*
         sel.fb_slots = fb_whole;
         sel.fb_count = fb;
         CP_CUDA(launch_spec_select(sel, s));
+        if ((st = confirm(fine, hier ? kCandFine : stage == kStageList ? kCandTrial : kCandGrid)) != CP_OK) return st;
     }
-    const int kind = hier ? kCandFine : stage == kStageList ? kCandTrial : kCandGrid;
-    PairArgs l = over_candidates(p, fine, kind, n_slots);
-    l.queue = queue_word(p, kQueuesPerWave * w + (stage == kStageList ? kStageFull : kStageList));
-    CP_CUDA(launch_pair_direct(l, p->pair_grid, p->pair_smem, s));
+    const size_t smem = p->pair_smem + (size_t)p->max_n * sizeof(float) + kTile * sizeof(float);
     if (hier) {
-        CP_CUDA(launch_pair_direct(over_fallback(p, base, fb + 1, fb_coarse, p->kc, 1), p->pair_grid, p->pair_smem, s));
+        CP_CUDA(launch_pair_direct(over_fallback(p, base, fb + 1, fb_coarse, p->kc, 1), p->n_sm, smem, s));
         CP_CUDA(launch_topk(topk_args(p, w, fb + 1, fb_coarse), s));
-        CP_CUDA(launch_pair_direct(over_fallback(p, fine, fb, fb_whole, 2 * p->J + 1, p->grid.top_k), p->pair_grid,
-                                   p->pair_smem, s));
+        CP_CUDA(launch_pair_direct(over_fallback(p, fine, fb, fb_whole, 2 * p->J + 1, p->grid.top_k), p->n_sm, smem, s));
     } else {
         CP_CUDA(launch_pair_direct(over_fallback(p, base, fb, fb_whole, stage == kStageList ? p->n_trials : p->grid.n_freq, 1),
-                                   p->pair_grid, p->pair_smem, s));
+                                   p->n_sm, smem, s));
     }
     if (ev_idx) {
         CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx) + 1], s, rec_flags(p)));
@@ -838,7 +835,8 @@ cp_status enqueue_search(cp_plan_t p, cudaStream_t s)
     }
     int ev = 0;
     for (int w = 0; w < (int)p->waves.size(); w++) {
-        if ((st = enqueue_wave_w(p, w, s)) != CP_OK) return st;
+        if ((st = enqueue_wave_w(p, w, p->grid.hierarchical == CP_SEARCH_FULL ? p->sfull.on : p->ssearch.on, s)) != CP_OK)
+            return st;
         if (p->bands) {
             if ((st = enqueue_values(p, kStageList, w, nullptr, s, &ev)) != CP_OK) return st;
         } else if (!p->grid.hierarchical) {
@@ -928,9 +926,9 @@ cp_status read_timings(cp_plan_t p)
 // Workspace of the pair spectrum per plan.  A chunk's transforms pass through the
 // L2 cache better the fewer there are, and the allocation costs the plan time.
 constexpr size_t kSpecWorkspace = (size_t)1 << 30;
-size_t spec_bytes(const SpecPlan& sp, int logq)
+size_t spec_bytes(const SpecPlan& sp, int logq, int max_n)
 {
-    return (sizeof(float2) << logq) + (size_t)(sp.p_ld + sp.row) * sizeof(float) + 1024;
+    return (sizeof(float2) << logq) + (size_t)(sp.p_ld + sp.row) * sizeof(float) + confirm_bytes(max_n) + 1024;
 }
 
 // Whether one kind of pass of the direct-form curves goes through the pair
@@ -988,7 +986,8 @@ void plan_spec(cp_plan_t p, SpecPlan& sp, const float* st_per_curve, double poin
         if (w.cls == 0) largest = std::max<int64_t>(largest, w.slot_end - w.slot_begin);
     sp.p_ld = (int64_t)(std::ldexp(2.0, hi) / kSpecOver) + 2 * kSpecPad;
     sp.row = row;
-    const size_t per = spec_bytes(sp, hi);
+    sp.points = (int64_t)points;       // an upper bound: the coarse and the fine points together
+    const size_t per = spec_bytes(sp, hi, p->max_n);
     if (budget && budget < per) return;
     if (!budget) budget = std::max(kSpecWorkspace, per);
     sp.on = true;
@@ -997,13 +996,11 @@ void plan_spec(cp_plan_t p, SpecPlan& sp, const float* st_per_curve, double poin
     sp.chunk = (int)std::min<int64_t>({largest, (int64_t)(budget / per), (int64_t)kSpecMaxChunk});
     for (const Wave& w : p->waves)
         if (w.cls == 0) sp.chunks += (w.slot_end - w.slot_begin + sp.chunk - 1) / sp.chunk;
-    // cells per spreading item: about four items per SM for a chunk, between 512 and 8192
-    const int ul = spec_logq(n_out(usual_nh, l_usual));
-    const double cells = std::ldexp(2.0, ul ? std::min(hi, ul) : hi) * 0.5 * (double)sp.chunk;
-    sp.seg = 512;
-    while (sp.seg < 8192 && cells / (double)(2 * sp.seg) > 4.0 * (double)p->n_sm) sp.seg *= 2;
+    sp.seg_items = (4 * p->n_sm + sp.chunk - 1) / sp.chunk;   // about four spreading items per SM and chunk
     p->spec_fc_min = fc_min;
 }
+
+constexpr int kSpecMaxPeaks = 20;      // coarse peaks whose candidates still fit a list
 
 void plan_spectra(cp_plan_t p, const float* st_per_curve)
 {
@@ -1029,7 +1026,7 @@ void plan_spectra(cp_plan_t p, const float* st_per_curve)
         sp.interp = true;
         sp.f_top = (g.f_min + (double)(p->kc - 1) * g.coarse_df) * (1.0 + 1e-9);
         sp.f_top = std::max(sp.f_top, full.f_top);
-        if (g.top_k <= 40 && fine <= (int64_t)1 << 20 && p->kc < (int64_t)1 << 30)
+        if (g.top_k <= kSpecMaxPeaks && fine <= (int64_t)1 << 20 && p->kc < (int64_t)1 << 30)
             plan_spec(p, sp, st_per_curve, (double)(p->kc + fine), fine, 0,
                       [&](int f) { return (p->kc + f - 1) / f + g.top_k * ((W + f - 1) / f); });
         p->ssearch = sp;
@@ -1041,7 +1038,7 @@ void plan_spectra(cp_plan_t p, const float* st_per_curve)
                   [&](int f) { return (int64_t)(p->n_trials + f - 1) / f; });
         p->ssearch = sp;
     }
-    if (p->ssearch.on) ws = (size_t)p->ssearch.chunk * spec_bytes(p->ssearch, p->ssearch.max_logq);
+    if (p->ssearch.on) ws = (size_t)p->ssearch.chunk * spec_bytes(p->ssearch, p->ssearch.max_logq, p->max_n);
     if (g.n_freq < (int64_t)1 << 30 && (g.hierarchical == CP_SEARCH_FULL || ws))
         plan_spec(p, full, st_per_curve, (double)g.n_freq, g.n_freq, ws, [&](int f) { return (g.n_freq + f - 1) / f; });
     p->sfull = full;
@@ -1384,17 +1381,24 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         close_wave(sb, (int)n_curves);
     }
 
+    p->spec_seg_max = spec_seg_max(p->max_n);
     plan_spectra(p, opt.sigma_t_per_curve);
     const bool spec = p->spec();
+    // magnitude-kernel tiles of the direct-form curves: only for passes that go through the pair sum
+    p->keep_w = !p->sfull.on || (g.hierarchical != CP_SEARCH_FULL && !p->ssearch.on);
+    if (!p->keep_w) max_tiles32 = 0;
     const int spec_chunks = std::max(p->sfull.chunks, p->ssearch.chunks);
     auto largest = [&](auto per) { return std::max(p->sfull.on ? per(p->sfull) : 0, p->ssearch.on ? per(p->ssearch) : 0); };
     const size_t sx_bytes = largest([](const SpecPlan& q) { return ((size_t)q.chunk << q.max_logq) * sizeof(float2); });
     const size_t sp_bytes = largest([](const SpecPlan& q) { return (size_t)q.chunk * q.p_ld * sizeof(float); });
+    const size_t svblk_bytes = largest([](const SpecPlan& q) {
+        return (size_t)q.chunk * ((q.points + kSpecBlock - 1) / kSpecBlock) * sizeof(unsigned int);
+    });
     const size_t srow_bytes = largest([](const SpecPlan& q) { return (size_t)q.chunk * q.row * sizeof(float); });
 
     // device allocation (one block)
     const int64_t np = p->n_points, nc = n_curves;
-    const int nq = kQueuesPerWave * (int)p->waves.size() + (spec ? 2 * spec_chunks + (int)p->waves.size() : 0);
+    const int nq = kQueuesPerWave * (int)p->waves.size() + (spec ? spec_chunks + (int)p->waves.size() : 0);
     p->n_u64 = 1 + nc + nq;
     struct Part { void** dst; size_t bytes; };
     const bool hier = g.hierarchical == CP_SEARCH_COARSE_FINE;
@@ -1435,7 +1439,9 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         {(void**)&p->d_sx, sx_bytes},
         {(void**)&p->d_sP, sp_bytes},
         {(void**)&p->d_srow, srow_bytes},
+        {(void**)&p->d_spart, spec ? (size_t)std::max(p->sfull.chunk, p->ssearch.chunk) * confirm_bytes(p->max_n) : 0},
         {(void**)&p->d_tw, spec ? (size_t)kSpecTwiddles * sizeof(float2) : 0},
+        {(void**)&p->d_svblk, svblk_bytes},
         {(void**)&p->d_svmax, spec ? (size_t)nc * sizeof(unsigned int) : 0},
         {(void**)&p->d_scand, spec ? (size_t)nc * kSpecCand * sizeof(int32_t) : 0},
         {(void**)&p->d_sfb, spec ? 2 * (size_t)nc * sizeof(int32_t) : 0},
@@ -1519,7 +1525,8 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     p->opt.sigma_t_per_curve = nullptr;
 
     if (spec) {
-        CP_CUDA(spec_prepare(p->np2max, p->max_n, std::max(p->sfull.seg, p->ssearch.seg)));
+        CP_CUDA(spec_prepare(p->np2max, p->max_n, p->spec_seg_max));
+        CP_CUDA(prepare_selected(p->pair_smem + (size_t)(p->max_n + kTile) * sizeof(float)));
         CP_CUDA(launch_spec_twiddle(p->d_tw, p->stream));
     }
 
@@ -1562,7 +1569,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
             if (w.cls == 0) {
                 const int64_t chunks = (w.slot_end - w.slot_begin + sp.chunk - 1) / sp.chunk;
                 const int transform = 1 + (sp.min_logq <= kSpecOneLogQ ? 1 : 0) + (sp.max_logq > kSpecOneLogQ ? 2 : 0);
-                p->launches_per_search += 2 + chunks * (transform + (hier ? 6 : 2));
+                p->launches_per_search += (hier ? 1 : 0) + chunks * (transform + (hier ? 9 : 4));
             }
     return CP_OK;
 }
@@ -1634,7 +1641,7 @@ static cp_status periodogram_impl(cp_plan_t p, float* out)
     stage_host_inputs(p);
     if ((st = enqueue_inputs(p, p->stream)) == CP_OK && (st = enqueue_stats(p, p->stream)) == CP_OK) {
         for (int w = 0; w < (int)p->waves.size() && st == CP_OK; w++) {
-            st = enqueue_wave_w(p, w, p->stream);
+            st = enqueue_wave_w(p, w, p->sfull.on, p->stream);
             if (st == CP_OK) st = enqueue_values(p, kStageFull, w, out, p->stream, nullptr);
         }
     }

@@ -80,6 +80,10 @@ enum Stage : int { kStageFull = 0, kStageCoarse = 1, kStageFine = 2, kStageList 
 // rank (2J+1) + (j+J).
 enum Candidates : int { kCandNone = 0, kCandGrid = 1, kCandCoarse = 2, kCandTrial = 3, kCandFine = 4 };
 
+constexpr int kConfirmCand = 32;             // candidate entries per curve (one ballot)
+constexpr int kConfirmMaxChunk = 64;         // curves per launch
+constexpr int kConfirmSmem = 114 * 1024;     // trig table and magnitudes (one frequency pair of the longest curve)
+
 // Direct-form pair tiling: a warp owns a 32 x 32 tile of (row i, col j)
 // pairs of the upper block triangle; lane (a, b) = (lane / 8, lane % 8)
 // holds rows i = I0 + a + 4k (k < 8) and columns j = J0 + b + 8m (m < 4).
@@ -169,7 +173,7 @@ struct PairArgs {
     int32_t n_trials;
     float* trial_stat;           // list stage: nCKP per trial (may be null)
     // launches over chosen frequencies or curves (pair spectrum, cp_spec.cu):
-    int64_t upc;                 // > 0: upc units per curve
+    int64_t upc;                 // units per curve of a launch over fb_slots
     int32_t candidates;          // Candidates kind of cand (kCandNone: every unit of the stage)
     int32_t n_cand;
     const int32_t* cand;         // [n_curves * n_cand] entries, -1 after the last
@@ -343,6 +347,10 @@ cudaError_t launch_pair_tensor(const TensorArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_stats(const StatsArgs& a, int n_curves, cudaStream_t s);
 cudaError_t launch_build_w(const BuildWArgs& a, cudaStream_t s);
 cudaError_t launch_pair_direct(const PairArgs& a, int grid, size_t smem, cudaStream_t s);
+// The pair sum at the candidate entries; part: confirm_bytes(max_n) per slot (part_ld f2).
+cudaError_t launch_confirm(const PairArgs& a, void* part, int64_t part_ld, int n_sm, int max_n, cudaStream_t s);
+size_t confirm_bytes(int max_n);
+cudaError_t prepare_selected(size_t pair_smem);   // launches over candidates or fb_slots
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t s);
 cudaError_t launch_finalize(const FinalArgs& a, cudaStream_t s);
 cudaError_t launch_zero_u64(unsigned long long* p, int64_t n, cudaStream_t s);

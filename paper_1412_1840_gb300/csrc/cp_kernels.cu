@@ -288,6 +288,18 @@ __device__ __forceinline__ void decode_tile(int t, int nb, int& bi, int& bj)
     bj = b + rem;
 }
 
+// The constant 2^(-beta/2) that the cos form's w carries (see pair_item); 1 in the sin form.
+__device__ __forceinline__ float w_scale(const CurveParams& P)
+{
+    const float tsc = P.tscale * P.tscale * 0.70710678f;
+    return P.sigma_t >= kCosFormMinSigma ? exp2f(-(tsc * tsc)) : 1.0f;
+}
+
+__device__ __forceinline__ float w_of(float ypi, float ypj, float ip_hi, float ip_lo, float scale)
+{
+    return ((gauss_g(ypi, ypj) - ip_hi) - ip_lo) * scale;
+}
+
 __global__ void __launch_bounds__(256) k_build_w(const BuildWArgs a)
 {
     const int lane = threadIdx.x & 31;
@@ -307,8 +319,7 @@ __global__ void __launch_bounds__(256) k_build_w(const BuildWArgs a)
     const int la = lane >> 3, lb = lane & 7;
     // cos-form curves: w carries the exponent's constant term, w 2^(-beta/2), so
     // that the pair kernel's exponent is the bare product sum (see pair_item)
-    const float tsc = P.tscale * P.tscale * 0.70710678f;
-    const float wscale = P.sigma_t >= kCosFormMinSigma ? exp2f(-(tsc * tsc)) : 1.0f;
+    const float wscale = w_scale(P);
     float ypc[kColsPerLane];
     int jj[kColsPerLane];
 #pragma unroll
@@ -324,8 +335,7 @@ __global__ void __launch_bounds__(256) k_build_w(const BuildWArgs a)
         float w[kColsPerLane];
 #pragma unroll
         for (int m = 0; m < kColsPerLane; m++) {
-            const float g = gauss_g(ypr, ypc[m]);
-            w[m] = (i < jj[m] && jj[m] < n) ? ((g - P.ip_hi) - P.ip_lo) * wscale : 0.f;
+            w[m] = (i < jj[m] && jj[m] < n) ? w_of(ypr, ypc[m], P.ip_hi, P.ip_lo, wscale) : 0.f;
         }
         reinterpret_cast<float4*>(dst)[k * 32 + lane] = make_float4(w[0], w[1], w[2], w[3]);
     }
@@ -362,64 +372,128 @@ constexpr int kTableGroups = 2;
 // The cos form's rounding is absolute, about beta 2^-24 in the exponent, so it
 // is used only for sigma_t >= kCosFormMinSigma (beta <= 32: below 3e-6 per term;
 // the exponent then lies in [-beta/2, beta/2], within FP32 range).
+// The item's sum at one frequency pair (SCf, NSf: that pair's table): (f, f').
+template <bool COSF>
+__device__ __forceinline__ f2 pair_item_at(const ulonglong2* SCf, const f2* NSf, int rbase, int cbase,
+                                           const f2 (&w01)[kItemRows], const f2 (&w23)[kItemRows])
+{
+    ulonglong2 col[kColsPerLane];
+#pragma unroll
+    for (int m = 0; m < kColsPerLane; m++) col[m] = SCf[cbase + 8 * m];
+    f2 tf0 = 0ull, tf1 = 0ull, tg0 = 0ull, tg1 = 0ull;
+#pragma unroll
+    for (int k = 0; k < kItemRows; k++) {
+        const int i = rbase + 4 * k;
+        float e[kColsPerLane][2];
+        if (COSF) {
+            const ulonglong2 R = SCf[i];   // ((S_i(f), S_i(f')), (C_i(f), C_i(f')))
+#pragma unroll
+            for (int m = 0; m < kColsPerLane; m++) {
+                const f2 a2 = fma2(R.y, col[m].y, mul2(R.x, col[m].x));
+                float a0, a1;
+                upk(a2, a0, a1);
+                e[m][0] = ex2_approx(a0);
+                e[m][1] = ex2_approx(a1);
+            }
+        } else {
+            const f2 A = SCf[i].y;   // (c_i(f), c_i(f'))
+            const f2 B = NSf[i];     // (-s_i(f), -s_i(f'))
+#pragma unroll
+            for (int m = 0; m < kColsPerLane; m++) {
+                const f2 t2 = mul2(B, col[m].y);
+                const f2 d2 = fma2(A, col[m].x, t2);
+                const f2 q2 = mul2(d2, d2);
+                float q0, q1;
+                upk(q2, q0, q1);
+                e[m][0] = ex2_approx(-q0);
+                e[m][1] = ex2_approx(-q1);
+            }
+        }
+        tf0 = fma2(w01[k], pk(e[0][0], e[1][0]), tf0);
+        tf1 = fma2(w23[k], pk(e[2][0], e[3][0]), tf1);
+        tg0 = fma2(w01[k], pk(e[0][1], e[1][1]), tg0);
+        tg1 = fma2(w23[k], pk(e[2][1], e[3][1]), tg1);
+    }
+    float fx, fy, gx, gy;
+    upk(add2(tf0, tf1), fx, fy);
+    upk(add2(tg0, tg1), gx, gy);
+    return pk(fx + fy, gx + gy);
+}
+
 template <bool COSF>
 __device__ __forceinline__ void pair_item(const ulonglong2* SC, const f2* NS, int npad, int nfp, int rbase,
                                           int cbase, const f2 (&w01)[kItemRows],
                                           const f2 (&w23)[kItemRows], f2 (&acc)[kFcMax / 2])
 {
 #pragma unroll
-    for (int fp = 0; fp < kFcMax / 2; fp++) {
-        if (fp < nfp) {
-            const ulonglong2* SCf = SC + fp * npad;
-            const f2* NSf = NS + fp * npad;
-            ulonglong2 col[kColsPerLane];
+    for (int fp = 0; fp < kFcMax / 2; fp++)
+        if (fp < nfp)
+            acc[fp] = add2(acc[fp], pair_item_at<COSF>(SC + fp * npad, NS + fp * npad, rbase, cbase, w01, w23));
+}
+
+// The item's w from the curve's scaled magnitudes (as k_build_w stores them).
+__device__ __forceinline__ void item_w(const float* Y, int n, int rbase, int cbase, float ip_hi, float ip_lo, float scale,
+                                       f2 (&w01)[kItemRows], f2 (&w23)[kItemRows])
+{
+    float yc[kColsPerLane];
 #pragma unroll
-            for (int m = 0; m < kColsPerLane; m++) col[m] = SCf[cbase + 8 * m];
-            f2 tf0 = 0ull, tf1 = 0ull, tg0 = 0ull, tg1 = 0ull;
+    for (int m = 0; m < kColsPerLane; m++) yc[m] = Y[cbase + 8 * m];
 #pragma unroll
-            for (int k = 0; k < kItemRows; k++) {
-                const int i = rbase + 4 * k;
-                float e[kColsPerLane][2];
-                if (COSF) {
-                    const ulonglong2 R = SCf[i];   // ((S_i(f), S_i(f')), (C_i(f), C_i(f')))
+    for (int k = 0; k < kItemRows; k++) {
+        const int i = rbase + 4 * k;
+        const float yr = Y[i];
+        float w[kColsPerLane];
 #pragma unroll
-                    for (int m = 0; m < kColsPerLane; m++) {
-                        const f2 a2 = fma2(R.y, col[m].y, mul2(R.x, col[m].x));
-                        float a0, a1;
-                        upk(a2, a0, a1);
-                        e[m][0] = ex2_approx(a0);
-                        e[m][1] = ex2_approx(a1);
-                    }
-                } else {
-                    const f2 A = SCf[i].y;   // (c_i(f), c_i(f'))
-                    const f2 B = NSf[i];     // (-s_i(f), -s_i(f'))
-#pragma unroll
-                    for (int m = 0; m < kColsPerLane; m++) {
-                        const f2 t2 = mul2(B, col[m].y);
-                        const f2 d2 = fma2(A, col[m].x, t2);
-                        const f2 q2 = mul2(d2, d2);
-                        float q0, q1;
-                        upk(q2, q0, q1);
-                        e[m][0] = ex2_approx(-q0);
-                        e[m][1] = ex2_approx(-q1);
-                    }
-                }
-                tf0 = fma2(w01[k], pk(e[0][0], e[1][0]), tf0);
-                tf1 = fma2(w23[k], pk(e[2][0], e[3][0]), tf1);
-                tg0 = fma2(w01[k], pk(e[0][1], e[1][1]), tg0);
-                tg1 = fma2(w23[k], pk(e[2][1], e[3][1]), tg1);
-            }
-            float fx, fy, gx, gy;
-            upk(add2(tf0, tf1), fx, fy);
-            upk(add2(tg0, tg1), gx, gy);
-            acc[fp] = add2(acc[fp], pk(fx + fy, gx + gy));
+        for (int m = 0; m < kColsPerLane; m++) {
+            const int j = cbase + 8 * m;
+            w[m] = (i < j && j < n) ? w_of(yr, yc[m], ip_hi, ip_lo, scale) : 0.f;
         }
+        w01[k] = pk(w[0], w[1]);
+        w23[k] = pk(w[2], w[3]);
     }
 }
 
-// SEL: a launch over chosen frequencies (candidate lists) or chosen curves
-// (fb_slots) of the pair-spectrum path; its own instantiation, so that the
-// units of a plain launch carry none of it.
+// Trig table entry of one point at a frequency pair (phases p0, p1).
+__device__ __forceinline__ void table_entry(bool cosf, float ts, uint64_t p0, uint64_t p1, ulonglong2& sc, f2& ns)
+{
+    float s0, c0, s1, c1;
+    if (cosf) {
+        sincos2pi_turns((uint32_t)(p0 >> 32), s0, c0);
+        sincos2pi_turns((uint32_t)(p1 >> 32), s1, c1);
+    } else {
+        sincospi_turns((uint32_t)(p0 >> 32), s0, c0);
+        sincospi_turns((uint32_t)(p1 >> 32), s1, c1);
+    }
+    s0 *= ts; c0 *= ts; s1 *= ts; c1 *= ts;
+    sc = make_ulonglong2(pk(s0, s1), pk(c0, c1));
+    ns = pk(-s0, -s1);
+}
+
+// Phase of point `at` (index in the CSR arrays) at candidate entry e.
+__device__ __forceinline__ uint64_t cand_phase(const PairArgs& a, const int32_t* tl, int c, int64_t at, int e)
+{
+    const uint64_t base = a.ph_base[at], st = a.ph_step[at];
+    if (a.candidates == kCandTrial) return base + (uint64_t)max(tl[e], 0) * st;
+    if (a.candidates != kCandFine) return base + (uint64_t)e * st;
+    const int W = 2 * a.fine_half + 1, pk_ = e / W;
+    return base + (uint64_t)a.peaks[(int64_t)c * a.top_k + pk_] * a.ph_coarse[at] +
+           (uint64_t)(int64_t)(e - pk_ * W - a.fine_half) * st;
+}
+
+// The value at candidate entry e (admissible already) replaces the spectrum's; its key.
+__device__ __forceinline__ unsigned long long cand_emit(const PairArgs& a, int c, int e, float v)
+{
+    if (a.candidates == kCandGrid && a.out) a.out[(int64_t)c * a.out_ld + e] = v;
+    if (a.candidates == kCandCoarse) a.coarse_out[(int64_t)c * a.n_freq + e] = v;
+    if (a.candidates == kCandTrial && a.trial_stat) a.trial_stat[(int64_t)c * a.n_trials + e] = v;
+    return a.candidates == kCandCoarse ? 0ull : make_key(v, (uint32_t)e);
+}
+
+// SEL: a launch over chosen curves (fb_slots), those that the pair-spectrum path
+// leaves to the pair sum; its own instantiation, so that the units of a plain
+// launch carry none of it.  Its w come from the magnitudes
+// instead of stored tiles (one more exponential per pair and unit), so that
+// plans whose every pass goes through the spectrum keep no tiles.
 template <bool SEL>
 __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs a)
 {
@@ -435,14 +509,14 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
         if (tid == 0) s_unit = (long long)atomicAdd(a.queue, 1ull) + a.unit_begin;
         __syncthreads();
         const long long u = s_unit;
-        if (u >= (SEL && a.fb_count ? (long long)*a.fb_count * a.upc : a.unit_end)) break;
+        if (u >= (SEL ? (long long)*a.fb_count * a.upc : a.unit_end)) break;
 
         int slot;
         long long chunk;
         if (SEL) {
             const int64_t q = u / a.upc;
             chunk = u - q * a.upc;
-            slot = a.fb_count ? a.fb_slots[q] : a.slot_begin + (int)q;
+            slot = a.fb_slots[q];
         } else {
             int lo = a.slot_begin, hi = a.slot_end - 1;
             while (lo < hi) {
@@ -463,13 +537,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
         int count;
         int peak = 0;
         uint64_t peak_mult = 0;  // fine: coarse peak index (phase offset kpeak * coarse_i)
-        const int32_t* ce = SEL ? a.cand + (int64_t)c * a.n_cand : nullptr;   // candidate entries
-        if (SEL && a.candidates != kCandNone) {
-            kfirst = chunk * fc;
-            count = 0;
-            while (count < fc && kfirst + count < a.n_cand && ce[kfirst + count] >= 0) count++;
-            if (count == 0) continue;
-        } else if (a.stage == kStageFine) {
+        if (a.stage == kStageFine) {
             const int W = 2 * a.fine_half + 1;
             const int upp = (W + fc - 1) / fc;
             peak = (int)(chunk / upp);
@@ -510,17 +578,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
                 if (a.stage == kStageFine) ph += peak_mult * a.ph_coarse[off + i];
                 for (int fp = fp0; fp < fp1; fp++, ph += 2 * st) {
                     uint64_t p0 = ph, p1 = ph + st;
-                    if (SEL && a.candidates != kCandNone) {
-                        auto phase = [&](int e) -> uint64_t {
-                            if (a.candidates == kCandTrial) return base + (uint64_t)max(tl[e], 0) * st;
-                            if (a.candidates != kCandFine) return base + (uint64_t)e * st;
-                            const int W = 2 * a.fine_half + 1, pk = e / W;
-                            return base + (uint64_t)a.peaks[(int64_t)c * a.top_k + pk] * a.ph_coarse[off + i] +
-                                   (uint64_t)(int64_t)(e - pk * W - a.fine_half) * st;
-                        };
-                        p0 = phase(ce[kfirst + 2 * fp]);
-                        p1 = 2 * fp + 1 < count ? phase(ce[kfirst + 2 * fp + 1]) : p0;
-                    } else if (a.stage == kStageList) {
+                    if (a.stage == kStageList) {
                         // grid indices of list positions kfirst + 2 fp (+1); a missing entry evaluates k = 0
                         const long long q0 = kfirst + 2 * fp;
                         const int k0 = q0 < a.n_trials ? max(tl[q0], 0) : 0;
@@ -528,17 +586,9 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
                         p0 = base + (uint64_t)k0 * st;
                         p1 = base + (uint64_t)k1 * st;
                     }
-                    float s0, c0, s1, c1;
-                    if (cosf) {
-                        sincos2pi_turns((uint32_t)(p0 >> 32), s0, c0);
-                        sincos2pi_turns((uint32_t)(p1 >> 32), s1, c1);
-                    } else {
-                        sincospi_turns((uint32_t)(p0 >> 32), s0, c0);
-                        sincospi_turns((uint32_t)(p1 >> 32), s1, c1);
-                    }
-                    s0 *= ts; c0 *= ts; s1 *= ts; c1 *= ts;
-                    SC[fp * npad + i] = make_ulonglong2(pk(s0, s1), pk(c0, c1));
-                    if (!cosf) NS[fp * npad + i] = pk(-s0, -s1);   // the cos form reads SC only
+                    f2 ns;
+                    table_entry(cosf, ts, p0, p1, SC[fp * npad + i], ns);
+                    if (!cosf) NS[fp * npad + i] = ns;   // the cos form reads SC only
                 }
             } else {
                 for (int fp = fp0; fp < fp1; fp++) {
@@ -547,12 +597,17 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
                 }
             }
         }
+        float* Y = reinterpret_cast<float*>(SC) + (size_t)(fc >> 1) * npad * 6;   // SEL: after the tables
+        if (SEL)
+            for (int i = tid; i < npad; i += kPairThreads) Y[i] = i < n ? a.yp[off + i] : 0.f;
+        const float wscale = SEL ? w_scale(P) : 1.0f;
         __syncthreads();
 
         const int nb = npad / kTile;
         const int ntiles = nb * (nb + 1) / 2;
         const int nitems = kItemsPerTile * ntiles;   // (tile, row part): 4 kItemRows x 32 pairs per warp item
-        const float4* Wc = reinterpret_cast<const float4*>(a.W + (a.wtile_start[slot] - a.wtile_base) * kTileFloats);
+        const float4* Wc =
+            SEL ? nullptr : reinterpret_cast<const float4*>(a.W + (a.wtile_start[slot] - a.wtile_base) * kTileFloats);
         f2 acc[kFcMax / 2];                      // per f-pair: (sum at f, sum at f')
 #pragma unroll
         for (int q = 0; q < kFcMax / 2; q++) acc[q] = 0ull;
@@ -570,8 +625,13 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
 #pragma unroll 1
         for (; item < nitems; item += NW) {
             f2 w01[kItemRows], w23[kItemRows];
+            int bi, bj;
+            decode_tile(item / kItemsPerTile, nb, bi, bj);
+            const int rbase = bi * kTile + (item % kItemsPerTile) * (4 * kItemRows) + la;
+            const int cbase = bj * kTile + lb;
+            if (SEL) item_w(Y, n, rbase, cbase, P.ip_hi, P.ip_lo, wscale, w01, w23);
 #pragma unroll
-            for (int k = 0; k < kItemRows; k++) {
+            for (int k = 0; k < (SEL ? 0 : kItemRows); k++) {
                 const float4 wv = kPrefetchW ? wn[k] : __ldg(w_ptr(item, k));
                 w01[k] = pk(wv.x, wv.y);
                 w23[k] = pk(wv.z, wv.w);
@@ -581,10 +641,6 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
 #pragma unroll
                 for (int k = 0; k < kItemRows; k++) wn[k] = __ldg(w_ptr(nxt, k));
             }
-            int bi, bj;
-            decode_tile(item / kItemsPerTile, nb, bi, bj);
-            const int rbase = bi * kTile + (item % kItemsPerTile) * (4 * kItemRows) + la;
-            const int cbase = bj * kTile + lb;
             if (cosf) pair_item<true>(SC, NS, npad, nfp, rbase, cbase, w01, w23, acc);
             else pair_item<false>(SC, NS, npad, nfp, rbase, cbase, w01, w23, acc);
         }
@@ -615,14 +671,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
                 for (int w = 0; w < NW; w++) S += s_red[w][lane];
                 const float v = (2.0f * S + P.diag) * P.norm;
                 const long long kk = kfirst + lane;
-                if (SEL && a.candidates != kCandNone) {
-                    // admissible already; the value also replaces the spectrum's
-                    const int e = ce[kk];
-                    if (a.candidates == kCandGrid && a.out) a.out[(int64_t)c * a.out_ld + e] = v;
-                    if (a.candidates == kCandCoarse) a.coarse_out[(int64_t)c * a.n_freq + e] = v;
-                    if (a.candidates == kCandTrial && a.trial_stat) a.trial_stat[(int64_t)c * a.n_trials + e] = v;
-                    if (a.candidates != kCandCoarse) key = make_key(v, (uint32_t)e);
-                } else if (a.stage == kStageFull) {
+                if (a.stage == kStageFull) {
                     if (a.out) a.out[(int64_t)c * a.out_ld + kk] = v;
                     if (!excluded_k(a.ex.full_k, a.ex.n, kk)) key = make_key(v, (uint32_t)kk);
                 } else if (a.stage == kStageCoarse) {
@@ -647,6 +696,149 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
                 if (lane == 0 && key) atomicMax(a.best_key + c, key);
             }
         }
+    }
+}
+
+// ===========================================================================
+// k_confirm / k_confirm_sum: the pair sum at the candidate
+// entries, for a chunk of curves.  A unit of k_pair_direct would run
+// its few frequencies on one SM (0.8 ms for one frequency of a 4,000-sample
+// curve, 50 us for the 12 coarse points of a 650-sample one).  Here the tiles are
+// spread over the chip: k_confirm stores every tile's sum per lane, and
+// k_confirm_sum adds them in k_pair_direct's order (lane by lane over the tiles
+// of each of its warps, then lanes, then warps), so the value is the same to the
+// last bit.
+// ===========================================================================
+constexpr int kConfirmThreads = 256;
+constexpr int kConfirmWarps = kConfirmThreads / 32;
+
+__global__ void __launch_bounds__(kConfirmThreads) k_confirm(const PairArgs a, f2* part, int64_t part_ld, int group)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_pre[kConfirmMaxChunk + 1];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int la = lane >> 3, lb = lane & 7;
+    const int nc = a.slot_end - a.slot_begin;
+    if (warp == 0) {
+        int base = 0;
+        for (int c0 = 0; c0 < nc; c0 += 32) {
+            int v = 0;
+            if (c0 + lane < nc) {
+                const int c = a.order[a.slot_begin + c0 + lane];
+                if (a.cand[(int64_t)c * a.n_cand] >= 0) v = (tiles_of(a.cp[c].n) + group - 1) / group;
+            }
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += t;
+            }
+            if (c0 + lane < nc) s_pre[c0 + lane + 1] = base + v;
+            base += __shfl_sync(0xffffffffu, v, 31);
+        }
+        if (lane == 0) s_pre[0] = 0;
+    }
+    __syncthreads();
+    for (int item = blockIdx.x; item < s_pre[nc]; item += gridDim.x) {
+        int lo = 0, hi = nc - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_pre[mid] <= item) lo = mid; else hi = mid - 1;
+        }
+        const int c = a.order[a.slot_begin + lo];
+        const CurveParams& P = a.cp[c];
+        const int n = P.n, npad = (n + kTile - 1) & ~(kTile - 1), nb = npad / kTile, ntiles = nb * (nb + 1) / 2;
+        const int64_t off = P.off;
+        const int32_t* ce = a.cand + (int64_t)c * a.n_cand;
+        const int32_t* tl = a.trials + (int64_t)c * a.n_trials;
+        int count = 0;
+        {
+            const int e = lane < a.n_cand ? ce[lane] : -1;
+            count = __popc(__ballot_sync(0xffffffffu, e >= 0));
+        }
+        const bool cosf = P.sigma_t >= kCosFormMinSigma;
+        const float ts = cosf ? P.tscale * P.tscale * 0.70710678f : P.tscale;
+        const float wscale = w_scale(P);
+        // frequency pairs per pass: as many as the table holds
+        const int room = (kConfirmSmem - npad * 4) / (npad * 24);
+        const int step = min(room, (count + 1) >> 1);
+        float* Y = reinterpret_cast<float*>(smem);
+        ulonglong2* SC = reinterpret_cast<ulonglong2*>(Y + npad);
+        f2* NS = reinterpret_cast<f2*>(SC + step * npad);
+        const int t0 = (item - s_pre[lo]) * group, t1 = min(t0 + group, ntiles);
+        f2* dst = part + (int64_t)lo * part_ld;
+        for (int f0 = 0; 2 * f0 < count; f0 += step) {
+            const int nfp = min(step, ((count + 1) >> 1) - f0);
+            __syncthreads();
+            for (int q = tid; q < nfp * npad; q += kConfirmThreads) {
+                const int fp = q / npad, i = q - fp * npad;
+                if (f0 == 0 && fp == 0) Y[i] = i < n ? a.yp[off + i] : 0.f;
+                ulonglong2 sc = make_ulonglong2(0ull, 0ull);
+                f2 ns = 0ull;
+                if (i < n) {
+                    const int e0 = 2 * (f0 + fp), e1 = e0 + 1 < count ? e0 + 1 : e0;
+                    table_entry(cosf, ts, cand_phase(a, tl, c, off + i, ce[e0]), cand_phase(a, tl, c, off + i, ce[e1]), sc, ns);
+                }
+                SC[q] = sc;
+                if (!cosf) NS[q] = ns;
+            }
+            __syncthreads();
+            for (int t = t0 + warp; t < t1; t += kConfirmWarps) {
+                int bi, bj;
+                decode_tile(t, nb, bi, bj);
+                const int rbase = bi * kTile + la, cbase = bj * kTile + lb;
+                f2 w01[kItemRows], w23[kItemRows];
+                item_w(Y, n, rbase, cbase, P.ip_hi, P.ip_lo, wscale, w01, w23);
+                for (int fp = 0; fp < nfp; fp++) {
+                    const f2 v = cosf ? pair_item_at<true>(SC + fp * npad, NS + fp * npad, rbase, cbase, w01, w23)
+                                      : pair_item_at<false>(SC + fp * npad, NS + fp * npad, rbase, cbase, w01, w23);
+                    dst[((int64_t)(f0 + fp) * ntiles + t) * 32 + lane] = v;
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kPairThreads) k_confirm_sum(const PairArgs a, const f2* part, int64_t part_ld)
+{
+    constexpr int NW = kPairThreads / 32;
+    __shared__ float s_red[NW][2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int c = a.order[a.slot_begin + blockIdx.x], fp = blockIdx.y;
+    const int32_t* ce = a.cand + (int64_t)c * a.n_cand;
+    if (ce[2 * fp] < 0) return;
+    const CurveParams& P = a.cp[c];
+    const int nb = (P.n + kTile - 1) / kTile, ntiles = nb * (nb + 1) / 2;
+    const f2* src = part + (int64_t)blockIdx.x * part_ld + (int64_t)fp * ntiles * 32 + lane;
+    f2 acc = 0ull;
+    int t = warp;
+    for (; t + 3 * NW < ntiles; t += 4 * NW) {
+        f2 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) v[q] = src[(int64_t)(t + q * NW) * 32];
+#pragma unroll
+        for (int q = 0; q < 4; q++) acc = add2(acc, v[q]);
+    }
+    for (; t < ntiles; t += NW) acc = add2(acc, src[(int64_t)t * 32]);
+    float vf, vg;
+    upk(acc, vf, vg);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        vf += __shfl_xor_sync(0xffffffffu, vf, o);
+        vg += __shfl_xor_sync(0xffffffffu, vg, o);
+    }
+    if (lane == 0) {
+        s_red[warp][0] = vf;
+        s_red[warp][1] = vg;
+    }
+    __syncthreads();
+    if (tid < 2 && ce[2 * fp + tid] >= 0) {
+        float S = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; w++) S += s_red[w][tid];
+        const float v = (2.0f * S + P.diag) * P.norm;
+        const unsigned long long key = cand_emit(a, c, ce[2 * fp + tid], v);
+        if (key) atomicMax(a.best_key + c, key);
     }
 }
 
@@ -780,7 +972,7 @@ cudaError_t launch_build_w(const BuildWArgs& a, cudaStream_t s)
 
 cudaError_t launch_pair_direct(const PairArgs& a, int grid, size_t smem, cudaStream_t s)
 {
-    if (a.upc > 0) k_pair_direct<true><<<grid, kPairThreads, smem, s>>>(a);
+    if (a.fb_count) k_pair_direct<true><<<grid, kPairThreads, smem, s>>>(a);
     else k_pair_direct<false><<<grid, kPairThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
@@ -797,6 +989,30 @@ cudaError_t launch_finalize(const FinalArgs& a, cudaStream_t s)
 {
     k_finalize<<<(a.n_curves + 255) / 256, 256, 0, s>>>(a);
     return cudaGetLastError();
+}
+
+cudaError_t launch_confirm(const PairArgs& a, void* part, int64_t part_ld, int n_sm, int max_n, cudaStream_t s)
+{
+    const int n = a.slot_end - a.slot_begin;
+    if (n <= 0) return cudaSuccess;
+    if (n > kConfirmMaxChunk || a.n_cand != kConfirmCand) return cudaErrorInvalidValue;
+    // tiles per item: enough items for two per SM, at least one tile a warp, at most eight
+    const int64_t tiles = (int64_t)n * tiles_of(max_n);
+    int group = kConfirmWarps;
+    while (group < 8 * kConfirmWarps && tiles / group > 6 * n_sm) group += kConfirmWarps;
+    k_confirm<<<2 * n_sm, kConfirmThreads, kConfirmSmem, s>>>(a, static_cast<f2*>(part), part_ld, group);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_confirm_sum<<<dim3(n, kConfirmCand / 2), kPairThreads, 0, s>>>(a, static_cast<const f2*>(part), part_ld);
+    return cudaGetLastError();
+}
+
+size_t confirm_bytes(int max_n) { return (size_t)tiles_of(max_n) * 32 * sizeof(f2) * (kConfirmCand / 2); }
+
+cudaError_t prepare_selected(size_t pair_smem)
+{
+    cudaError_t e = raise_dyn_smem((const void*)k_confirm, kConfirmSmem);
+    return e == cudaSuccess ? raise_dyn_smem((const void*)k_pair_direct<true>, pair_smem) : e;
 }
 
 int pair_direct_threads() { return kPairThreads; }
@@ -824,8 +1040,6 @@ cudaError_t raise_dyn_smem(const void* func, size_t bytes)
 cudaError_t prepare_kernels(int np2max, size_t pair_smem)
 {
     cudaError_t e = raise_dyn_smem((const void*)k_stats, stats_smem_bytes(np2max));
-    if (e != cudaSuccess) return e;
-    e = raise_dyn_smem((const void*)k_pair_direct<true>, pair_smem);
     if (e != cudaSuccess) return e;
     return raise_dyn_smem((const void*)k_pair_direct<false>, pair_smem);
 }

@@ -35,9 +35,9 @@
 // transform).
 //
 // Measured (GB300; N 300-1000, 49,981 frequencies, sigma_t rule): best period of
-// 384 curves 715.8 ms by the pair sum alone, 7.4 ms through the spectrum, results
-// identical; 12 periodograms 25.3 -> 0.42 ms, error against FP64 3.4e-7 -> 7.5e-8;
-// coarse-then-fine search of 256 curves 81.4 -> 7.5 ms, results identical.
+// 384 curves 717 ms by the pair sum alone, 4.6 ms through the spectrum, results
+// identical; 12 periodograms 25.3 -> 0.29 ms, error against FP64 3.2e-7 -> 8.6e-8;
+// coarse-then-fine search of 256 curves 81.0 -> 4.7 ms, results identical.
 #include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -69,10 +69,11 @@ __constant__ float c_kbO[4][4] = {{4.896753093e-01f, -2.389145815e-01f, 5.541547
 // z = sqrt(shape^2 - (4 pi m / H)^2) >= 14 here, so 2 z e^-z.
 __device__ __forceinline__ float kb_inverse(float r)     // r = m / H
 {
-    const float om = 4.0f * (float)CP_PI * r;
-    const float o2 = om * om;
-    const float z = sqrtf(kKbShape * kKbShape - o2);
-    return kKbInv0 * (1.0f / kKbShape) * z * ex2_approx(1.4426950408889634f * __fdividef(o2, z + kKbShape));
+    const float o2 = (16.0f * (float)(CP_PI * CP_PI)) * (r * r);
+    float z, q;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(z) : "f"(fmaf(-(16.0f * (float)(CP_PI * CP_PI)) * r, r, kKbShape * kKbShape)));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(z + kKbShape));
+    return (kKbInv0 / kKbShape) * z * ex2_approx(1.4426950408889634f * o2 * q);
 }
 
 // Weights of the 8 cells l - 3 .. l + 4 around a point z = f - 1/2 off the middle of cells l, l + 1.
@@ -107,39 +108,44 @@ __device__ __host__ inline int spec_logq_of(int64_t n_out)
 
 __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a)
 {
+    // FP64 runs at 1.7 operations/clk/SM here, so only the differences and their fixed-point
+    // form are FP64; the times (all >= 0) are compared as the integers of their bits.
     extern __shared__ __align__(16) unsigned char smem[];
-    double* ts = reinterpret_cast<double*>(smem);
+    long long* ts = reinterpret_cast<long long*>(smem);
     int32_t* ix = reinterpret_cast<int32_t*>(ts + a.np2max);
     __shared__ double s_a[kMillerMax + 2];
-    __shared__ double s_max[kSpecPrepThreads / 32];
+    __shared__ float s_f[kMillerMax + 2];
+    __shared__ long long s_max[kSpecPrepThreads / 32];
     __shared__ double s_cpd, s_T, s_inv;
-    __shared__ int s_unsorted, s_n0, s_nh;
+    __shared__ int s_n0, s_nh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int c = a.order[a.slot_begin + blockIdx.x];
     const CurveParams& P = a.cp[c];
     const int n = P.n;
     const int64_t off = P.off;
-    int np2 = 1;
-    while (np2 < n) np2 <<= 1;
-    if (tid == 0) s_unsorted = 0;
-    __syncthreads();
     const double t0 = P.t0;
-    double tmax = 0.0;
+    long long tmax = 0;
     for (int i = tid; i < n; i += kSpecPrepThreads) {
-        const double t = a.times[off + i] - t0;
+        long long t = __double_as_longlong(a.times[off + i] - t0);
+        if (t < 0) t = t == (long long)0x8000000000000000ull ? 0 : 0x7ff8000000000000ll;   // -0; a NaN
         ts[i] = t;
         ix[i] = i;
-        tmax = fmax(tmax, t);
-        if (!isfinite(t)) tmax = INFINITY;
-        if (i > 0 && !(a.times[off + i - 1] <= a.times[off + i])) s_unsorted = 1;
+        tmax = t > tmax ? t : tmax;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tmax = fmax(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+    for (int o = 16; o > 0; o >>= 1) {
+        const long long t = __shfl_xor_sync(0xffffffffu, tmax, o);
+        tmax = t > tmax ? t : tmax;
+    }
     if (lane == 0) s_max[warp] = tmax;
     __syncthreads();
-    if (s_unsorted) {
+    bool ordered = true;
+    for (int i = tid; i + 1 < n; i += kSpecPrepThreads) ordered = ordered && ts[i] <= ts[i + 1];
+    if (!__syncthreads_and(ordered)) {
+        int np2 = 1;
+        while (np2 < n) np2 <<= 1;
         for (int i = n + tid; i < np2; i += kSpecPrepThreads) {
-            ts[i] = INFINITY;
+            ts[i] = 0x7fffffffffffffffll;
             ix[i] = i;
         }
         for (int k = 2; k <= np2; k <<= 1) {
@@ -148,7 +154,7 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
                 for (int i = tid; i < np2; i += kSpecPrepThreads) {
                     const int q = i ^ j;
                     if (q > i) {
-                        const double u = ts[i], v = ts[q];
+                        const long long u = ts[i], v = ts[q];
                         const int iu = ix[i], iv = ix[q];
                         if ((u > v || (u == v && iu > iv)) == ((i & k) == 0)) {
                             ts[i] = v; ts[q] = u;
@@ -161,15 +167,15 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
         __syncthreads();
     }
     if (tid == 0) {
-        double T = 0.0;
-        for (int w = 0; w < kSpecPrepThreads / 32; w++) T = fmax(T, s_max[w]);
+        for (int w = 0; w < kSpecPrepThreads / 32; w++) tmax = s_max[w] > tmax ? s_max[w] : tmax;
+        const double T = __longlong_as_double(tmax);
         s_T = T;
         // a_n = 2 e^-k I_n(k) by the backward recurrence I_{n-1} = I_{n+1} + (2n/k) I_n,
         // normalised by a_0 + sum a_n = 1.  One thread's chain of FP64 FMAs; all that
         // can be done by the other threads is left to them below.
         const float st = P.sigma_t;
         int n0 = 0;
-        if (st >= 0.09f && st < 1e3f && isfinite(T)) {
+        if (st >= 0.09f && st < 1e3f && tmax < 0x7ff0000000000000ll) {
             const double s2 = (double)st * (double)st, two_k = 2.0 * s2;      // 2 / k
             n0 = min(kMillerMax, (int)(14.0f + 10.0f / st));
             double hi = 0.0, cur = 1e-200, sum = 0.0, qk = (double)n0 * two_k;
@@ -188,19 +194,18 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
         s_nh = 1;
     }
     __syncthreads();
-    {
-        // harmonics kept: the smallest count whose tail is below kSpecTail
-        const int n0 = s_n0;
-        if (tid < n0 && tid >= 1) {
-            float tail = 0.f;
-            for (int q = n0; q > tid - 1; q--) tail += 2.0f * (float)(s_a[q] * s_inv);
-            if (tail > (float)kSpecTail) atomicMax(&s_nh, tid);      // without harmonic tid the tail is too large
-        }
+    // harmonics kept: the smallest count whose tail is below kSpecTail
+    const int n0 = s_n0;
+    if (tid <= n0 && n0) s_f[tid] = (float)((tid ? 2.0 : 1.0) * s_a[tid] * s_inv);
+    __syncthreads();
+    if (tid <= n0 && tid >= 1) {
+        float tail = 0.f;
+        for (int q = n0; q >= tid; q--) tail += s_f[q];
+        if (tail > (float)kSpecTail) atomicMax(&s_nh, tid);      // without harmonic tid the tail is too large
     }
     __syncthreads();
-    const int nh = s_n0 ? s_nh : kSpecMaxHarm + 1;
-    if (tid < nh && nh <= kSpecMaxHarm)
-        a.coef[(int64_t)c * kSpecMaxHarm + tid] = (float)(2.0 * s_a[tid + 1] * s_inv);
+    const int nh = n0 ? s_nh : kSpecMaxHarm + 1;
+    if (tid < nh && nh <= kSpecMaxHarm) a.coef[(int64_t)c * kSpecMaxHarm + tid] = s_f[tid + 1];
     if (tid == 0) {
         SpecCurve S;
         S.nh = 0;
@@ -240,14 +245,16 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
                 S.support = sup >= (double)S.H ? (int32_t)S.H : min((int32_t)S.H, ((int32_t)sup + 3) & ~3);
             }
         }
+        // segments: about seg_items of them per curve, of 512 cells at least
+        S.seg = min(a.seg_max, max(512, ((S.support / a.seg_items) + 511) & ~511));
         a.sc[c] = S;
-        s_cpd = S.cells_per_day;
+        s_cpd = S.cells_per_day * 4294967296.0;
         a.vmax[c] = 0u;
     }
     __syncthreads();
     const double cpd = s_cpd;
     for (int i = tid; i < n; i += kSpecPrepThreads) {
-        a.xs[off + i] = (uint64_t)__double2ll_rn(ts[i] * cpd * 4294967296.0);
+        a.xs[off + i] = (uint64_t)__double2ll_rn(__longlong_as_double(ts[i]) * cpd);
         a.ys[off + i] = a.yp[off + ix[i]];
     }
 }
@@ -255,12 +262,18 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
 // ===========================================================================
 // k_spec_spread: one item = (curve, segment of cells).  With the times sorted,
 // the pairs of a segment are one range of j per row i (and per fold of the
-// period); the ranges are found by bisection, counted, and the threads take
-// pairs evenly across rows.  Cells are 64-bit integers of 2^-28 quanta: the
-// low word, started at 2^31, takes a shared-memory integer add whose carry or
-// borrow (rare) goes to the high word.
+// period).  A warp takes 16 rows, half its lanes bisecting for the first j, half
+// for the last, and then 32 pairs at a time across the rows.  Cells are 64-bit
+// integers of 2^-28 quanta: the low word, started at 2^31, takes a shared-memory
+// integer add whose carry or borrow (rare) goes to the high word, so the sums are
+// exact and do not depend on the order.  Bound by instructions issued, about 120
+// per 32 pairs: the 8 cells of a pair lie at constant offsets (a margin on both
+// sides of the segment takes what falls outside; at 0 and at half the period the
+// margin is folded back when the segment is written).
 // ===========================================================================
 constexpr int kSpreadThreads = 512;
+constexpr int kSpreadMargin = 16;                // cells on either side of a segment
+constexpr int kSpreadRows = 16;                  // rows a warp takes at a time
 constexpr float kQuanta = 268435456.0f;          // 2^28 per unit of weight
 
 __device__ __forceinline__ int lower_bound_x(const uint64_t* x, int lo, int hi, uint64_t v)
@@ -307,23 +320,22 @@ __device__ __forceinline__ int item_curve(const int* pre, int nc, int item)
 // INTERP: the weights are divided by the interpolation window's transform at the
 // pair's time difference (all differences lie below half of the half period).
 template <bool INTERP>
-__global__ void __launch_bounds__(kSpreadThreads) k_spec_spread(const SpecArgs a, int max_n)
+__global__ void __launch_bounds__(kSpreadThreads, 2) k_spec_spread(const SpecArgs a, int max_n)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t* X = reinterpret_cast<uint64_t*>(smem);
+    // low and high words of the cells A - margin .. A + seg + margin, then the curve's samples
+    uint32_t* cl = reinterpret_cast<uint32_t*>(smem);
+    const int words = a.seg_max + 2 * kSpreadMargin;
+    int32_t* ch = reinterpret_cast<int32_t*>(cl + words);
+    uint64_t* X = reinterpret_cast<uint64_t*>(ch + words);
     float* Y = reinterpret_cast<float*>(X + max_n);
-    int* pre = reinterpret_cast<int*>(Y + max_n);            // pairs before row i (max_n + 1)
-    int* jlo = pre + max_n + 1;                              // first j of row i
-    uint32_t* cl = reinterpret_cast<uint32_t*>(jlo + max_n + 1);
-    int32_t* ch = reinterpret_cast<int32_t*>(cl + a.seg);
-    __shared__ int s_item, s_wsum[kSpreadThreads / 32];
+    __shared__ int s_item;
     __shared__ int s_pre[kSpecMaxChunk + 1];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nc = a.slot_end - a.slot_begin;
-    const int seg = a.seg;
     item_prefix(s_pre, nc, [&](int i) {
         const SpecCurve& S = a.sc[a.order[a.slot_begin + i]];
-        return S.nh ? (S.support + seg - 1) / seg : 0;
+        return S.nh ? (S.support + S.seg - 1) / S.seg : 0;
     });
     const int total = s_pre[nc];
     int loaded = -1;
@@ -346,10 +358,10 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spec_spread(const SpecArgs a
             loaded = ci;
         }
         const int H = (int)S.H;
-        const int A = (item - s_pre[ci]) * seg, B = min(A + seg, S.support);
-        for (int i = tid; i < seg; i += kSpreadThreads) {
-            cl[i] = 0x80000000u;
-            ch[i] = 0;
+        const int A = (item - s_pre[ci]) * S.seg, B = min(A + S.seg, S.support), len = B - A;
+        for (int i = tid; i < (len + 2 * kSpreadMargin) / 4; i += kSpreadThreads) {
+            reinterpret_cast<uint4*>(cl)[i] = make_uint4(0x80000000u, 0x80000000u, 0x80000000u, 0x80000000u);
+            reinterpret_cast<int4*>(ch)[i] = make_int4(0, 0, 0, 0);
         }
         __syncthreads();
         const float iph = P.ip_hi, ipl = P.ip_lo;
@@ -358,87 +370,88 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spec_spread(const SpecArgs a
         // folded interval of the differences that touch the segment (window half-width 4, half-cell centres)
         const int flo = A - 5 > 0 ? A - 5 : 0, fhi = B + 5 < H ? B + 5 : H;
         for (int r = 0; (uint64_t)r * (uint64_t)H << 32 <= span; r++) {
-            const uint64_t ulo = (r & 1) ? (uint64_t)(r + 1) * H - fhi : (uint64_t)r * H + flo;
-            const uint64_t uhi = (r & 1) ? (uint64_t)(r + 1) * H - flo : (uint64_t)r * H + fhi;
-            if ((ulo << 32) > span) continue;
-            // pairs per row, prefix over the rows
-            const int per = (n + kSpreadThreads - 1) / kSpreadThreads;
-            const int i0 = tid * per, i1 = min(n, i0 + per);
-            int sum = 0;
-            for (int i = i0; i < i1; i++) {
-                const uint64_t xi = X[i];
-                const int lo = lower_bound_x(X, i + 1, n, xi + (ulo << 32));
-                const int hi = lower_bound_x(X, lo, n, xi + (uhi << 32));
-                jlo[i] = lo;
-                pre[i + 1] = hi - lo;
-                sum += hi - lo;
-            }
-            int incl = sum;
+            const bool odd = r & 1;
+            const uint64_t ulo = (odd ? (uint64_t)(r + 1) * H - fhi : (uint64_t)r * H + flo) << 32;
+            const uint64_t uhi = (odd ? (uint64_t)(r + 1) * H - flo : (uint64_t)r * H + fhi) << 32;
+            if (ulo > span) continue;
+            // cell position of a difference d: +-(d - fold) less half a cell, relative to A - margin
+            const uint64_t fold = (uint64_t)(odd ? r + 1 : r) * (uint64_t)H << 32;
+            const uint64_t shift = ((uint64_t)(uint32_t)(kSpreadMargin - A) << 32) - 0x80000000ull;
+            for (int g = warp; g * kSpreadRows < n; g += kSpreadThreads / 32) {
+                const int row = min(g * kSpreadRows + (lane & (kSpreadRows - 1)), n - 1);
+                const int bound = lower_bound_x(X, row + 1, n, X[row] + (lane < kSpreadRows ? ulo : uhi));
+                int cnt = __shfl_down_sync(0xffffffffu, bound, kSpreadRows) - bound;   // lanes below kSpreadRows
+                if (lane >= kSpreadRows || g * kSpreadRows + lane >= n) cnt = 0;
+                int incl = cnt;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            if (lane == 31) s_wsum[warp] = incl;
-            __syncthreads();
-            int base = 0;
-            for (int w = 0; w < warp; w++) base += s_wsum[w];
-            int run = base + incl - sum;
-            for (int i = i0; i < i1; i++) {
-                run += pre[i + 1];
-                pre[i + 1] = run;
-            }
-            if (tid == 0) pre[0] = 0;
-            __syncthreads();
-            const int np = pre[n];
-            const uint64_t fold = (uint64_t)((r & 1) ? r + 1 : r) * (uint64_t)H << 32;
-            for (int p0 = warp * 32; p0 < np; p0 += kSpreadThreads) {
-                // row of the warp's first pair by bisection, then a short walk per lane
-                int lo = 0, hi = n - 1;
-                while (lo < hi) {
-                    const int m = (lo + hi + 1) >> 1;
-                    if (pre[m] <= p0) lo = m; else hi = m - 1;
+                for (int o = 1; o < kSpreadRows; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += t;
                 }
-                const int p = p0 + lane;
-                if (p >= np) continue;
-                int i = lo;
-                while (pre[i + 1] <= p) i++;
-                const int j = jlo[i] + (p - pre[i]);
-                const uint64_t d = X[j] - X[i];
-                const uint64_t u = ((r & 1) ? fold - d : d - fold) - 0x80000000ull;    // cells from the first centre
-                const int l = (int)((int64_t)u >> 32);
-                const float z = (float)(uint32_t)u * 2.3283064365386963e-10f - 0.5f;
-                float w = ((gauss_g(Y[i], Y[j]) - iph) - ipl) * kQuanta;
-                if (INTERP) w *= kb_inverse(((float)l + (z + 1.0f)) * inv_h);
-                float q[8];
-                kb_weights(z, q);
-                const int l0 = l - 3 - A;
+                const int np = __shfl_sync(0xffffffffu, incl, kSpreadRows - 1);
+                const int start = bound - (incl - cnt);      // j of pair p of this row: start + p
+                for (int p0 = 0; p0 < np; p0 += 32) {
+                    const int p = p0 + lane;
+                    // row of pair p: how many rows end at or before it
+                    int q = 0;
 #pragma unroll
-                for (int k = 0; k < 8; k++) {
-                    const int v = __float2int_rn(w * q[k]);
-                    int t = l0 + k;                                  // cell relative to A
-                    if (t + A < 0) t = -1 - (t + A) - A;             // folds at 0 and at half the period
-                    else if (t + A >= H) t = 2 * H - 1 - (t + A) - A;
-                    if ((unsigned)t < (unsigned)(B - A)) {
-                        const uint32_t old = atomicAdd(&cl[t], (uint32_t)v);
-                        const int up = (v >> 31) + (old + (uint32_t)v < old ? 1 : 0);
-                        if (up) atomicAdd(&ch[t], up);
+                    for (int o = kSpreadRows / 2; o > 0; o >>= 1) {
+                        const int e = __shfl_sync(0xffffffffu, incl, q + o - 1);
+                        if (e <= p) q += o;
+                    }
+                    const int j = __shfl_sync(0xffffffffu, start, q) + p;
+                    if (p < np) {
+                        const int i = g * kSpreadRows + q;
+                        const uint64_t d = X[j] - X[i];
+                        const uint64_t u = (odd ? fold - d : d - fold) + shift;
+                        const int t = (int)(u >> 32);
+                        const float z = (float)(uint32_t)u * 2.3283064365386963e-10f - 0.5f;
+                        float w = ((gauss_g(Y[i], Y[j]) - iph) - ipl) * kQuanta;
+                        if (INTERP) w *= kb_inverse(((float)(t + A - kSpreadMargin) + (z + 1.0f)) * inv_h);
+                        float k[8];
+                        kb_weights(z, k);
+                        if ((unsigned)(t - 3) <= (unsigned)(len + 2 * kSpreadMargin - 8)) {
+                            uint32_t* at = cl + (t - 3);
+                            int up[8], any = 0;
+#pragma unroll
+                            for (int m = 0; m < 8; m++) {
+                                const int v = __float2int_rn(w * k[m]);
+                                const uint32_t old = atomicAdd(at + m, (uint32_t)v);
+                                up[m] = (v >> 31) + (old + (uint32_t)v < old ? 1 : 0);
+                                any |= up[m];
+                            }
+                            if (any) {
+#pragma unroll
+                                for (int m = 0; m < 8; m++)
+                                    if (up[m]) atomicAdd(ch + (t - 3) + m, up[m]);
+                            }
+                        }
                     }
                 }
             }
-            __syncthreads();
         }
         __syncthreads();
         // cells 4b .. 4b + 3 in the order of the half-length transform: g[2j] at j, g[2j+1] from the
         // end, two reals per complex value
         float2* x = a.x + (int64_t)ci * a.x_ld;
         const int Q = H >> 1;
-        for (int b = tid; b < (B - A) >> 2; b += kSpreadThreads) {
-            float g[4];
+        auto cell = [&](int t) {
+            return fmaf((float)ch[t], 16.0f, (float)(int)(cl[t] - 0x80000000u) * (1.0f / kQuanta));
+        };
+        for (int b = tid; b < len >> 2; b += kSpreadThreads) {
+            const int4 h = reinterpret_cast<const int4*>(ch + kSpreadMargin)[b];
+            const uint4 l = reinterpret_cast<const uint4*>(cl + kSpreadMargin)[b];
+            float g[4] = {fmaf((float)h.x, 16.0f, (float)(int)(l.x - 0x80000000u) * (1.0f / kQuanta)),
+                          fmaf((float)h.y, 16.0f, (float)(int)(l.y - 0x80000000u) * (1.0f / kQuanta)),
+                          fmaf((float)h.z, 16.0f, (float)(int)(l.z - 0x80000000u) * (1.0f / kQuanta)),
+                          fmaf((float)h.w, 16.0f, (float)(int)(l.w - 0x80000000u) * (1.0f / kQuanta))};
+            if (A == 0 && b < kSpreadMargin / 4) {            // cell -1 - i folds to cell i
 #pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const long long v = ((long long)ch[4 * b + q] << 32) + (long long)cl[4 * b + q] - 0x80000000ll;
-                g[q] = (float)v * (1.0f / kQuanta);
+                for (int m = 0; m < 4; m++) g[m] += cell(kSpreadMargin - 1 - (4 * b + m));
+            }
+            if (B == H && 4 * b + 4 > len - kSpreadMargin) {  // cell H + i folds to cell H - 1 - i
+#pragma unroll
+                for (int m = 0; m < 4; m++) g[m] += cell(kSpreadMargin + 2 * len - 1 - (4 * b + m));
             }
             const int bb = (A >> 2) + b;
             x[bb] = make_float2(g[0], g[2]);
@@ -449,91 +462,115 @@ __global__ void __launch_bounds__(kSpreadThreads) k_spec_spread(const SpecArgs a
 
 // ===========================================================================
 // Complex transforms in registers and shared memory.  512 threads hold 8192
-// points, 16 each: radix-16 steps, the last one 2, 4 or 8.
+// points, 16 each: radix-16 steps, the last one 2, 4 or 8.  Complex values are
+// f32x2 pairs, so an addition is one instruction; 64 registers a thread let two
+// CTAs share an SM, one's loads and barriers under the other's arithmetic.
 // ===========================================================================
 constexpr int kFftThreads = 512;
 constexpr int kFftPoints = 16 * kFftThreads;
-constexpr int kTwLog = 13;                       // twiddle table exp(-2 pi i k / 8192)
 
-__device__ __forceinline__ float2 cmul(float2 a, float2 b)
+typedef f2 cx;                                   // (re, im)
+__device__ __forceinline__ cx cadd(cx a, cx b) { return add2(a, b); }
+__device__ __forceinline__ cx csub(cx a, cx b) { return fma2(b, pk(-1.f, -1.f), a); }
+__device__ __forceinline__ cx cmul(cx a, cx b)
 {
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+    float ax, ay, bx, by;
+    upk(a, ax, ay);
+    upk(b, bx, by);
+    return fma2(pk(ax, ax), b, mul2(pk(ay, ay), pk(-by, bx)));
 }
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cmi(float2 a) { return make_float2(a.y, -a.x); }   // times -i
-
-__device__ __forceinline__ void dft4(float2& a, float2& b, float2& c, float2& d)
+__device__ __forceinline__ cx cmi(cx a)          // times -i
 {
-    const float2 s0 = cadd(a, c), s1 = csub(a, c), s2 = cadd(b, d), s3 = cmi(csub(b, d));
+    float x, y;
+    upk(a, x, y);
+    return pk(y, -x);
+}
+
+__device__ __forceinline__ void dft4(cx& a, cx& b, cx& c, cx& d)
+{
+    const cx s0 = cadd(a, c), s1 = csub(a, c), s2 = cadd(b, d), s3 = csub(b, d);
     a = cadd(s0, s2);
-    b = cadd(s1, s3);
     c = csub(s0, s2);
-    d = csub(s1, s3);
+    float x1, y1, x3, y3;
+    upk(s1, x1, y1);
+    upk(s3, x3, y3);
+    b = pk(x1 + y3, y1 - x3);                    // s1 - i s3
+    d = pk(x1 - y3, y1 + x3);
 }
 
 template <int R>
-__device__ __forceinline__ void dft(float2* v)
+__device__ __forceinline__ void dft(cx* v)
 {
+    constexpr float h = 0.70710678118654752f;
     if constexpr (R == 2) {
-        const float2 t = csub(v[0], v[1]);
+        const cx t = csub(v[0], v[1]);
         v[0] = cadd(v[0], v[1]);
         v[1] = t;
     } else if constexpr (R == 4) {
         dft4(v[0], v[1], v[2], v[3]);
     } else if constexpr (R == 8) {
-        const float h = 0.70710678118654752f;
         dft4(v[0], v[2], v[4], v[6]);
         dft4(v[1], v[3], v[5], v[7]);
-        // after: even part E_k = v[2k], odd part O_k = v[2k + 1]
-        const float2 o0 = v[1], o1 = make_float2(h * (v[3].x + v[3].y), h * (v[3].y - v[3].x)), o2 = cmi(v[5]),
-                     o3 = make_float2(h * (v[7].y - v[7].x), -h * (v[7].x + v[7].y));
-        const float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
+        // even part E_k = v[2k], odd part O_k = v[2k + 1]
+        const cx o0 = v[1], o1 = cmul(v[3], pk(h, -h)), o2 = cmi(v[5]), o3 = cmul(v[7], pk(-h, -h));
+        const cx e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
         v[0] = cadd(e0, o0); v[4] = csub(e0, o0);
         v[1] = cadd(e1, o1); v[5] = csub(e1, o1);
         v[2] = cadd(e2, o2); v[6] = csub(e2, o2);
         v[3] = cadd(e3, o3); v[7] = csub(e3, o3);
     } else {
-        constexpr float c1 = 0.92387953251128674f, s1 = 0.38268343236508977f, h = 0.70710678118654752f;
+        constexpr float c1 = 0.92387953251128674f, s1 = 0.38268343236508977f;
 #pragma unroll
         for (int k = 0; k < 4; k++) dft4(v[k], v[k + 4], v[k + 8], v[k + 12]);
         // v[k + 4 q] holds part q of column k: twiddle exp(-2 pi i k q / 16), then across the columns
-        v[5] = cmul(v[5], make_float2(c1, -s1));
-        v[9] = cmul(v[9], make_float2(h, -h));
-        v[13] = cmul(v[13], make_float2(s1, -c1));
-        v[6] = cmul(v[6], make_float2(h, -h));
+        v[5] = cmul(v[5], pk(c1, -s1));
+        v[9] = cmul(v[9], pk(h, -h));
+        v[13] = cmul(v[13], pk(s1, -c1));
+        v[6] = cmul(v[6], pk(h, -h));
         v[10] = cmi(v[10]);
-        v[14] = cmul(v[14], make_float2(-h, -h));
-        v[7] = cmul(v[7], make_float2(s1, -c1));
-        v[11] = cmul(v[11], make_float2(-h, -h));
-        v[15] = cmul(v[15], make_float2(-c1, s1));
-        float2 o[16];
+        v[14] = cmul(v[14], pk(-h, -h));
+        v[7] = cmul(v[7], pk(s1, -c1));
+        v[11] = cmul(v[11], pk(-h, -h));
+        v[15] = cmul(v[15], pk(-c1, s1));
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            dft4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        for (int q = 0; q < 4; q++) dft4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        // transpose: output q + 4 k from v[4 q + k]
 #pragma unroll
-            for (int k = 0; k < 4; k++) o[q + 4 * k] = v[4 * q + k];
-        }
+        for (int q = 0; q < 4; q++)
 #pragma unroll
-        for (int q = 0; q < 16; q++) v[q] = o[q];
+            for (int k = q + 1; k < 4; k++) {
+                const cx t = v[4 * q + k];
+                v[4 * q + k] = v[4 * k + q];
+                v[4 * k + q] = t;
+            }
     }
 }
 
-// Column c, element i of the block's 8192 points in shared memory (one pad
-// every 16 elements): columns fastest in the first pass, elements in the second.
+// Twiddle factors exp(-2 pi i r k / (NS R)) of a step of radix R after NS points:
+// [r - 1][k], k < NS, so that a warp's loads are consecutive.  Tables in one
+// array: (16, 16), (16, 8), (256, 2), (256, 4), (256, 8), (256, 16), (4096, 2).
+__host__ __device__ constexpr int tw_offset(int ns, int r)
+{
+    return ns == 16    ? (r == 16 ? 0 : 240)
+           : ns == 256 ? 352 + 256 * (r == 2 ? 0 : r == 4 ? 1 : r == 8 ? 4 : 11)
+                       : 352 + 256 * 26;
+}
+
+// Column c, element i of the block's 8192 points in shared memory (a pad every
+// 16 elements; columns fastest in the first pass, elements in the second, whose
+// columns start 4 elements apart in the banks).
 template <int LOGN, bool CFAST>
 __device__ __forceinline__ int fft_addr(int c, int i)
 {
     constexpr int N = 1 << LOGN, C = kFftPoints / N;
-    return CFAST ? (i + (i >> 4)) * C + c : c * (N + N / 16) + i + (i >> 4);
+    return CFAST ? (i + (i >> 4)) * C + c : c * (N + N / 16 + 4) + i + (i >> 4);
 }
 
-// On entry v[r] = element j + r N/16 of column c (j < N/16).  On return the
-// transform's elements are in shared memory (LAST_IN_SMEM) or in v: v[b R + r]
-// = element j + b N/16 + r N/R, R the last radix.  `on` masks idle threads
-// (every thread takes the barriers).
+// On entry v[r] = element j + r N/16 of column c (j < N/16).  On return v[b R + r]
+// = element j + b N/16 + r N/R of the transform, R the last radix.  `on` masks
+// idle threads (every thread takes the barriers).
 template <int LOGN, int DONE, bool CFAST>
-__device__ __forceinline__ void fft_rest(float2* v, float2* sm, const float2* __restrict__ tw, int c, int j, bool on)
+__device__ __forceinline__ void fft_rest(cx* v, cx* sm, const cx* __restrict__ tw, int c, int j, bool on)
 {
     constexpr int N = 1 << LOGN, NT = N / 16;
     constexpr int LEFT = LOGN - DONE;                 // bits still to do
@@ -552,7 +589,7 @@ __device__ __forceinline__ void fft_rest(float2* v, float2* sm, const float2* __
             const int k = (j + b * NT) & (NS - 1);
 #pragma unroll
             for (int r = 1; r < R; r++)
-                v[b * R + r] = cmul(v[b * R + r], __ldg(tw + ((r * k) << (kTwLog - DONE - (LEFT >= 4 ? 4 : LEFT)))));
+                v[b * R + r] = cmul(v[b * R + r], __ldg(tw + tw_offset(NS, R) + (r - 1) * NS + k));
             dft<R>(v + b * R);
         }
         if constexpr (LEFT > 4) {
@@ -571,7 +608,7 @@ __device__ __forceinline__ void fft_rest(float2* v, float2* sm, const float2* __
 }
 
 template <int LOGN, bool CFAST>
-__device__ __forceinline__ void fft_block(float2* v, float2* sm, const float2* __restrict__ tw, int c, int j, bool on)
+__device__ __forceinline__ void fft_block(cx* v, cx* sm, const cx* __restrict__ tw, int c, int j, bool on)
 {
     dft<16>(v);
     if (on) {
@@ -582,47 +619,79 @@ __device__ __forceinline__ void fft_block(float2* v, float2* sm, const float2* _
 }
 
 // exp(-2 pi i U / 2^32)
-__device__ __forceinline__ float2 cis_neg(uint32_t U)
+__device__ __forceinline__ cx cis_neg(uint32_t U)
 {
     float s, c;
     sincos2pi_turns(U, s, c);
-    return make_float2(c, -s);
+    return pk(c, -s);
 }
 
-constexpr int fft_smem_floats2() { return kFftPoints + kFftPoints / 16; }
+// sin and cos of x, |x| <= pi / 4, by Taylor polynomials (remainders below 2e-9)
+__device__ __forceinline__ void sincos_small(float x, float& s, float& c)
+{
+    const float x2 = x * x;
+    float p = fmaf(x2, 1.0f / 362880.0f, -1.0f / 5040.0f);
+    p = fmaf(x2, p, 1.0f / 120.0f);
+    p = fmaf(x2, p, -1.0f / 6.0f);
+    s = fmaf(x2 * x, p, x);
+    float q = fmaf(x2, -1.0f / 3628800.0f, 1.0f / 40320.0f);
+    q = fmaf(x2, q, -1.0f / 720.0f);
+    q = fmaf(x2, q, 1.0f / 24.0f);
+    q = fmaf(x2, q, -0.5f);
+    c = fmaf(x2, q, 1.0f);
+}
+
+// Bits of the second pass's length.  512 points make 16 rows of a block, so its
+// eight mirror pairs write 32-byte runs; longer ones only where the first pass
+// would exceed 2048.
+__host__ __device__ constexpr int spec_log2(int logq)
+{
+    return logq >= 20 ? (logq - 11 > 9 ? logq - 11 : 9) : logq >= 18 ? 9 : logq >> 1;
+}
+
+constexpr int fft_smem_floats2() { return kFftPoints + kFftPoints / 16 + 4 * 64; }
 
 template <int LOGN>
-__device__ __forceinline__ void fft1_item(const SpecArgs& a, const SpecCurve& S, float2* x, int blk, float2* sm)
+__device__ __forceinline__ void fft1_item(const SpecArgs& a, const SpecCurve& S, cx* x, int blk, cx* sm)
 {
     constexpr int N = 1 << LOGN, C = kFftPoints / N, NT = N / 16;
     constexpr int LEFT = (LOGN & 3) == 0 ? 4 : (LOGN & 3);
     constexpr int R = 1 << LEFT, B = 16 / R;
     const int tid = threadIdx.x, c = tid % C, j = tid / C;
-    const int Q = 1 << S.logq, log2q = S.logq - LOGN, Q2 = 1 << log2q;
+    const int Q = 1 << S.logq, log2q = S.logq - LOGN;
     const int col = blk * C + c;
     const int zlo = S.support >> 2, zhi = Q - zlo;       // x is zero in [zlo, zhi)
-    float2 v[16];
+    cx v[16];
 #pragma unroll
     for (int r = 0; r < 16; r++) {
         const int l = ((j + r * NT) << log2q) + col;
-        v[r] = l < zlo || l >= zhi ? x[l] : make_float2(0.f, 0.f);
+        v[r] = l < zlo || l >= zhi ? x[l] : 0ull;
     }
-    fft_block<LOGN, true>(v, sm, a.tw, c, j, true);
+    fft_block<LOGN, true>(v, sm, reinterpret_cast<const cx*>(a.tw), c, j, true);
+    // times exp(-2 pi i k1 col / Q), k1 = j + b NT + r N/R: one sine and cosine each for j, NT and N/R,
+    // the others by products
+    const int sh = 32 - S.logq;
+    const cx sr = cis_neg((uint32_t)((N / R) * col) << sh);
+    const cx sb = B > 1 ? cis_neg((uint32_t)(NT * col) << sh) : 0ull;
+    cx wb = cis_neg((uint32_t)(j * col) << sh);
+    cx* xo = x + ((int64_t)j << log2q) + col;
 #pragma unroll
-    for (int b = 0; b < B; b++)
+    for (int b = 0; b < B; b++) {
+        cx w = wb;
 #pragma unroll
         for (int r = 0; r < R; r++) {
-            const int k1 = j + b * NT + r * (N / R);
-            const uint32_t m = (uint32_t)(k1 * col) & (uint32_t)(Q - 1);
-            x[(k1 << log2q) + col] = cmul(v[b * R + r], cis_neg(m << (32 - S.logq)));
+            xo[(b * NT + r * (N / R)) << log2q] = cmul(v[b * R + r], w);
+            if (r + 1 < R)      // every fourth afresh: products of at most three roundings
+                w = (r & 3) == 3 ? cis_neg((uint32_t)((j + b * NT + (r + 1) * (N / R)) * col) << sh) : cmul(w, sr);
         }
-    (void)Q2;
+        if (b + 1 < B) wb = cmul(wb, sb);
+    }
 }
 
-__global__ void __launch_bounds__(kFftThreads) k_spec_fft1(const SpecArgs a)
+__global__ void __launch_bounds__(kFftThreads, 2) k_spec_fft1(const SpecArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    float2* sm = reinterpret_cast<float2*>(smem);
+    cx* sm = reinterpret_cast<cx*>(smem);
     __shared__ int s_pre[kSpecMaxChunk + 1];
     const int nc = a.slot_end - a.slot_begin;
     item_prefix(s_pre, nc, [&](int i) {
@@ -632,9 +701,9 @@ __global__ void __launch_bounds__(kFftThreads) k_spec_fft1(const SpecArgs a)
     for (int item = blockIdx.x; item < s_pre[nc]; item += gridDim.x) {
         const int ci = item_curve(s_pre, nc, item);
         const SpecCurve S = a.sc[a.order[a.slot_begin + ci]];
-        float2* x = a.x + (int64_t)ci * a.x_ld;
+        cx* x = reinterpret_cast<cx*>(a.x + (int64_t)ci * a.x_ld);
         const int blk = item - s_pre[ci];
-        switch ((S.logq + 1) >> 1) {
+        switch (S.logq - spec_log2(S.logq)) {
         case 7: fft1_item<7>(a, S, x, blk, sm); break;
         case 8: fft1_item<8>(a, S, x, blk, sm); break;
         case 9: fft1_item<9>(a, S, x, blk, sm); break;
@@ -648,35 +717,35 @@ __global__ void __launch_bounds__(kFftThreads) k_spec_fft1(const SpecArgs a)
 // The four pair-spectrum values of X[m] and X[Q - m] (x the transform of the
 // packed reals): V the half-length real transform, C[m] = Re(c_m V[m]),
 // C[H - m] = -Im(c_m V[m]), c_m = exp(-i pi m / (2 H)).
-__device__ __forceinline__ void spec_emit(const SpecCurve& S, float* P, int m, float2 xa, float2 xb)
+__device__ __forceinline__ void spec_emit(const SpecCurve& S, float* P, int m, cx pa, cx pb)
 {
     const int Q = 1 << S.logq, H = 2 * Q;
-    const float inv_h = 1.0f / (float)H;
-    const float2 E = make_float2(0.5f * (xa.x + xb.x), 0.5f * (xa.y - xb.y));
-    const float2 O = make_float2(0.5f * (xa.y + xb.y), -0.5f * (xa.x - xb.x));
-    const float2 c4 = cis_neg((uint32_t)m << (31 - S.logq));                  // exp(-2 pi i m / H)
-    const float2 cm = cis_neg((uint32_t)m << (29 - S.logq));                  // exp(-2 pi i m / (4 H))
-    const float2 WO = cmul(c4, O);
-    const float2 v1 = cmul(cm, cadd(E, WO));
-    const float2 d = csub(E, WO);
-    // V[Q - m] = conj(E - W O), c_{Q-m} = exp(-i pi / 4) conj(c_m)
+    const float inv_h = 1.0f / (float)H, fm = (float)m;      // m <= Q / 2 (or the row Q1 / 2's up to Q)
+    float xa, ya, xb, yb;
+    upk(pa, xa, ya);
+    upk(pb, xb, yb);
+    const float ex = 0.5f * (xa + xb), ey = 0.5f * (ya - yb), ox = 0.5f * (ya + yb), oy = -0.5f * (xa - xb);
+    float s4, c4, sm_, cm;
+    sincos2pi_turns((uint32_t)m << (31 - S.logq), s4, c4);
+    sincos_small((float)(0.5 * CP_PI) * fm * inv_h, sm_, cm);                // pi m / (2 H) <= pi / 4
+    const float wx = fmaf(c4, ox, s4 * oy), wy = fmaf(c4, oy, -s4 * ox);     // exp(-i a) O
+    // V[m] = E + W O times c_m = exp(-i pi m / (2 H)); V[Q - m] = conj(E - W O), c_{Q-m} = exp(-i pi/4) conj(c_m)
     const float h = 0.70710678118654752f;
-    const float2 cq = make_float2(h * (cm.x - cm.y), -h * (cm.x + cm.y));
-    const float2 v2 = cmul(cq, make_float2(d.x, -d.y));
-    const int m1 = m, m2 = Q - m, m3 = H - m, m4 = Q + m;
-    if (m1 < S.n_out) {
-        const float p = v1.x * kb_inverse((float)m1 * inv_h);
-        P[m1] = p;
-        if (m1 <= 4) P[-m1] = p;                          // the interpolation reads across 0
+    const float ux = ex + wx, uy = ey + wy, dx = ex - wx, dy = wy - ey;
+    const float qx = h * (cm + sm_), qy = h * (sm_ - cm);
+    const int m2 = Q - m, m3 = H - m, m4 = Q + m;
+    if (m < S.n_out) {
+        const float p = fmaf(cm, ux, sm_ * uy) * kb_inverse(fm * inv_h);
+        P[m] = p;
+        if (m <= 4) P[-m] = p;                            // the interpolation reads across 0
     }
-    if (m2 < S.n_out) P[m2] = v2.x * kb_inverse((float)m2 * inv_h);
-    if (m3 < S.n_out) P[m3] = -v1.y * kb_inverse((float)m3 * inv_h);
-    if (m4 < S.n_out) P[m4] = -v2.y * kb_inverse((float)m4 * inv_h);
+    if (m2 < S.n_out) P[m2] = fmaf(qx, dx, -qy * dy) * kb_inverse((float)m2 * inv_h);
+    if (m3 < S.n_out) P[m3] = fmaf(sm_, ux, -cm * uy) * kb_inverse((float)m3 * inv_h);
+    if (m4 < S.n_out) P[m4] = -fmaf(qx, dy, qy * dx) * kb_inverse((float)m4 * inv_h);
 }
 
 template <int LOGN>
-__device__ __forceinline__ void fft2_item(const SpecArgs& a, const SpecCurve& S, const float2* x, float* P, int blk,
-                                          float2* sm)
+__device__ __forceinline__ void fft2_item(const SpecArgs& a, const SpecCurve& S, const cx* x, float* P, int blk, cx* sm)
 {
     constexpr int N = 1 << LOGN, C = kFftPoints / N, NT = N / 16;
     constexpr int LEFT = (LOGN & 3) == 0 ? 4 : (LOGN & 3);
@@ -687,10 +756,10 @@ __device__ __forceinline__ void fft2_item(const SpecArgs& a, const SpecCurve& S,
     // rows a0 .. a0 + C/2 - 1 and their mirror rows Q1 - a (row 0 with row Q1 / 2: each its own mirror)
     const int ar = a0 + (c < C / 2 ? c : c - C / 2);
     const int row = c < C / 2 ? ar : (ar == 0 ? Q1 >> 1 : Q1 - ar);
-    float2 v[16];
+    cx v[16];
 #pragma unroll
     for (int r = 0; r < 16; r++) v[r] = x[((int64_t)row << LOGN) + j + r * NT];
-    fft_block<LOGN, false>(v, sm, a.tw, c, j, true);
+    fft_block<LOGN, false>(v, sm, reinterpret_cast<const cx*>(a.tw), c, j, true);
     __syncthreads();
 #pragma unroll
     for (int b = 0; b < B; b++)
@@ -713,10 +782,10 @@ __device__ __forceinline__ void fft2_item(const SpecArgs& a, const SpecCurve& S,
     }
 }
 
-__global__ void __launch_bounds__(kFftThreads) k_spec_fft2(const SpecArgs a)
+__global__ void __launch_bounds__(kFftThreads, 2) k_spec_fft2(const SpecArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    float2* sm = reinterpret_cast<float2*>(smem);
+    cx* sm = reinterpret_cast<cx*>(smem);
     __shared__ int s_pre[kSpecMaxChunk + 1];
     const int nc = a.slot_end - a.slot_begin;
     item_prefix(s_pre, nc, [&](int i) {
@@ -726,10 +795,10 @@ __global__ void __launch_bounds__(kFftThreads) k_spec_fft2(const SpecArgs a)
     for (int item = blockIdx.x; item < s_pre[nc]; item += gridDim.x) {
         const int ci = item_curve(s_pre, nc, item);
         const SpecCurve S = a.sc[a.order[a.slot_begin + ci]];
-        const float2* x = a.x + (int64_t)ci * a.x_ld;
+        const cx* x = reinterpret_cast<const cx*>(a.x + (int64_t)ci * a.x_ld);
         float* P = a.P + (int64_t)ci * a.p_ld + kSpecPad;
         const int blk = item - s_pre[ci];
-        switch (S.logq >> 1) {
+        switch (spec_log2(S.logq)) {
         case 7: fft2_item<7>(a, S, x, P, blk, sm); break;
         case 8: fft2_item<8>(a, S, x, P, blk, sm); break;
         case 9: fft2_item<9>(a, S, x, P, blk, sm); break;
@@ -742,7 +811,7 @@ __global__ void __launch_bounds__(kFftThreads) k_spec_fft2(const SpecArgs a)
 
 // Short transforms (Q <= 8192): one CTA per curve, both passes in one.
 template <int LOGN>
-__device__ __forceinline__ void fft_one(const SpecArgs& a, const SpecCurve& S, const float2* x, float* P, float2* sm)
+__device__ __forceinline__ void fft_one(const SpecArgs& a, const SpecCurve& S, const cx* x, float* P, cx* sm)
 {
     constexpr int N = 1 << LOGN, NT = N / 16;
     constexpr int LEFT = (LOGN & 3) == 0 ? 4 : (LOGN & 3);
@@ -751,13 +820,13 @@ __device__ __forceinline__ void fft_one(const SpecArgs& a, const SpecCurve& S, c
     const bool on = tid < NT;
     const int j = on ? tid : 0;
     const int zlo = S.support >> 2, zhi = N - zlo;
-    float2 v[16];
+    cx v[16];
 #pragma unroll
     for (int r = 0; r < 16; r++) {
         const int l = j + r * NT;
-        v[r] = l < zlo || l >= zhi ? x[l] : make_float2(0.f, 0.f);
+        v[r] = l < zlo || l >= zhi ? x[l] : 0ull;
     }
-    fft_block<LOGN, false>(v, sm, a.tw, 0, j, on);
+    fft_block<LOGN, false>(v, sm, reinterpret_cast<const cx*>(a.tw), 0, j, on);
     __syncthreads();
     if (on) {
 #pragma unroll
@@ -770,14 +839,14 @@ __device__ __forceinline__ void fft_one(const SpecArgs& a, const SpecCurve& S, c
         spec_emit(S, P, k, sm[fft_addr<LOGN, false>(0, k)], sm[fft_addr<LOGN, false>(0, (N - k) & (N - 1))]);
 }
 
-__global__ void __launch_bounds__(kFftThreads) k_spec_fft_one(const SpecArgs a)
+__global__ void __launch_bounds__(kFftThreads, 2) k_spec_fft_one(const SpecArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    float2* sm = reinterpret_cast<float2*>(smem);
+    cx* sm = reinterpret_cast<cx*>(smem);
     const int ci = blockIdx.x;
     const SpecCurve S = a.sc[a.order[a.slot_begin + ci]];
     if (!S.nh || S.logq > kSpecOneLogQ) return;
-    const float2* x = a.x + (int64_t)ci * a.x_ld;
+    const cx* x = reinterpret_cast<const cx*>(a.x + (int64_t)ci * a.x_ld);
     float* P = a.P + (int64_t)ci * a.p_ld + kSpecPad;
     switch (S.logq) {
     case 8: fft_one<8>(a, S, x, P, sm); break;
@@ -851,6 +920,7 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_sum(const SpecArgs a)
 #pragma unroll
             for (int w = 1; w < kSumThreads / 32; w++) key = max(key, s_key[w]);
             if (key) atomicMax(a.vmax + c, key);
+            a.vblk[(int64_t)ci * a.vb_ld + (item - s_pre[ci])] = key;
         }
         __syncthreads();
     }
@@ -936,6 +1006,7 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
 #pragma unroll
             for (int w = 1; w < kSumThreads / 32; w++) key = max(key, s_key[w]);
             if (key) atomicMax(a.vmax + c, key);
+            a.vblk[(int64_t)ci * a.vb_ld + (item - s_pre[ci])] = key;
         }
         __syncthreads();
     }
@@ -976,8 +1047,8 @@ __device__ __forceinline__ void write_sorted(const int32_t* s_k, int n, int32_t*
 
 __global__ void __launch_bounds__(kSelThreads) k_spec_select(const SpecArgs a)
 {
-    __shared__ int s_n;
-    __shared__ int32_t s_k[kSpecCand];
+    __shared__ int s_n, s_hot;
+    __shared__ int32_t s_k[kSpecCand], s_blk[kSpecCand];
     const int ci = blockIdx.x, tid = threadIdx.x;
     const int c = a.order[a.slot_begin + ci];
     const CurveParams& P = a.cp[c];
@@ -986,17 +1057,35 @@ __global__ void __launch_bounds__(kSelThreads) k_spec_select(const SpecArgs a)
     __syncthreads();
     const bool spec = a.sc[c].nh != 0 && !a.sc[c].whole;
     const unsigned int top = a.vmax[c];
+    if (tid == 0) s_hot = 0;
+    __syncthreads();
     if (spec && top) {
         const float v0 = from_orderable(top);
         const float thr = v0 - spec_margin(v0, P);
+        const unsigned int othr = orderable(thr);
         const float* row = a.rows + (a.rows_by_curve ? (int64_t)c : (int64_t)ci) * a.row_ld;
-        const int count = spec_count(a, c);
-        for (int k = tid; k < count; k += kSelThreads) {
-            if (row[k] >= thr) {
-                const int g = a.stage == kSpecList ? a.trials[(int64_t)c * a.n_trials + k] : k;
-                if (a.stage != kSpecFine && excluded_k(a.ex.full_k, a.ex.n, g)) continue;
-                const int pos = atomicAdd(&s_n, 1);
-                if (pos < kSpecCand) s_k[pos] = k;
+        const int count = spec_count(a, c), per = a.interp ? kSumThreads : kSumThreads * kSumPer;
+        // only the blocks whose largest admissible value reaches the threshold are read again
+        for (int b = tid; b * per < count; b += kSelThreads)
+            if (a.vblk[(int64_t)ci * a.vb_ld + b] >= othr) {
+                const int pos = atomicAdd(&s_hot, 1);
+                if (pos < kSpecCand) s_blk[pos] = b;
+            }
+        __syncthreads();
+        const int hot = s_hot;
+        if (hot > kSpecCand) {                       // at least as many entries
+            if (tid == 0) s_n = hot;
+        } else {
+            for (int h = 0; h < hot; h++) {
+                const int k1 = min(count, (s_blk[h] + 1) * per);
+                for (int k = s_blk[h] * per + tid; k < k1; k += kSelThreads) {
+                    if (row[k] >= thr) {
+                        const int g = a.stage == kSpecList ? a.trials[(int64_t)c * a.n_trials + k] : k;
+                        if (a.stage != kSpecFine && excluded_k(a.ex.full_k, a.ex.n, g)) continue;
+                        const int pos = atomicAdd(&s_n, 1);
+                        if (pos < kSpecCand) s_k[pos] = k;
+                    }
+                }
             }
         }
     }
@@ -1016,11 +1105,14 @@ __global__ void __launch_bounds__(kSelThreads) k_spec_select(const SpecArgs a)
 // every other comparison is decided by more than the margin.
 // ===========================================================================
 constexpr int kPeakRaw = 256;
+constexpr int kPeakThreads = 1024;
+constexpr int kPeakRow = 24576;                  // row points kept in shared memory
 
-__global__ void __launch_bounds__(kSelThreads) k_spec_peaks(const SpecArgs a)
+__global__ void __launch_bounds__(kPeakThreads) k_spec_peaks(const SpecArgs a)
 {
+    extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned int s_hist[256], s_prefix, s_need;
-    __shared__ float s_max[kSelThreads / 32];
+    __shared__ float s_max[kPeakThreads / 32];
     __shared__ int s_n, s_m;
     __shared__ int32_t s_raw[kPeakRaw], s_k[kSpecCand];
     const int ci = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1037,8 +1129,14 @@ __global__ void __launch_bounds__(kSelThreads) k_spec_peaks(const SpecArgs a)
         }
         return;
     }
+    if (K <= kPeakRow) {
+        float* row = reinterpret_cast<float*>(smem);
+        for (int k = tid; k < K; k += kPeakThreads) row[k] = v[k];
+        v = row;
+        __syncthreads();
+    }
     float vm = 0.f;
-    for (int k = tid; k < K; k += kSelThreads) vm = fmaxf(vm, fabsf(v[k]));
+    for (int k = tid; k < K; k += kPeakThreads) vm = fmaxf(vm, fabsf(v[k]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) vm = fmaxf(vm, __shfl_xor_sync(0xffffffffu, vm, o));
     if (lane == 0) s_max[warp] = vm;
@@ -1050,7 +1148,7 @@ __global__ void __launch_bounds__(kSelThreads) k_spec_peaks(const SpecArgs a)
     }
     __syncthreads();
 #pragma unroll
-    for (int w = 0; w < kSelThreads / 32; w++) vm = fmaxf(vm, s_max[w]);
+    for (int w = 0; w < kPeakThreads / 32; w++) vm = fmaxf(vm, s_max[w]);
     const float m = spec_margin(vm, P);
     auto sure = [&](int k) {
         const float x = v[k];
@@ -1060,32 +1158,45 @@ __global__ void __launch_bounds__(kSelThreads) k_spec_peaks(const SpecArgs a)
     bool enough = true;
     for (int pass = 0; pass < 4 && enough; pass++) {
         const int shift = 24 - 8 * pass;
-        for (int i = tid; i < 256; i += kSelThreads) s_hist[i] = 0u;
+        for (int i = tid; i < 256; i += kPeakThreads) s_hist[i] = 0u;
         __syncthreads();
         const unsigned int prefix = s_prefix, need = s_need;
-        for (int k = tid; k < K; k += kSelThreads) {
+        for (int k = tid; k < K; k += kPeakThreads) {
             const unsigned int u = orderable(v[k]);
             if ((pass == 0 || (u >> (shift + 8)) == prefix) && sure(k)) atomicAdd(&s_hist[(u >> shift) & 255u], 1u);
         }
         __syncthreads();
-        if (tid == 0) {
-            unsigned int cum = 0;
-            int d = 255;
-            for (; d >= 0; d--) {
-                if (cum + s_hist[d] >= need) break;
-                cum += s_hist[d];
+        if (warp == 0) {
+            // lane l owns digits 255 - 8l .. 248 - 8l; the one holding the need-th largest
+            unsigned int h[8], sum = 0;
+#pragma unroll
+            for (int x = 0; x < 8; x++) sum += h[x] = s_hist[255 - 8 * lane - x];
+            unsigned int incl = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
             }
-            if (d < 0) s_need = 0u;                      // fewer than top_k (first pass only)
-            else {
-                s_prefix = (prefix << 8) | (unsigned)d;
-                s_need = need - cum;
+            unsigned int cum = incl - sum;
+            if (cum < need && need <= incl) {
+                bool found = false;
+#pragma unroll
+                for (int x = 0; x < 8; x++) {
+                    if (!found && cum + h[x] >= need) {
+                        found = true;
+                        s_prefix = (prefix << 8) | (255u - 8u * lane - x);
+                        s_need = need - cum;
+                    }
+                    cum += h[x];
+                }
             }
+            if (lane == 31 && incl < need) s_need = 0u;      // fewer than top_k (first pass only)
         }
         __syncthreads();
         enough = s_need != 0u;
     }
     const float floor_v = enough ? from_orderable(s_prefix) - m : -INFINITY;
-    for (int k = tid; k < K; k += kSelThreads) {
+    for (int k = tid; k < K; k += kPeakThreads) {
         const float x = v[k];
         if (!(x >= floor_v) || excluded_k(a.ex.coarse_k, a.ex.n, k)) continue;
         const float l = k > 0 ? v[k - 1] : -INFINITY, h = k < K - 1 ? v[k + 1] : -INFINITY;
@@ -1148,34 +1259,53 @@ __global__ void __launch_bounds__(kSpecCand) k_spec_rank(const SpecArgs a)
 // ---------------------------------------------------------------------------
 __global__ void k_spec_twiddle(float2* tw)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    double s, c;
-    sincospi(-2.0 * (double)k / (double)(1 << kTwLog), &s, &c);
-    tw[k] = make_float2((float)c, (float)s);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int ns[7] = {16, 16, 256, 256, 256, 256, 4096}, rr[7] = {16, 8, 2, 4, 8, 16, 2};
+    for (int t = 0; t < 7; t++) {
+        const int e = i - tw_offset(ns[t], rr[t]);
+        if (e >= 0 && e < (rr[t] - 1) * ns[t]) {
+            const int r = e / ns[t] + 1, k = e % ns[t];
+            double s, c;
+            sincospi(-2.0 * (double)(r * k) / (double)(ns[t] * rr[t]), &s, &c);
+            tw[i] = make_float2((float)c, (float)s);
+        }
+    }
 }
 
 cudaError_t launch_spec_twiddle(float2* tw, cudaStream_t s)
 {
-    k_spec_twiddle<<<(1 << kTwLog) / 256, 256, 0, s>>>(tw);
+    static_assert(tw_offset(4096, 2) + 4096 <= kSpecTwiddles, "twiddle tables");
+    k_spec_twiddle<<<kSpecTwiddles / 256, 256, 0, s>>>(tw);
     return cudaGetLastError();
 }
 
 static size_t prep_smem(int np2max) { return (size_t)np2max * (sizeof(double) + sizeof(int32_t)); }
 static size_t fft_smem() { return (size_t)fft_smem_floats2() * sizeof(float2); }
 
+// Shared memory of the spreading kernel: two CTAs share an SM where the curve
+// leaves room for at least 4096 cells each.
 size_t spec_spread_smem(int max_n, int seg)
 {
-    return (size_t)max_n * (sizeof(uint64_t) + sizeof(float)) + 2 * (size_t)(max_n + 1) * sizeof(int) + (size_t)seg * 8;
+    return (size_t)max_n * (sizeof(uint64_t) + sizeof(float)) + 8 * (size_t)(seg + 2 * kSpreadMargin);
 }
 
-cudaError_t spec_prepare(int np2max, int max_n, int seg)
+int spec_seg_max(int max_n)
+{
+    const size_t half = 112 * 1024;
+    int seg = 4096;
+    while (seg < 16384 && spec_spread_smem(max_n, seg + 512) <= half) seg += 512;
+    return seg;
+}
+
+cudaError_t spec_prepare(int np2max, int max_n, int seg_max)
 {
     cudaError_t e = raise_dyn_smem((const void*)k_spec_prep, prep_smem(np2max));
-    if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_spread<false>, spec_spread_smem(max_n, seg));
-    if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_spread<true>, spec_spread_smem(max_n, seg));
+    if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_spread<false>, spec_spread_smem(max_n, seg_max));
+    if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_spread<true>, spec_spread_smem(max_n, seg_max));
     if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_fft1, fft_smem());
     if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_fft2, fft_smem());
     if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_fft_one, fft_smem());
+    if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_spec_peaks, kPeakRow * sizeof(float));
     return e;
 }
 
@@ -1192,7 +1322,7 @@ cudaError_t launch_spec_transform(const SpecArgs& a, int n_sm, int max_n, bool o
     const int n = a.slot_end - a.slot_begin;
     if (n <= 0) return cudaSuccess;
     if (n > kSpecMaxChunk) return cudaErrorInvalidValue;
-    const size_t smem = spec_spread_smem(max_n, a.seg);
+    const size_t smem = spec_spread_smem(max_n, a.seg_max);
     if (a.interp) k_spec_spread<true><<<2 * n_sm, kSpreadThreads, smem, s>>>(a, max_n);
     else k_spec_spread<false><<<2 * n_sm, kSpreadThreads, smem, s>>>(a, max_n);
     cudaError_t e = cudaGetLastError();
@@ -1226,7 +1356,7 @@ cudaError_t launch_spec_select(const SpecArgs& a, cudaStream_t s)
 
 cudaError_t launch_spec_peaks(const SpecArgs& a, cudaStream_t s)
 {
-    k_spec_peaks<<<a.slot_end - a.slot_begin, kSelThreads, 0, s>>>(a);
+    k_spec_peaks<<<a.slot_end - a.slot_begin, kPeakThreads, a.n_freq <= kPeakRow ? (size_t)a.n_freq * sizeof(float) : 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -16,11 +16,12 @@ constexpr int kSpecMaxHarm = 64;       // harmonics kept per curve
 constexpr int kSpecMinLogQ = 8;        // complex transform length 2^logq
 constexpr int kSpecMaxLogQ = 22;
 constexpr int kSpecOneLogQ = 13;       // up to this length one CTA transforms a curve
-constexpr int kSpecCand = 64;          // frequencies per curve evaluated again by the pair sum
-constexpr int kSpecMaxChunk = 64;      // curves per chunk
+constexpr int kSpecCand = kConfirmCand;// frequencies per curve evaluated again by the pair sum
+constexpr int kSpecMaxChunk = kConfirmMaxChunk;   // curves per chunk
 constexpr double kSpecTail = 2e-8;     // harmonics left out: at most this much of the kernel's peak
 constexpr double kSpecOver = 1.1;      // transform length over the highest frequency needed, at least
 
+constexpr int kSpecBlock = 256;        // values per block at least (one item of the value kernels)
 constexpr int kSpecPad = 8;            // pair-spectrum values kept before index 0 (P(-nu) = P(nu))
 
 // Which frequencies a launch evaluates.
@@ -36,6 +37,7 @@ struct SpecCurve {
     int32_t support;        // cells that can be non-zero, a multiple of 4 (H: all)
     int32_t n_out;          // pair-spectrum values needed
     float one_minus_a0;
+    int32_t seg;            // cells per spreading item
     int32_t whole;          // set when a curve's candidates do not fit its list
 };
 
@@ -65,7 +67,8 @@ struct SpecArgs {
     int32_t n_trials;
     int slot_begin, slot_end;     // curves of this launch
     int np2max;
-    int seg;                      // cells per spreading item
+    int seg_max;                  // cells per spreading item at most
+    int seg_items;                // spreading items per curve wanted
     float2* x;                    // chunk workspace: transform data, x_ld per curve
     int64_t x_ld;
     float* P;                     // pair spectrum, p_ld per curve (index 0 at kSpecPad)
@@ -74,6 +77,8 @@ struct SpecArgs {
     int64_t row_ld;
     int rows_by_curve;
     unsigned int* vmax;           // [n_curves] largest admissible value (orderable bits)
+    unsigned int* vblk;           // the same per block of a launch's values, vb_ld per curve of the chunk
+    int64_t vb_ld;
     int32_t* cand;                // [n_curves * kSpecCand] candidate entries, -1 after the last
     int32_t* fb_slots;            // slots that the pair sum evaluates whole
     int* fb_count;
@@ -82,10 +87,10 @@ struct SpecArgs {
     Exclusion ex;
 };
 
-constexpr int kSpecTwiddles = 8192;
+constexpr int kSpecTwiddles = 11264;
 cudaError_t launch_spec_twiddle(float2* tw, cudaStream_t s);   // fills kSpecTwiddles entries
 cudaError_t spec_prepare(int np2max, int max_n, int seg);
-size_t spec_spread_smem(int max_n, int seg);
+int spec_seg_max(int max_n);           // cells per spreading item that shared memory holds
 cudaError_t launch_spec_prep(const SpecArgs& a, cudaStream_t s);
 // pair spectrum of one chunk (slot_end - slot_begin <= kSpecMaxChunk)
 cudaError_t launch_spec_transform(const SpecArgs& a, int n_sm, int max_n, bool one_pass, bool two_pass, cudaStream_t s);

@@ -111,10 +111,10 @@ def test_best_frequency_is_the_pair_sums(integer, f_min):
     same(best, via_noalloc(b, g, 0.3))
 
 
-# coarse_df T from 0.5 to 4, one peak to 40 (the most that goes through the spectrum), windows that
+# coarse_df T from 0.5 to 4, one peak to 20 (the most that goes through the spectrum), windows that
 # overlap and that leave the band
 @pytest.mark.parametrize("span,coarse_df,top_k,half,sigma_t", [(500.0, 1e-3, 10, 2e-3, 0.45), (2500.0, 1e-3, 1, 2e-3, 0.3),
-                                                               (2500.0, 1.6e-3, 40, 1e-3, 0.25), (1733.0, 7e-4, 5, 5e-3, 0.12)])
+                                                               (2500.0, 1.6e-3, 20, 1e-3, 0.25), (1733.0, 7e-4, 5, 5e-3, 0.12)])
 @pytest.mark.parametrize("integer", [False, True])
 def test_coarse_fine_is_the_pair_sums(span, coarse_df, top_k, half, sigma_t, integer):
     b = batch(64, 150, 300, span, seed=14, integer=integer)
