@@ -103,7 +103,7 @@ struct cp_plan_s {
     std::vector<int64_t> offsets;
     cp_freq_grid grid{};
     cp_options opt{};
-    int max_n = 0, np2max = 1;
+    int max_n = 0, np2max = 32;
     int64_t kc = 0;   // coarse grid points
     int J = 0;        // fine half-width in steps
     bool bands = false;          // bands method (Section 3.1)
@@ -122,6 +122,7 @@ struct cp_plan_s {
     std::vector<Wave> waves;
     size_t pair_smem = 0;
     int pair_grid = 0;
+    int pair_warps = 16;               // warps per block of the pair kernel
     bool tensor = false;               // CP_FORM_TENSOR
     uint32_t wait_limit = 1u << 26;    // polls per bounded device wait (tensor form)
     int n_max = 0;                     // harmonics of the tensor form
@@ -153,6 +154,8 @@ struct cp_plan_s {
     float* d_yp = nullptr;
     uint64_t *d_ph_base = nullptr, *d_ph_full = nullptr, *d_ph_coarse = nullptr, *d_ph_fine = nullptr;
     float* d_stpc = nullptr;
+    double* d_parts = nullptr;           // partial sums of the statistics (IP, rounding error)
+    int ip_blocks = 0;                   // see stats_blocks
     int32_t* d_order = nullptr;
     int64_t *d_unit_full = nullptr, *d_unit_coarse = nullptr, *d_unit_fine = nullptr, *d_wtile = nullptr;
     int64_t* d_unit_list = nullptr;
@@ -168,6 +171,7 @@ struct cp_plan_s {
     int32_t *d_peaks = nullptr, *d_npeaks = nullptr;
     unsigned long long* d_u64 = nullptr;  // [status | best_key (n_curves) | queues]
     int64_t n_u64 = 0;
+    void* d_res = nullptr;                // results of a search: status word, then the arrays below
     int64_t* d_res_idx = nullptr;
     double* d_res_freq = nullptr;
     float* d_res_stat = nullptr;
@@ -212,6 +216,7 @@ namespace {
 inline unsigned long long* status_word(cp_plan_t p) { return p->d_u64; }
 inline unsigned long long* best_keys(cp_plan_t p) { return p->d_u64 + 1; }
 inline unsigned long long* queue_word(cp_plan_t p, int i) { return p->d_u64 + 1 + p->n_curves + i; }
+size_t results_bytes(size_t nc) { return 8 + nc * (8 + 8 + 4 + 4 + 1); }
 constexpr int kQueuesPerWave = 4;   // one work counter per (wave, stage)
 
 constexpr int kCoefStride = kTcMaxHarmonics;   // a_1..a_48 stored per curve (largest class)
@@ -449,6 +454,12 @@ cp_status enqueue_stats(cp_plan_t p, cudaStream_t s)
     a.alpha = p->opt.alpha;
     a.np2max = p->np2max;
     a.status = reinterpret_cast<int*>(status_word(p));
+    a.ip_blocks = p->ip_blocks;
+    a.rho_blocks = std::max(p->ip_blocks, 1);
+    a.ip_parts = p->d_parts;
+    a.rho_parts = p->d_parts + p->n_curves * std::max(p->ip_blocks, 1);
+    a.ip_count = reinterpret_cast<unsigned int*>(p->d_u64 + p->n_u64 - p->n_curves);
+    a.rho_count = a.ip_count + p->n_curves;
     a.wrho = p->tensor ? p->d_wrho : nullptr;
     a.wrho_bf16 = w_bf16(p->opt.dtype) ? 1 : 0;
     CP_CUDA(launch_stats(a, (int)p->n_curves, s));
@@ -631,7 +642,7 @@ cp_status enqueue_pair(cp_plan_t p, int stage, int w, float* out, cudaStream_t s
         t.ft = tensor_freqs_per_unit(t.n_max, t.zsplit != 0);
         CP_CUDA(launch_pair_tensor(t, p->n_sm, s));
     } else {
-        CP_CUDA(launch_pair_direct(a, p->pair_grid, p->pair_smem, s));
+        CP_CUDA(launch_pair_direct(a, p->pair_warps, p->pair_grid, p->pair_smem, s));
     }
     if (ev_idx) {
         CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx) + 1], s, rec_flags(p)));
@@ -775,12 +786,12 @@ cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float*
     }
     const size_t smem = p->pair_smem + (size_t)p->max_n * sizeof(float) + kTile * sizeof(float);
     if (hier) {
-        CP_CUDA(launch_pair_direct(over_fallback(p, base, fb + 1, fb_coarse, p->kc, 1), p->n_sm, smem, s));
+        CP_CUDA(launch_pair_direct(over_fallback(p, base, fb + 1, fb_coarse, p->kc, 1), 16, p->n_sm, smem, s));
         CP_CUDA(launch_topk(topk_args(p, w, fb + 1, fb_coarse), s));
-        CP_CUDA(launch_pair_direct(over_fallback(p, fine, fb, fb_whole, 2 * p->J + 1, p->grid.top_k), p->n_sm, smem, s));
+        CP_CUDA(launch_pair_direct(over_fallback(p, fine, fb, fb_whole, 2 * p->J + 1, p->grid.top_k), 16, p->n_sm, smem, s));
     } else {
         CP_CUDA(launch_pair_direct(over_fallback(p, base, fb, fb_whole, stage == kStageList ? p->n_trials : p->grid.n_freq, 1),
-                                   p->n_sm, smem, s));
+                                   16, p->n_sm, smem, s));
     }
     if (ev_idx) {
         CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx) + 1], s, rec_flags(p)));
@@ -868,14 +879,11 @@ cp_status enqueue_search(cp_plan_t p, cudaStream_t s)
     f.best_stat = p->d_res_stat;
     f.is_periodic = p->d_res_per;
     f.psnr = p->d_res_psnr;
+    f.status = status_word(p);
+    f.status_out = reinterpret_cast<unsigned long long*>(p->d_res);
     CP_CUDA(launch_finalize(f, s));
     const size_t nc = (size_t)p->n_curves;
-    CP_CUDA(cudaMemcpyAsync(p->h_res_idx, p->d_res_idx, nc * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    CP_CUDA(cudaMemcpyAsync(p->h_res_freq, p->d_res_freq, nc * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CP_CUDA(cudaMemcpyAsync(p->h_res_stat, p->d_res_stat, nc * sizeof(float), cudaMemcpyDeviceToHost, s));
-    CP_CUDA(cudaMemcpyAsync(p->h_res_per, p->d_res_per, nc, cudaMemcpyDeviceToHost, s));
-    CP_CUDA(cudaMemcpyAsync(p->h_res_psnr, p->d_res_psnr, nc * sizeof(float), cudaMemcpyDeviceToHost, s));
-    CP_CUDA(cudaMemcpyAsync(p->h_status, p->d_u64, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+    CP_CUDA(cudaMemcpyAsync(p->h_status, p->d_res, results_bytes(nc), cudaMemcpyDeviceToHost, s));   // all results
     CP_CUDA(cudaEventRecordWithFlags(p->ev_step1, s, rec_flags(p)));
     return CP_OK;
 }
@@ -1237,6 +1245,17 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         const int tb = tune_bucket(tune, (int)n);
         p->fc[c] = fc_for((int)n, tb >= 0 ? tune.direct_fc[tb] : kFcMax);
     }
+    // Short curves have fewer tiles than a block of 16 warps has shares: blocks of 4 warps, four to an
+    // SM, overlap one's trig table and sums with another's tiles (64 curves x 1,000 frequencies: N = 40
+    // 159 -> 65 us, 100 223 -> 136, 150 266 -> 186, 250 481 -> 390; at 420 only with 8 frequencies a
+    // unit, 1152 -> 1069; at 650 slower).  The table of a unit must leave room for four blocks.
+    if (max_n <= kShortCurve) {
+        p->pair_warps = 4;
+        for (int64_t c = 0; c < n_curves; c++) {
+            const int n = (int)(offsets[c + 1] - offsets[c]);
+            while (p->fc[c] > 2 && (n + kTile - 1) / kTile * kTile * p->fc[c] * 12 > kShortTable) p->fc[c] >>= 1;
+        }
+    }
     p->max_band_points = (max_n + 9) / 10;   // a band holds at most ceil(N/10) samples
     p->n_points = offsets[n_curves];
     p->max_n = max_n;
@@ -1399,7 +1418,8 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     // device allocation (one block)
     const int64_t np = p->n_points, nc = n_curves;
     const int nq = kQueuesPerWave * (int)p->waves.size() + (spec ? spec_chunks + (int)p->waves.size() : 0);
-    p->n_u64 = 1 + nc + nq;
+    p->ip_blocks = stats_blocks(nc, max_n, p->n_sm);
+    p->n_u64 = 1 + nc + nq + nc;      // status, keys, work counters, two 32-bit counts per curve
     struct Part { void** dst; size_t bytes; };
     const bool hier = g.hierarchical == CP_SEARCH_COARSE_FINE;
     const bool bnd = p->bands;
@@ -1413,6 +1433,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         {(void**)&p->d_ph_full, np * sizeof(uint64_t)},
         {(void**)&p->d_ph_coarse, hier ? np * sizeof(uint64_t) : 0},
         {(void**)&p->d_ph_fine, hier ? np * sizeof(uint64_t) : 0},
+        {(void**)&p->d_parts, (size_t)2 * nc * std::max(p->ip_blocks, 1) * sizeof(double)},
         {(void**)&p->d_stpc, opt.sigma_t_mode == CP_SIGMA_T_PER_CURVE ? nc * sizeof(float) : 0},
         {(void**)&p->d_order, nc * sizeof(int32_t)},
         {(void**)&p->d_unit_full, (nc + 1) * sizeof(int64_t)},
@@ -1449,11 +1470,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         {(void**)&p->d_peaks, hier ? (size_t)nc * g.top_k * sizeof(int32_t) : 0},
         {(void**)&p->d_npeaks, hier ? nc * sizeof(int32_t) : 0},
         {(void**)&p->d_u64, (size_t)p->n_u64 * sizeof(unsigned long long)},
-        {(void**)&p->d_res_idx, nc * sizeof(int64_t)},
-        {(void**)&p->d_res_freq, nc * sizeof(double)},
-        {(void**)&p->d_res_stat, nc * sizeof(float)},
-        {(void**)&p->d_res_per, (size_t)nc},
-        {(void**)&p->d_res_psnr, nc * sizeof(float)},
+        {(void**)&p->d_res, results_bytes(nc)},
     };
     size_t total = 0;
     for (auto& q : parts) total = align_up(total, 256) + q.bytes;
@@ -1469,12 +1486,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     }
     // pinned host block
     std::vector<Part> hparts = {
-        {(void**)&p->h_res_idx, nc * sizeof(int64_t)},
-        {(void**)&p->h_res_freq, nc * sizeof(double)},
-        {(void**)&p->h_res_stat, nc * sizeof(float)},
-        {(void**)&p->h_res_per, (size_t)nc},
-        {(void**)&p->h_res_psnr, nc * sizeof(float)},
-        {(void**)&p->h_status, sizeof(unsigned long long)},
+        {(void**)&p->h_status, results_bytes(nc)},
         {(void**)&p->h_times, p->host_inputs && !p->host_pinned ? np * sizeof(double) : 0},
         {(void**)&p->h_mags, p->host_inputs && !p->host_pinned ? np * sizeof(float) : 0},
         {(void**)&p->h_errs, p->host_inputs && !p->host_pinned ? np * sizeof(float) : 0},
@@ -1490,6 +1502,17 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
             o += q.bytes;
         }
     }
+
+    // the results' arrays, at the same places on both sides (one copy)
+    auto results = [nc](void* base, int64_t** idx, double** freq, float** stat, float** psnr, uint8_t** per) {
+        *idx = static_cast<int64_t*>(base) + 1;
+        *freq = reinterpret_cast<double*>(*idx + nc);
+        *stat = reinterpret_cast<float*>(*freq + nc);
+        *psnr = *stat + nc;
+        *per = reinterpret_cast<uint8_t*>(*psnr + nc);
+    };
+    results(p->d_res, &p->d_res_idx, &p->d_res_freq, &p->d_res_stat, &p->d_res_psnr, &p->d_res_per);
+    results(p->h_status, &p->h_res_idx, &p->h_res_freq, &p->h_res_stat, &p->h_res_psnr, &p->h_res_per);
 
     // per-curve constants and schedule tables
     std::vector<CurveParams> cps(nc);
@@ -1544,7 +1567,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         if (p->class_count[class_rank(nm)]) CP_CUDA(prepare_tensor_kernel(nm));   // one CTA per SM
     {
         int occ = 1;
-        CP_CUDA(pair_direct_occupancy(&occ, p->pair_smem));
+        CP_CUDA(pair_direct_occupancy(&occ, p->pair_warps, p->pair_smem));
         p->pair_grid = p->n_sm * std::max(occ, 1);
     }
 
@@ -1561,7 +1584,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         CP_CUDA(cudaEventCreate(&p->ev_bands1));
     }
     p->launches_per_search =
-        2 /* zero, stats */ + (p->tensor ? 1 : 0) /* harmonic coefficients */ + (bnd ? 2 : 0) /* bands, window */ +
+        2 /* zero, stats */ + (p->ip_blocks ? 1 : 0) + (p->tensor ? 2 : 0) /* rounding sums, harmonic coefficients */ + (bnd ? 2 : 0) /* bands, window */ +
         (int64_t)p->waves.size() * (hier ? 4 : 2) + 1 /* finalize */;
     const SpecPlan& sp = hier || bnd ? p->ssearch : p->sfull;
     if (sp.on)

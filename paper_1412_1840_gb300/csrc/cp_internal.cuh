@@ -28,6 +28,8 @@ namespace cpk {
 constexpr int kMaxN = 4096;            // largest curve the kernels accept
 constexpr int kTableBytes = 196608;    // shared trig table budget of the direct kernel (192 KB)
 constexpr int kFcMax = 16;             // frequencies per work unit (direct form)
+constexpr int kShortCurve = 448;       // largest N of a batch for blocks of 4 warps (direct form)
+constexpr int kShortTable = 55296;     // their trig table: four blocks to an SM (54 KB)
 
 // Per-curve parameters, indexed by the caller's curve number.
 struct CurveParams {
@@ -202,7 +204,22 @@ struct StatsArgs {
     int* status;
     float* wrho;      // tensor form: per sample, sum_j of the 16-bit rounding error of w_ij (else null)
     int wrho_bf16;    // that operand is BF16 hi + lo (else FP16)
+    // pair sums of few curves spread over several CTAs a curve (see stats_blocks)
+    int ip_blocks;             // 0: in k_stats
+    int rho_blocks;
+    double *ip_parts, *rho_parts;           // [n_curves * blocks]
+    unsigned int *ip_count, *rho_count;     // [n_curves], zero before the call
 };
+
+// CTAs per curve for the N^2 sums of the statistics: one (with the curve's other
+// work) when there are curves for every SM or the curves are short, else enough
+// for four a SM, at least 16 rows each.
+inline int stats_blocks(int64_t n_curves, int max_n, int n_sm)
+{
+    if (n_curves >= n_sm || max_n <= 256) return 0;
+    const int64_t want = (4 * (int64_t)n_sm + n_curves - 1) / n_curves, most = max_n / 16;
+    return (int)(want < most ? want : most);
+}
 
 struct BuildWArgs {
     const CurveParams* cp;
@@ -243,6 +260,8 @@ struct FinalArgs {
     float* best_stat;
     uint8_t* is_periodic;
     float* psnr;
+    const unsigned long long* status;   // copied to status_out with the results (null: not)
+    unsigned long long* status_out;
 };
 
 // Tensor form (cp_tensor.cu).
@@ -346,7 +365,7 @@ cudaError_t launch_pair_tensor(const TensorArgs& a, int grid, cudaStream_t s);
 // Launchers (cp_kernels.cu); return the launch error.
 cudaError_t launch_stats(const StatsArgs& a, int n_curves, cudaStream_t s);
 cudaError_t launch_build_w(const BuildWArgs& a, cudaStream_t s);
-cudaError_t launch_pair_direct(const PairArgs& a, int grid, size_t smem, cudaStream_t s);
+cudaError_t launch_pair_direct(const PairArgs& a, int warps, int grid, size_t smem, cudaStream_t s);   // warps: 16 or 4 a block
 // The pair sum at the candidate entries; part: confirm_bytes(max_n) per slot (part_ld f2).
 cudaError_t launch_confirm(const PairArgs& a, void* part, int64_t part_ld, int n_sm, int max_n, cudaStream_t s);
 size_t confirm_bytes(int max_n);
@@ -355,7 +374,7 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t s);
 cudaError_t launch_finalize(const FinalArgs& a, cudaStream_t s);
 cudaError_t launch_zero_u64(unsigned long long* p, int64_t n, cudaStream_t s);
 int pair_direct_threads();
-cudaError_t pair_direct_occupancy(int* blocks_per_sm, size_t smem);
+cudaError_t pair_direct_occupancy(int* blocks_per_sm, int warps, size_t smem);
 size_t stats_smem_bytes(int np2max);
 cudaError_t prepare_kernels(int np2max, size_t pair_smem);
 // sigma_t of the skewness rule for every curve (one CTA per curve), from
@@ -376,16 +395,23 @@ const char* last_error_buffer();
 
 // ---------------------------------------------------------------------------
 // FP64-exact phase in 64-bit fixed point: frac(a * b) * 2^64 (mod 2^64).
-// p + e == a*b exactly (FMA error-free product); frac(p) is exact in FP64.
 // ---------------------------------------------------------------------------
+// By integers: the 106-bit product of the significands, shifted by the exponents
+// and rounded (FP64 arithmetic runs at 1.7 operations/clk/SM, and this is done up to
+// four times a sample).  a, b >= 0; a zero, subnormal or non-finite factor gives 0.
 __device__ __forceinline__ uint64_t fixfrac(double a, double b)
 {
-    double p = a * b;
-    double e = fma(a, b, -p);
-    double fr = p - floor(p);                    // [0, 1), exact
-    uint64_t hi = __double2ull_rn(fr * 18446744073709551616.0);   // fr has <= 53 significant bits
-    long long lo = __double2ll_rn(e * 18446744073709551616.0);
-    return hi + (uint64_t)lo;
+    const uint64_t ua = (uint64_t)__double_as_longlong(a), ub = (uint64_t)__double_as_longlong(b);
+    const int ea = (int)(ua >> 52) & 0x7ff, eb = (int)(ub >> 52) & 0x7ff;
+    if (ea == 0 || eb == 0 || ea == 0x7ff || eb == 0x7ff) return 0;
+    const uint64_t ma = (ua & 0xfffffffffffffull) | 0x10000000000000ull, mb = (ub & 0xfffffffffffffull) | 0x10000000000000ull;
+    const uint64_t lo = ma * mb, hi = __umul64hi(ma, mb);
+    const int s = ea + eb - 2 * 1075 + 64;           // the product times 2^s, modulo 2^64
+    if (s >= 0) return s < 64 ? lo << s : 0;
+    const int r = -s;
+    if (r < 64) return ((lo >> r) | (hi << (64 - r))) + ((lo >> (r - 1)) & 1u);
+    if (r == 64) return hi + (lo >> 63);
+    return r < 128 ? (hi >> (r - 64)) + ((hi >> (r - 65)) & 1u) : 0;
 }
 
 // sin(pi x), cos(pi x) for the phase x = U / 2^32 (turns of pi), up to a

@@ -50,6 +50,114 @@ __device__ __forceinline__ int snr_bin(double p)
     return b;
 }
 
+// Ascending bitonic sort of np2 floats (a power of two, at least 32) by T threads
+// of whole warps: strides below 32 stay in a warp's registers, a barrier separates
+// only the longer ones (15 instead of 55 at 1024).  Other is a second array
+// sorted alike (or the same pointer: one array).
+template <int T>
+__device__ __forceinline__ void sort_floats(float* a, float* other, int np2)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    const bool two = other != a;
+    for (int k = 32; k <= np2; k <<= 1) {
+        for (int j = k >> 1; j >= 32; j >>= 1) {
+            __syncthreads();
+            for (int p = tid; p < np2 >> 1; p += T) {
+                const int i = ((p & ~(j - 1)) << 1) | (p & (j - 1)), o = i | j;
+                const bool up = (i & k) == 0;
+                float u = a[i], v = a[o];
+                if ((u > v) == up) { a[i] = v; a[o] = u; }
+                if (two) {
+                    u = other[i];
+                    v = other[o];
+                    if ((u > v) == up) { other[i] = v; other[o] = u; }
+                }
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < np2; i += T) {
+            float u = a[i], v = two ? other[i] : 0.f;
+            for (int kk = k == 32 ? 2 : k; kk <= k; kk <<= 1) {
+#pragma unroll
+                for (int j = 16; j > 0; j >>= 1) {
+                    if (j >= kk) continue;
+                    const bool low = ((i & kk) == 0) == ((lane & j) == 0);     // keeps the smaller
+                    const float u2 = __shfl_xor_sync(0xffffffffu, u, j);
+                    u = (u2 < u) == low ? u2 : u;
+                    if (two) {
+                        const float v2 = __shfl_xor_sync(0xffffffffu, v, j);
+                        v = (v2 < v) == low ? v2 : v;
+                    }
+                }
+            }
+            a[i] = u;
+            if (two) other[i] = v;
+        }
+    }
+    __syncthreads();
+}
+
+// Block sum of one double per thread in a fixed order (lanes, then warps); thread 0 gets it.
+__device__ __forceinline__ double stats_sum(double v, double* s_red)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if (lane == 0) s_red[warp] = v;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < kStatsThreads / 32; w++) t += s_red[w];
+    return t;
+}
+
+// This block's part of sum_{i<j} g_ij: rows block, block + blocks, ... dealt to the
+// warps, lanes along j, each lane a compensated (Kahan) FP32 sum whose remainder is
+// kept, so that nothing is lost beyond FP32's second order; FP64 only at the end.
+__device__ __forceinline__ double ip_part(const float* y, int n, int block, int blocks)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
+    for (int i = block + blocks * warp; i < n; i += blocks * (kStatsThreads / 32)) {
+        const float yi = y[i];
+        int j = i + 1 + lane;
+        for (; j + 32 < n; j += 64) {
+            float d = gauss_g(yi, y[j]) - c0, t = s0 + d;
+            c0 = (t - s0) - d;
+            s0 = t;
+            d = gauss_g(yi, y[j + 32]) - c1;
+            t = s1 + d;
+            c1 = (t - s1) - d;
+            s1 = t;
+        }
+        if (j < n) {
+            const float d = gauss_g(yi, y[j]) - c0, t = s0 + d;
+            c0 = (t - s0) - d;
+            s0 = t;
+        }
+    }
+    return ((double)s0 - (double)c0) + ((double)s1 - (double)c1);
+}
+
+// IP and what follows from it: ip = (N + 2 sum_{i<j} g_ij) / N^2.
+__device__ __forceinline__ void set_ip(CurveParams* P, double s2)
+{
+    const double nn = (double)P->n;
+    const double ip = (nn + 2.0 * s2) / (nn * nn);
+    const float iph = (float)ip;
+    P->ip = ip;
+    P->ip_hi = iph;
+    P->ip_lo = (float)(ip - (double)iph);
+    P->norm = (float)(sqrt(nn) / (nn * nn * ip * sqrt(2.0 * CP_PI) * sqrt((double)P->sigma_t)));
+    P->diag = (float)(nn * (1.0 - ip));
+}
+
+// One CTA per curve.  FP64 runs at 1.7 operations/clk/SM: the phase steps are
+// integer products of the significands, the scalars are dealt to three warps, and
+// the pair sum of IP is FP32.  With few long curves the pair sum is left to k_ip
+// (a.ip_blocks blocks a curve).  70 us for 12 curves of up to 1,000 samples and
+// 568 us for three of up to 4,096 before, 19 and 31 us now (with k_ip).
 __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -59,7 +167,7 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
     float* ypl = es + a.np2max;
     __shared__ double s_red[kStatsThreads / 32];
     __shared__ double s_t0;
-    __shared__ float s_yref, s_gamma, s_iph, s_ipl;
+    __shared__ float s_yref, s_gamma;
     __shared__ int s_bad;
 
     const int c = blockIdx.x;
@@ -67,7 +175,7 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
     CurveParams* P = a.cp + c;
     const int64_t off = P->off;
     const int n = P->n;
-    int np2 = 1;
+    int np2 = 32;
     while (np2 < n) np2 <<= 1;
     if (tid == 0) s_bad = 0;
     __syncthreads();
@@ -79,50 +187,41 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
             const double t = a.times[off + i];
             const float y = a.mags[off + i];
             const float e = a.errs[off + i];
-            if (!isfinite(t) || !isfinite(y) || !isfinite(e)) s_bad = 1;
+            if ((__double2hiint(t) & 0x7ff00000) == 0x7ff00000 || !isfinite(y) || !isfinite(e)) s_bad = 1;
             ts[i] = t;
             ys[i] = y;
             es[i] = e;
-            tmin = fmin(tmin, t);
+            ypl[i] = y;
+            tmin = t < tmin ? t : tmin;
         } else {
             ys[i] = INFINITY;
             es[i] = INFINITY;
         }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tmin = fmin(tmin, __shfl_xor_sync(0xffffffffu, tmin, o));
+    for (int o = 16; o > 0; o >>= 1) {
+        const double t = __shfl_xor_sync(0xffffffffu, tmin, o);
+        tmin = t < tmin ? t : tmin;
+    }
     if (lane == 0) s_red[warp] = tmin;
-    __syncthreads();
+
+    // 2. magnitudes and error bars in ascending order
+    sort_floats<kStatsThreads>(ys, es, np2);
+
+    // 3. per-curve scalars (FP64), one thread of three warps
     if (tid == 0) {
         double m = s_red[0];
-        for (int w = 1; w < kStatsThreads / 32; w++) m = fmin(m, s_red[w]);
+        for (int w = 1; w < kStatsThreads / 32; w++) m = s_red[w] < m ? s_red[w] : m;
         s_t0 = m;
-    }
-
-    // 2. bitonic sort of magnitudes and error bars (ascending)
-    for (int k = 2; k <= np2; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            __syncthreads();
-            for (int i = tid; i < np2; i += kStatsThreads) {
-                const int ixj = i ^ j;
-                if (ixj > i) {
-                    const bool up = (i & k) == 0;
-                    float u = ys[i], v = ys[ixj];
-                    if ((u > v) == up) { ys[i] = v; ys[ixj] = u; }
-                    u = es[i]; v = es[ixj];
-                    if ((u > v) == up) { es[i] = v; es[ixj] = u; }
-                }
-            }
-        }
-    }
-    __syncthreads();
-
-    // 3. per-curve scalars (FP64, one thread)
-    if (tid == 0) {
+        P->t0 = m;
         const double sy = median_sorted(es, n);
-        const double yref = median_sorted(ys, n);
-        const double q1 = quantile_sorted(ys, n, 0.25), q3 = quantile_sorted(ys, n, 0.75);
-        const double psnr = 0.7413 * (q3 - q1) / ((double)a.alpha * sy);
+        if (!(sy > 0.0) || !isfinite(sy)) s_bad = 1;
+        const double gamma = sqrt(1.4426950408889634 / (2.0 * sy * sy));
+        P->sigma_y = (float)sy;
+        s_yref = (float)median_sorted(ys, n);
+        s_gamma = (float)gamma;
+        P->gamma = (float)gamma;
+    } else if (tid == 32) {
         double st;
         if (a.sigma_t_mode == 1) {
             st = (double)a.sigma_t_per_curve[c];
@@ -131,100 +230,37 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
         } else {
             st = (double)a.sigma_t;
         }
-        if (!(sy > 0.0) || !isfinite(sy) || !(st > 0.0) || !isfinite(st)) s_bad = 1;
+        if (!(st > 0.0) || !isfinite(st)) s_bad = 1;
         const float stf = (float)st;
         // the planned harmonic count no longer covers this sigma_t: the host re-plans
         if (stf < P->st_floor) atomicOr(a.status, 4);
-        P->sigma_y = (float)sy;
         P->sigma_t = stf;
-        P->psnr = (float)psnr;
-        P->th = c_th[snr_bin(psnr)];
-        P->t0 = s_t0;
-        const double gamma = sqrt(1.4426950408889634 / (2.0 * sy * sy));
-        s_yref = (float)yref;
-        s_gamma = (float)gamma;
-        P->gamma = (float)gamma;
         // sqrt(beta), beta = sqrt(2 log2 e) / sigma_t
         P->tscale = (float)sqrt(sqrt(2.0 * 1.4426950408889634) / (double)stf);
+    } else if (tid == 64) {
+        const double sy = median_sorted(es, n);
+        const double q1 = quantile_sorted(ys, n, 0.25), q3 = quantile_sorted(ys, n, 0.75);
+        const double psnr = 0.7413 * (q3 - q1) / ((double)a.alpha * sy);
+        P->psnr = (float)psnr;
+        P->th = c_th[snr_bin(psnr)];
     }
     __syncthreads();
 
     // 4. scaled magnitudes y' = (y - y_ref) * gamma (same values feed IP and W)
     const float yref = s_yref, gamma = s_gamma;
     for (int i = tid; i < n; i += kStatsThreads) {
-        const float v = (a.mags[off + i] - yref) * gamma;
+        const float v = (ypl[i] - yref) * gamma;
         ypl[i] = v;
         a.yp[off + i] = v;
     }
     __syncthreads();
 
-    // 5. IP: ip = (N + 2 sum_{i<j} g_ij) / N^2.  Each row is summed in FP32 with
-    //    Kahan compensation (error ~1 ulp of the row sum, independent of its
-    //    length) and the rows are accumulated in FP64; an FP64 add per pair
-    //    would cost more than the rest of the kernel (2.3 DFMA/clk/SM).
-    double acc = 0.0;
-    for (int i = tid; i < n; i += kStatsThreads) {
-        const float yi = ypl[i];
-        float sum = 0.f, comp = 0.f;
-        for (int j = i + 1; j < n; j++) {
-            const float y = gauss_g(yi, ypl[j]) - comp;
-            const float t = sum + y;
-            comp = (t - sum) - y;
-            sum = t;
-        }
-        acc += (double)sum - (double)comp;
+    // 5. IP
+    if (a.ip_blocks == 0) {
+        const double s2 = stats_sum(ip_part(ypl, n, 0, 1), s_red);
+        if (tid == 0) set_ip(P, s2);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    __syncthreads();
-    if (lane == 0) s_red[warp] = acc;
-    __syncthreads();
-    if (tid == 0) {
-        double s2 = 0.0;
-        for (int w = 0; w < kStatsThreads / 32; w++) s2 += s_red[w];
-        const double nn = (double)n;
-        const double ip = (nn + 2.0 * s2) / (nn * nn);
-        const float iph = (float)ip;
-        P->ip = ip;
-        P->ip_hi = iph;
-        P->ip_lo = (float)(ip - (double)iph);
-        s_iph = iph;
-        s_ipl = P->ip_lo;
-        P->norm = (float)(sqrt(nn) / (nn * nn * ip * sqrt(2.0 * CP_PI) * sqrt((double)P->sigma_t)));
-        P->diag = (float)(nn * (1.0 - ip));
-        if (s_bad) atomicOr(a.status, 1);
-    }
-
-    // 5b. tensor form: per sample i, the sum over j of the rounding error of the
-    //     16-bit operand w_ij = (g_ij - ip_hi) - ip_lo (the same FP32 values the
-    //     tile builder rounds), and its total.  With these the tensor epilogue
-    //     removes the error's coherent part: for a Z column x with mean xm the
-    //     operand error adds xm^2 sum(dW) + 2 xm drho^T (x - xm), which does not
-    //     average out where x is nearly constant over the samples (low f T, or
-    //     aliases of the sampling).  Full rows in a fixed order: deterministic.
-    if (a.wrho) {
-        __syncthreads();
-        const float iph = s_iph, ipl = s_ipl;
-        const bool bf = a.wrho_bf16 != 0;
-        double tot = 0.0;
-        for (int i = tid; i < n; i += kStatsThreads) {
-            const float yi = ypl[i];
-            float sum = 0.f;
-            for (int j = 0; j < n; j++) sum += w16_err((gauss_g(yi, ypl[j]) - iph) - ipl, bf);
-            a.wrho[off + i] = sum;
-            tot += (double)sum;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-        __syncthreads();
-        if (lane == 0) s_red[warp] = tot;
-        __syncthreads();
-        if (tid == 0) {
-            double t = 0.0;
-            for (int w = 0; w < kStatsThreads / 32; w++) t += s_red[w];
-            P->dwsum = (float)t;
-        }
-    }
+    if (tid == 0 && s_bad) atomicOr(a.status, 1);
 
     // 6. fixed-point phase steps of t - t0 for each grid the search uses
     const double t0 = s_t0;
@@ -235,6 +271,78 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
         if (a.hierarchical) {
             a.ph_coarse[off + i] = fixfrac(a.coarse_df, tp);
             a.ph_fine[off + i] = fixfrac(a.fine_df, tp);
+        }
+    }
+}
+
+// IP of few curves: a.ip_blocks CTAs a curve; the last to finish adds the parts in
+// order and takes the steps that follow.
+__global__ void __launch_bounds__(kStatsThreads) k_ip(const StatsArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    float* y = reinterpret_cast<float*>(smem);
+    __shared__ double s_red[kStatsThreads / 32];
+    __shared__ int s_last;
+    const int c = blockIdx.x, tid = threadIdx.x, nb = a.ip_blocks;
+    CurveParams* P = a.cp + c;
+    const int n = P->n;
+    for (int i = tid; i < n; i += kStatsThreads) y[i] = a.yp[P->off + i];
+    __syncthreads();
+    const double part = stats_sum(ip_part(y, n, blockIdx.y, nb), s_red);
+    if (tid == 0) {
+        a.ip_parts[(int64_t)c * nb + blockIdx.y] = part;
+        __threadfence();
+        s_last = atomicAdd(a.ip_count + c, 1u) == (unsigned)nb - 1u;
+        if (s_last) {
+            __threadfence();
+            double s2 = 0.0;
+            for (int b = 0; b < nb; b++) s2 += __ldcg(a.ip_parts + (int64_t)c * nb + b);
+            set_ip(P, s2);
+        }
+    }
+}
+
+// Tensor form: per sample i, the sum over j of the rounding error of the 16-bit
+// operand w_ij = (g_ij - ip_hi) - ip_lo (the same FP32 values the tile builder
+// rounds), and its total.  With these the tensor epilogue removes the error's
+// coherent part: for a Z column x with mean xm the operand error adds
+// xm^2 sum(dW) + 2 xm drho^T (x - xm), which does not average out where x is nearly
+// constant over the samples (low f T, or aliases of the sampling).  A warp per row,
+// a.rho_blocks CTAs per curve; fixed order: deterministic.
+__global__ void __launch_bounds__(kStatsThreads) k_wrho(const StatsArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    float* y = reinterpret_cast<float*>(smem);
+    __shared__ double s_red[kStatsThreads / 32];
+    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = a.rho_blocks;
+    CurveParams* P = a.cp + c;
+    const int n = P->n;
+    const int64_t off = P->off;
+    for (int i = tid; i < n; i += kStatsThreads) y[i] = a.yp[off + i];
+    __syncthreads();
+    const float iph = P->ip_hi, ipl = P->ip_lo;
+    const bool bf = a.wrho_bf16 != 0;
+    double tot = 0.0;
+    for (int i = blockIdx.y + nb * warp; i < n; i += nb * (kStatsThreads / 32)) {
+        const float yi = y[i];
+        float s = 0.f;
+        for (int j = lane; j < n; j += 32) s += w16_err((gauss_g(yi, y[j]) - iph) - ipl, bf);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) {
+            a.wrho[off + i] = s;
+            tot += (double)s;
+        }
+    }
+    const double part = stats_sum(tot, s_red);
+    if (tid == 0) {
+        a.rho_parts[(int64_t)c * nb + blockIdx.y] = part;
+        __threadfence();
+        if (atomicAdd(a.rho_count + c, 1u) == (unsigned)nb - 1u) {
+            __threadfence();
+            double t = 0.0;
+            for (int b = 0; b < nb; b++) t += __ldcg(a.rho_parts + (int64_t)c * nb + b);
+            P->dwsum = (float)t;
         }
     }
 }
@@ -251,23 +359,10 @@ __global__ void __launch_bounds__(kStatsThreads) k_sigma_t_rule(const float* mag
     const int c = blockIdx.x, tid = threadIdx.x;
     const int64_t off = offsets[c];
     const int n = (int)(offsets[c + 1] - off);
-    int np2 = 1;
+    int np2 = 32;
     while (np2 < n) np2 <<= 1;
     for (int i = tid; i < np2; i += kStatsThreads) ys[i] = i < n ? mags[off + i] : INFINITY;
-    for (int k = 2; k <= np2; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            __syncthreads();
-            for (int i = tid; i < np2; i += kStatsThreads) {
-                const int ixj = i ^ j;
-                if (ixj > i) {
-                    const bool up = (i & k) == 0;
-                    const float u = ys[i], v = ys[ixj];
-                    if ((u > v) == up) { ys[i] = v; ys[ixj] = u; }
-                }
-            }
-        }
-    }
-    __syncthreads();
+    sort_floats<kStatsThreads>(ys, ys, np2);
     if (tid == 0) out[c] = (float)sigma_t_rule(ys, n);
 }
 
@@ -350,8 +445,7 @@ constexpr int kPairThreads = 512;
 // shared memory serves (rows x columns) / (rows + columns) evaluations, so the
 // whole-tile item needs a third fewer shared-memory loads per evaluation.
 constexpr int kItemRows = 8;
-constexpr int kItemsPerTile = kRowsPerLane / kItemRows;
-constexpr bool kPrefetchW = kItemRows == 4;   // next item's W in registers (the half-tile item only)
+static_assert(kItemRows == kRowsPerLane && kFcMax == 16, "whole-tile items, 16 sums per share");
 // The unit's trig table is built by one thread per (point, half of the
 // frequency pairs): each point's phase and step are loaded twice per unit
 // instead of once per frequency pair, and the threads' shares stay even
@@ -494,10 +588,30 @@ __device__ __forceinline__ unsigned long long cand_emit(const PairArgs& a, int c
 // launch carry none of it.  Its w come from the magnitudes
 // instead of stored tiles (one more exponential per pair and unit), so that
 // plans whose every pass goes through the spectrum keep no tiles.
-template <bool SEL>
-__global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs a)
+// Butterfly reduce-scatter of 16 values: on return lane l holds the warp's sum of
+// x[l >> 1] (the same pairs in the same order as 16 separate butterflies).
+__device__ __forceinline__ float reduce_scatter16(float (&x)[16], int lane)
+{
+#pragma unroll
+    for (int half = 8, bit = 4; half > 0; half >>= 1, bit--) {
+        const bool upper = (lane >> bit) & 1;
+#pragma unroll
+        for (int q = 0; q < half; q++) {
+            const float recv = __shfl_xor_sync(0xffffffffu, upper ? x[q] : x[q + half], 1 << bit);
+            x[q] = (upper ? x[q + half] : x[q]) + recv;
+        }
+    }
+    return x[0] + __shfl_xor_sync(0xffffffffu, x[0], 1);
+}
+
+// WARPS: a unit's tiles are always summed as by kPairThreads / 32 warps (each
+// every 16th tile, then lanes, then warps); a block of fewer warps takes several
+// of these shares in turn, with the same result.
+template <bool SEL, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_pair_direct(const PairArgs a)
 {
     constexpr int NW = kPairThreads / 32;
+    constexpr int T = 32 * WARPS;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long s_unit;
     __shared__ float s_red[NW][kFcMax];
@@ -568,7 +682,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
         // step are loaded once for the whole group, and the phase advances by two
         // grid steps per pair (exact in the 2^-64 fixed point).
         const int gsz = (nfp + kTableGroups - 1) / kTableGroups;
-        for (int it = tid; it < kTableGroups * npad; it += kPairThreads) {
+        for (int it = tid; it < kTableGroups * npad; it += T) {
             const int gi = it / npad, i = it - gi * npad;
             const int fp0 = gi * gsz, fp1 = min(nfp, fp0 + gsz);
             if (i < n) {
@@ -599,68 +713,47 @@ __global__ void __launch_bounds__(kPairThreads, 1) k_pair_direct(const PairArgs 
         }
         float* Y = reinterpret_cast<float*>(SC) + (size_t)(fc >> 1) * npad * 6;   // SEL: after the tables
         if (SEL)
-            for (int i = tid; i < npad; i += kPairThreads) Y[i] = i < n ? a.yp[off + i] : 0.f;
+            for (int i = tid; i < npad; i += T) Y[i] = i < n ? a.yp[off + i] : 0.f;
         const float wscale = SEL ? w_scale(P) : 1.0f;
         __syncthreads();
 
         const int nb = npad / kTile;
         const int ntiles = nb * (nb + 1) / 2;
-        const int nitems = kItemsPerTile * ntiles;   // (tile, row part): 4 kItemRows x 32 pairs per warp item
+        const int nitems = ntiles;                   // a warp item is a whole tile
         const float4* Wc =
             SEL ? nullptr : reinterpret_cast<const float4*>(a.W + (a.wtile_start[slot] - a.wtile_base) * kTileFloats);
-        f2 acc[kFcMax / 2];                      // per f-pair: (sum at f, sum at f')
-#pragma unroll
-        for (int q = 0; q < kFcMax / 2; q++) acc[q] = 0ull;
-
-        // W of an item: rows (item % kItemsPerTile) * kItemRows + k of the stored tile
-        auto w_ptr = [&](int it, int k) {
-            return Wc + (int64_t)(it / kItemsPerTile) * (kTileFloats / 4) + ((it % kItemsPerTile) * kItemRows + k) * 32 + lane;
-        };
-        float4 wn[kPrefetchW ? kItemRows : 1];
-        int item = warp;
-        if (kPrefetchW && item < nitems) {
-#pragma unroll
-            for (int k = 0; k < kItemRows; k++) wn[k] = __ldg(w_ptr(item, k));
-        }
 #pragma unroll 1
-        for (; item < nitems; item += NW) {
-            f2 w01[kItemRows], w23[kItemRows];
-            int bi, bj;
-            decode_tile(item / kItemsPerTile, nb, bi, bj);
-            const int rbase = bi * kTile + (item % kItemsPerTile) * (4 * kItemRows) + la;
-            const int cbase = bj * kTile + lb;
-            if (SEL) item_w(Y, n, rbase, cbase, P.ip_hi, P.ip_lo, wscale, w01, w23);
-#pragma unroll
-            for (int k = 0; k < (SEL ? 0 : kItemRows); k++) {
-                const float4 wv = kPrefetchW ? wn[k] : __ldg(w_ptr(item, k));
-                w01[k] = pk(wv.x, wv.y);
-                w23[k] = pk(wv.z, wv.w);
+        for (int share = warp; share < NW; share += WARPS) {
+            if (share >= nitems) {                   // a short curve's shares without a tile
+                if (lane < 16) s_red[share][lane] = 0.f;
+                continue;
             }
-            const int nxt = item + NW;
-            if (kPrefetchW && nxt < nitems) {
+            f2 acc[kFcMax / 2];                      // per f-pair: (sum at f, sum at f')
 #pragma unroll
-                for (int k = 0; k < kItemRows; k++) wn[k] = __ldg(w_ptr(nxt, k));
-            }
-            if (cosf) pair_item<true>(SC, NS, npad, nfp, rbase, cbase, w01, w23, acc);
-            else pair_item<false>(SC, NS, npad, nfp, rbase, cbase, w01, w23, acc);
-        }
-
-        // warp reduction of the 2*nfp frequency sums, then a fixed-order CTA sum
+            for (int q = 0; q < kFcMax / 2; q++) acc[q] = 0ull;
+#pragma unroll 1
+            for (int item = share; item < nitems; item += NW) {
+                f2 w01[kItemRows], w23[kItemRows];
+                int bi, bj;
+                decode_tile(item, nb, bi, bj);
+                const int rbase = bi * kTile + la;
+                const int cbase = bj * kTile + lb;
+                if (SEL) item_w(Y, n, rbase, cbase, P.ip_hi, P.ip_lo, wscale, w01, w23);
 #pragma unroll
-        for (int fp = 0; fp < kFcMax / 2; fp++) {
-            if (fp < nfp) {
-                float vf, vg;
-                upk(acc[fp], vf, vg);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    vf += __shfl_xor_sync(0xffffffffu, vf, o);
-                    vg += __shfl_xor_sync(0xffffffffu, vg, o);
+                for (int k = 0; k < (SEL ? 0 : kItemRows); k++) {
+                    const float4 wv = __ldg(Wc + (int64_t)item * (kTileFloats / 4) + k * 32 + lane);
+                    w01[k] = pk(wv.x, wv.y);
+                    w23[k] = pk(wv.z, wv.w);
                 }
-                if (lane == 0) {
-                    s_red[warp][2 * fp] = vf;
-                    s_red[warp][2 * fp + 1] = vg;
-                }
+                if (cosf) pair_item<true>(SC, NS, npad, nfp, rbase, cbase, w01, w23, acc);
+                else pair_item<false>(SC, NS, npad, nfp, rbase, cbase, w01, w23, acc);
             }
+            // the share's frequency sums over the lanes, then (below) a fixed-order sum over the shares
+            float x[16];
+#pragma unroll
+            for (int fp = 0; fp < kFcMax / 2; fp++) upk(acc[fp], x[2 * fp], x[2 * fp + 1]);
+            const float v = reduce_scatter16(x, lane);
+            if ((lane & 1) == 0) s_red[share][lane >> 1] = v;
         }
         __syncthreads();
         if (warp == 0) {
@@ -899,37 +992,35 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(const TopkArgs a)
 __global__ void k_finalize(const FinalArgs a)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c == 0 && a.status_out) *a.status_out = *a.status;
     if (c >= a.n_curves) return;
     const unsigned long long key = a.best_key[c];
-    if (key == 0ull) {   // no admissible candidate (cannot happen for valid grids)
-        a.best_idx[c] = -1;
-        a.best_freq[c] = __longlong_as_double(0x7ff8000000000000ll);
-        a.best_stat[c] = __int_as_float(0x7fc00000);
-        a.is_periodic[c] = 0;
-        a.psnr[c] = a.cp[c].psnr;
-        return;
+    int64_t kout = -1;   // no admissible candidate
+    double f = __longlong_as_double(0x7ff8000000000000ll);
+    float v = __int_as_float(0x7fc00000);
+    if (key != 0ull) {
+        v = from_orderable((uint32_t)(key >> 32));
+        const uint32_t idx = 0xffffffffu - (uint32_t)(key & 0xffffffffu);
+        kout = (int64_t)idx;
+        if (a.hierarchical == CP_SEARCH_BANDS) {
+            const uint32_t k = (uint32_t)a.trials[(int64_t)c * a.n_trials + idx];   // list position -> grid index
+            kout = (int64_t)k;
+            f = __dadd_rn(a.f_min, __dmul_rn((double)k, a.df));
+        } else if (a.hierarchical) {
+            const int W = 2 * a.fine_half + 1;
+            const int p = (int)(idx / (uint32_t)W);
+            const int j = (int)(idx % (uint32_t)W) - a.fine_half;
+            const double fpk = __dadd_rn(a.f_min, __dmul_rn((double)a.peaks[(int64_t)c * a.top_k + p], a.coarse_df));
+            f = __dadd_rn(fpk, __dmul_rn((double)j, a.fine_df));
+        } else {
+            f = __dadd_rn(a.f_min, __dmul_rn((double)idx, a.df));
+        }
     }
-    const float v = from_orderable((uint32_t)(key >> 32));
-    const uint32_t idx = 0xffffffffu - (uint32_t)(key & 0xffffffffu);
-    double f;
-    uint32_t kout = idx;
-    if (a.hierarchical == CP_SEARCH_BANDS) {
-        kout = (uint32_t)a.trials[(int64_t)c * a.n_trials + idx];   // list position -> grid index
-        f = __dadd_rn(a.f_min, __dmul_rn((double)kout, a.df));
-    } else if (a.hierarchical) {
-        const int W = 2 * a.fine_half + 1;
-        const int p = (int)(idx / (uint32_t)W);
-        const int j = (int)(idx % (uint32_t)W) - a.fine_half;
-        const double fpk = __dadd_rn(a.f_min, __dmul_rn((double)a.peaks[(int64_t)c * a.top_k + p], a.coarse_df));
-        f = __dadd_rn(fpk, __dmul_rn((double)j, a.fine_df));
-    } else {
-        f = __dadd_rn(a.f_min, __dmul_rn((double)idx, a.df));
-    }
-    a.best_idx[c] = (int64_t)kout;
-    a.best_freq[c] = f;
-    a.best_stat[c] = v;
-    a.is_periodic[c] = v > a.cp[c].th ? 1 : 0;
-    a.psnr[c] = a.cp[c].psnr;
+    if (a.best_idx) a.best_idx[c] = kout;
+    if (a.best_freq) a.best_freq[c] = f;
+    if (a.best_stat) a.best_stat[c] = v;
+    if (a.is_periodic) a.is_periodic[c] = v > a.cp[c].th ? 1 : 0;
+    if (a.psnr) a.psnr[c] = a.cp[c].psnr;
 }
 
 __global__ void k_zero_u64(unsigned long long* p, int64_t n)
@@ -949,7 +1040,17 @@ cudaError_t launch_stats(const StatsArgs& a, int n_curves, cudaStream_t s)
 {
     const size_t smem = stats_smem_bytes(a.np2max);
     k_stats<<<n_curves, kStatsThreads, smem, s>>>(a);
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    const size_t ysmem = (size_t)a.np2max * sizeof(float);
+    if (e == cudaSuccess && a.ip_blocks) {
+        k_ip<<<dim3(n_curves, a.ip_blocks), kStatsThreads, ysmem, s>>>(a);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess && a.wrho) {
+        k_wrho<<<dim3(n_curves, a.rho_blocks), kStatsThreads, ysmem, s>>>(a);
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 cudaError_t launch_sigma_t_rule(const float* mags, const int64_t* offsets, int n_curves, int np2max, float* out,
@@ -970,10 +1071,11 @@ cudaError_t launch_build_w(const BuildWArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_pair_direct(const PairArgs& a, int grid, size_t smem, cudaStream_t s)
+cudaError_t launch_pair_direct(const PairArgs& a, int warps, int grid, size_t smem, cudaStream_t s)
 {
-    if (a.fb_count) k_pair_direct<true><<<grid, kPairThreads, smem, s>>>(a);
-    else k_pair_direct<false><<<grid, kPairThreads, smem, s>>>(a);
+    if (a.fb_count) k_pair_direct<true, 16><<<grid, kPairThreads, smem, s>>>(a);
+    else if (warps == 4) k_pair_direct<false, 4><<<grid, 128, smem, s>>>(a);
+    else k_pair_direct<false, 16><<<grid, kPairThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1012,7 +1114,7 @@ size_t confirm_bytes(int max_n) { return (size_t)tiles_of(max_n) * 32 * sizeof(f
 cudaError_t prepare_selected(size_t pair_smem)
 {
     cudaError_t e = raise_dyn_smem((const void*)k_confirm, kConfirmSmem);
-    return e == cudaSuccess ? raise_dyn_smem((const void*)k_pair_direct<true>, pair_smem) : e;
+    return e == cudaSuccess ? raise_dyn_smem((const void*)k_pair_direct<true, 16>, pair_smem) : e;
 }
 
 int pair_direct_threads() { return kPairThreads; }
@@ -1041,14 +1143,17 @@ cudaError_t prepare_kernels(int np2max, size_t pair_smem)
 {
     cudaError_t e = raise_dyn_smem((const void*)k_stats, stats_smem_bytes(np2max));
     if (e != cudaSuccess) return e;
-    return raise_dyn_smem((const void*)k_pair_direct<false>, pair_smem);
+    e = raise_dyn_smem((const void*)k_pair_direct<false, 4>, pair_smem);
+    if (e != cudaSuccess) return e;
+    return raise_dyn_smem((const void*)k_pair_direct<false, 16>, pair_smem);
 }
 
-cudaError_t pair_direct_occupancy(int* blocks_per_sm, size_t smem)
+cudaError_t pair_direct_occupancy(int* blocks_per_sm, int warps, size_t smem)
 {
-    cudaError_t e = raise_dyn_smem((const void*)k_pair_direct<false>, smem);
+    const void* k = warps == 4 ? (const void*)k_pair_direct<false, 4> : (const void*)k_pair_direct<false, 16>;
+    cudaError_t e = raise_dyn_smem(k, smem);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_pair_direct<false>, kPairThreads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, 32 * warps, smem);
 }
 
 cudaError_t launch_zero_u64(unsigned long long* p, int64_t n, cudaStream_t s)

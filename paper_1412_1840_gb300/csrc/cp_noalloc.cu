@@ -171,16 +171,22 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         order[pos] = c;
     }
     const int64_t n_points = offsets[n_curves];
-    int np2max = 1;
+    int np2max = 32;
     while (np2max < max_n) np2max <<= 1;
     unit_full[0] = unit_coarse[0] = unit_fine[0] = wtile[0] = 0;
+    // blocks of 4 warps for a batch of short curves, as in a plan (cp_api.cu)
+    const int warps = max_n <= kShortCurve ? 4 : 16;
+    auto fc_of = [warps](int npad) {
+        int fc = kFcMax;
+        while (fc > 2 && npad * fc * 12 > (warps == 4 ? kShortTable : kTableBytes)) fc >>= 1;
+        return fc;
+    };
     size_t pair_smem = 0;
     for (int s = 0; s < n_curves; s++) {
         const int c = order[s];
         const int n = (int)(offsets[c + 1] - offsets[c]);
         const int npad = (n + kTile - 1) / kTile * kTile;
-        int fc = kFcMax;
-        while (fc > 2 && (size_t)npad * fc * 12 > (size_t)kTableBytes) fc >>= 1;
+        const int fc = fc_of(npad);
         unit_full[s + 1] = unit_full[s] + (g.n_freq + fc - 1) / fc;
         unit_coarse[s + 1] = unit_coarse[s] + (g.hierarchical ? (kc + fc - 1) / fc : 0);
         unit_fine[s + 1] = unit_fine[s] + (g.hierarchical ? (int64_t)g.top_k * ((2 * J + 1 + fc - 1) / fc) : 0);
@@ -192,13 +198,13 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         cps[c].off = offsets[c];
         cps[c].n = (int32_t)(offsets[c + 1] - offsets[c]);
         const int npad = (cps[c].n + kTile - 1) / kTile * kTile;
-        int fc = kFcMax;
-        while (fc > 2 && (size_t)npad * fc * 12 > (size_t)kTableBytes) fc >>= 1;
-        cps[c].fc = fc;
+        cps[c].fc = fc_of(npad);
     }
 
-    int dev = 0;
+    int dev = 0, nsm = 1;
     NA_CUDA(cudaGetDevice(&dev));
+    NA_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int ip_blocks = stats_blocks(n_curves, max_n, nsm);
     void* base = nullptr;
     cp_status st = scratch_base(dev, &base);
     if (st != CP_OK) return st;
@@ -206,39 +212,47 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     // carve the scratch array (one wave: all W tiles must fit)
     Carve cv{static_cast<char*>(base), 0};
     const int nc = (int)n_curves;
-    CurveParams* d_cp = cv.take<CurveParams>(nc);
+    // tables from the host, in one copy: parameters, order, unit and tile prefix sums
+    const size_t table_bytes = nc * sizeof(CurveParams) + 4 * (nc + 1) * sizeof(int64_t) + nc * sizeof(int32_t);
+    char* d_table = cv.take<char>(table_bytes);
+    CurveParams* d_cp = reinterpret_cast<CurveParams*>(d_table);
+    int64_t* d_unit_full = reinterpret_cast<int64_t*>(d_cp + nc);
+    int64_t* d_unit_coarse = d_unit_full + nc + 1;
+    int64_t* d_unit_fine = d_unit_coarse + nc + 1;
+    int64_t* d_wtile = d_unit_fine + nc + 1;
+    int32_t* d_order = reinterpret_cast<int32_t*>(d_wtile + nc + 1);
     float* d_yp = cv.take<float>(n_points);
     uint64_t* d_ph_base = cv.take<uint64_t>(n_points);
     uint64_t* d_ph_full = cv.take<uint64_t>(n_points);
     uint64_t* d_ph_coarse = g.hierarchical ? cv.take<uint64_t>(n_points) : nullptr;
     uint64_t* d_ph_fine = g.hierarchical ? cv.take<uint64_t>(n_points) : nullptr;
-    int32_t* d_order = cv.take<int32_t>(nc);
-    int64_t* d_unit_full = cv.take<int64_t>(nc + 1);
-    int64_t* d_unit_coarse = cv.take<int64_t>(nc + 1);
-    int64_t* d_unit_fine = cv.take<int64_t>(nc + 1);
-    int64_t* d_wtile = cv.take<int64_t>(nc + 1);
     float* d_W = cv.take<float>((size_t)wtile[nc] * kTileFloats);
     float* d_coarse = g.hierarchical ? cv.take<float>((size_t)nc * kc) : nullptr;
     int32_t* d_peaks = g.hierarchical ? cv.take<int32_t>((size_t)nc * g.top_k) : nullptr;
     int32_t* d_npeaks = g.hierarchical ? cv.take<int32_t>(nc) : nullptr;
-    const int64_t n_u64 = 1 + nc + 3;
+    const int64_t n_u64 = 1 + nc + 3 + nc;
     unsigned long long* d_u64 = cv.take<unsigned long long>(n_u64);
-    int64_t* d_idx = cv.take<int64_t>(nc);
-    double* d_freq = cv.take<double>(nc);
-    float* d_stat = cv.take<float>(nc);
-    uint8_t* d_per = cv.take<uint8_t>(nc);
-    float* d_psnr = cv.take<float>(nc);
+    double* d_parts = cv.take<double>((size_t)nc * (ip_blocks > 0 ? ip_blocks : 1));
     if (cv.used > kScratchBytes)
         return nfail(CP_EUNSUPPORTED, "cp_best_period_noalloc: batch needs more than CP_NOALLOC_SCRATCH_BYTES");
 
     cudaStream_t s = (cudaStream_t)cuda_stream;
     SyncOnError guard{s, true};
-    NA_CUDA(cudaMemcpyAsync(d_cp, cps, nc * sizeof(CurveParams), cudaMemcpyHostToDevice, s));
-    NA_CUDA(cudaMemcpyAsync(d_order, order, nc * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    NA_CUDA(cudaMemcpyAsync(d_unit_full, unit_full, (nc + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-    NA_CUDA(cudaMemcpyAsync(d_unit_coarse, unit_coarse, (nc + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-    NA_CUDA(cudaMemcpyAsync(d_unit_fine, unit_fine, (nc + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-    NA_CUDA(cudaMemcpyAsync(d_wtile, wtile, (nc + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    {
+        char table[kMaxCurves * (sizeof(CurveParams) + 4 * sizeof(int64_t) + sizeof(int32_t)) + 4 * sizeof(int64_t)];
+        char* at = table;
+        auto put = [&at](const void* src, size_t bytes) {
+            std::memcpy(at, src, bytes);
+            at += bytes;
+        };
+        put(cps, nc * sizeof(CurveParams));
+        put(unit_full, (nc + 1) * sizeof(int64_t));
+        put(unit_coarse, (nc + 1) * sizeof(int64_t));
+        put(unit_fine, (nc + 1) * sizeof(int64_t));
+        put(wtile, (nc + 1) * sizeof(int64_t));
+        put(order, nc * sizeof(int32_t));
+        NA_CUDA(cudaMemcpyAsync(d_table, table, table_bytes, cudaMemcpyHostToDevice, s));
+    }
     NA_CUDA(launch_zero_u64(d_u64, n_u64, s));   // status, best keys and work counters start at zero
 
     StatsArgs sa{};
@@ -261,6 +275,9 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     sa.alpha = 1.0f;
     sa.np2max = np2max;
     sa.status = reinterpret_cast<int*>(d_u64);
+    sa.ip_blocks = ip_blocks;
+    sa.ip_parts = d_parts;
+    sa.ip_count = reinterpret_cast<unsigned int*>(d_u64 + 1 + nc + 3);
     NA_CUDA(prepare_kernels(np2max, pair_smem));
     NA_CUDA(launch_stats(sa, nc, s));
 
@@ -276,9 +293,8 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     bw.tile_end = wtile[nc];
     NA_CUDA(launch_build_w(bw, s));
 
-    int occ = 1, nsm = 1;
-    NA_CUDA(pair_direct_occupancy(&occ, pair_smem));
-    NA_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    int occ = 1;
+    NA_CUDA(pair_direct_occupancy(&occ, warps, pair_smem));
     PairArgs pa{};
     pa.cp = d_cp;
     pa.order = d_order;
@@ -310,7 +326,7 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         pa.unit_begin = 0;
         pa.unit_end = unit_full[nc];
         pa.queue = d_u64 + 1 + nc;
-        NA_CUDA(launch_pair_direct(pa, nsm * (occ > 0 ? occ : 1), pair_smem, s));
+        NA_CUDA(launch_pair_direct(pa, warps, nsm * (occ > 0 ? occ : 1), pair_smem, s));
     } else {
         pa.stage = kStageCoarse;
         pa.unit_start = d_unit_coarse;
@@ -320,7 +336,7 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         pa.unit_begin = 0;
         pa.unit_end = unit_coarse[nc];
         pa.queue = d_u64 + 1 + nc + 1;
-        NA_CUDA(launch_pair_direct(pa, nsm * (occ > 0 ? occ : 1), pair_smem, s));
+        NA_CUDA(launch_pair_direct(pa, warps, nsm * (occ > 0 ? occ : 1), pair_smem, s));
         TopkArgs ta{};
         ta.coarse = d_coarse;
         ta.order = d_order;
@@ -337,7 +353,7 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         pa.step = g.fine_df;
         pa.unit_end = unit_fine[nc];
         pa.queue = d_u64 + 1 + nc + 2;
-        NA_CUDA(launch_pair_direct(pa, nsm * (occ > 0 ? occ : 1), pair_smem, s));
+        NA_CUDA(launch_pair_direct(pa, warps, nsm * (occ > 0 ? occ : 1), pair_smem, s));
     }
     FinalArgs fa{};
     fa.cp = d_cp;
@@ -351,16 +367,11 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     fa.df = g.df;
     fa.coarse_df = g.coarse_df;
     fa.fine_df = g.fine_df;
-    fa.best_idx = d_idx;
-    fa.best_freq = d_freq;
-    fa.best_stat = d_stat;
-    fa.is_periodic = d_per;
-    fa.psnr = d_psnr;
+    fa.best_idx = best_idx;          // straight to the caller's arrays (null: not wanted)
+    fa.best_freq = best_freq;
+    fa.best_stat = best_stat;
+    fa.is_periodic = is_periodic;
     NA_CUDA(launch_finalize(fa, s));
-    if (best_idx) NA_CUDA(cudaMemcpyAsync(best_idx, d_idx, nc * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-    if (best_freq) NA_CUDA(cudaMemcpyAsync(best_freq, d_freq, nc * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    if (best_stat) NA_CUDA(cudaMemcpyAsync(best_stat, d_stat, nc * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    if (is_periodic) NA_CUDA(cudaMemcpyAsync(is_periodic, d_per, nc, cudaMemcpyDeviceToDevice, s));
     unsigned long long status = 0;
     NA_CUDA(cudaMemcpyAsync(&status, d_u64, sizeof(status), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));

@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 import paper_1412_1840_gb300 as cp  # noqa: E402
 
 TOL = 1e-5
-PLAIN = 5      # launches of a search whose curves the pair sum evaluates at every frequency
+PLAIN = 6      # most launches of a search whose curves the pair sum evaluates at every frequency
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -123,7 +123,7 @@ def test_coarse_fine_is_the_pair_sums(span, coarse_df, top_k, half, sigma_t, int
     dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (b.times, b.mags, b.errs)]
     with cp.Plan(*dev, b.offsets, cp.grid_from(g), sigma_t=sigma_t) as p:
         best = p.best_period()
-        assert p.info()["launches_per_search"] > 7
+        assert p.info()["launches_per_search"] > 8
         same(p.best_period(), best)
     same(best, via_noalloc(b, g, sigma_t))
 
