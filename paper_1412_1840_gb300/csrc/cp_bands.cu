@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kBandsThreads) k_bands(const BandsArgs a)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t off = a.cp[c].off;
     const int n = a.cp[c].n;
-    int np2 = 1;
+    int np2 = 32;
     while (np2 < n) np2 <<= 1;
 
     // (magnitude, sample index) keys; -0 ranks with +0
@@ -93,17 +93,29 @@ __global__ void __launch_bounds__(kBandsThreads) k_bands(const BandsArgs a)
         }
         keys[i] = k;
     }
-    for (int k = 2; k <= np2; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
+    // strides below 32 stay in a warp's registers
+    for (int k = 32; k <= np2; k <<= 1) {
+        for (int j = k >> 1; j >= 32; j >>= 1) {
             __syncthreads();
-            for (int i = tid; i < np2; i += kBandsThreads) {
-                const int ixj = i ^ j;
-                if (ixj > i) {
-                    const bool up = (i & k) == 0;
-                    const unsigned long long u = keys[i], v = keys[ixj];
-                    if ((u > v) == up) { keys[i] = v; keys[ixj] = u; }
+            for (int p = tid; p < np2 >> 1; p += kBandsThreads) {
+                const int i = ((p & ~(j - 1)) << 1) | (p & (j - 1)), o = i | j;
+                const unsigned long long u = keys[i], v = keys[o];
+                if ((u > v) == ((i & k) == 0)) { keys[i] = v; keys[o] = u; }
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < np2; i += kBandsThreads) {
+            unsigned long long u = keys[i];
+            for (int kk = k == 32 ? 2 : k; kk <= k; kk <<= 1) {
+#pragma unroll
+                for (int j = 16; j > 0; j >>= 1) {
+                    if (j >= kk) continue;
+                    const unsigned long long o = __shfl_xor_sync(0xffffffffu, u, j);
+                    const bool low = ((i & kk) == 0) == ((lane & j) == 0);
+                    u = (o < u) == low ? o : u;
                 }
             }
+            keys[i] = u;
         }
     }
     __syncthreads();
@@ -774,20 +786,38 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 2) k_window_refine(const Wi
     // Only candidates that can still reach the first n_t trials matter: with the n_t
     // certain maxima of the list bounding the n_t-th trial's value from below by L,
     // a candidate whose value is below L by more than its error bound cannot.
+    // FP32 with directed rounding: the cut errs on the safe side.
     int rel = cnt;
-    if (lane == 0) {                               // FP32 with directed rounding: the cut errs on the safe side
-        int secured = 0;
+    {
+        int secured = 0, after = cnt;              // first entry behind the n_t-th certain maximum
         float L = INFINITY;
-        for (int r = 0; r < cnt; r++) {
-            const float v = fv[r], er = win_err(v, e);
-            if (secured >= n_t && __fadd_ru(v, er) < L) { rel = r; break; }
-            if (!(kk[r] & 0x40000000) && secured < n_t) {
-                secured++;
-                L = fminf(L, __fsub_rd(v, er));
+        for (int r0 = 0; r0 < cnt && secured < n_t; r0 += 32) {
+            const int r = r0 + lane;
+            const bool sure = r < cnt && !(kk[r] & 0x40000000);
+            const uint32_t bal = __ballot_sync(0xffffffffu, sure);
+            const int rank = secured + __popc(bal & ((1u << lane) - 1u));
+            if (sure && rank < n_t) {
+                L = fminf(L, __fsub_rd(fv[r], win_err(fv[r], e)));
+                if (rank == n_t - 1) after = r + 1;
+            }
+            secured += __popc(bal);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            L = fminf(L, __shfl_xor_sync(0xffffffffu, L, o));
+            after = min(after, __shfl_xor_sync(0xffffffffu, after, o));
+        }
+        if (secured >= n_t) {
+            for (int r0 = after; r0 < cnt; r0 += 32) {
+                const int r = r0 + lane;
+                const uint32_t bal = __ballot_sync(0xffffffffu, r < cnt && __fadd_ru(fv[r], win_err(fv[r], e)) < L);
+                if (bal) {
+                    rel = r0 + __ffs(bal) - 1;
+                    break;
+                }
             }
         }
     }
-    rel = __shfl_sync(0xffffffffu, rel, 0);
 
     // Decide what the FP32 bounds leave open: first with the accurate FP32 value
     // (a bound about ten times tighter), then in FP64, repeated until nothing is
@@ -800,35 +830,47 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 2) k_window_refine(const Wi
     for (int r = lane; r < rel; r += 32) eb[r] = win_err(fv[r], e);
     __syncwarp();
     for (int tier = 1;; tier = 2) {
-        if (lane == 0) {                           // drop the rejected entries, sort the rest
-            int kept = 0;                          // (values >= 0: their bit patterns order as integers)
-            for (int r = 0; r < rel; r++) {
-                const int t = kk[r];
-                if (t < 0) continue;
-                const double v = val[r];
-                const long long vb = __double_as_longlong(v);
-                const float bv = eb[r], f = fv[r];
-                const int k = t & 0x0fffffff;
-                int q = kept;
-                while (q > 0) {
-                    const long long pb = __double_as_longlong(val[q - 1]);
-                    if (!(pb < vb || (pb == vb && (kk[q - 1] & 0x0fffffff) > k))) break;
-                    val[q] = val[q - 1];
-                    eb[q] = eb[q - 1];
-                    fv[q] = fv[q - 1];
-                    kk[q] = kk[q - 1];
-                    q--;
+        {                                          // drop the rejected entries (in order)
+            int kept = 0;
+            for (int r0 = 0; r0 < rel; r0 += 32) {
+                const int r = r0 + lane;
+                const int t = r < rel ? kk[r] : -1;
+                const double v = r < rel ? val[r] : 0.0;
+                const float bv = r < rel ? eb[r] : 0.f, f = r < rel ? fv[r] : 0.f;
+                const uint32_t bal = __ballot_sync(0xffffffffu, t >= 0);
+                if (t >= 0) {                      // never ahead of the entries still to be read
+                    const int q = kept + __popc(bal & ((1u << lane) - 1u));
+                    val[q] = v;
+                    eb[q] = bv;
+                    fv[q] = f;
+                    kk[q] = t;
                 }
-                val[q] = v;
-                eb[q] = bv;
-                fv[q] = f;
-                kk[q] = t;
-                kept++;
+                kept += __popc(bal);
+                __syncwarp();
             }
             rel = kept;
         }
-        rel = __shfl_sync(0xffffffffu, rel, 0);
-        __syncwarp();
+        // sort: value descending (values >= 0: their bit patterns order as integers), ties to the
+        // lower k.  The list is nearly in order, so odd-even exchanges end after a few rounds.
+        for (bool moved = true; moved;) {
+            bool any = false;
+            for (int odd = 0; odd < 2; odd++) {
+                for (int r = 2 * lane + odd; r + 1 < rel; r += 64) {
+                    const long long va = __double_as_longlong(val[r]), vb = __double_as_longlong(val[r + 1]);
+                    const int ta = kk[r], tb = kk[r + 1];
+                    if (va < vb || (va == vb && (ta & 0x0fffffff) > (tb & 0x0fffffff))) {
+                        const float ea = eb[r], fa = fv[r];
+                        val[r] = __longlong_as_double(vb); val[r + 1] = __longlong_as_double(va);
+                        eb[r] = eb[r + 1]; eb[r + 1] = ea;
+                        fv[r] = fv[r + 1]; fv[r + 1] = fa;
+                        kk[r] = tb; kk[r + 1] = ta;
+                        any = true;
+                    }
+                }
+                __syncwarp();
+            }
+            moved = __any_sync(0xffffffffu, any);
+        }
         float ebmax = 0.f;
         for (int r = lane; r < rel; r += 32) ebmax = fmaxf(ebmax, eb[r]);
 #pragma unroll
@@ -863,8 +905,15 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 2) k_window_refine(const Wi
         __syncwarp();
         if (open == 0) break;
         for (int r = 0; r < rel; r++) {
+            if ((r & 31) == 0) {                   // the open ones of the next 32
+                open = __ballot_sync(0xffffffffu, r + lane < rel && (kk[min(r + lane, rel - 1)] & 0x20000000));
+                if (!open) {
+                    r += 31;
+                    continue;
+                }
+            }
+            if (!((uint32_t)open >> (r & 31) & 1u)) continue;
             const int tag = kk[r];
-            if (!(tag & 0x20000000)) continue;
             const int k = tag & 0x0fffffff;
             if (tag & 0x10000000) {                // exact already: nothing to recompute
                 if (lane == 0) kk[r] = tag & ~0x20000000;
