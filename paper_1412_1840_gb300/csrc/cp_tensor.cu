@@ -208,22 +208,24 @@ __global__ void __launch_bounds__(256) k_build_w16(const BuildW16Args a)
 }
 
 // ===========================================================================
-// k_harmonic_coef: a_n = 2 e^-k I_n(k), n = 1..n_max, per curve (one warp),
+// k_harmonic_coef: a_n = 2 e^-k I_n(k), n = 1..n_max, per curve (four warps),
 // trapezoid rule on (1/pi) int_0^pi e^{k(cos t - 1)} cos(n t) dt.  The
 // integrand is evaluated in FP32 (relative error ~1e-5 at most, from the
 // exponent's rounding at k <= 100 and n^2 2^-24 from the Chebyshev recurrence
 // for cos(n t), n <= 32; beyond 32, cos(n t) is evaluated directly on the
 // exactly reduced angle (n k mod 2M) / M turns of pi; far below the tensor
-// form's 1e-3), each lane sums its <= M/32 points in FP32, and the warp sum is
+// form's 1e-3), each lane sums its <= M/128 points in FP32, and the rest is
 // FP64.  (FP64 transcendentals run at 1.68 operations/clk/SM here; this took
-// 0.4 ms per 4096 curves in FP64.)  Written at coef[c * stride + n - 1].
+// 0.4 ms per 4096 curves in FP64.)  Bound by one curve's chain: with one warp a
+// curve and a 64-bit modulo per point and harmonic above 32, 114 us.  Written at coef[c * stride + n - 1].
 // ===========================================================================
-__global__ void __launch_bounds__(256) k_harmonic_coef(const CurveParams* cp, int n_curves, int n_max, int stride,
+constexpr int kCoefWarps = 4;
+__global__ void __launch_bounds__(32 * kCoefWarps) k_harmonic_coef(const CurveParams* cp, int n_curves, int n_max, int stride,
                                                        float* coef)
 {
-    const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
+    __shared__ double s_sum[kCoefWarps][kTcMaxHarmonics];
+    const int c = blockIdx.x, warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    if (c >= n_curves) return;
     const float st = cp[c].sigma_t;
     const float kap = 1.0f / (st * st);
     // quadrature points: enough for the integrand's width ~1/sqrt(k) and the
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(256) k_harmonic_coef(const CurveParams* cp, in
     float acc[kTcMaxHarmonics];
 #pragma unroll
     for (int q = 0; q < kTcMaxHarmonics; q++) acc[q] = 0.f;
-    for (int k = lane; k <= M; k += 32) {
+    for (int k = threadIdx.x; k <= M; k += 32 * kCoefWarps) {
         float sn, ct;
         sincospif((float)k / (float)M, &sn, &ct);
         const float wgt = (k == 0 || k == M) ? 0.5f : 1.0f;
@@ -245,17 +247,29 @@ __global__ void __launch_bounds__(256) k_harmonic_coef(const CurveParams* cp, in
             cm2 = cm1;
             cm1 = cn;
         }
+        if (n_max > 32) {
+            int r = (int)((32ll * k) % (2 * M));         // (q + 1) k mod 2M, one addition a harmonic
 #pragma unroll
-        for (int q = 32; q < kTcMaxHarmonics; q++)
-            if (q < n_max)
-                acc[q] = fmaf(e, cospif((float)(((int64_t)(q + 1) * k) % (2 * M)) / (float)M), acc[q]);
+            for (int q = 32; q < kTcMaxHarmonics; q++) {
+                r += k;
+                r -= r >= 2 * M ? 2 * M : 0;
+                if (q < n_max) acc[q] = fmaf(e, cospif((float)r / (float)M), acc[q]);
+            }
+        }
     }
 #pragma unroll
     for (int q = 0; q < kTcMaxHarmonics; q++) {
         double v = (double)acc[q];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0 && q < n_max) coef[(int64_t)c * stride + q] = (float)(2.0 * v / (double)M);
+        if (lane == 0) s_sum[warp][q] = v;
+    }
+    __syncthreads();
+    const int q = threadIdx.x;
+    if (q < n_max) {
+        double v = 0.0;
+        for (int w = 0; w < kCoefWarps; w++) v += s_sum[w][q];
+        coef[(int64_t)c * stride + q] = (float)(2.0 * v / (double)M);
     }
 }
 
@@ -1023,7 +1037,7 @@ cudaError_t launch_harmonic_coef(const CurveParams* cp, int n_curves, int n_max,
                                  cudaStream_t s)
 {
     if (n_max < 1 || n_max > kTcMaxHarmonics || stride < n_max) return cudaErrorInvalidValue;
-    k_harmonic_coef<<<(n_curves + 7) / 8, 256, 0, s>>>(cp, n_curves, n_max, stride, coef);
+    k_harmonic_coef<<<n_curves, 32 * kCoefWarps, 0, s>>>(cp, n_curves, n_max, stride, coef);
     return cudaGetLastError();
 }
 
