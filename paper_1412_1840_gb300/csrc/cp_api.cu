@@ -121,8 +121,7 @@ struct cp_plan_s {
     std::vector<int64_t> unit_full, unit_coarse, unit_fine, unit_list, wtile;
     std::vector<Wave> waves;
     size_t pair_smem = 0;
-    int pair_grid = 0;
-    int pair_warps = 16;               // warps per block of the pair kernel
+    int pair_grid[2] = {0, 0};         // blocks of 16 warps, of 4
     bool tensor = false;               // CP_FORM_TENSOR
     uint32_t wait_limit = 1u << 26;    // polls per bounded device wait (tensor form)
     int n_max = 0;                     // harmonics of the tensor form
@@ -642,7 +641,8 @@ cp_status enqueue_pair(cp_plan_t p, int stage, int w, float* out, cudaStream_t s
         t.ft = tensor_freqs_per_unit(t.n_max, t.zsplit != 0);
         CP_CUDA(launch_pair_tensor(t, p->n_sm, s));
     } else {
-        CP_CUDA(launch_pair_direct(a, p->pair_warps, p->pair_grid, p->pair_smem, s));
+        const int warps = pair_warps(p->max_n, a.unit_end - a.unit_begin, p->n_sm);
+        CP_CUDA(launch_pair_direct(a, warps, p->pair_grid[warps == 4], p->pair_smem, s));
     }
     if (ev_idx) {
         CP_CUDA(cudaEventRecordWithFlags(p->ev_pair[2 * (*ev_idx) + 1], s, rec_flags(p)));
@@ -696,6 +696,8 @@ SpecArgs spec_args(cp_plan_t p, const SpecPlan& sp, const PairArgs& base)
     a.ex = exclusion_of(p);
     return a;
 }
+
+int spec_chunk_max(cp_plan_t p) { return std::max(p->sfull.chunk, p->ssearch.chunk); }
 
 // Units over whole curves of a fallback list.
 PairArgs over_fallback(cp_plan_t p, PairArgs f, const int* count, const int32_t* slots, int64_t points, int64_t times)
@@ -755,7 +757,8 @@ cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float*
         l.n_cand = kSpecCand;
         l.slot_begin = a.slot_begin;
         l.slot_end = a.slot_end;
-        CP_CUDA(launch_confirm(l, p->d_spart, (int64_t)(confirm_bytes(p->max_n) / sizeof(f2)), p->n_sm, p->max_n, s));
+        CP_CUDA(launch_confirm(l, p->d_spart, (int64_t)(confirm_bytes(p->max_n) / sizeof(f2)),
+                               spec_chunk_max(p), p->n_sm, p->max_n, s));
         return CP_OK;
     };
     for (int b = wv.slot_begin, k = chunk0; b < wv.slot_end; b += sp.chunk, k++) {
@@ -949,16 +952,20 @@ void plan_spec(cp_plan_t p, SpecPlan& sp, const float* st_per_curve, double poin
                Units units)
 {
     const int64_t top = sp.m0 + sp.mq * (p->grid.n_freq - 1);
-    // longest period that a spectrum is made for when the frequencies are interpolated: 4 T <= this
-    // (curves observed for longer are evaluated by the pair sum); and a usual one
-    const double step = p->grid.hierarchical == CP_SEARCH_COARSE_FINE ? p->grid.coarse_df : p->grid.df;
-    const double l_cap = (p->grid.hierarchical == CP_SEARCH_COARSE_FINE ? 32.0 : 4.0) / step;
-    const double l_usual = (p->grid.hierarchical == CP_SEARCH_COARSE_FINE ? 10.0 : 1.0) / step;
+    // Longest period that a spectrum is made for when the frequencies are interpolated: 4 T <= this
+    // (curves observed for longer are evaluated by the pair sum), and a usual one.  The longer cap is
+    // taken where its workspace leaves chunks of 32 curves: a curve whose step is coarser than its
+    // resolution fits it, and smaller chunks cost the others more than it gains (15 curves a chunk
+    // instead of 31: 9.8 against 7.5 ms for 256 coarse-then-fine searches).
+    const bool hier = p->grid.hierarchical == CP_SEARCH_COARSE_FINE;
+    const double step = hier ? p->grid.coarse_df : p->grid.df;
+    const double l_caps[2] = {(hier ? 32.0 : 8.0) / step, (hier ? 13.0 : 2.0) / step};
+    const double l_usual = (hier ? 10.0 : 1.0) / step;
     auto n_out = [&](int nh, double l) {
         return sp.interp ? (int64_t)std::min(1e10, nh * sp.f_top * l + 16.0) : (int64_t)nh * top + 1;
     };
-    double t_pair = 0, t_spec = 0;
-    int lo = kSpecMaxLogQ + 1, hi = 0, fc_min = kFcMax;
+    double t_pair = 0, t_short = 0, t_spec = 0, n_units = 0;
+    int lo = kSpecMaxLogQ + 1, hi[2] = {0, 0}, fc_min = kFcMax, n_max = 0;
     const int usual_nh = spec_harmonics(0.4);
     float last_st = -1.f;
     int nh = 0;
@@ -969,41 +976,57 @@ void plan_spec(cp_plan_t p, SpecPlan& sp, const float* st_per_curve, double poin
                          : p->opt.sigma_t_mode == CP_SIGMA_T_PER_CURVE ? st_per_curve[c] : 0.1f;
         if (st != last_st) nh = spec_harmonics(last_st = st);
         const double n = (double)(p->offsets[c + 1] - p->offsets[c]), pairs = 0.5 * n * (n - 1);
-        // pair sum: per unit of fc frequencies about 4 us for its trig table and sums and 6 us (at 16
-        // frequencies) for every 16 tiles, one unit per SM at a time (measured at N = 150 and 650)
-        const double whole = (double)units(p->fc[c]) *
-                             (4e-6 + 6e-6 * p->fc[c] / kFcMax * std::ceil(tiles_of((int)n) / 16.0)) / p->n_sm;
+        // Pair sum, per unit of fc frequencies and SM.  16 warps: about 4 us for the trig table and the
+        // sums and 6 us (at 16 frequencies) for every 16 tiles (measured at N = 150 to 860).  Blocks of 4
+        // warps: 0.5 us and 0.41 us a tile (N = 75: 3.1 us a unit, 150 6.7, 200 11.8, 310 23).
+        const double u = (double)units(p->fc[c]) / p->n_sm, part = (double)p->fc[c] / kFcMax, tiles = tiles_of((int)n);
+        const double whole = u * (4e-6 + 6e-6 * part * std::ceil(tiles / 16.0));
+        n_units += u;
+        n_max = std::max(n_max, (int)n);
         fc_min = std::min(fc_min, p->fc[c]);
         t_pair += whole;
+        t_short += u * (0.5e-6 + 0.41e-6 * part * tiles);
         if (!nh) {
             t_spec += whole;
             continue;
         }
-        int lq = spec_logq(n_out(nh, l_cap));
-        if (!lq) lq = kSpecMaxLogQ;          // a curve that needs more is evaluated by the pair sum
         const int usual = p->opt.sigma_t_mode == CP_SIGMA_T_RULE ? usual_nh : nh;
         const int ul = spec_logq(n_out(usual, l_usual));
         t_spec += ul ? pairs * 8e-12 + std::ldexp(1.4e-11, ul) + points * usual * (sp.interp ? 2e-11 : 6e-12) : whole;
-        lo = std::min(lo, sp.interp ? kSpecMinLogQ : spec_logq(top + 1) ? spec_logq(top + 1) : lq);
-        hi = std::max(hi, lq);
+        for (int k = 0; k < 2; k++) {
+            int lq = spec_logq(n_out(nh, l_caps[k]));
+            if (!lq) lq = kSpecMaxLogQ;      // a curve that needs more is evaluated by the pair sum
+            hi[k] = std::max(hi[k], lq);
+            if (k) lo = std::min(lo, sp.interp ? kSpecMinLogQ : spec_logq(top + 1) ? spec_logq(top + 1) : lq);
+        }
     }
-    const double launches = p->grid.hierarchical == CP_SEARCH_COARSE_FINE ? 160e-6 : 110e-6;
-    if (!hi || t_spec + launches >= t_pair) return;
+    if (!hi[1]) return;
+    if (pair_warps(p->max_n, (int64_t)(n_units * p->n_sm), p->n_sm) == 4) t_pair = std::min(t_pair, t_short);
     int64_t largest = 0;
     for (const Wave& w : p->waves)
         if (w.cls == 0) largest = std::max<int64_t>(largest, w.slot_end - w.slot_begin);
-    sp.p_ld = (int64_t)(std::ldexp(2.0, hi) / kSpecOver) + 2 * kSpecPad;
     sp.row = row;
     sp.points = (int64_t)points;       // an upper bound: the coarse and the fine points together
-    const size_t per = spec_bytes(sp, hi, p->max_n);
+    size_t per = 0;
+    for (int h : hi) {
+        sp.max_logq = h;
+        sp.p_ld = (int64_t)(std::ldexp(2.0, h) / kSpecOver) + 2 * kSpecPad;
+        per = spec_bytes(sp, h, p->max_n);
+        if ((budget ? budget : kSpecWorkspace) / per >= (size_t)std::min<int64_t>(largest, 32)) break;
+    }
     if (budget && budget < per) return;
     if (!budget) budget = std::max(kSpecWorkspace, per);
-    sp.on = true;
     sp.min_logq = lo;
-    sp.max_logq = hi;
     sp.chunk = (int)std::min<int64_t>({largest, (int64_t)(budget / per), (int64_t)kSpecMaxChunk});
+    sp.chunks = 0;
     for (const Wave& w : p->waves)
         if (w.cls == 0) sp.chunks += (w.slot_end - w.slot_begin + sp.chunk - 1) / sp.chunk;
+    // What the spectrum's launches add (measured at 1 to 114 short curves): a part once, a part for
+    // every chunk, and the candidates' pair sums of the longest curve
+    t_spec += hier ? 50e-6 + 50e-6 * sp.chunks : 30e-6 + 30e-6 * sp.chunks;
+    t_spec += 1e-6 * std::ceil(tiles_of(n_max) / 16.0);
+    if (t_spec >= t_pair) return;
+    sp.on = true;
     sp.seg_items = (4 * p->n_sm + sp.chunk - 1) / sp.chunk;   // about four spreading items per SM and chunk
     p->spec_fc_min = fc_min;
 }
@@ -1245,17 +1268,12 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         const int tb = tune_bucket(tune, (int)n);
         p->fc[c] = fc_for((int)n, tb >= 0 ? tune.direct_fc[tb] : kFcMax);
     }
-    // Short curves have fewer tiles than a block of 16 warps has shares: blocks of 4 warps, four to an
-    // SM, overlap one's trig table and sums with another's tiles (64 curves x 1,000 frequencies: N = 40
-    // 159 -> 65 us, 100 223 -> 136, 150 266 -> 186, 250 481 -> 390; at 420 only with 8 frequencies a
-    // unit, 1152 -> 1069; at 650 slower).  The table of a unit must leave room for four blocks.
-    if (max_n <= kShortCurve) {
-        p->pair_warps = 4;
+    // the tables of short curves leave room for four blocks to an SM (pair_warps)
+    if (max_n <= kShortCurve)
         for (int64_t c = 0; c < n_curves; c++) {
             const int n = (int)(offsets[c + 1] - offsets[c]);
             while (p->fc[c] > 2 && (n + kTile - 1) / kTile * kTile * p->fc[c] * 12 > kShortTable) p->fc[c] >>= 1;
         }
-    }
     p->max_band_points = (max_n + 9) / 10;   // a band holds at most ceil(N/10) samples
     p->n_points = offsets[n_curves];
     p->max_n = max_n;
@@ -1460,7 +1478,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         {(void**)&p->d_sx, sx_bytes},
         {(void**)&p->d_sP, sp_bytes},
         {(void**)&p->d_srow, srow_bytes},
-        {(void**)&p->d_spart, spec ? (size_t)std::max(p->sfull.chunk, p->ssearch.chunk) * confirm_bytes(p->max_n) : 0},
+        {(void**)&p->d_spart, spec ? (size_t)spec_chunk_max(p) * confirm_bytes(p->max_n) + confirm_extra_bytes() : 0},
         {(void**)&p->d_tw, spec ? (size_t)kSpecTwiddles * sizeof(float2) : 0},
         {(void**)&p->d_svblk, svblk_bytes},
         {(void**)&p->d_svmax, spec ? (size_t)nc * sizeof(unsigned int) : 0},
@@ -1551,6 +1569,8 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         CP_CUDA(spec_prepare(p->np2max, p->max_n, p->spec_seg_max));
         CP_CUDA(prepare_selected(p->pair_smem + (size_t)(p->max_n + kTile) * sizeof(float)));
         CP_CUDA(launch_spec_twiddle(p->d_tw, p->stream));
+        CP_CUDA(cudaMemsetAsync((char*)p->d_spart + (size_t)spec_chunk_max(p) * confirm_bytes(p->max_n), 0,
+                                confirm_extra_bytes(), p->stream));
     }
 
     // launch geometry of the persistent pair kernel
@@ -1565,10 +1585,10 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     }
     for (int nm : {4, 8, 12, 16, 32, 48})
         if (p->class_count[class_rank(nm)]) CP_CUDA(prepare_tensor_kernel(nm));   // one CTA per SM
-    {
+    for (int warps : {16, 4}) {
         int occ = 1;
-        CP_CUDA(pair_direct_occupancy(&occ, p->pair_warps, p->pair_smem));
-        p->pair_grid = p->n_sm * std::max(occ, 1);
+        CP_CUDA(pair_direct_occupancy(&occ, warps, p->pair_smem));
+        p->pair_grid[warps == 4] = p->n_sm * std::max(occ, 1);
     }
 
     // events

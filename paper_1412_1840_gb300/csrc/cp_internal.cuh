@@ -31,6 +31,17 @@ constexpr int kFcMax = 16;             // frequencies per work unit (direct form
 constexpr int kShortCurve = 448;       // largest N of a batch for blocks of 4 warps (direct form)
 constexpr int kShortTable = 55296;     // their trig table: four blocks to an SM (54 KB)
 
+// Warps per block of the direct form's pair kernel.  Short curves have fewer tiles than a block of 16
+// warps has shares: blocks of 4 warps, four to an SM, overlap one's trig table and sums with another's
+// tiles (64 curves x 1,000 frequencies: N = 40 159 -> 65 us, 100 223 -> 136, 150 266 -> 186, 250
+// 481 -> 390; at 420 only with 8 frequencies a unit, 1152 -> 1069; at 650 slower).  They need a unit
+// for every block: with fewer, a unit on 16 warps ends sooner (one curve of N = 330, 122 units: 86
+// against 108 us a call).
+inline int pair_warps(int max_n, int64_t units, int n_sm)
+{
+    return max_n <= kShortCurve && units >= (int64_t)4 * n_sm ? 4 : 16;
+}
+
 // Per-curve parameters, indexed by the caller's curve number.
 struct CurveParams {
     int64_t off;      // first sample in the CSR arrays
@@ -211,13 +222,14 @@ struct StatsArgs {
     unsigned int *ip_count, *rho_count;     // [n_curves], zero before the call
 };
 
-// CTAs per curve for the N^2 sums of the statistics: one (with the curve's other
-// work) when there are curves for every SM or the curves are short, else enough
-// for four a SM, at least 16 rows each.
+// CTAs per curve for the N^2 sums of the statistics: one, with the curve's other
+// work, when there are curves enough for eight a SM or the curves are short, else
+// enough for eight a SM, at least 16 rows each.  (384 curves of up to 1,000 samples:
+// 101 us in k_stats alone, the longest curves' sums finishing last.)
 inline int stats_blocks(int64_t n_curves, int max_n, int n_sm)
 {
-    if (n_curves >= n_sm || max_n <= 256) return 0;
-    const int64_t want = (4 * (int64_t)n_sm + n_curves - 1) / n_curves, most = max_n / 16;
+    const int64_t want = (8 * (int64_t)n_sm + n_curves - 1) / n_curves, most = max_n / 16;
+    if (max_n <= 512 || want < 2) return 0;
     return (int)(want < most ? want : most);
 }
 
@@ -366,9 +378,11 @@ cudaError_t launch_pair_tensor(const TensorArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_stats(const StatsArgs& a, int n_curves, cudaStream_t s);
 cudaError_t launch_build_w(const BuildWArgs& a, cudaStream_t s);
 cudaError_t launch_pair_direct(const PairArgs& a, int warps, int grid, size_t smem, cudaStream_t s);   // warps: 16 or 4 a block
-// The pair sum at the candidate entries; part: confirm_bytes(max_n) per slot (part_ld f2).
-cudaError_t launch_confirm(const PairArgs& a, void* part, int64_t part_ld, int n_sm, int max_n, cudaStream_t s);
+// The pair sum at the candidate entries; part: confirm_bytes(max_n) for each of chunk slots (part_ld
+// f2 apart), then confirm_extra_bytes() that start at zero.
+cudaError_t launch_confirm(const PairArgs& a, void* part, int64_t part_ld, int chunk, int n_sm, int max_n, cudaStream_t s);
 size_t confirm_bytes(int max_n);
+size_t confirm_extra_bytes();
 cudaError_t prepare_selected(size_t pair_smem);   // launches over candidates or fb_slots
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t s);
 cudaError_t launch_finalize(const FinalArgs& a, cudaStream_t s);

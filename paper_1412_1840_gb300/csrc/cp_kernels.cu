@@ -10,6 +10,7 @@
 //   k_topk         coarse-grid local maxima for the coarse-then-fine search
 //                  (the bands method of Section 3.1 is in cp_bands.cu)
 //   k_finalize     best frequency, nCKP and Table tab:th discriminator
+#include <algorithm>
 #include <cstdint>
 #include <map>
 #include <mutex>
@@ -98,6 +99,7 @@ __device__ __forceinline__ void sort_floats(float* a, float* other, int np2)
 }
 
 // Block sum of one double per thread in a fixed order (lanes, then warps); thread 0 gets it.
+template <int T>
 __device__ __forceinline__ double stats_sum(double v, double* s_red)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -108,18 +110,19 @@ __device__ __forceinline__ double stats_sum(double v, double* s_red)
     __syncthreads();
     double t = 0.0;
     if (threadIdx.x == 0)
-        for (int w = 0; w < kStatsThreads / 32; w++) t += s_red[w];
+        for (int w = 0; w < T / 32; w++) t += s_red[w];
     return t;
 }
 
 // This block's part of sum_{i<j} g_ij: rows block, block + blocks, ... dealt to the
 // warps, lanes along j, each lane a compensated (Kahan) FP32 sum whose remainder is
 // kept, so that nothing is lost beyond FP32's second order; FP64 only at the end.
+template <int T>
 __device__ __forceinline__ double ip_part(const float* y, int n, int block, int blocks)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float s0 = 0.f, c0 = 0.f, s1 = 0.f, c1 = 0.f;
-    for (int i = block + blocks * warp; i < n; i += blocks * (kStatsThreads / 32)) {
+    for (int i = block + blocks * warp; i < n; i += blocks * (T / 32)) {
         const float yi = y[i];
         int j = i + 1 + lane;
         for (; j + 32 < n; j += 64) {
@@ -156,16 +159,17 @@ __device__ __forceinline__ void set_ip(CurveParams* P, double s2)
 // One CTA per curve.  FP64 runs at 1.7 operations/clk/SM: the phase steps are
 // integer products of the significands, the scalars are dealt to three warps, and
 // the pair sum of IP is FP32.  With few long curves the pair sum is left to k_ip
-// (a.ip_blocks blocks a curve).  70 us for 12 curves of up to 1,000 samples and
-// 568 us for three of up to 4,096 before, 19 and 31 us now (with k_ip).
-__global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
+// (a.ip_blocks blocks a curve).  With k_ip: 12 curves of up to 1,000 samples 70 ->
+// 28 us, three of up to 4,096 568 -> 93 us; a curve of 150 samples 18 -> 14 us.
+template <int T>
+__global__ void __launch_bounds__(T) k_stats(const StatsArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     double* ts = reinterpret_cast<double*>(smem);
     float* ys = reinterpret_cast<float*>(ts + a.np2max);
     float* es = ys + a.np2max;
     float* ypl = es + a.np2max;
-    __shared__ double s_red[kStatsThreads / 32];
+    __shared__ double s_red[T / 32];
     __shared__ double s_t0;
     __shared__ float s_yref, s_gamma;
     __shared__ int s_bad;
@@ -182,7 +186,7 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
 
     // 1. load, validate, min t
     double tmin = INFINITY;
-    for (int i = tid; i < np2; i += kStatsThreads) {
+    for (int i = tid; i < np2; i += T) {
         if (i < n) {
             const double t = a.times[off + i];
             const float y = a.mags[off + i];
@@ -206,12 +210,12 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
     if (lane == 0) s_red[warp] = tmin;
 
     // 2. magnitudes and error bars in ascending order
-    sort_floats<kStatsThreads>(ys, es, np2);
+    sort_floats<T>(ys, es, np2);
 
     // 3. per-curve scalars (FP64), one thread of three warps
     if (tid == 0) {
         double m = s_red[0];
-        for (int w = 1; w < kStatsThreads / 32; w++) m = s_red[w] < m ? s_red[w] : m;
+        for (int w = 1; w < T / 32; w++) m = s_red[w] < m ? s_red[w] : m;
         s_t0 = m;
         P->t0 = m;
         const double sy = median_sorted(es, n);
@@ -248,7 +252,7 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
 
     // 4. scaled magnitudes y' = (y - y_ref) * gamma (same values feed IP and W)
     const float yref = s_yref, gamma = s_gamma;
-    for (int i = tid; i < n; i += kStatsThreads) {
+    for (int i = tid; i < n; i += T) {
         const float v = (ypl[i] - yref) * gamma;
         ypl[i] = v;
         a.yp[off + i] = v;
@@ -257,14 +261,14 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
 
     // 5. IP
     if (a.ip_blocks == 0) {
-        const double s2 = stats_sum(ip_part(ypl, n, 0, 1), s_red);
+        const double s2 = stats_sum<T>(ip_part<T>(ypl, n, 0, 1), s_red);
         if (tid == 0) set_ip(P, s2);
     }
     if (tid == 0 && s_bad) atomicOr(a.status, 1);
 
     // 6. fixed-point phase steps of t - t0 for each grid the search uses
     const double t0 = s_t0;
-    for (int i = tid; i < n; i += kStatsThreads) {
+    for (int i = tid; i < n; i += T) {
         const double tp = ts[i] - t0;
         a.ph_base[off + i] = fixfrac(a.f_min, tp);
         a.ph_full[off + i] = fixfrac(a.df, tp);
@@ -273,6 +277,22 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(const StatsArgs a)
             a.ph_fine[off + i] = fixfrac(a.fine_df, tp);
         }
     }
+}
+
+// Adds the blocks' parts of a curve in the last block to arrive (*last, all threads
+// agree), in a fixed order; thread 0 gets the sum.  At most kStatsThreads blocks.
+__device__ __forceinline__ double last_block_sum(double part, double* parts, unsigned int* count, int blocks,
+                                                 double* s_red, int* last)
+{
+    if (threadIdx.x == 0) {
+        parts[blockIdx.y] = part;
+        __threadfence();
+        *last = atomicAdd(count, 1u) == (unsigned)blocks - 1u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!*last) return 0.0;
+    return stats_sum<kStatsThreads>((int)threadIdx.x < blocks ? __ldcg(parts + threadIdx.x) : 0.0, s_red);
 }
 
 // IP of few curves: a.ip_blocks CTAs a curve; the last to finish adds the parts in
@@ -288,18 +308,9 @@ __global__ void __launch_bounds__(kStatsThreads) k_ip(const StatsArgs a)
     const int n = P->n;
     for (int i = tid; i < n; i += kStatsThreads) y[i] = a.yp[P->off + i];
     __syncthreads();
-    const double part = stats_sum(ip_part(y, n, blockIdx.y, nb), s_red);
-    if (tid == 0) {
-        a.ip_parts[(int64_t)c * nb + blockIdx.y] = part;
-        __threadfence();
-        s_last = atomicAdd(a.ip_count + c, 1u) == (unsigned)nb - 1u;
-        if (s_last) {
-            __threadfence();
-            double s2 = 0.0;
-            for (int b = 0; b < nb; b++) s2 += __ldcg(a.ip_parts + (int64_t)c * nb + b);
-            set_ip(P, s2);
-        }
-    }
+    const double part = stats_sum<kStatsThreads>(ip_part<kStatsThreads>(y, n, blockIdx.y, nb), s_red);
+    const double s2 = last_block_sum(part, a.ip_parts + (int64_t)c * nb, a.ip_count + c, nb, s_red, &s_last);
+    if (tid == 0 && s_last) set_ip(P, s2);
 }
 
 // Tensor form: per sample i, the sum over j of the rounding error of the 16-bit
@@ -314,6 +325,7 @@ __global__ void __launch_bounds__(kStatsThreads) k_wrho(const StatsArgs a)
     extern __shared__ __align__(16) unsigned char smem[];
     float* y = reinterpret_cast<float*>(smem);
     __shared__ double s_red[kStatsThreads / 32];
+    __shared__ int s_last;
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = a.rho_blocks;
     CurveParams* P = a.cp + c;
     const int n = P->n;
@@ -334,17 +346,9 @@ __global__ void __launch_bounds__(kStatsThreads) k_wrho(const StatsArgs a)
             tot += (double)s;
         }
     }
-    const double part = stats_sum(tot, s_red);
-    if (tid == 0) {
-        a.rho_parts[(int64_t)c * nb + blockIdx.y] = part;
-        __threadfence();
-        if (atomicAdd(a.rho_count + c, 1u) == (unsigned)nb - 1u) {
-            __threadfence();
-            double t = 0.0;
-            for (int b = 0; b < nb; b++) t += __ldcg(a.rho_parts + (int64_t)c * nb + b);
-            P->dwsum = (float)t;
-        }
-    }
+    const double part = stats_sum<kStatsThreads>(tot, s_red);
+    const double t = last_block_sum(part, a.rho_parts + (int64_t)c * nb, a.rho_count + c, nb, s_red, &s_last);
+    if (tid == 0 && s_last) P->dwsum = (float)t;
 }
 
 // ===========================================================================
@@ -802,10 +806,11 @@ __global__ void __launch_bounds__(32 * WARPS, 16 / WARPS) k_pair_direct(const Pa
 // of each of its warps, then lanes, then warps), so the value is the same to the
 // last bit.
 // ===========================================================================
-constexpr int kConfirmThreads = 256;
+constexpr int kConfirmThreads = 512;
 constexpr int kConfirmWarps = kConfirmThreads / 32;
 
-__global__ void __launch_bounds__(kConfirmThreads) k_confirm(const PairArgs a, f2* part, int64_t part_ld, int group)
+__global__ void __launch_bounds__(kConfirmThreads) k_confirm(const PairArgs a, f2* part, int64_t part_ld, int group,
+                                                             int smem_bytes)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_pre[kConfirmMaxChunk + 1];
@@ -852,18 +857,28 @@ __global__ void __launch_bounds__(kConfirmThreads) k_confirm(const PairArgs a, f
         const float ts = cosf ? P.tscale * P.tscale * 0.70710678f : P.tscale;
         const float wscale = w_scale(P);
         // frequency pairs per pass: as many as the table holds
-        const int room = (kConfirmSmem - npad * 4) / (npad * 24);
+        const int room = (smem_bytes - npad * 4) / (npad * 24);
         const int step = min(room, (count + 1) >> 1);
         float* Y = reinterpret_cast<float*>(smem);
         ulonglong2* SC = reinterpret_cast<ulonglong2*>(Y + npad);
         f2* NS = reinterpret_cast<f2*>(SC + step * npad);
         const int t0 = (item - s_pre[lo]) * group, t1 = min(t0 + group, ntiles);
         f2* dst = part + (int64_t)lo * part_ld;
+        int bi0, bi1, bj0, bj1;
+        decode_tile(t0, nb, bi0, bj0);
+        decode_tile(t1 - 1, nb, bi1, bj1);
+        if (bi0 != bi1) {                         // several tile rows: every column from the first row on
+            bj0 = bi0;
+            bj1 = nb - 1;
+        }
         for (int f0 = 0; 2 * f0 < count; f0 += step) {
             const int nfp = min(step, ((count + 1) >> 1) - f0);
             __syncthreads();
             for (int q = tid; q < nfp * npad; q += kConfirmThreads) {
                 const int fp = q / npad, i = q - fp * npad;
+                // only the points of the group's tile rows and columns
+                const int b = i / kTile;
+                if (!((b >= bi0 && b <= bi1) || (b >= bj0 && b <= bj1))) continue;
                 if (f0 == 0 && fp == 0) Y[i] = i < n ? a.yp[off + i] : 0.f;
                 ulonglong2 sc = make_ulonglong2(0ull, 0ull);
                 f2 ns = 0ull;
@@ -892,45 +907,80 @@ __global__ void __launch_bounds__(kConfirmThreads) k_confirm(const PairArgs a, f
     }
 }
 
-__global__ void __launch_bounds__(kPairThreads) k_confirm_sum(const PairArgs a, const f2* part, int64_t part_ld)
+// A block per (curve, share of k_pair_direct's 16 warps): its warps load 64 tiles at
+// a time, the first adds them in order; a curve's last block adds the shares.  (One
+// block for all shares pulled 2 MB through one SM for a 4,000-sample curve; one
+// warp a share waited for memory every 16 tiles: 56 and 44 us.)
+constexpr int kSumWarps = 4, kSumLoads = 16;
+
+__global__ void __launch_bounds__(32 * kSumWarps) k_confirm_sum(const PairArgs a, const f2* part, int64_t part_ld,
+                                                                float2* shares, unsigned int* arrived)
 {
-    constexpr int NW = kPairThreads / 32;
-    __shared__ float s_red[NW][2];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int c = a.order[a.slot_begin + blockIdx.x], fp = blockIdx.y;
+    constexpr int NW = kPairThreads / 32, B = kSumWarps * kSumLoads;
+    __shared__ f2 s_v[B][32];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, share = blockIdx.y;
+    const int c = a.order[a.slot_begin + blockIdx.x];
     const int32_t* ce = a.cand + (int64_t)c * a.n_cand;
-    if (ce[2 * fp] < 0) return;
     const CurveParams& P = a.cp[c];
     const int nb = (P.n + kTile - 1) / kTile, ntiles = nb * (nb + 1) / 2;
-    const f2* src = part + (int64_t)blockIdx.x * part_ld + (int64_t)fp * ntiles * 32 + lane;
-    f2 acc = 0ull;
-    int t = warp;
-    for (; t + 3 * NW < ntiles; t += 4 * NW) {
-        f2 v[4];
+    const int mine = (ntiles - share + NW - 1) / NW;           // tiles share, share + 16, ...
+    float2* sums = shares + (int64_t)blockIdx.x * (kConfirmCand / 2) * NW;
+    int pairs = 0;
+    for (; 2 * pairs < a.n_cand && ce[2 * pairs] >= 0; pairs++) {
+        const f2* src = part + (int64_t)blockIdx.x * part_ld + ((int64_t)pairs * ntiles + share) * 32 + lane;
+        f2 acc = 0ull, v[kSumLoads];
+        auto load = [&](int t0) {
 #pragma unroll
-        for (int q = 0; q < 4; q++) v[q] = src[(int64_t)(t + q * NW) * 32];
+            for (int q = 0; q < kSumLoads; q++) {
+                const int t = t0 + warp * kSumLoads + q;
+                v[q] = t < mine ? src[(int64_t)t * (NW * 32)] : 0ull;
+            }
+        };
+        load(0);
+        for (int t0 = 0; t0 < mine; t0 += B) {
+            __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 4; q++) acc = add2(acc, v[q]);
+            for (int q = 0; q < kSumLoads; q++) s_v[warp * kSumLoads + q][lane] = v[q];
+            __syncthreads();
+            if (t0 + B < mine) load(t0 + B);
+            if (warp == 0) {
+                const int m = min(B, mine - t0);
+#pragma unroll 8
+                for (int q = 0; q < m; q++) acc = add2(acc, s_v[q][lane]);
+            }
+        }
+        if (warp == 0) {
+            float vf, vg;
+            upk(acc, vf, vg);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                vf += __shfl_xor_sync(0xffffffffu, vf, o);
+                vg += __shfl_xor_sync(0xffffffffu, vg, o);
+            }
+            if (lane == 0) sums[pairs * NW + share] = make_float2(vf, vg);
+        }
     }
-    for (; t < ntiles; t += NW) acc = add2(acc, src[(int64_t)t * 32]);
-    float vf, vg;
-    upk(acc, vf, vg);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        vf += __shfl_xor_sync(0xffffffffu, vf, o);
-        vg += __shfl_xor_sync(0xffffffffu, vg, o);
-    }
-    if (lane == 0) {
-        s_red[warp][0] = vf;
-        s_red[warp][1] = vg;
+    if (pairs == 0) return;
+    if (tid == 0) {
+        __threadfence();
+        const bool last = atomicAdd(arrived + blockIdx.x, 1u) == NW - 1u;
+        if (last) arrived[blockIdx.x] = 0u;     // for the next launch
+        s_last = last;
+        __threadfence();
     }
     __syncthreads();
-    if (tid < 2 && ce[2 * fp + tid] >= 0) {
+    if (!s_last) return;
+    for (int e = tid; e < 2 * pairs; e += 32 * kSumWarps) {
+        if (ce[e] < 0) continue;
         float S = 0.f;
 #pragma unroll
-        for (int w = 0; w < NW; w++) S += s_red[w][tid];
+        for (int w = 0; w < NW; w++) {
+            const float2 v = __ldcg(sums + (e >> 1) * NW + w);
+            S += (e & 1) ? v.y : v.x;
+        }
         const float v = (2.0f * S + P.diag) * P.norm;
-        const unsigned long long key = cand_emit(a, c, ce[2 * fp + tid], v);
+        const unsigned long long key = cand_emit(a, c, ce[e], v);
         if (key) atomicMax(a.best_key + c, key);
     }
 }
@@ -1036,10 +1086,17 @@ __global__ void k_zero_u64(unsigned long long* p, int64_t n)
 // ---------------------------------------------------------------------------
 namespace cpk {
 
+static bool stats_wide(const StatsArgs& a, int n_curves)
+{
+    return (a.ip_blocks > 0 && a.np2max >= 1024) || (a.np2max >= 512 && n_curves <= 128);
+}
+
 cudaError_t launch_stats(const StatsArgs& a, int n_curves, cudaStream_t s)
 {
     const size_t smem = stats_smem_bytes(a.np2max);
-    k_stats<<<n_curves, kStatsThreads, smem, s>>>(a);
+    // few curves, not the shortest: more threads for each curve's sort and sums
+    if (stats_wide(a, n_curves)) k_stats<1024><<<n_curves, 1024, smem, s>>>(a);
+    else k_stats<kStatsThreads><<<n_curves, kStatsThreads, smem, s>>>(a);
     cudaError_t e = cudaGetLastError();
     const size_t ysmem = (size_t)a.np2max * sizeof(float);
     if (e == cudaSuccess && a.ip_blocks) {
@@ -1093,20 +1150,32 @@ cudaError_t launch_finalize(const FinalArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_confirm(const PairArgs& a, void* part, int64_t part_ld, int n_sm, int max_n, cudaStream_t s)
+cudaError_t launch_confirm(const PairArgs& a, void* part, int64_t part_ld, int chunk, int n_sm, int max_n, cudaStream_t s)
 {
     const int n = a.slot_end - a.slot_begin;
     if (n <= 0) return cudaSuccess;
     if (n > kConfirmMaxChunk || a.n_cand != kConfirmCand) return cudaErrorInvalidValue;
-    // tiles per item: enough items for two per SM, at least one tile a warp, at most eight
+    // tiles per item: one to four a warp, so that there are a few items for every SM
     const int64_t tiles = (int64_t)n * tiles_of(max_n);
     int group = kConfirmWarps;
-    while (group < 8 * kConfirmWarps && tiles / group > 6 * n_sm) group += kConfirmWarps;
-    k_confirm<<<2 * n_sm, kConfirmThreads, kConfirmSmem, s>>>(a, static_cast<f2*>(part), part_ld, group);
+    while (group < 4 * kConfirmWarps && tiles / group > 4 * n_sm) group += kConfirmWarps;
+    // trig table: at least one frequency pair of the longest curve
+    const int npad = (max_n + kTile - 1) & ~(kTile - 1);
+    const int smem = std::min(kConfirmSmem, std::max(npad * 28, 104 * 1024));
+    k_confirm<<<n_sm, kConfirmThreads, smem, s>>>(a, static_cast<f2*>(part), part_ld, group, smem);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_confirm_sum<<<dim3(n, kConfirmCand / 2), kPairThreads, 0, s>>>(a, static_cast<const f2*>(part), part_ld);
+    // after the tiles' sums: the shares' sums of every slot and frequency pair, the slots' arrival counts
+    float2* shares = reinterpret_cast<float2*>(static_cast<f2*>(part) + part_ld * chunk);
+    unsigned int* arrived = reinterpret_cast<unsigned int*>(shares + kConfirmMaxChunk * kConfirmCand / 2 * 16);
+    k_confirm_sum<<<dim3(n, kPairThreads / 32), 32 * kSumWarps, 0, s>>>(a, static_cast<const f2*>(part), part_ld, shares,
+                                                                       arrived);
     return cudaGetLastError();
+}
+
+size_t confirm_extra_bytes()
+{
+    return (size_t)kConfirmMaxChunk * (kConfirmCand / 2) * (16 * sizeof(float2) + sizeof(unsigned int));
 }
 
 size_t confirm_bytes(int max_n) { return (size_t)tiles_of(max_n) * 32 * sizeof(f2) * (kConfirmCand / 2); }
@@ -1141,7 +1210,8 @@ cudaError_t raise_dyn_smem(const void* func, size_t bytes)
 
 cudaError_t prepare_kernels(int np2max, size_t pair_smem)
 {
-    cudaError_t e = raise_dyn_smem((const void*)k_stats, stats_smem_bytes(np2max));
+    cudaError_t e = raise_dyn_smem((const void*)k_stats<kStatsThreads>, stats_smem_bytes(np2max));
+    if (e == cudaSuccess) e = raise_dyn_smem((const void*)k_stats<1024>, stats_smem_bytes(np2max));
     if (e != cudaSuccess) return e;
     e = raise_dyn_smem((const void*)k_pair_direct<false, 4>, pair_smem);
     if (e != cudaSuccess) return e;

@@ -174,11 +174,11 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     int np2max = 32;
     while (np2max < max_n) np2max <<= 1;
     unit_full[0] = unit_coarse[0] = unit_fine[0] = wtile[0] = 0;
-    // blocks of 4 warps for a batch of short curves, as in a plan (cp_api.cu)
-    const int warps = max_n <= kShortCurve ? 4 : 16;
-    auto fc_of = [warps](int npad) {
+    // a batch of short curves leaves room for blocks of 4 warps, as in a plan (cp_api.cu)
+    const int table = max_n <= kShortCurve ? kShortTable : kTableBytes;
+    auto fc_of = [table](int npad) {
         int fc = kFcMax;
-        while (fc > 2 && npad * fc * 12 > (warps == 4 ? kShortTable : kTableBytes)) fc >>= 1;
+        while (fc > 2 && npad * fc * 12 > table) fc >>= 1;
         return fc;
     };
     size_t pair_smem = 0;
@@ -293,8 +293,12 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     bw.tile_end = wtile[nc];
     NA_CUDA(launch_build_w(bw, s));
 
-    int occ = 1;
-    NA_CUDA(pair_direct_occupancy(&occ, warps, pair_smem));
+    auto pair = [&](const PairArgs& a) {
+        const int warps = pair_warps(max_n, a.unit_end - a.unit_begin, nsm);
+        int occ = 1;
+        const cudaError_t e = pair_direct_occupancy(&occ, warps, pair_smem);
+        return e ? e : launch_pair_direct(a, warps, nsm * (occ > 0 ? occ : 1), pair_smem, s);
+    };
     PairArgs pa{};
     pa.cp = d_cp;
     pa.order = d_order;
@@ -326,7 +330,7 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         pa.unit_begin = 0;
         pa.unit_end = unit_full[nc];
         pa.queue = d_u64 + 1 + nc;
-        NA_CUDA(launch_pair_direct(pa, warps, nsm * (occ > 0 ? occ : 1), pair_smem, s));
+        NA_CUDA(pair(pa));
     } else {
         pa.stage = kStageCoarse;
         pa.unit_start = d_unit_coarse;
@@ -336,7 +340,7 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         pa.unit_begin = 0;
         pa.unit_end = unit_coarse[nc];
         pa.queue = d_u64 + 1 + nc + 1;
-        NA_CUDA(launch_pair_direct(pa, warps, nsm * (occ > 0 ? occ : 1), pair_smem, s));
+        NA_CUDA(pair(pa));
         TopkArgs ta{};
         ta.coarse = d_coarse;
         ta.order = d_order;
@@ -353,7 +357,7 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         pa.step = g.fine_df;
         pa.unit_end = unit_fine[nc];
         pa.queue = d_u64 + 1 + nc + 2;
-        NA_CUDA(launch_pair_direct(pa, warps, nsm * (occ > 0 ? occ : 1), pair_smem, s));
+        NA_CUDA(pair(pa));
     }
     FinalArgs fa{};
     fa.cp = d_cp;

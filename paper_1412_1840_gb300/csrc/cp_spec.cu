@@ -245,8 +245,10 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
                 S.support = sup >= (double)S.H ? (int32_t)S.H : min((int32_t)S.H, ((int32_t)sup + 3) & ~3);
             }
         }
-        // segments: about seg_items of them per curve, of 512 cells at least
-        S.seg = min(a.seg_max, max(512, ((S.support / a.seg_items) + 511) & ~511));
+        // segments: seg_items of them per curve or more, about 16384 pairs each (a dense curve's
+        // segment of 512 cells near zero difference took 270 us), of 128 cells at least
+        const int items = max(a.seg_items, (int)(((int64_t)n * n) >> 15));
+        S.seg = min(a.seg_max, max(128, (S.support / items + 127) & ~127));
         a.sc[c] = S;
         s_cpd = S.cells_per_day * 4294967296.0;
         a.vmax[c] = 0u;
@@ -264,7 +266,7 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
 // the pairs of a segment are one range of j per row i (and per fold of the
 // period).  A warp takes 16 rows, half its lanes bisecting for the first j, half
 // for the last, and then 32 pairs at a time across the rows.  Cells are 64-bit
-// integers of 2^-28 quanta: the low word, started at 2^31, takes a shared-memory
+// integers of 2^-26 quanta: the low word, started at 2^31, takes a shared-memory
 // integer add whose carry or borrow (rare) goes to the high word, so the sums are
 // exact and do not depend on the order.  Bound by instructions issued, about 120
 // per 32 pairs: the 8 cells of a pair lie at constant offsets (a margin on both
@@ -274,15 +276,19 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
 constexpr int kSpreadThreads = 512;
 constexpr int kSpreadMargin = 16;                // cells on either side of a segment
 constexpr int kSpreadRows = 16;                  // rows a warp takes at a time
-constexpr float kQuanta = 268435456.0f;          // 2^28 per unit of weight
+// Quanta per unit of weight, 2^26: a contribution is rounded by 4e-9 r.m.s., below the
+// 1.7e-8 of w itself, and the low word spans +-32, which even thousands of pairs on a
+// cell rarely leave.
+constexpr float kQuanta = 67108864.0f;
 
-__device__ __forceinline__ int lower_bound_x(const uint64_t* x, int lo, int hi, uint64_t v)
+// First index in [lo, n) whose cell (high word of x) is at least v; steps: a power of two above n / 2.
+__device__ __forceinline__ int lower_bound_cell(const uint64_t* x, int lo, int n, int steps, uint32_t v)
 {
-    while (lo < hi) {
-        const int m = (lo + hi) >> 1;
-        if (x[m] < v) lo = m + 1; else hi = m;
-    }
-    return lo;
+    const uint32_t* h = reinterpret_cast<const uint32_t*>(x) + 1;
+    int pos = lo - 1;
+    for (int s = steps; s > 0; s >>= 1)
+        if (pos + s < n && h[2 * (pos + s)] < v) pos += s;
+    return pos + 1;
 }
 
 // Items of a launch: counts per curve as a prefix in shared memory.
@@ -329,9 +335,9 @@ __global__ void __launch_bounds__(kSpreadThreads, 2) k_spec_spread(const SpecArg
     int32_t* ch = reinterpret_cast<int32_t*>(cl + words);
     uint64_t* X = reinterpret_cast<uint64_t*>(ch + words);
     float* Y = reinterpret_cast<float*>(X + max_n);
-    __shared__ int s_item;
+    __shared__ int s_item, s_group;
     __shared__ int s_pre[kSpecMaxChunk + 1];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int nc = a.slot_end - a.slot_begin;
     item_prefix(s_pre, nc, [&](int i) {
         const SpecCurve& S = a.sc[a.order[a.slot_begin + i]];
@@ -359,6 +365,7 @@ __global__ void __launch_bounds__(kSpreadThreads, 2) k_spec_spread(const SpecArg
         }
         const int H = (int)S.H;
         const int A = (item - s_pre[ci]) * S.seg, B = min(A + S.seg, S.support), len = B - A;
+        if (tid == 0) s_group = 0;
         for (int i = tid; i < (len + 2 * kSpreadMargin) / 4; i += kSpreadThreads) {
             reinterpret_cast<uint4*>(cl)[i] = make_uint4(0x80000000u, 0x80000000u, 0x80000000u, 0x80000000u);
             reinterpret_cast<int4*>(ch)[i] = make_int4(0, 0, 0, 0);
@@ -367,19 +374,31 @@ __global__ void __launch_bounds__(kSpreadThreads, 2) k_spec_spread(const SpecArg
         const float iph = P.ip_hi, ipl = P.ip_lo;
         const float inv_h = 1.0f / (float)H;
         const uint64_t span = X[n - 1];
-        // folded interval of the differences that touch the segment (window half-width 4, half-cell centres)
-        const int flo = A - 5 > 0 ? A - 5 : 0, fhi = B + 5 < H ? B + 5 : H;
-        for (int r = 0; (uint64_t)r * (uint64_t)H << 32 <= span; r++) {
+        // folded interval of the differences that touch the segment (window half-width 4, half-cell
+        // centres, differences of whole cells off by one at most; a pair that whole cells put on the
+        // wrong side of a fold lands in the margin there, which folds it back)
+        const int flo = A - 6 > 0 ? A - 6 : 0, fhi = B + 6 < H ? B + 6 : H;
+        int steps = 1;
+        while (steps < n) steps <<= 1;
+        // (fold, row group) go to the warps as they become free
+        const int groups = (n + kSpreadRows - 1) / kSpreadRows;
+        const int folds = (int)(span / ((uint64_t)H << 32)) + 1;
+        const uint64_t shift = ((uint64_t)(uint32_t)(kSpreadMargin - A) << 32) - 0x80000000ull;
+        for (;;) {
+            int ticket = 0;
+            if (lane == 0) ticket = atomicAdd(&s_group, 1);
+            ticket = __shfl_sync(0xffffffffu, ticket, 0);
+            if (ticket >= folds * groups) break;
+            const int r = ticket / groups, g = ticket - r * groups;
             const bool odd = r & 1;
-            const uint64_t ulo = (odd ? (uint64_t)(r + 1) * H - fhi : (uint64_t)r * H + flo) << 32;
-            const uint64_t uhi = (odd ? (uint64_t)(r + 1) * H - flo : (uint64_t)r * H + fhi) << 32;
-            if (ulo > span) continue;
+            const uint32_t ulo = odd ? (uint32_t)(r + 1) * H - fhi : (uint32_t)r * H + flo;
+            const uint32_t uhi = odd ? (uint32_t)(r + 1) * H - flo : (uint32_t)r * H + fhi;
+            if (ulo > (uint32_t)(span >> 32) + 1u) continue;
             // cell position of a difference d: +-(d - fold) less half a cell, relative to A - margin
             const uint64_t fold = (uint64_t)(odd ? r + 1 : r) * (uint64_t)H << 32;
-            const uint64_t shift = ((uint64_t)(uint32_t)(kSpreadMargin - A) << 32) - 0x80000000ull;
-            for (int g = warp; g * kSpreadRows < n; g += kSpreadThreads / 32) {
+            {
                 const int row = min(g * kSpreadRows + (lane & (kSpreadRows - 1)), n - 1);
-                const int bound = lower_bound_x(X, row + 1, n, X[row] + (lane < kSpreadRows ? ulo : uhi));
+                const int bound = lower_bound_cell(X, row + 1, n, steps, (uint32_t)(X[row] >> 32) + (lane < kSpreadRows ? ulo : uhi));
                 int cnt = __shfl_down_sync(0xffffffffu, bound, kSpreadRows) - bound;   // lanes below kSpreadRows
                 if (lane >= kSpreadRows || g * kSpreadRows + lane >= n) cnt = 0;
                 int incl = cnt;
@@ -436,15 +455,15 @@ __global__ void __launch_bounds__(kSpreadThreads, 2) k_spec_spread(const SpecArg
         float2* x = a.x + (int64_t)ci * a.x_ld;
         const int Q = H >> 1;
         auto cell = [&](int t) {
-            return fmaf((float)ch[t], 16.0f, (float)(int)(cl[t] - 0x80000000u) * (1.0f / kQuanta));
+            return fmaf((float)ch[t], 64.0f, (float)(int)(cl[t] - 0x80000000u) * (1.0f / kQuanta));
         };
         for (int b = tid; b < len >> 2; b += kSpreadThreads) {
             const int4 h = reinterpret_cast<const int4*>(ch + kSpreadMargin)[b];
             const uint4 l = reinterpret_cast<const uint4*>(cl + kSpreadMargin)[b];
-            float g[4] = {fmaf((float)h.x, 16.0f, (float)(int)(l.x - 0x80000000u) * (1.0f / kQuanta)),
-                          fmaf((float)h.y, 16.0f, (float)(int)(l.y - 0x80000000u) * (1.0f / kQuanta)),
-                          fmaf((float)h.z, 16.0f, (float)(int)(l.z - 0x80000000u) * (1.0f / kQuanta)),
-                          fmaf((float)h.w, 16.0f, (float)(int)(l.w - 0x80000000u) * (1.0f / kQuanta))};
+            float g[4] = {fmaf((float)h.x, 64.0f, (float)(int)(l.x - 0x80000000u) * (1.0f / kQuanta)),
+                          fmaf((float)h.y, 64.0f, (float)(int)(l.y - 0x80000000u) * (1.0f / kQuanta)),
+                          fmaf((float)h.z, 64.0f, (float)(int)(l.z - 0x80000000u) * (1.0f / kQuanta)),
+                          fmaf((float)h.w, 64.0f, (float)(int)(l.w - 0x80000000u) * (1.0f / kQuanta))};
             if (A == 0 && b < kSpreadMargin / 4) {            // cell -1 - i folds to cell i
 #pragma unroll
                 for (int m = 0; m < 4; m++) g[m] += cell(kSpreadMargin - 1 - (4 * b + m));
@@ -931,6 +950,9 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_sum(const SpecArgs a)
 // trial list), each harmonic interpolated from 8 pair-spectrum values.  The
 // position n f L is an integer multiple of the fixed-point f L (32.32).
 // ===========================================================================
+constexpr int kInterpBlock = kSumThreads / 4;      // frequencies per block of the interpolation
+static_assert(kInterpBlock == kSpecBlock, "block maxima");
+
 __device__ __forceinline__ int spec_count(const SpecArgs& a, int c)
 {
     return a.stage == kSpecFine ? a.n_peaks[c] * (2 * a.fine_half + 1) : a.stage == kSpecList ? a.n_trials : (int)a.n_freq;
@@ -945,7 +967,7 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
     const int nc = a.slot_end - a.slot_begin;
     item_prefix(s_pre, nc, [&](int i) {
         const int c = a.order[a.slot_begin + i];
-        return a.sc[c].nh && !a.sc[c].whole ? (spec_count(a, c) + kSumThreads - 1) / kSumThreads : 0;
+        return a.sc[c].nh && !a.sc[c].whole ? (spec_count(a, c) + kInterpBlock - 1) / kInterpBlock : 0;
     });
     for (int item = blockIdx.x; item < s_pre[nc]; item += gridDim.x) {
         const int ci = item_curve(s_pre, nc, item);
@@ -955,11 +977,14 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
         if (tid < S.nh) s_a[tid] = a.coef[(int64_t)c * kSpecMaxHarm + tid];
         __syncthreads();
         const float* Ps = a.P + (int64_t)ci * a.p_ld + kSpecPad;
-        const int q = (item - s_pre[ci]) * kSumThreads + tid;
+        // four threads a frequency, each every fourth harmonic (one thread's chain of up to 64
+        // dependent fetches took 55 us a launch, however few the frequencies)
+        const int q = (item - s_pre[ci]) * kInterpBlock + (tid >> 2), part = tid & 3;
         unsigned int key = 0u;
-        if (q < spec_count(a, c)) {
-            double f;
-            bool ok = true, live = true;          // admissible as the best; evaluated at all
+        const bool in = q < spec_count(a, c);
+        bool ok = in, live = in;                  // admissible as the best; evaluated at all
+        double f = 0.0;
+        if (in) {
             if (a.stage == kSpecFine) {
                 const int W = 2 * a.fine_half + 1, pk = q / W;
                 const double fpk = grid_freq(a.f_min, (double)a.peaks[(int64_t)c * a.top_k + pk], a.coarse_df);
@@ -975,14 +1000,13 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
                 f = grid_freq(a.f_min, (double)q, a.step);
                 ok = a.stage == kSpecFull && !excluded_k(a.ex.full_k, a.ex.n, q);
             }
-            float v = 0.f;
-            if (live) {
-                const uint64_t step = (uint64_t)__double2ll_rn(f * S.L * 4294967296.0);
-                uint64_t pos = 0;
-                float s = 0.f;
+        }
+        float s = 0.f;
+        if (live) {
+            const uint64_t step = (uint64_t)__double2ll_rn(f * S.L * 4294967296.0);
+            uint64_t pos = step * (uint64_t)(part + 1);
 #pragma unroll 2
-                for (int h = 0; h < S.nh; h++) {
-                    pos += step;
+            for (int h = part; h < S.nh; h += 4, pos += 4 * step) {
                     float w[8];
                     kb_weights((float)(uint32_t)pos * 2.3283064365386963e-10f - 0.5f, w);
                     const float* p = Ps + ((int)(pos >> 32) - 3);
@@ -990,9 +1014,12 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
 #pragma unroll
                     for (int k = 0; k < 8; k++) t = fmaf(w[k], p[k], t);
                     s = fmaf(s_a[h], t, s);
-                }
-                v = fmaf(2.0f, s, P.diag * S.one_minus_a0) * P.norm;
             }
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (in && part == 0) {
+            float v = live ? fmaf(2.0f, s, P.diag * S.one_minus_a0) * P.norm : 0.f;
             if (a.stage == kSpecFine && !ok) v = -INFINITY;
             if (a.stage == kSpecList && !live) v = __int_as_float(0x7fc00000);
             a.rows[(a.rows_by_curve ? (int64_t)c : (int64_t)ci) * a.row_ld + q] = v;
@@ -1064,7 +1091,7 @@ __global__ void __launch_bounds__(kSelThreads) k_spec_select(const SpecArgs a)
         const float thr = v0 - spec_margin(v0, P);
         const unsigned int othr = orderable(thr);
         const float* row = a.rows + (a.rows_by_curve ? (int64_t)c : (int64_t)ci) * a.row_ld;
-        const int count = spec_count(a, c), per = a.interp ? kSumThreads : kSumThreads * kSumPer;
+        const int count = spec_count(a, c), per = a.interp ? kInterpBlock : kSumThreads * kSumPer;
         // only the blocks whose largest admissible value reaches the threshold are read again
         for (int b = tid; b * per < count; b += kSelThreads)
             if (a.vblk[(int64_t)ci * a.vb_ld + b] >= othr) {

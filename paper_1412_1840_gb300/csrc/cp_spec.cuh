@@ -21,7 +21,7 @@ constexpr int kSpecMaxChunk = kConfirmMaxChunk;   // curves per chunk
 constexpr double kSpecTail = 2e-8;     // harmonics left out: at most this much of the kernel's peak
 constexpr double kSpecOver = 1.1;      // transform length over the highest frequency needed, at least
 
-constexpr int kSpecBlock = 256;        // values per block at least (one item of the value kernels)
+constexpr int kSpecBlock = 64;         // values per block at least (one item of the value kernels)
 constexpr int kSpecPad = 8;            // pair-spectrum values kept before index 0 (P(-nu) = P(nu))
 
 // Which frequencies a launch evaluates.

@@ -151,3 +151,13 @@ def test_curves_outside_the_spectrums_range():
     adm = ~np.any([(f >= lo) & (f <= hi) for lo, hi in g.exclude], axis=0)
     want = [np.flatnonzero(adm)[np.argmax(rows[c][adm])] for c in keep]
     np.testing.assert_array_equal(left["best_idx"][keep], want)
+
+
+@pytest.mark.parametrize("n", [40, 300, 448])
+def test_pair_sum_is_the_same_on_either_block_size(n):
+    """Short curves run on blocks of 4 warps once every SM has four of its units
+    (below that: 16 warps): the sums' order, hence every bit, is the same."""
+    b = batch(1, n, n, 900.0)
+    few, many = 2000, 16 * 4 * 160          # fewer units than 4 per SM at 8 a unit; more at 16 a unit
+    rows = [run(b, synth.Grid(0.01, 1e-4, k), sigma_t=0.08)[0] for k in (few, many)]
+    np.testing.assert_array_equal(rows[0][0], rows[1][0, :few])
