@@ -133,6 +133,7 @@ struct cp_plan_s {
     SpecPlan sfull, ssearch;           // the uniform grid; the coarse-then-fine or bands search
     int spec_fc_min = kFcMax;
     int spec_seg_max = 0;
+    size_t spec_budget = 0;            // workspace of the pair spectrum at most
     bool keep_w = true;                // some pass of the direct-form curves reads W tiles
     bool spec() const { return sfull.on || ssearch.on; }
     SpecCurve* d_sc = nullptr;
@@ -725,9 +726,9 @@ cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float*
     int chunk0 = 0;      // chunks of the waves before this one
     for (int v = 0; v < w; v++)
         if (p->waves[v].cls == 0) chunk0 += (p->waves[v].slot_end - p->waves[v].slot_begin + sp.chunk - 1) / sp.chunk;
-    // work counters: spreading items per chunk, then two fallback counts per wave
+    // work counters: two per chunk, then two fallback counts per wave
     unsigned long long* q0 = queue_word(p, kQueuesPerWave * (int)p->waves.size());
-    int* fb = reinterpret_cast<int*>(q0 + sp.chunks + w);              // [0] whole curves, [1] coarse rows
+    int* fb = reinterpret_cast<int*>(q0 + 2 * sp.chunks + w);              // [0] whole curves, [1] coarse rows
     int32_t* fb_whole = p->d_sfb;
     int32_t* fb_coarse = p->d_sfb + p->n_curves;
 
@@ -764,7 +765,7 @@ cp_status enqueue_spec(cp_plan_t p, const SpecPlan& sp, int stage, int w, float*
     for (int b = wv.slot_begin, k = chunk0; b < wv.slot_end; b += sp.chunk, k++) {
         a.slot_begin = b;
         a.slot_end = std::min(b + sp.chunk, wv.slot_end);
-        a.queue = q0 + k;
+        a.queue = q0 + 2 * k;
         CP_CUDA(launch_spec_transform(a, p->n_sm, p->max_n, sp.min_logq <= kSpecOneLogQ, sp.max_logq > kSpecOneLogQ, s));
         CP_CUDA(launch_spec_values(a, p->n_sm, s));
         SpecArgs sel = a;
@@ -934,16 +935,18 @@ cp_status read_timings(cp_plan_t p)
     return CP_OK;
 }
 
-// Workspace of the pair spectrum per plan.  A chunk's transforms pass through the
-// L2 cache better the fewer there are, and the allocation costs the plan time.
-constexpr size_t kSpecWorkspace = (size_t)1 << 30;
+// Workspace of the pair spectrum per plan (at most an eighth of the free memory, or one
+// curve's).  Every chunk ends in latency-bound kernels and half-empty last waves: 384 curves
+// of 300 to 1,000 samples at 49,981 frequencies take 4.44 ms with 1 GB (13 chunks), 4.14 with
+// 2, 3.94 with 4 (4 chunks), 3.79 with 8; allocating 4 GB costs a plan 0.3 ms.
+constexpr size_t kSpecWorkspace = (size_t)4 << 30;
 size_t spec_bytes(const SpecPlan& sp, int logq, int max_n)
 {
     return (sizeof(float2) << logq) + (size_t)(sp.p_ld + sp.row) * sizeof(float) + confirm_bytes(max_n) + 1024;
 }
 
 // Whether one kind of pass of the direct-form curves goes through the pair
-// spectrum, and its workspace (budget 0: kSpecWorkspace, or one curve's).  `points`: frequencies per curve; `units`: pair-sum
+// spectrum, and its workspace (budget 0: spec_budget, or one curve's).  `points`: frequencies per curve; `units`: pair-sum
 // units of a curve at f frequencies per unit.  The pair sum takes N (N - 1) / 2
 // exponentials per frequency; the spectrum a few operations per pair, the
 // transform, and nh products (interpolated: 8 nh) per frequency, and more launches.
@@ -1012,12 +1015,14 @@ void plan_spec(cp_plan_t p, SpecPlan& sp, const float* st_per_curve, double poin
         sp.max_logq = h;
         sp.p_ld = (int64_t)(std::ldexp(2.0, h) / kSpecOver) + 2 * kSpecPad;
         per = spec_bytes(sp, h, p->max_n);
-        if ((budget ? budget : kSpecWorkspace) / per >= (size_t)std::min<int64_t>(largest, 32)) break;
+        if ((budget ? budget : p->spec_budget) / per >= (size_t)std::min<int64_t>(largest, 32)) break;
     }
     if (budget && budget < per) return;
-    if (!budget) budget = std::max(kSpecWorkspace, per);
+    if (!budget) budget = std::max(p->spec_budget, per);
     sp.min_logq = lo;
     sp.chunk = (int)std::min<int64_t>({largest, (int64_t)(budget / per), (int64_t)kSpecMaxChunk});
+    const int64_t chunks = (largest + sp.chunk - 1) / sp.chunk;
+    sp.chunk = (int)((largest + chunks - 1) / chunks);       // of about equal sizes: a short last one leaves the chip idle
     sp.chunks = 0;
     for (const Wave& w : p->waves)
         if (w.cls == 0) sp.chunks += (w.slot_end - w.slot_begin + sp.chunk - 1) / sp.chunk;
@@ -1419,6 +1424,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     }
 
     p->spec_seg_max = spec_seg_max(p->max_n);
+    p->spec_budget = std::min<size_t>(kSpecWorkspace, free_b / 8);
     plan_spectra(p, opt.sigma_t_per_curve);
     const bool spec = p->spec();
     // magnitude-kernel tiles of the direct-form curves: only for passes that go through the pair sum
@@ -1435,7 +1441,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
 
     // device allocation (one block)
     const int64_t np = p->n_points, nc = n_curves;
-    const int nq = kQueuesPerWave * (int)p->waves.size() + (spec ? spec_chunks + (int)p->waves.size() : 0);
+    const int nq = kQueuesPerWave * (int)p->waves.size() + (spec ? 2 * spec_chunks + (int)p->waves.size() : 0);
     p->ip_blocks = stats_blocks(nc, max_n, p->n_sm);
     p->n_u64 = 1 + nc + nq + nc;      // status, keys, work counters, two 32-bit counts per curve
     struct Part { void** dst; size_t bytes; };

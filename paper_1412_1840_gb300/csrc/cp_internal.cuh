@@ -94,7 +94,7 @@ enum Stage : int { kStageFull = 0, kStageCoarse = 1, kStageFine = 2, kStageList 
 enum Candidates : int { kCandNone = 0, kCandGrid = 1, kCandCoarse = 2, kCandTrial = 3, kCandFine = 4 };
 
 constexpr int kConfirmCand = 32;             // candidate entries per curve (one ballot)
-constexpr int kConfirmMaxChunk = 64;         // curves per launch
+constexpr int kConfirmMaxChunk = 192;        // curves per launch
 constexpr int kConfirmSmem = 114 * 1024;     // trig table and magnitudes (one frequency pair of the longest curve)
 
 // Direct-form pair tiling: a warp owns a 32 x 32 tile of (row i, col j)

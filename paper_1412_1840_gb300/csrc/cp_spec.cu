@@ -806,12 +806,19 @@ __global__ void __launch_bounds__(kFftThreads, 2) k_spec_fft2(const SpecArgs a)
     extern __shared__ __align__(16) unsigned char smem[];
     cx* sm = reinterpret_cast<cx*>(smem);
     __shared__ int s_pre[kSpecMaxChunk + 1];
+    __shared__ int s_next;
     const int nc = a.slot_end - a.slot_begin;
     item_prefix(s_pre, nc, [&](int i) {
         const SpecCurve& S = a.sc[a.order[a.slot_begin + i]];
         return S.nh && S.logq > kSpecOneLogQ ? 1 << (S.logq - 13) : 0;
     });
-    for (int item = blockIdx.x; item < s_pre[nc]; item += gridDim.x) {
+    // Items are started in order, by ticket: the runs that neighbouring items write are half a sector
+    // each above 2^19 points, and meet in L2 only if their blocks keep together (71 curves of 2^20
+    // points in one launch: 1400 us with a fixed stride of the grid, against 960 in three launches).
+    int item = blockIdx.x;
+    while (item < s_pre[nc]) {
+        int next = 0;
+        if (threadIdx.x == 0) next = (int)gridDim.x + (int)atomicAdd(a.queue + 1, 1ull);
         const int ci = item_curve(s_pre, nc, item);
         const SpecCurve S = a.sc[a.order[a.slot_begin + ci]];
         const cx* x = reinterpret_cast<const cx*>(a.x + (int64_t)ci * a.x_ld);
@@ -825,6 +832,9 @@ __global__ void __launch_bounds__(kFftThreads, 2) k_spec_fft2(const SpecArgs a)
         default: fft2_item<11>(a, S, x, P, blk, sm); break;
         }
         __syncthreads();
+        if (threadIdx.x == 0) s_next = next;
+        __syncthreads();
+        item = s_next;
     }
 }
 

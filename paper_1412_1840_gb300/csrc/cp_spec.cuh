@@ -82,7 +82,7 @@ struct SpecArgs {
     int32_t* cand;                // [n_curves * kSpecCand] candidate entries, -1 after the last
     int32_t* fb_slots;            // slots that the pair sum evaluates whole
     int* fb_count;
-    unsigned long long* queue;    // spreading items
+    unsigned long long* queue;    // two work counters of the chunk: spreading, second transform pass
     const float2* tw;             // twiddle factors, see launch_spec_twiddle
     Exclusion ex;
 };

@@ -66,6 +66,10 @@ CASES = [
     (64, 60, 130, 700.0, 0.00143, 1e-3, 3500, 0.5),
     (6, 200, 400, 1733.0, 1.0 / 1733.0, 1e-4, 6000, 0.1),
     (6, 300, 400, 5000.0, 0.0123457, 1e-3, 5000, 0.3),   # longer than the spectra are made for
+    # more curves than one launch takes
+    (200, 60, 90, 300.0, 0.01, 2e-3, 1500, 0.4),
+    # transforms of 2^20 points
+    (2, 300, 400, 1500.0, 0.0, 1e-4, 40000, 0.1),
 ]
 
 
