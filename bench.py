@@ -1,9 +1,10 @@
 """Throughput benchmark of the GB300 CKP periodogram (arXiv:1412.1840).
 
 One step = one best-period search over one synthetic batch through the C ABI
-(cp_best_period): per-curve scalars, magnitude-kernel tiles, the pair sum at
-every trial frequency, normalisation, argmax / coarse-then-fine search and the
-Table tab:th discriminator.
+(cp_best_period): per-curve scalars, the pair spectrum and the statistic at
+every trial frequency (or the pair sum, where that is cheaper), the pair sum at
+the candidates for the best, normalisation, argmax / coarse-then-fine search and
+the Table tab:th discriminator.
 
 Default workload (N=1): 4096 lightcurves, N ~ U{300..1000}, seasonal sampling
 over 2500 d, grid 0.002-5 1/d step 1e-4 (49,981 frequencies), direct form,
@@ -13,8 +14,9 @@ sigma_t from the Bowley-skewness rule.
             around each step; L2 flushed between steps)
   e2e       the same through host (pinned) buffers: H2D of the inputs and D2H
             of the results inside every timed step
-  roofline  the pair-sum kernel against the SFU/FP32 pipe ceiling (one ex2 per
-            pair-frequency evaluation, 32 ex2/clk/SM)
+  roofline  the pair spectrum's kernels against the measured copy bandwidth (the
+            transforms' least traffic); where the pair sum evaluates every frequency,
+            that kernel against the SFU ceiling (one ex2 per pair-frequency, 32/clk/SM)
   cpu_baseline  the FP64 oracle timed on the host cores on a bounded sample
   tensor    the tensor-core form on the same batch (FP16 or BF16 operands, per-curve
             harmonics): device-resident rate, its roofline against the measured
@@ -55,6 +57,28 @@ def sfu_ex2_per_clk_sm():
 # same curve hit L2, so a full launch moves (this ratio) x (its tile bytes).
 DRAM_PER_W_BYTE_DIRECT = 1.034
 DRAM_PER_W_BYTE_TENSOR = 1.044
+
+
+def spectrum_bytes(sigma_t, g):
+    """Least memory traffic of the pair spectrum of curves with these sigma_t on a uniform grid from a
+    multiple of df (csrc/cp_spec.cu): the cells and the data between the two transform passes each
+    written and read once, the spectrum written and read once, the values written once."""
+    top = int(round(g.f_min / g.df)) + g.n_freq - 1
+    total = 0.0
+    for st, count in zip(*np.unique(np.round(np.asarray(sigma_t, np.float64), 3), return_counts=True)):
+        k = 1.0 / (st * st)                     # a_n = 2 e^-k I_n(k) by the backward recurrence
+        n0 = min(130, int(14 + 10 / st))
+        a = np.zeros(n0 + 2)
+        a[n0] = 1e-200
+        for n in range(n0, 0, -1):
+            a[n - 1] = a[n + 1] + 2.0 * n / k * a[n]
+        a[1:] *= 2.0
+        tail = np.cumsum((a / a.sum())[::-1])[::-1]           # tail[n] = a_n + a_{n+1} + ...
+        nh = int(np.argmax(tail[1:] <= 2e-8))                 # harmonics kept
+        n_out = nh * top + 1
+        q = 2.0 ** np.ceil(np.log2(max(1.1 * n_out / 2.0, 256.0)))
+        total += count * (4 * 8 * q + 2 * 4 * n_out + 4 * g.n_freq)
+    return total
 
 
 def measured_peaks():
@@ -318,6 +342,7 @@ def main():
         barrier()
     step_ms = [ev0[k].elapsed_time(ev1[k]) for k in range(args.steps)]
     info = plan.info()
+    sigma_t = plan.curve_stats()["sigma_t"]
     total_s = max_over_ranks(sum(step_ms) / 1e3, device=dev)
     value = n_job * args.steps / total_s
     plan.close()
@@ -503,7 +528,7 @@ def main():
                 ent["roofline_frac"] = hi_["tensor_flops_search"] / (np.mean(km) / 1e3) / 1e12 / \
                     measured_peaks()["bf16_tflops_sustained"]
                 ent["dtype"] = "fp16"
-            else:
+            elif hi_["w_bytes_direct"]:        # every frequency by the pair sum
                 ent["roofline_frac"] = hi_["pair_freq_search"] / (np.mean(km) / 1e3) / \
                     (sfu_ex2_per_clk_sm() * hi_["n_sm"] * SM_MAX_MHZ * 1e6)
             hier[fname] = ent
@@ -551,8 +576,9 @@ def main():
             else:
                 ent["note"] = "no warm-up step (kernels already loaded by the runs above; the first call " \
                               "instantiates its CUDA graph inside the timed step)"
-                ent["roofline_frac"] = tinfo["pair_freq_search"] / (tinfo["last_pair_kernel_ms"] / 1e3) / \
-                    (sfu_ex2_per_clk_sm() * tinfo["n_sm"] * SM_MAX_MHZ * 1e6)
+                if tinfo["w_bytes_direct"]:
+                    ent["roofline_frac"] = tinfo["pair_freq_search"] / (tinfo["last_pair_kernel_ms"] / 1e3) / \
+                        (sfu_ex2_per_clk_sm() * tinfo["n_sm"] * SM_MAX_MHZ * 1e6)
             thr[fname] = ent
         rel = np.abs(res["tensor"].astype(np.float64) - res["direct"]) / \
             np.maximum(np.abs(res["direct"].astype(np.float64)), 1e-30)
@@ -600,6 +626,14 @@ def main():
                      "avg_launch_ms": float(np.mean(pair_ms))},
         "clocks": clocks,
     }
+    if args.form == "direct" and not info["w_bytes_direct"]:      # through the pair spectrum
+        peaks = measured_peaks()
+        line["roofline"] = {"bound": "hbm", "peak": peaks["hbm_gbs"], "unit": "GB/s", "kernel": "k_spec_*",
+                            "peak_basis": "copy bandwidth, " + peaks["source"], "avg_launch_ms": float(np.mean(pair_ms))}
+        if not (g.hierarchical or getattr(g, "bands", False)):
+            least = spectrum_bytes(sigma_t, g)
+            line["roofline"].update(achieved=least / pair_s / 1e9, frac=least / pair_s / 1e9 / peaks["hbm_gbs"],
+                                    traffic=least, traffic_basis="least traffic of the transforms (not measured)")
     if args.form == "tensor":
         peaks = measured_peaks()
         tflops = info["tensor_flops_search"] / (info["last_tensor_kernel_ms"] / 1e3) / 1e12

@@ -49,7 +49,9 @@ typedef enum {
 typedef struct cp_plan_s *cp_plan_t;
 
 /* Evaluation form. */
-enum { CP_FORM_DIRECT = 0, /* FP32 pair sum, FP64-exact fixed-point phases          */
+enum { CP_FORM_DIRECT = 0, /* FP32 pair sum, FP64-exact fixed-point phases, or the */
+                           /* pair spectrum (FP32) where that takes less time; the  */
+                           /* best frequency is the pair sum's either way           */
        CP_FORM_TENSOR = 1  /* Fourier/Bessel series, FP16/BF16 tcgen05 GEMMs        */ };
 /* Operand type of the tensor form (FP32 accumulation in every case).
  * FP16: 11 significand bits; meets 1e-3 of the peak with single operands.
@@ -322,9 +324,11 @@ typedef struct {
     int64_t n_curves;
     int64_t n_points;             /* sum N                                             */
     double pair_freq_full;        /* sum_c N(N-1)/2 * n_freq: one uniform-grid pass     */
-    double pair_freq_search;      /* pair-frequency evaluations of one cp_best_period   */
+    double pair_freq_search;      /* the same for the frequencies of a cp_best_period   */
+                                  /* (the pair spectrum gets by with far fewer)       */
     int64_t launches_per_search;  /* kernels one cp_best_period launches                */
-    float last_pair_kernel_ms;    /* device time of the pair-sum kernel(s), last call   */
+    float last_pair_kernel_ms;    /* device time of the pair-sum or pair-spectrum       */
+                                  /* kernels, last call                               */
     float last_step_ms;           /* device time of the whole last cp_best_period       */
     int32_t n_sm;                 /* SMs of the plan's device                           */
     int32_t max_n;                /* largest N in the batch                             */
@@ -341,7 +345,8 @@ typedef struct {
     double window_terms_search;   /* bands method: spectral-window terms (band point x  */
                                   /* grid frequency) of one cp_best_period              */
     double w_bytes_direct;        /* bytes of the magnitude-kernel tiles one search     */
-    double w_bytes_tensor;        /* builds for the direct / tensor-form curves         */
+    double w_bytes_tensor;        /* builds for the direct / tensor-form curves (none   */
+                                  /* for direct curves through the pair spectrum)     */
     int64_t replans;              /* plans rebuilt after a curve's sigma_t left the     */
                                   /* range of its harmonic count (see cp_options.n_max) */
     int64_t bands_exact_scans;    /* bands method, last search: (curve, band) lists     */
@@ -374,9 +379,9 @@ cp_status cp_bessel_coefficients(double sigma_t, int32_t n_max, double *out);
  * for their own pools at start-up, latency-bounded pipelines that must not
  * enter the allocator, or plug-ins whose host owns the allocator.
  *
- * It runs the direct form (same kernels and results as cp_best_period with
- * CP_FORM_DIRECT, CP_SIGMA_T_FIXED, alpha = 1) and allocates nothing: every
- * intermediate buffer lives in one static device array of
+ * It runs the direct form's pair sum at every frequency (same results as
+ * cp_best_period with CP_FORM_DIRECT, CP_SIGMA_T_FIXED, alpha = 1) and
+ * allocates nothing: every intermediate buffer lives in one static device array of
  * CP_NOALLOC_SCRATCH_BYTES that each GPU loading the library holds until the
  * process exits.  Its first call on a device looks up that array's device
  * address (cudaGetSymbolAddress) with the device current.

@@ -1853,10 +1853,14 @@ cp_status cp_get_plan_info(cp_plan_t p, cp_plan_info* info)
     info->last_bands_kernel_ms = p->last_bands_ms;
     info->reserved0 = 0.f;
     info->window_terms_search = p->window_terms;
+    // a search through the pair spectrum builds no direct-form tiles
+    const bool spec = p->grid.hierarchical == CP_SEARCH_FULL ? p->sfull.on : p->ssearch.on;
     double wd = 0, wt = 0;
-    for (const Wave& w : p->waves)
-        (w.cls ? wt : wd) += (double)(w.tile_end - w.tile_begin) *
-                             (w.cls ? (double)tensor_tile_bytes(w_bf16(p->opt.dtype)) : (double)kTileFloats * 4);
+    for (const Wave& w : p->waves) {
+        const double tiles = (double)(w.tile_end - w.tile_begin);
+        if (w.cls) wt += tiles * (double)tensor_tile_bytes(w_bf16(p->opt.dtype));
+        else if (!spec) wd += tiles * (double)kTileFloats * 4;
+    }
     info->w_bytes_direct = wd;
     info->w_bytes_tensor = wt;
     info->replans = p->replans;
