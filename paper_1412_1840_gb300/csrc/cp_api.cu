@@ -831,6 +831,7 @@ cp_status enqueue_search(cp_plan_t p, cudaStream_t s)
         CP_CUDA(launch_bands(b, (int)p->n_curves, s));
         WindowArgs wa{};
         wa.cp = p->d_cp;
+        wa.order = p->d_order;
         wa.band_of = p->d_band_of;
         wa.kept = p->d_kept;
         wa.ph_base = p->d_ph_base;

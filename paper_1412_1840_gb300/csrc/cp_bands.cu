@@ -292,7 +292,8 @@ __global__ void __launch_bounds__(kWinThreads) k_window(const WindowArgs a)
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NW = kWinThreads / 32;
-    const int c = blockIdx.x / a.n_bands, b = blockIdx.x - c * a.n_bands;
+    // longest curves first: 4 blocks fit an SM, and the last wave is the shorter the smaller its bands
+    const int slot = blockIdx.x / a.n_bands, b = blockIdx.x - slot * a.n_bands, c = a.order[slot];
     const int K = a.n_freq, n_t = win_candidates(a.n_t);   // candidates kept per band
     const int64_t off = a.cp[c].off;
     const int n = a.cp[c].n;

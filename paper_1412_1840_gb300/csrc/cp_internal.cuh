@@ -342,6 +342,7 @@ struct BandsArgs {
 
 struct WindowArgs {
     const CurveParams* cp;
+    const int32_t* order;         // slot -> curve, longest first
     const int8_t* band_of;
     const int32_t* kept;
     const uint64_t* ph_base;      // frac(f_min (t - t0)) in 2^-64 turns
