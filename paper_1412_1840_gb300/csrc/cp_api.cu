@@ -642,7 +642,7 @@ cp_status enqueue_pair(cp_plan_t p, int stage, int w, float* out, cudaStream_t s
         t.ft = tensor_freqs_per_unit(t.n_max, t.zsplit != 0);
         CP_CUDA(launch_pair_tensor(t, p->n_sm, s));
     } else {
-        const int warps = pair_warps(p->max_n, a.unit_end - a.unit_begin, p->n_sm);
+        const int warps = pair_warps(p->pair_smem, p->max_n, a.unit_end - a.unit_begin, p->n_sm);
         CP_CUDA(launch_pair_direct(a, warps, p->pair_grid[warps == 4], p->pair_smem, s));
     }
     if (ev_idx) {
@@ -1005,7 +1005,7 @@ void plan_spec(cp_plan_t p, SpecPlan& sp, const float* st_per_curve, double poin
         }
     }
     if (!hi[1]) return;
-    if (pair_warps(p->max_n, (int64_t)(n_units * p->n_sm), p->n_sm) == 4) t_pair = std::min(t_pair, t_short);
+    if (pair_warps(p->pair_smem, p->max_n, (int64_t)(n_units * p->n_sm), p->n_sm) == 4) t_pair = std::min(t_pair, t_short);
     int64_t largest = 0;
     for (const Wave& w : p->waves)
         if (w.cls == 0) largest = std::max<int64_t>(largest, w.slot_end - w.slot_begin);
@@ -1274,12 +1274,6 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         const int tb = tune_bucket(tune, (int)n);
         p->fc[c] = fc_for((int)n, tb >= 0 ? tune.direct_fc[tb] : kFcMax);
     }
-    // the tables of short curves leave room for four blocks to an SM (pair_warps)
-    if (max_n <= kShortCurve)
-        for (int64_t c = 0; c < n_curves; c++) {
-            const int n = (int)(offsets[c + 1] - offsets[c]);
-            while (p->fc[c] > 2 && (n + kTile - 1) / kTile * kTile * p->fc[c] * 12 > kShortTable) p->fc[c] >>= 1;
-        }
     p->max_band_points = (max_n + 9) / 10;   // a band holds at most ceil(N/10) samples
     p->n_points = offsets[n_curves];
     p->max_n = max_n;
@@ -1300,6 +1294,14 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     p->device = opt.device;
     CP_CUDA(cudaSetDevice(p->device));
     CP_CUDA(cudaDeviceGetAttribute(&p->n_sm, cudaDevAttrMultiProcessorCount, p->device));
+    {
+        const int64_t points = p->bands ? p->n_trials : g.hierarchical == CP_SEARCH_COARSE_FINE ? p->kc : g.n_freq;
+        const int table = pair_table(max_n, (points + kFcMax - 1) / kFcMax * n_curves, p->n_sm);
+        for (int64_t c = 0; c < n_curves; c++) {
+            const int n = (int)(offsets[c + 1] - offsets[c]);
+            while (p->fc[c] > 2 && (n + kTile - 1) / kTile * kTile * p->fc[c] * 12 > table) p->fc[c] >>= 1;
+        }
+    }
     p->stream = (cudaStream_t)stream;
     CP_CUDA(cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking));
 

@@ -37,9 +37,20 @@ constexpr int kShortTable = 55296;     // their trig table: four blocks to an SM
 // 481 -> 390; at 420 only with 8 frequencies a unit, 1152 -> 1069; at 650 slower).  They need a unit
 // for every block: with fewer, a unit on 16 warps ends sooner (one curve of N = 330, 122 units: 86
 // against 108 us a call).
-inline int pair_warps(int max_n, int64_t units, int n_sm)
+inline int pair_warps(size_t table, int max_n, int64_t units, int n_sm)
 {
-    return max_n <= kShortCurve && units >= (int64_t)4 * n_sm ? 4 : 16;
+    return max_n <= kShortCurve && table <= (size_t)kShortTable && units >= (int64_t)4 * n_sm ? 4 : 16;
+}
+
+// Bytes of a unit's trig table at most, hence its frequencies, for a batch of `units` units of kFcMax
+// frequencies.  Short curves: the small table where it gives blocks of 4 warps their units, and where
+// there are so few units that halving them fills more of the chip (one curve of N = 420 at 900
+// frequencies: 120 -> 104 us); between the two, whole units on 16 warps (8 curves of N = 40 to 420 at
+// 900: 160 -> 144 us).
+inline int pair_table(int max_n, int64_t units, int n_sm)
+{
+    const bool between = units >= (int64_t)2 * n_sm && units < (int64_t)4 * n_sm;
+    return max_n <= kShortCurve && !between ? kShortTable : kTableBytes;
 }
 
 // Per-curve parameters, indexed by the caller's curve number.

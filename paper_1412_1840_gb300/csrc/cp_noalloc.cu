@@ -174,8 +174,10 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     int np2max = 32;
     while (np2max < max_n) np2max <<= 1;
     unit_full[0] = unit_coarse[0] = unit_fine[0] = wtile[0] = 0;
-    // a batch of short curves leaves room for blocks of 4 warps, as in a plan (cp_api.cu)
-    const int table = max_n <= kShortCurve ? kShortTable : kTableBytes;
+    int dev = 0, nsm = 1;
+    NA_CUDA(cudaGetDevice(&dev));
+    NA_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int table = pair_table(max_n, ((g.hierarchical ? kc : g.n_freq) + kFcMax - 1) / kFcMax * n_curves, nsm);
     auto fc_of = [table](int npad) {
         int fc = kFcMax;
         while (fc > 2 && npad * fc * 12 > table) fc >>= 1;
@@ -201,9 +203,6 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         cps[c].fc = fc_of(npad);
     }
 
-    int dev = 0, nsm = 1;
-    NA_CUDA(cudaGetDevice(&dev));
-    NA_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int ip_blocks = stats_blocks(n_curves, max_n, nsm);
     void* base = nullptr;
     cp_status st = scratch_base(dev, &base);
@@ -294,7 +293,7 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     NA_CUDA(launch_build_w(bw, s));
 
     auto pair = [&](const PairArgs& a) {
-        const int warps = pair_warps(max_n, a.unit_end - a.unit_begin, nsm);
+        const int warps = pair_warps(pair_smem, max_n, a.unit_end - a.unit_begin, nsm);
         int occ = 1;
         const cudaError_t e = pair_direct_occupancy(&occ, warps, pair_smem);
         return e ? e : launch_pair_direct(a, warps, nsm * (occ > 0 ? occ : 1), pair_smem, s);

@@ -160,8 +160,10 @@ def test_curves_outside_the_spectrums_range():
 @pytest.mark.parametrize("n", [40, 300, 448])
 def test_pair_sum_is_the_same_on_either_block_size(n):
     """Short curves run on blocks of 4 warps once every SM has four of its units
-    (below that: 16 warps): the sums' order, hence every bit, is the same."""
+    (below that: 16 warps, on whole or halved units): the sums' order, hence
+    every bit, is the same."""
     b = batch(1, n, n, 900.0)
-    few, many = 2000, 16 * 4 * 160          # fewer units than 4 per SM at 8 a unit; more at 16 a unit
-    rows = [run(b, synth.Grid(0.01, 1e-4, k), sigma_t=0.08)[0] for k in (few, many)]
-    np.testing.assert_array_equal(rows[0][0], rows[1][0, :few])
+    ks = (2000, 6400, 16 * 4 * 160)         # units of 16 frequencies: fewer than 2 per SM, than 4 per SM, more
+    rows = [run(b, synth.Grid(0.01, 1e-4, k), sigma_t=0.08)[0][0] for k in ks]
+    for k, row in zip(ks, rows):
+        np.testing.assert_array_equal(row, rows[-1][:k])
