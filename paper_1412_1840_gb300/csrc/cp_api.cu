@@ -1029,7 +1029,7 @@ void plan_spec(cp_plan_t p, SpecPlan& sp, const float* st_per_curve, double poin
         if (w.cls == 0) sp.chunks += (w.slot_end - w.slot_begin + sp.chunk - 1) / sp.chunk;
     // What the spectrum's launches add (measured at 1 to 114 short curves): a part once, a part for
     // every chunk, and the candidates' pair sums of the longest curve
-    t_spec += hier ? 50e-6 + 50e-6 * sp.chunks : 30e-6 + 30e-6 * sp.chunks;
+    t_spec += hier ? 45e-6 + 45e-6 * sp.chunks : 22e-6 + 28e-6 * sp.chunks;
     t_spec += 1e-6 * std::ceil(tiles_of(n_max) / 16.0);
     if (t_spec >= t_pair) return;
     sp.on = true;

@@ -160,7 +160,7 @@ __device__ __forceinline__ void set_ip(CurveParams* P, double s2)
 // integer products of the significands, the scalars are dealt to three warps, and
 // the pair sum of IP is FP32.  With few long curves the pair sum is left to k_ip
 // (a.ip_blocks blocks a curve).  With k_ip: 12 curves of up to 1,000 samples 70 ->
-// 28 us, three of up to 4,096 568 -> 93 us; a curve of 150 samples 18 -> 14 us.
+// 28 us, three of up to 4,096 568 -> 41 us (and 18 in k_ip); a curve of 150 samples 18 -> 14 us.
 template <int T>
 __global__ void __launch_bounds__(T) k_stats(const StatsArgs a)
 {
