@@ -18,7 +18,6 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
-#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -402,15 +401,15 @@ constexpr uint64_t kPoolKeep = 16u << 20;
 cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s)
 {
     static std::mutex mutex;
-    static std::map<int, cudaMemPool_t> pools;
+    static cudaMemPool_t pools[64];          // by device ordinal
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    if (dev >= 64) return cudaMallocAsync(p, bytes, s);
     cudaMemPool_t pool = nullptr;
     {
         std::lock_guard<std::mutex> lock(mutex);
-        auto it = pools.find(dev);
-        if (it == pools.end()) {
+        if (!pools[dev]) {
             cudaMemPoolProps props{};
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
@@ -424,9 +423,8 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s)
                 return e;
             }
             pools[dev] = pool;
-        } else {
-            pool = it->second;
         }
+        pool = pools[dev];
     }
     return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
