@@ -90,8 +90,18 @@ __global__ void __launch_bounds__(kCleanThreads) k_prep_stats(const double* time
     const float cutf = __double2float_ru(mean + 3.0 * sqrt(var));
 
     // weighted chi^2 sums (weights 1 / e^2) and unweighted moments of the kept samples, about the
-    // curve's first sample (so that single-pass sums lose nothing)
-    const double tref = times[off], xref = (double)mags[off];
+    // first kept sample: single-pass sums then lose nothing to a large common offset, and a dropped
+    // sample (not finite, or a sentinel value) has no part in them
+    int first = 0;
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        const uint32_t kept = __ballot_sync(0xffffffffu, i < n && errs[off + i] < cutf);
+        if (kept) {
+            first = i0 + __ffs(kept) - 1;
+            break;
+        }
+    }
+    const double tref = times[off + first], xref = (double)mags[off + first];
     int cnt = 0;
     double S = 0, St = 0, Sx = 0, Stt = 0, Stx = 0, ut = 0, ux = 0, utt = 0, utx = 0, uxx = 0;
     for (int i = lane; i < n; i += 32) {

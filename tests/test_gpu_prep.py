@@ -99,3 +99,38 @@ def test_two_level_search_finds_the_second_mode():
     with cp.Plan(td, w, ed, off, g, sigma_t=0.4) as p:
         f1 = p.best_period()["best_freq"][0]
     assert abs(f1 - 1 / P1) < 3e-4, (f1, 1 / P1)
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, 1e30, 1e9, 99.999])
+@pytest.mark.parametrize("lead", [1, 40])
+def test_dropped_first_samples_have_no_part_in_the_fit(value, lead):
+    """Curves whose first samples fail the error-bar cut and carry a value that
+    is not finite or a sentinel (magnitudes and, for the non-finite ones, times):
+    the fit of the kept samples is the oracle's.  Trends of both signs, noise,
+    and kept magnitudes that are all equal (no variance: r = 0)."""
+    rng = np.random.default_rng(54)
+    sizes = np.array([999, 900, 640, 700])
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    t = synth.seasonal_times(rng, sizes, 2500.0)
+    m = 17.0 + rng.normal(0, 0.05, t.shape[0])
+    e = rng.uniform(0.03, 0.08, t.shape[0])
+    for c, slope in enumerate([2e-3, -2e-3, 0.0, None]):
+        a, z = off[c], off[c + 1]
+        m[a:z] = 17.1 if slope is None else m[a:z] + slope * (t[a:z] - t[a])
+        m[a:a + lead] = value
+        if not np.isfinite(value):
+            t[a:a + lead] = value
+        e[a:a + lead] = 3.0
+    b = synth.Batch(t, m.astype(np.float32), e.astype(np.float32), off, np.zeros(4), np.zeros(4, bool),
+                    np.zeros(4, np.int8))
+    ot, ox, oe, oo, res = oracle.batch_preprocess(b)
+    assert [bool(r["detrended"]) for r in res] == [True, True, False, False] and res[3]["r"] == 0.0
+    assert all(oo[c + 1] - oo[c] == sizes[c] - lead for c in range(4))
+    d = cp.cp_preprocess(torch.from_numpy(b.times).cuda(), torch.from_numpy(b.mags).cuda(),
+                         torch.from_numpy(b.errs).cuda(), b.offsets)
+    np.testing.assert_array_equal(d["offsets_all"], oo)
+    np.testing.assert_array_equal(d["flags"], [3, 3, 1, 1])
+    for c, r in enumerate(res):
+        np.testing.assert_allclose(d["fit"][c], [r["a0"], r["a1"], r["r"]], rtol=1e-9, atol=1e-12)
+    np.testing.assert_array_equal(d["times"].cpu().numpy(), ot)
+    np.testing.assert_allclose(d["mags"].cpu().numpy(), ox, rtol=0, atol=4e-6 * max(1.0, np.abs(ox).max()))
