@@ -134,7 +134,6 @@ struct cp_plan_s {
     int spec_fc_min = kFcMax;
     int spec_seg_max = 0;
     size_t spec_budget = 0;            // workspace of the pair spectrum at most
-    bool keep_w = true;                // some pass of the direct-form curves reads W tiles
     bool spec() const { return sfull.on || ssearch.on; }
     SpecCurve* d_sc = nullptr;
     float* d_scoef = nullptr;
@@ -386,24 +385,28 @@ int tune_bucket(const cp_tuning& t, int n)
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Failure-injection hook for tests: with CP_FAIL_ALLOC=k in the environment,
-// the k-th allocation (device or pinned host, counted from 1) of one cp_plan
-// call reports cudaErrorMemoryAllocation without allocating.  The plan must
-// then return CP_ENOMEM and release everything it allocated before.
+// Failure-injection hook for tests: with CP_FAIL_ALLOC=1 in the environment
+// cp_plan's allocations of the device block report cudaErrorMemoryAllocation
+// without allocating, with 2 that of the pinned host block.  The plan must then
+// return CP_ENOMEM and release everything it allocated before.  With
+// CP_FAIL_ALLOC_ABOVE_KB=n device blocks of more than n KB fail (a plan whose
+// pair spectrum does not fit evaluates by the pair sum).
 struct AllocHook {
-    int target = 0, count = 0;
+    int target = 0;
+    size_t limit = ~(size_t)0;
     AllocHook()
     {
         if (const char* env = std::getenv("CP_FAIL_ALLOC")) target = std::atoi(env);
+        if (const char* env = std::getenv("CP_FAIL_ALLOC_ABOVE_KB")) limit = (size_t)std::atoll(env) << 10;
     }
-    cudaError_t device(void** p, size_t bytes)
+    cudaError_t device(void** p, size_t bytes) const
     {
-        if (++count == target) return cudaErrorMemoryAllocation;
+        if (target == 1 || bytes > limit) return cudaErrorMemoryAllocation;
         return cudaMalloc(p, bytes);
     }
-    cudaError_t pinned(void** p, size_t bytes)
+    cudaError_t pinned(void** p, size_t bytes) const
     {
-        if (++count == target) return cudaErrorMemoryAllocation;
+        if (target == 2) return cudaErrorMemoryAllocation;
         return cudaMallocHost(p, bytes);
     }
 };
@@ -1429,80 +1432,95 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
     p->spec_seg_max = spec_seg_max(p->max_n);
     p->spec_budget = std::min<size_t>(kSpecWorkspace, free_b / 8);
     plan_spectra(p, opt.sigma_t_per_curve);
-    const bool spec = p->spec();
-    // magnitude-kernel tiles of the direct-form curves: only for passes that go through the pair sum
-    p->keep_w = !p->sfull.on || (g.hierarchical != CP_SEARCH_FULL && !p->ssearch.on);
-    if (!p->keep_w) max_tiles32 = 0;
-    const int spec_chunks = std::max(p->sfull.chunks, p->ssearch.chunks);
-    auto largest = [&](auto per) { return std::max(p->sfull.on ? per(p->sfull) : 0, p->ssearch.on ? per(p->ssearch) : 0); };
-    const size_t sx_bytes = largest([](const SpecPlan& q) { return ((size_t)q.chunk << q.max_logq) * sizeof(float2); });
-    const size_t sp_bytes = largest([](const SpecPlan& q) { return (size_t)q.chunk * q.p_ld * sizeof(float); });
-    const size_t svblk_bytes = largest([](const SpecPlan& q) {
-        return (size_t)q.chunk * ((q.points + kSpecBlock - 1) / kSpecBlock) * sizeof(unsigned int);
-    });
-    const size_t srow_bytes = largest([](const SpecPlan& q) { return (size_t)q.chunk * q.row * sizeof(float); });
-
-    // device allocation (one block)
-    const int64_t np = p->n_points, nc = n_curves;
-    const int nq = kQueuesPerWave * (int)p->waves.size() + (spec ? 2 * spec_chunks + (int)p->waves.size() : 0);
-    p->ip_blocks = stats_blocks(nc, max_n, p->n_sm);
-    p->n_u64 = 1 + nc + nq + nc;      // status, keys, work counters, two 32-bit counts per curve
     struct Part { void** dst; size_t bytes; };
+    const int64_t np = p->n_points, nc = n_curves;
     const bool hier = g.hierarchical == CP_SEARCH_COARSE_FINE;
     const bool bnd = p->bands;
-    std::vector<Part> parts = {
-        {(void**)&p->d_times, p->host_inputs ? np * sizeof(double) : 0},
-        {(void**)&p->d_mags, p->host_inputs ? np * sizeof(float) : 0},
-        {(void**)&p->d_errs, p->host_inputs ? np * sizeof(float) : 0},
-        {(void**)&p->d_cp, nc * sizeof(CurveParams)},
-        {(void**)&p->d_yp, np * sizeof(float)},
-        {(void**)&p->d_ph_base, np * sizeof(uint64_t)},
-        {(void**)&p->d_ph_full, np * sizeof(uint64_t)},
-        {(void**)&p->d_ph_coarse, hier ? np * sizeof(uint64_t) : 0},
-        {(void**)&p->d_ph_fine, hier ? np * sizeof(uint64_t) : 0},
-        {(void**)&p->d_parts, (size_t)2 * nc * std::max(p->ip_blocks, 1) * sizeof(double)},
-        {(void**)&p->d_stpc, opt.sigma_t_mode == CP_SIGMA_T_PER_CURVE ? nc * sizeof(float) : 0},
-        {(void**)&p->d_order, nc * sizeof(int32_t)},
-        {(void**)&p->d_unit_full, (nc + 1) * sizeof(int64_t)},
-        {(void**)&p->d_unit_coarse, (nc + 1) * sizeof(int64_t)},
-        {(void**)&p->d_unit_fine, (nc + 1) * sizeof(int64_t)},
-        {(void**)&p->d_wtile, (nc + 1) * sizeof(int64_t)},
-        {(void**)&p->d_unit_list, bnd ? (nc + 1) * sizeof(int64_t) : 0},
-        {(void**)&p->d_band_of, bnd ? (size_t)np : 0},
-        {(void**)&p->d_kept, bnd ? (size_t)nc * g.n_bands * sizeof(int32_t) : 0},
-        {(void**)&p->d_trials, bnd ? (size_t)nc * p->n_trials * sizeof(int32_t) : 0},
-        {(void**)&p->d_wcand, bnd ? (size_t)nc * 2 * p->n_trials * sizeof(unsigned long long) : 0},
-        {(void**)&p->d_trial_stat, bnd ? (size_t)nc * p->n_trials * sizeof(float) : 0},
-        {(void**)&p->d_excl_f, p->excl_f.size() * sizeof(double)},
-        {(void**)&p->d_excl_full, p->excl_full.size() * sizeof(int32_t)},
-        {(void**)&p->d_excl_coarse, p->excl_coarse.size() * sizeof(int32_t)},
-        {(void**)&p->d_W, (size_t)max_tiles32 * tile32_bytes},
-        {(void**)&p->d_W16, (size_t)max_tiles16 * tile16_bytes},
-        {(void**)&p->d_coef, p->tensor ? (size_t)nc * kCoefStride * sizeof(float) : 0},
-        {(void**)&p->d_wrho, p->tensor ? np * sizeof(float) : 0},
-        {(void**)&p->d_sc, spec ? (size_t)nc * sizeof(SpecCurve) : 0},
-        {(void**)&p->d_scoef, spec ? (size_t)nc * kSpecMaxHarm * sizeof(float) : 0},
-        {(void**)&p->d_sxs, spec ? np * sizeof(uint64_t) : 0},
-        {(void**)&p->d_sys, spec ? np * sizeof(float) : 0},
-        {(void**)&p->d_sx, sx_bytes},
-        {(void**)&p->d_sP, sp_bytes},
-        {(void**)&p->d_srow, srow_bytes},
-        {(void**)&p->d_spart, spec ? (size_t)spec_chunk_max(p) * confirm_bytes(p->max_n) + confirm_extra_bytes() : 0},
-        {(void**)&p->d_tw, spec ? (size_t)kSpecTwiddles * sizeof(float2) : 0},
-        {(void**)&p->d_svblk, svblk_bytes},
-        {(void**)&p->d_svmax, spec ? (size_t)nc * sizeof(unsigned int) : 0},
-        {(void**)&p->d_scand, spec ? (size_t)nc * kSpecCand * sizeof(int32_t) : 0},
-        {(void**)&p->d_sfb, spec ? 2 * (size_t)nc * sizeof(int32_t) : 0},
-        {(void**)&p->d_coarse, hier ? (size_t)nc * p->kc * sizeof(float) : 0},
-        {(void**)&p->d_peaks, hier ? (size_t)nc * g.top_k * sizeof(int32_t) : 0},
-        {(void**)&p->d_npeaks, hier ? nc * sizeof(int32_t) : 0},
-        {(void**)&p->d_u64, (size_t)p->n_u64 * sizeof(unsigned long long)},
-        {(void**)&p->d_res, results_bytes(nc)},
-    };
+    p->ip_blocks = stats_blocks(nc, max_n, p->n_sm);
+
+    // device allocation (one block)
+    std::vector<Part> parts;
     size_t total = 0;
-    for (auto& q : parts) total = align_up(total, 256) + q.bytes;
-    AllocHook alloc;
-    CP_CUDA(alloc.device(&p->dblock, std::max<size_t>(total, 256)));
+    auto lay_out = [&] {
+        const bool spec = p->spec();
+        // magnitude-kernel tiles of the direct-form curves: only for passes that go through the pair sum
+        const bool keep_w = !p->sfull.on || (g.hierarchical != CP_SEARCH_FULL && !p->ssearch.on);
+        const int spec_chunks = std::max(p->sfull.chunks, p->ssearch.chunks);
+        auto largest = [&](auto per) { return std::max(p->sfull.on ? per(p->sfull) : 0, p->ssearch.on ? per(p->ssearch) : 0); };
+        const size_t sx_bytes = largest([](const SpecPlan& q) { return ((size_t)q.chunk << q.max_logq) * sizeof(float2); });
+        const size_t sp_bytes = largest([](const SpecPlan& q) { return (size_t)q.chunk * q.p_ld * sizeof(float); });
+        const size_t svblk_bytes = largest([](const SpecPlan& q) {
+            return (size_t)q.chunk * ((q.points + kSpecBlock - 1) / kSpecBlock) * sizeof(unsigned int);
+        });
+        const size_t srow_bytes = largest([](const SpecPlan& q) { return (size_t)q.chunk * q.row * sizeof(float); });
+        const int nq = kQueuesPerWave * (int)p->waves.size() + (spec ? 2 * spec_chunks + (int)p->waves.size() : 0);
+        p->n_u64 = 1 + nc + nq + nc;      // status, keys, work counters, two 32-bit counts per curve
+        parts = {
+            {(void**)&p->d_times, p->host_inputs ? np * sizeof(double) : 0},
+            {(void**)&p->d_mags, p->host_inputs ? np * sizeof(float) : 0},
+            {(void**)&p->d_errs, p->host_inputs ? np * sizeof(float) : 0},
+            {(void**)&p->d_cp, nc * sizeof(CurveParams)},
+            {(void**)&p->d_yp, np * sizeof(float)},
+            {(void**)&p->d_ph_base, np * sizeof(uint64_t)},
+            {(void**)&p->d_ph_full, np * sizeof(uint64_t)},
+            {(void**)&p->d_ph_coarse, hier ? np * sizeof(uint64_t) : 0},
+            {(void**)&p->d_ph_fine, hier ? np * sizeof(uint64_t) : 0},
+            {(void**)&p->d_parts, (size_t)2 * nc * std::max(p->ip_blocks, 1) * sizeof(double)},
+            {(void**)&p->d_stpc, opt.sigma_t_mode == CP_SIGMA_T_PER_CURVE ? nc * sizeof(float) : 0},
+            {(void**)&p->d_order, nc * sizeof(int32_t)},
+            {(void**)&p->d_unit_full, (nc + 1) * sizeof(int64_t)},
+            {(void**)&p->d_unit_coarse, (nc + 1) * sizeof(int64_t)},
+            {(void**)&p->d_unit_fine, (nc + 1) * sizeof(int64_t)},
+            {(void**)&p->d_wtile, (nc + 1) * sizeof(int64_t)},
+            {(void**)&p->d_unit_list, bnd ? (nc + 1) * sizeof(int64_t) : 0},
+            {(void**)&p->d_band_of, bnd ? (size_t)np : 0},
+            {(void**)&p->d_kept, bnd ? (size_t)nc * g.n_bands * sizeof(int32_t) : 0},
+            {(void**)&p->d_trials, bnd ? (size_t)nc * p->n_trials * sizeof(int32_t) : 0},
+            {(void**)&p->d_wcand, bnd ? (size_t)nc * 2 * p->n_trials * sizeof(unsigned long long) : 0},
+            {(void**)&p->d_trial_stat, bnd ? (size_t)nc * p->n_trials * sizeof(float) : 0},
+            {(void**)&p->d_excl_f, p->excl_f.size() * sizeof(double)},
+            {(void**)&p->d_excl_full, p->excl_full.size() * sizeof(int32_t)},
+            {(void**)&p->d_excl_coarse, p->excl_coarse.size() * sizeof(int32_t)},
+            {(void**)&p->d_W, keep_w ? (size_t)max_tiles32 * tile32_bytes : 0},
+            {(void**)&p->d_W16, (size_t)max_tiles16 * tile16_bytes},
+            {(void**)&p->d_coef, p->tensor ? (size_t)nc * kCoefStride * sizeof(float) : 0},
+            {(void**)&p->d_wrho, p->tensor ? np * sizeof(float) : 0},
+            {(void**)&p->d_sc, spec ? (size_t)nc * sizeof(SpecCurve) : 0},
+            {(void**)&p->d_scoef, spec ? (size_t)nc * kSpecMaxHarm * sizeof(float) : 0},
+            {(void**)&p->d_sxs, spec ? np * sizeof(uint64_t) : 0},
+            {(void**)&p->d_sys, spec ? np * sizeof(float) : 0},
+            {(void**)&p->d_sx, sx_bytes},
+            {(void**)&p->d_sP, sp_bytes},
+            {(void**)&p->d_srow, srow_bytes},
+            {(void**)&p->d_spart, spec ? (size_t)spec_chunk_max(p) * confirm_bytes(p->max_n) + confirm_extra_bytes() : 0},
+            {(void**)&p->d_tw, spec ? (size_t)kSpecTwiddles * sizeof(float2) : 0},
+            {(void**)&p->d_svblk, svblk_bytes},
+            {(void**)&p->d_svmax, spec ? (size_t)nc * sizeof(unsigned int) : 0},
+            {(void**)&p->d_scand, spec ? (size_t)nc * kSpecCand * sizeof(int32_t) : 0},
+            {(void**)&p->d_sfb, spec ? 2 * (size_t)nc * sizeof(int32_t) : 0},
+            {(void**)&p->d_coarse, hier ? (size_t)nc * p->kc * sizeof(float) : 0},
+            {(void**)&p->d_peaks, hier ? (size_t)nc * g.top_k * sizeof(int32_t) : 0},
+            {(void**)&p->d_npeaks, hier ? nc * sizeof(int32_t) : 0},
+            {(void**)&p->d_u64, (size_t)p->n_u64 * sizeof(unsigned long long)},
+            {(void**)&p->d_res, results_bytes(nc)},
+        };
+        total = 0;
+        for (auto& q : parts) total = align_up(total, 256) + q.bytes;
+    };
+    const AllocHook alloc;
+    auto device_block = [&] {
+        lay_out();
+        cudaError_t r = alloc.device(&p->dblock, std::max<size_t>(total, 256));
+        if (r == cudaErrorMemoryAllocation && p->spec()) {      // no room for the pair spectrum: the pair sum
+            cudaGetLastError();
+            p->sfull = p->ssearch = SpecPlan();
+            lay_out();
+            r = alloc.device(&p->dblock, std::max<size_t>(total, 256));
+        }
+        return r;
+    };
+    CP_CUDA(device_block());
+    const bool spec = p->spec();
     {
         size_t o = 0;
         for (auto& q : parts) {
