@@ -692,6 +692,7 @@ SpecArgs spec_args(cp_plan_t p, const SpecPlan& sp, const PairArgs& base)
     a.P = p->d_sP;
     a.p_ld = sp.p_ld;
     a.vmax = p->d_svmax;
+    a.vtop = p->d_svmax + p->n_curves;
     a.vblk = p->d_svblk;
     a.vb_ld = (sp.points + kSpecBlock - 1) / kSpecBlock;
     a.cand = p->d_scand;
@@ -1495,7 +1496,7 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
             {(void**)&p->d_spart, spec ? (size_t)spec_chunk_max(p) * confirm_bytes(p->max_n) + confirm_extra_bytes() : 0},
             {(void**)&p->d_tw, spec ? (size_t)kSpecTwiddles * sizeof(float2) : 0},
             {(void**)&p->d_svblk, svblk_bytes},
-            {(void**)&p->d_svmax, spec ? (size_t)nc * sizeof(unsigned int) : 0},
+            {(void**)&p->d_svmax, spec ? 2 * (size_t)nc * sizeof(unsigned int) : 0},
             {(void**)&p->d_scand, spec ? (size_t)nc * kSpecCand * sizeof(int32_t) : 0},
             {(void**)&p->d_sfb, spec ? 2 * (size_t)nc * sizeof(int32_t) : 0},
             {(void**)&p->d_coarse, hier ? (size_t)nc * p->kc * sizeof(float) : 0},

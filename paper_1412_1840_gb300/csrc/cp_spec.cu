@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(kSpecPrepThreads) k_spec_prep(const SpecArgs a
         a.sc[c] = S;
         s_cpd = S.cells_per_day * 4294967296.0;
         a.vmax[c] = 0u;
+        a.vtop[c] = 0u;
     }
     __syncthreads();
     const double cpd = s_cpd;
@@ -323,6 +324,32 @@ __device__ __forceinline__ int item_curve(const int* pre, int nc, int item)
         if (pre[m] <= item) lo = m; else hi = m - 1;
     }
     return lo;
+}
+
+// A block's largest admissible value and largest magnitude: into the curve's maxima, the first
+// also into the block's.  All threads call it.
+template <int WARPS>
+__device__ __forceinline__ void block_maxima(const SpecArgs& a, int c, int64_t blk, unsigned int key, unsigned int top,
+                                             unsigned int (&s_key)[WARPS], unsigned int (&s_top)[WARPS])
+{
+    key = __reduce_max_sync(0xffffffffu, key);
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) {
+        s_key[threadIdx.x >> 5] = key;
+        s_top[threadIdx.x >> 5] = top;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < WARPS; w++) {
+            key = max(key, s_key[w]);
+            top = max(top, s_top[w]);
+        }
+        if (key) atomicMax(a.vmax + c, key);
+        if (top) atomicMax(a.vtop + c, top);
+        a.vblk[blk] = key;
+    }
+    __syncthreads();
 }
 
 // INTERP: the weights are divided by the interpolation window's transform at the
@@ -905,8 +932,8 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_sum(const SpecArgs a)
 {
     __shared__ int s_pre[kSpecMaxChunk + 1];
     __shared__ float s_a[kSpecMaxHarm];
-    __shared__ unsigned int s_key[kSumThreads / 32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ unsigned int s_key[kSumThreads / 32], s_top[kSumThreads / 32];
+    const int tid = threadIdx.x;
     const int nc = a.slot_end - a.slot_begin;
     const int blocks = (int)((a.n_freq + kSumThreads * kSumPer - 1) / (kSumThreads * kSumPer));
     item_prefix(s_pre, nc, [&](int i) { return a.sc[a.order[a.slot_begin + i]].nh ? blocks : 0; });
@@ -938,7 +965,7 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_sum(const SpecArgs a)
                 s[q] = fmaf(an, Ps[at[q]], s[q]);
             }
         }
-        unsigned int key = 0u;
+        unsigned int key = 0u, top = 0u;
         float* row = a.rows + (a.rows_by_curve ? (int64_t)c : (int64_t)ci) * a.row_ld;
 #pragma unroll
         for (int q = 0; q < kSumPer; q++) {
@@ -946,20 +973,11 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_sum(const SpecArgs a)
             if (k < a.n_freq) {
                 const float v = fmaf(2.0f, s[q], P.diag * S.one_minus_a0) * P.norm;
                 row[k] = v;
+                top = max(top, __float_as_uint(fabsf(v)));
                 if (!excluded_k(a.ex.full_k, a.ex.n, k)) key = max(key, orderable(v));
             }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
-        if (lane == 0) s_key[warp] = key;
-        __syncthreads();
-        if (tid == 0) {
-#pragma unroll
-            for (int w = 1; w < kSumThreads / 32; w++) key = max(key, s_key[w]);
-            if (key) atomicMax(a.vmax + c, key);
-            a.vblk[(int64_t)ci * a.vb_ld + (item - s_pre[ci])] = key;
-        }
-        __syncthreads();
+        block_maxima(a, c, (int64_t)ci * a.vb_ld + (item - s_pre[ci]), key, top, s_key, s_top);
     }
 }
 
@@ -980,8 +998,8 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
 {
     __shared__ int s_pre[kSpecMaxChunk + 1];
     __shared__ float s_a[kSpecMaxHarm];
-    __shared__ unsigned int s_key[kSumThreads / 32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ unsigned int s_key[kSumThreads / 32], s_top[kSumThreads / 32];
+    const int tid = threadIdx.x;
     const int nc = a.slot_end - a.slot_begin;
     item_prefix(s_pre, nc, [&](int i) {
         const int c = a.order[a.slot_begin + i];
@@ -998,7 +1016,7 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
         // four threads a frequency, each every fourth harmonic (one thread's chain of up to 64
         // dependent fetches took 55 us a launch, however few the frequencies)
         const int q = (item - s_pre[ci]) * kInterpBlock + (tid >> 2), part = tid & 3;
-        unsigned int key = 0u;
+        unsigned int key = 0u, top = 0u;
         const bool in = q < spec_count(a, c);
         bool ok = in, live = in;                  // admissible as the best; evaluated at all
         double f = 0.0;
@@ -1038,32 +1056,24 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
         s += __shfl_xor_sync(0xffffffffu, s, 2);
         if (in && part == 0) {
             float v = live ? fmaf(2.0f, s, P.diag * S.one_minus_a0) * P.norm : 0.f;
+            top = __float_as_uint(fabsf(v));
             if (a.stage == kSpecFine && !ok) v = -INFINITY;
             if (a.stage == kSpecList && !live) v = __int_as_float(0x7fc00000);
             a.rows[(a.rows_by_curve ? (int64_t)c : (int64_t)ci) * a.row_ld + q] = v;
             if (ok) key = orderable(v);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
-        if (lane == 0) s_key[warp] = key;
-        __syncthreads();
-        if (tid == 0) {
-#pragma unroll
-            for (int w = 1; w < kSumThreads / 32; w++) key = max(key, s_key[w]);
-            if (key) atomicMax(a.vmax + c, key);
-            a.vblk[(int64_t)ci * a.vb_ld + (item - s_pre[ci])] = key;
-        }
-        __syncthreads();
+        block_maxima(a, c, (int64_t)ci * a.vb_ld + (item - s_pre[ci]), key, top, s_key, s_top);
     }
 }
 
 // Margin below which two values of a curve are not told apart by the spectrum:
-// 1e-5 of the largest value plus 1e-6 of the scale of a noise curve, several
+// 1e-5 of the largest magnitude in the row, admissible or not (an excluded peak
+// carries its error to the values beside it), plus 1e-6 of the scale of a noise curve, several
 // times the error of the pair sum and of the spectrum together (both below 2e-6
 // of the peak).
-__device__ __forceinline__ float spec_margin(float vmax, const CurveParams& P)
+__device__ __forceinline__ float spec_margin(float vtop, const CurveParams& P)
 {
-    return 1e-5f * fabsf(vmax) + 1e-6f * P.norm * (float)P.n;
+    return 1e-5f * vtop + 1e-6f * P.norm * (float)P.n;
 }
 
 // ===========================================================================
@@ -1105,8 +1115,7 @@ __global__ void __launch_bounds__(kSelThreads) k_spec_select(const SpecArgs a)
     if (tid == 0) s_hot = 0;
     __syncthreads();
     if (spec && top) {
-        const float v0 = from_orderable(top);
-        const float thr = v0 - spec_margin(v0, P);
+        const float thr = from_orderable(top) - spec_margin(__uint_as_float(a.vtop[c]), P);
         const unsigned int othr = orderable(thr);
         const float* row = a.rows + (a.rows_by_curve ? (int64_t)c : (int64_t)ci) * a.row_ld;
         const int count = spec_count(a, c), per = a.interp ? kInterpBlock : kSumThreads * kSumPer;

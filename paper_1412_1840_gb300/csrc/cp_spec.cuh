@@ -77,6 +77,7 @@ struct SpecArgs {
     int64_t row_ld;
     int rows_by_curve;
     unsigned int* vmax;           // [n_curves] largest admissible value (orderable bits)
+    unsigned int* vtop;           // [n_curves] largest magnitude of any value, excluded ones too (float bits)
     unsigned int* vblk;           // the same per block of a launch's values, vb_ld per curve of the chunk
     int64_t vb_ld;
     int32_t* cand;                // [n_curves * kSpecCand] candidate entries, -1 after the last
