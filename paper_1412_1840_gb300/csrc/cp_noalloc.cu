@@ -235,23 +235,24 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     if (cv.used > kScratchBytes)
         return nfail(CP_EUNSUPPORTED, "cp_best_period_noalloc: batch needs more than CP_NOALLOC_SCRATCH_BYTES");
 
+    // The copy's source and the status word below stand before the guard: they outlive every
+    // synchronisation of the stream, the guard's on an error among them.
+    char h_table[kMaxCurves * (sizeof(CurveParams) + 4 * sizeof(int64_t) + sizeof(int32_t)) + 4 * sizeof(int64_t)];
+    unsigned long long status = 0;
+    char* at = h_table;
+    auto put = [&at](const void* src, size_t bytes) {
+        std::memcpy(at, src, bytes);
+        at += bytes;
+    };
+    put(cps, nc * sizeof(CurveParams));
+    put(unit_full, (nc + 1) * sizeof(int64_t));
+    put(unit_coarse, (nc + 1) * sizeof(int64_t));
+    put(unit_fine, (nc + 1) * sizeof(int64_t));
+    put(wtile, (nc + 1) * sizeof(int64_t));
+    put(order, nc * sizeof(int32_t));
     cudaStream_t s = (cudaStream_t)cuda_stream;
     SyncOnError guard{s, true};
-    {
-        char table[kMaxCurves * (sizeof(CurveParams) + 4 * sizeof(int64_t) + sizeof(int32_t)) + 4 * sizeof(int64_t)];
-        char* at = table;
-        auto put = [&at](const void* src, size_t bytes) {
-            std::memcpy(at, src, bytes);
-            at += bytes;
-        };
-        put(cps, nc * sizeof(CurveParams));
-        put(unit_full, (nc + 1) * sizeof(int64_t));
-        put(unit_coarse, (nc + 1) * sizeof(int64_t));
-        put(unit_fine, (nc + 1) * sizeof(int64_t));
-        put(wtile, (nc + 1) * sizeof(int64_t));
-        put(order, nc * sizeof(int32_t));
-        NA_CUDA(cudaMemcpyAsync(d_table, table, table_bytes, cudaMemcpyHostToDevice, s));
-    }
+    NA_CUDA(cudaMemcpyAsync(d_table, h_table, table_bytes, cudaMemcpyHostToDevice, s));
     NA_CUDA(launch_zero_u64(d_u64, n_u64, s));   // status, best keys and work counters start at zero
 
     StatsArgs sa{};
@@ -375,7 +376,6 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     fa.best_stat = best_stat;
     fa.is_periodic = is_periodic;
     NA_CUDA(launch_finalize(fa, s));
-    unsigned long long status = 0;
     NA_CUDA(cudaMemcpyAsync(&status, d_u64, sizeof(status), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));
     guard.armed = false;
