@@ -203,7 +203,7 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         cps[c].fc = fc_of(npad);
     }
 
-    const int ip_blocks = stats_blocks(n_curves, max_n, nsm);
+    int ip_blocks = stats_blocks(n_curves, max_n, nsm);
     void* base = nullptr;
     cp_status st = scratch_base(dev, &base);
     if (st != CP_OK) return st;
@@ -229,9 +229,23 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     float* d_coarse = g.hierarchical ? cv.take<float>((size_t)nc * kc) : nullptr;
     int32_t* d_peaks = g.hierarchical ? cv.take<int32_t>((size_t)nc * g.top_k) : nullptr;
     int32_t* d_npeaks = g.hierarchical ? cv.take<int32_t>(nc) : nullptr;
-    const int64_t n_u64 = 1 + nc + 3 + nc;
-    unsigned long long* d_u64 = cv.take<unsigned long long>(n_u64);
-    double* d_parts = cv.take<double>((size_t)nc * (ip_blocks > 0 ? ip_blocks : 1));
+    // counters, then what spreads IP over several blocks; a batch that leaves no room for the latter
+    // does without (k_stats sums IP itself)
+    const size_t before = cv.used;
+    int64_t n_u64 = 0;
+    unsigned long long* d_u64 = nullptr;
+    double* d_parts = nullptr;
+    auto take_counters = [&] {
+        cv.used = before;
+        n_u64 = 1 + nc + 3 + (ip_blocks > 0 ? nc : 0);
+        d_u64 = cv.take<unsigned long long>(n_u64);
+        if (ip_blocks > 0) d_parts = cv.take<double>((size_t)nc * ip_blocks);
+    };
+    take_counters();
+    if (cv.used > kScratchBytes && ip_blocks > 0) {
+        ip_blocks = 0;
+        take_counters();
+    }
     if (cv.used > kScratchBytes)
         return nfail(CP_EUNSUPPORTED, "cp_best_period_noalloc: batch needs more than CP_NOALLOC_SCRATCH_BYTES");
 

@@ -150,3 +150,25 @@ def test_noalloc_rejects_bad_arguments_before_the_gpu():
     st = L.cp_best_period_noalloc(t.data_ptr(), m.data_ptr(), e.data_ptr(), off.ctypes.data, b.n_curves,
                                   ctypes.byref(inf), ctypes.c_float(0.3), None, None, None, None, None)
     assert st == cp.CP_EINVAL
+
+
+def test_noalloc_batch_that_fills_the_scratch_array():
+    """Eight curves of 1,000 samples whose coarse grid fills the scratch array up
+    to the last 256 bytes of its plainest layout: one 256-byte aligned array each
+    for the parameters (80 bytes a curve), order, four tables, magnitudes, phases,
+    tiles, coarse values, peaks, counters and results."""
+    up = lambda x: (x + 255) // 256 * 256
+    nc, n = 8, 1000
+    tiles = nc * 32 * 33 // 2 * 4096
+    fixed = (up(80 * nc) + up(4 * nc * n) + 4 * up(8 * nc * n) + up(4 * nc) + 4 * up(8 * (nc + 1)) + tiles + 2 * up(4 * nc) +
+             up(8 * (4 + nc)) + 2 * up(8 * nc) + 2 * up(4 * nc) + up(nc))
+    kc = ((64 << 20) - fixed) // 256 * 256 // (4 * nc)
+    b = synth.ragged_batch(nc, seed=49, n_lo=n, n_hi=n)
+    g = synth.Grid(0.0, 2.0 ** -20, kc, hierarchical=True, coarse_df=2.0 ** -20, top_k=1, fine_df=2.0 ** -22,
+                   fine_halfwidth=2.0 ** -20)
+    same(via_noalloc(b, g, 0.45), via_plan(b, g, 0.45))
+    more = synth.Grid(0.0, 2.0 ** -20, kc + 200, hierarchical=True, coarse_df=2.0 ** -20, top_k=1, fine_df=2.0 ** -22,
+                      fine_halfwidth=2.0 ** -20)
+    with pytest.raises(cp.CpError) as e:
+        via_noalloc(b, more, 0.45)
+    assert e.value.status == cp.CP_EUNSUPPORTED
