@@ -11,6 +11,7 @@
 // until the process exits.  No cudaMalloc, cudaFree or allocating library
 // routine is called on this path.
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <mutex>
 
@@ -229,6 +230,12 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     float* d_coarse = g.hierarchical ? cv.take<float>((size_t)nc * kc) : nullptr;
     int32_t* d_peaks = g.hierarchical ? cv.take<int32_t>((size_t)nc * g.top_k) : nullptr;
     int32_t* d_npeaks = g.hierarchical ? cv.take<int32_t>(nc) : nullptr;
+    // results go straight to the caller's arrays, by way of the scratch array where one is off its
+    // type's alignment
+    auto aligned = [](const void* p, size_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; };
+    int64_t* d_idx = aligned(best_idx, sizeof(int64_t)) ? best_idx : cv.take<int64_t>(nc);
+    double* d_freq = aligned(best_freq, sizeof(double)) ? best_freq : cv.take<double>(nc);
+    float* d_stat = aligned(best_stat, sizeof(float)) ? best_stat : cv.take<float>(nc);
     // counters, then what spreads IP over several blocks; a batch that leaves no room for the latter
     // does without (k_stats sums IP itself)
     const size_t before = cv.used;
@@ -385,11 +392,14 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     fa.df = g.df;
     fa.coarse_df = g.coarse_df;
     fa.fine_df = g.fine_df;
-    fa.best_idx = best_idx;          // straight to the caller's arrays (null: not wanted)
-    fa.best_freq = best_freq;
-    fa.best_stat = best_stat;
+    fa.best_idx = d_idx;             // null: not wanted
+    fa.best_freq = d_freq;
+    fa.best_stat = d_stat;
     fa.is_periodic = is_periodic;
     NA_CUDA(launch_finalize(fa, s));
+    if (d_idx != best_idx) NA_CUDA(cudaMemcpyAsync(best_idx, d_idx, nc * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+    if (d_freq != best_freq) NA_CUDA(cudaMemcpyAsync(best_freq, d_freq, nc * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    if (d_stat != best_stat) NA_CUDA(cudaMemcpyAsync(best_stat, d_stat, nc * sizeof(float), cudaMemcpyDeviceToDevice, s));
     NA_CUDA(cudaMemcpyAsync(&status, d_u64, sizeof(status), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));
     guard.armed = false;

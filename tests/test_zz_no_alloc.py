@@ -172,3 +172,29 @@ def test_noalloc_batch_that_fills_the_scratch_array():
     with pytest.raises(cp.CpError) as e:
         via_noalloc(b, more, 0.45)
     assert e.value.status == cp.CP_EUNSUPPORTED
+
+
+def test_noalloc_results_at_any_address():
+    """Result arrays that are off their type's alignment (the header asks for
+    device memory, not for aligned addresses) are written all the same."""
+    import ctypes
+    b = synth.ragged_batch(9, seed=50, n_lo=60, n_hi=300)
+    g = synth.Grid(0.01, 1e-3, 500)
+    want = via_noalloc(b, g, 0.3)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    t, m, e = dev(b.times), dev(b.mags), dev(b.errs)
+    off = np.ascontiguousarray(b.offsets, np.int64)
+    grid = cp.grid_from(g)
+    n = b.n_curves
+    for shift in (1, 2, 4):
+        raw = torch.zeros(1024, dtype=torch.uint8, device="cuda")
+        at = [256 * k + shift for k in range(4)]
+        torch.cuda.synchronize()
+        st = cp.lib().cp_best_period_noalloc(t.data_ptr(), m.data_ptr(), e.data_ptr(), off.ctypes.data, n,
+                                             ctypes.byref(grid), ctypes.c_float(0.3), None,
+                                             *(raw.data_ptr() + a for a in at))
+        assert st == cp.CP_OK
+        h = raw.cpu().numpy()
+        got = [h[a:a + n * np.dtype(d).itemsize].copy().view(d) for a, d in zip(at, ("i8", "f8", "f4", "u1"))]
+        for x, key in zip(got, ("best_idx", "best_freq", "best_stat", "is_periodic")):
+            np.testing.assert_array_equal(x.astype(want[key].dtype), want[key], err_msg=key)
