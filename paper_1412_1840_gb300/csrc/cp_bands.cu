@@ -839,6 +839,7 @@ __global__ void __launch_bounds__(32 * kRefineWarps, 2) k_window_refine(const Wi
                 const double v = r < rel ? val[r] : 0.0;
                 const float bv = r < rel ? eb[r] : 0.f, f = r < rel ? fv[r] : 0.f;
                 const uint32_t bal = __ballot_sync(0xffffffffu, t >= 0);
+                __syncwarp();                      // a vote orders no memory: these reads before the writes below
                 if (t >= 0) {                      // never ahead of the entries still to be read
                     const int q = kept + __popc(bal & ((1u << lane) - 1u));
                     val[q] = v;
