@@ -157,8 +157,9 @@ typedef struct {
  *                      class 8, 16, 32, 12, 48 run in the tensor form; a curve
  *                      whose class bit is clear runs in the direct form.
  * Curves above the last bucket, and plans without tuning, use the built-in
- * choices (16 frequencies per unit where they fit; every class in the tensor
- * form).  Results never depend on the tuning beyond the form's own rounding.
+ * choices (16 frequencies per unit where they fit, fewer for batches of short
+ * curves; every class in the tensor form).  Results never depend on the tuning
+ * beyond the form's own rounding.
  */
 #define CP_TUNE_MAX_BUCKETS 16
 typedef struct {

@@ -365,16 +365,6 @@ Exclusion exclusion_of(cp_plan_t p)
 // outside capture the flag is not allowed.
 unsigned rec_flags(cp_plan_t p) { return p->capturing ? cudaEventRecordExternal : cudaEventRecordDefault; }
 
-// Frequencies per direct-form unit: the requested count (16 by default),
-// halved until the unit's trig table fits the kernel's shared-memory budget.
-int fc_for(int n, int want = kFcMax)
-{
-    const int npad = (n + kTile - 1) / kTile * kTile;
-    int f = want;
-    while (f > 2 && (size_t)npad * f * 12 > (size_t)kTableBytes) f >>= 1;
-    return f;
-}
-
 // Tuning bucket of a curve of n samples, or -1 (built-in choices).
 int tune_bucket(const cp_tuning& t, int n)
 {
@@ -1275,8 +1265,6 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
             return fail(CP_EUNSUPPORTED, "cp_plan: curve " + std::to_string(c) + " has " + std::to_string(n) +
                                              " samples; the maximum is " + std::to_string(kMaxN));
         max_n = std::max(max_n, (int)n);
-        const int tb = tune_bucket(tune, (int)n);
-        p->fc[c] = fc_for((int)n, tb >= 0 ? tune.direct_fc[tb] : kFcMax);
     }
     p->max_band_points = (max_n + 9) / 10;   // a band holds at most ceil(N/10) samples
     p->n_points = offsets[n_curves];
@@ -1302,8 +1290,8 @@ static cp_status plan_impl(const double* times, const float* mags, const float* 
         const int64_t points = p->bands ? p->n_trials : g.hierarchical == CP_SEARCH_COARSE_FINE ? p->kc : g.n_freq;
         const int table = pair_table(max_n, (points + kFcMax - 1) / kFcMax * n_curves, p->n_sm);
         for (int64_t c = 0; c < n_curves; c++) {
-            const int n = (int)(offsets[c + 1] - offsets[c]);
-            while (p->fc[c] > 2 && (n + kTile - 1) / kTile * kTile * p->fc[c] * 12 > table) p->fc[c] >>= 1;
+            const int n = (int)(offsets[c + 1] - offsets[c]), tb = tune_bucket(tune, n);
+            p->fc[c] = direct_fc(n, tb >= 0 ? tune.direct_fc[tb] : 0, table);
         }
     }
     p->stream = (cudaStream_t)stream;

@@ -53,6 +53,16 @@ inline int pair_table(int max_n, int64_t units, int n_sm)
     return max_n <= kShortCurve && !between ? kShortTable : kTableBytes;
 }
 
+// Frequencies per direct-form unit of a curve of n samples: a tuned count (0: none) halved until the
+// unit's trig table fits the kernel's, else kFcMax halved until it fits the batch's (pair_table).
+inline int direct_fc(int n, int tuned, int table)
+{
+    const int npad = (n + 31) / 32 * 32, room = tuned ? kTableBytes : table;
+    int fc = tuned ? tuned : kFcMax;
+    while (fc > 2 && npad * fc * 12 > room) fc >>= 1;
+    return fc;
+}
+
 // Per-curve parameters, indexed by the caller's curve number.
 struct CurveParams {
     int64_t off;      // first sample in the CSR arrays

@@ -179,17 +179,12 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
     NA_CUDA(cudaGetDevice(&dev));
     NA_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int table = pair_table(max_n, ((g.hierarchical ? kc : g.n_freq) + kFcMax - 1) / kFcMax * n_curves, nsm);
-    auto fc_of = [table](int npad) {
-        int fc = kFcMax;
-        while (fc > 2 && npad * fc * 12 > table) fc >>= 1;
-        return fc;
-    };
     size_t pair_smem = 0;
     for (int s = 0; s < n_curves; s++) {
         const int c = order[s];
         const int n = (int)(offsets[c + 1] - offsets[c]);
         const int npad = (n + kTile - 1) / kTile * kTile;
-        const int fc = fc_of(npad);
+        const int fc = direct_fc(n, 0, table);
         unit_full[s + 1] = unit_full[s] + (g.n_freq + fc - 1) / fc;
         unit_coarse[s + 1] = unit_coarse[s] + (g.hierarchical ? (kc + fc - 1) / fc : 0);
         unit_fine[s + 1] = unit_fine[s] + (g.hierarchical ? (int64_t)g.top_k * ((2 * J + 1 + fc - 1) / fc) : 0);
@@ -200,8 +195,7 @@ extern "C" cp_status cp_best_period_noalloc(const double* times, const float* ma
         std::memset(&cps[c], 0, sizeof(CurveParams));
         cps[c].off = offsets[c];
         cps[c].n = (int32_t)(offsets[c + 1] - offsets[c]);
-        const int npad = (cps[c].n + kTile - 1) / kTile * kTile;
-        cps[c].fc = fc_of(npad);
+        cps[c].fc = direct_fc(cps[c].n, 0, table);
     }
 
     int ip_blocks = stats_blocks(n_curves, max_n, nsm);
