@@ -2,15 +2,19 @@
 
 * frequencies per work unit of the direct form (2, 4, 8 or 16), and
 * for each harmonic class of the tensor form (8, 12, 16, 32, 48 harmonics)
-  whether the tensor form or the direct form is faster at that curve size (the
-  tensor form pads a curve to 128-row tiles, which costs most for small N).
-  Classes 8, 12 and 16 are compared with the direct form's cos-form exponent
+  whether the tensor form or the direct form's pair sum takes less time per
+  pair and frequency at that curve size (the tensor form pads a curve to
+  128-row tiles, which costs most for small N).
+  Classes 8, 12 and 16 are compared with the pair sum's cos-form exponent
   (sigma_t 0.3), classes 32 and 48, which serve sigma_t < 0.25, with its
   sin-form exponent (sigma_t 0.2), the one those curves run in.
 
 It times the pair kernels through the public API on synthetic curves of
-each size bucket (results do not depend on the data, only on N and the grid
-size) and writes a JSON table that ``tuning_from`` turns into the C ABI's
+each size bucket (times do not depend on the data, only on N and the grid
+size).  A plan takes the pair spectrum instead of the pair sum where that is
+faster, whatever the table says, and its time per pair and frequency falls with
+the grid's length: the grid timed here starts at F_MIN, too far up for any
+transform, so that every frequency goes through the pair sum.  It writes a JSON table that ``tuning_from`` turns into the C ABI's
 ``cp_tuning``:
 
     python -m paper_1412_1840_gb300.tune --out paper_1412_1840_gb300/tuning_gb300.json
@@ -33,6 +37,7 @@ from . import (CP_FORM_DIRECT, CP_FORM_TENSOR, CP_SIGMA_T_FIXED, Plan, cp_max_po
 # (lowest, highest] curve sizes of each bucket
 BUCKETS = [(2, 96), (96, 192), (192, 320), (320, 512), (512, 768), (768, 1024), (1024, 1536),
            (1536, 2048), (2048, 3072), (3072, 4096)]
+F_MIN, DF = 1e4, 1e-3       # 1/day; see above
 TABLE_BYTES = 196608        # shared trig table of the direct kernel (12 B per point and frequency)
 
 
@@ -59,6 +64,8 @@ def timed(t, y, e, off, grid, reps: int = 2, sigma_t: float = 0.3, **kw) -> dict
         for _ in range(reps):
             p.best_period()
         info = p.info()
+    if kw.get("form") != CP_FORM_TENSOR and info["w_bytes_direct"] == 0:
+        raise RuntimeError("the search went through the pair spectrum: not the pair sum's time")
     ms = info["last_tensor_kernel_ms"] if kw.get("form") == CP_FORM_TENSOR else info["last_direct_kernel_ms"]
     return {"ms": ms, "pair_freq_per_s": info["pair_freq_search"] / (ms * 1e-3)}
 
@@ -66,7 +73,7 @@ def timed(t, y, e, off, grid, reps: int = 2, sigma_t: float = 0.3, **kw) -> dict
 def tune(n_freq: int = 2048, target_pair_freq: float = 4e10, seed: int = 0, device: int = 0, log=print,
          classes=(8, 12, 16, 32, 48), base: dict | None = None) -> dict:
     rng = np.random.default_rng(seed)
-    grid = make_grid(0.01, 1e-3, n_freq)
+    grid = make_grid(F_MIN, DF, n_freq)
     out = {"n_freq": n_freq, "buckets": []}
     try:
         import torch

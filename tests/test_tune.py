@@ -3,6 +3,8 @@ merge of a partial run into an earlier table, with the kernel timings
 replaced by a deterministic stand-in."""
 import json
 
+import pytest
+
 import paper_1412_1840_gb300 as cp
 from paper_1412_1840_gb300 import tune as T
 
@@ -60,3 +62,30 @@ def test_merge_times_only_the_listed_classes(monkeypatch, tmp_path):
         for cls in ("8", "12", "16", "32"):
             assert b1["tensor"][cls] == b0["tensor"][cls]
         assert "48" in b1["tensor"] and "48" not in b0["tensor"]
+
+
+def test_a_search_that_bypasses_the_pair_sum_is_not_a_measurement(monkeypatch):
+    """The direct form's time stands for the pair kernel only if the search ran
+    it at every frequency (tiles of magnitude kernels were built)."""
+    class Plan:
+        def __init__(self, *a, **kw):
+            self.info_ = dict(w_bytes_direct=4096.0 * (kw.get("tuning") is not None), last_direct_kernel_ms=2.0,
+                              last_tensor_kernel_ms=1.0, pair_freq_search=1e6)
+
+        def __enter__(self):
+            return self
+
+        def __exit__(self, *a):
+            return False
+
+        def best_period(self):
+            return {}
+
+        def info(self):
+            return self.info_
+
+    monkeypatch.setattr(T, "Plan", Plan)
+    assert T.timed(None, None, None, None, None, form=cp.CP_FORM_DIRECT, tuning=1)["pair_freq_per_s"] == 5e8
+    assert T.timed(None, None, None, None, None, form=cp.CP_FORM_TENSOR, n_max=8)["pair_freq_per_s"] == 1e9
+    with pytest.raises(RuntimeError):
+        T.timed(None, None, None, None, None, form=cp.CP_FORM_DIRECT)
