@@ -16,7 +16,9 @@
 //   S(f) = sum_ij w_ij e_ij = N (1 - ip) + 2 sum_{i<j} w_ij e_ij
 //   nCKP = sqrt(N sigma_t) / IP * CKP = S sqrt(N) / (N^2 ip sqrt(2 pi) sqrt(sigma_t))
 #pragma once
+#include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -428,6 +430,22 @@ cudaError_t raise_dyn_smem(const void* func, size_t bytes);
 // Thread-local message returned by cp_last_error() (fixed buffer, no heap).
 cp_status set_error(cp_status s, const char* msg);
 const char* last_error_buffer();
+
+// ---------------------------------------------------------------------------
+// a / b, correctly rounded, for many a: rb = RN(1 / b), rl = recip_low(b, rb).
+// q = a (rb + rl) is within a unit of a / b (half of one and 2^-51), and then
+// one correction by its exact remainder rounds correctly (Markstein 1990), as
+// long as nothing overflows or is subnormal.  Without rl q can be off by up to
+// one and a half units, and neither the remainder nor the rounding is certain.
+// ---------------------------------------------------------------------------
+__host__ __device__ __forceinline__ double recip_low(double b, double rb) { return fma(-b, rb, 1.0) * rb; }
+__host__ __device__ __forceinline__ double div_by(double a, double b, double rb, double rl)
+{
+    const double q = fma(a, rb, a * rl);
+    uint64_t bits;                                  // FP64 comparisons are slow on the device
+    memcpy(&bits, &q, sizeof bits);
+    return (bits >> 52 & 0x7ff) == 0x7ff ? a * rb : fma(fma(-q, b, a), rb, q);
+}
 
 // ---------------------------------------------------------------------------
 // FP64-exact phase in 64-bit fixed point: frac(a * b) * 2^64 (mod 2^64).
