@@ -18,7 +18,9 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -503,11 +505,13 @@ extern "C" cp_status cp_whiten(const double* times, const float* mags, const int
     const size_t smem = whiten_smem_bytes(np2);
     char* tmp = nullptr;
     // offsets and periods in one copy
-    std::vector<char> h_in((size_t)(2 * nc + 1) * 8);
-    std::memcpy(h_in.data(), offsets, (size_t)(nc + 1) * 8);
-    std::memcpy(h_in.data() + (nc + 1) * 8, p0, (size_t)nc * 8);
-    PREP_CUDA(pool_alloc((void**)&tmp, h_in.size(), s));
-    PREP_CUDA(cudaMemcpyAsync(tmp, h_in.data(), h_in.size(), cudaMemcpyHostToDevice, s));
+    const size_t in_bytes = (size_t)(2 * nc + 1) * 8;
+    const std::unique_ptr<char[]> h_in(new (std::nothrow) char[in_bytes]);
+    if (!h_in) return pfail(CP_ENOMEM, "cp_whiten: host allocation failed");
+    std::memcpy(h_in.get(), offsets, (size_t)(nc + 1) * 8);
+    std::memcpy(h_in.get() + (nc + 1) * 8, p0, (size_t)nc * 8);
+    PREP_CUDA(pool_alloc((void**)&tmp, in_bytes, s));
+    PREP_CUDA(cudaMemcpyAsync(tmp, h_in.get(), in_bytes, cudaMemcpyHostToDevice, s));
     PREP_CUDA(raise_dyn_smem((const void*)k_whiten, smem));
     k_whiten<<<(unsigned)nc, kPrepThreads, smem, s>>>(times, mags, reinterpret_cast<const int64_t*>(tmp),
                                                       reinterpret_cast<const double*>(tmp + (nc + 1) * 8), window, np2,
@@ -516,5 +520,6 @@ extern "C" cp_status cp_whiten(const double* times, const float* mags, const int
     PREP_CUDA(cudaStreamSynchronize(s));
 done:
     if (tmp) cudaFreeAsync(tmp, s);
+    if (st != CP_OK) cudaStreamSynchronize(s);       // the copy may still read h_in
     return st;
 }
