@@ -35,15 +35,23 @@ def search(b, g, rows=False, **kw):
         return got, p.info()
 
 
-def by_the_pair_sum(monkeypatch, b, g, extra_kb, **kw):
-    """The same search on a plan that has room for the magnitude-kernel tiles only."""
+def by_the_pair_sum(monkeypatch, b, g, **kw):
+    """The same search on a plan that has room for the magnitude-kernel tiles, not for a spectrum."""
     nb = (np.diff(b.offsets) + 31) // 32
     tiles = int(np.sum(nb * (nb + 1) // 2)) * 4096
+    room = tiles + 60 * int(b.offsets[-1]) + (768 << 10)
+    if g.hierarchical:
+        room += 8 * b.n_curves * int((g.n_freq - 1) * g.df / g.coarse_df + 2)
     with monkeypatch.context() as m:
-        m.setenv("CP_FAIL_ALLOC_ABOVE_KB", str((tiles >> 10) + extra_kb))
+        m.setenv("CP_FAIL_ALLOC_ABOVE_KB", str(room >> 10))
         got, info = search(b, g, **kw)
     assert info["w_bytes_direct"] == tiles
     return got
+
+
+def same_search(got, want):
+    for key in ("best_idx", "best_freq", "best_stat", "is_periodic"):
+        np.testing.assert_array_equal(got[key], want[key], err_msg=key)
 
 
 def strong_batch(n_curves, n, span, seed, integer):
@@ -83,9 +91,7 @@ def test_best_beside_excluded_peaks_is_the_pair_sums(monkeypatch, n, n_curves, i
     best, info = search(b, g, sigma_t=0.3)
     assert info["w_bytes_direct"] == 0
     assert np.all(best["best_idx"] >= 0)
-    want = by_the_pair_sum(monkeypatch, b, g, 2560, sigma_t=0.3)
-    for key in ("best_idx", "best_freq", "best_stat", "is_periodic"):
-        np.testing.assert_array_equal(best[key], want[key], err_msg=key)
+    same_search(best, by_the_pair_sum(monkeypatch, b, g, sigma_t=0.3))
 
 
 @pytest.mark.parametrize("n", [700, 2000])
@@ -108,6 +114,106 @@ def test_ties_far_below_an_excluded_peak(monkeypatch, n, seed):
     g = synth.Grid(g0.f_min, g0.df, g0.n_freq, exclude=tuple(map(tuple, edges)))
     best, info = search(b, g, sigma_t=0.3)
     assert info["w_bytes_direct"] == 0 and int(best["best_idx"][0]) in left and len(left) >= 5
-    want = by_the_pair_sum(monkeypatch, b, g, 1536, sigma_t=0.3)
-    for key in ("best_idx", "best_freq", "best_stat", "is_periodic"):
-        np.testing.assert_array_equal(best[key], want[key], err_msg=key)
+    same_search(best, by_the_pair_sum(monkeypatch, b, g, sigma_t=0.3))
+
+
+def harmonics_of(sigma_t, tail=2e-8):
+    """Harmonics kept: a_n = 2 e^-k I_n(k), k = 1 / sigma_t^2, by the backward recurrence,
+    up to the first n whose remaining sum is at most `tail` of the kernel's peak."""
+    k = 1.0 / (sigma_t * sigma_t)
+    a = np.zeros(160)
+    a[140] = 1e-200
+    for n in range(140, 0, -1):
+        a[n - 1] = a[n + 1] + 2.0 * n / k * a[n]
+    a[1:] *= 2.0
+    rest = np.cumsum((a / a.sum())[::-1])[::-1]
+    return int(np.argmax(rest[1:] <= tail))
+
+
+def transform_log2(n_out):
+    """log2 of the complex transform for n_out entries: 1.1 times as many cells at least, two a point."""
+    lq = 8
+    while (2 << lq) < 1.1 * n_out:
+        lq += 1
+    return lq
+
+
+# transform length, sigma_t, f_min, df, steps of the spectrum per df, K, curves, N.
+# Up to 2^13 points one block transforms a curve; 2^22 is the longest.
+LENGTHS = [(8, 1.5, 0.0, 1e-3, 1, 78, 64, 2000), (9, 1.5, 0.0, 1e-3, 1, 155, 64, 1200), (10, 1.5, 0.0, 1e-3, 1, 311, 64, 700),
+           (11, 1.5, 0.0, 1e-3, 1, 621, 64, 500), (12, 1.5, 0.0, 1e-3, 1, 1241, 48, 400), (13, 1.5, 0.0, 1e-3, 1, 2482, 24, 400),
+           (14, 1.5, 0.0, 1e-3, 1, 2500, 24, 400), (21, 0.1, 0.0, 1e-4, 1, 49981, 2, 400), (22, 0.1, 5e-5, 1e-4, 2, 49981, 2, 400)]
+
+
+@pytest.mark.parametrize("case", LENGTHS, ids=["2^%d" % c[0] for c in LENGTHS])
+def test_every_transform_length(monkeypatch, case):
+    """Against the oracle: within 1e-5 of the curve's peak or, where the pair sum at every frequency
+    does not meet that (noise curves on a few frequencies: 1.8e-5 at sigma_t 1.5, N 2,000), within the
+    pair sum's own error."""
+    logq, st, f_min, df, q, K, n_curves, n = case
+    top = int(round(f_min / df * q)) + q * (K - 1)
+    assert transform_log2(harmonics_of(st) * top + 1) == logq
+    b = synth.ragged_batch(n_curves, seed=93, n_lo=n - 30, n_hi=n, span=900.0)
+    g = synth.Grid(f_min, df, K)
+    got, info = search(b, g, rows=True, sigma_t=st)
+    assert info["w_bytes_direct"] == 0
+    rows = got["rows"]
+    np.testing.assert_array_equal(got["best_idx"], rows.argmax(axis=1))
+    np.testing.assert_array_equal(got["best_stat"], rows.max(axis=1))
+    some = list(range(min(n_curves, 6)))
+    ks = np.unique(np.r_[0, 1, K - 1, np.random.default_rng(4).choice(K, 60, replace=False), got["best_idx"][some]])
+    ref = oracle.batch_nckp(b.subset(some), np.full(len(some), float(np.float32(st))), g.freqs()[ks])
+    peak = np.maximum(np.abs(ref).max(axis=1), np.abs(rows[some]).max(axis=1))
+    err = np.abs(rows[some][:, ks] - ref).max(axis=1) / peak
+    pair = by_the_pair_sum(monkeypatch, b, g, rows=True, sigma_t=st)
+    perr = np.abs(pair["rows"][some][:, ks] - ref).max(axis=1) / peak
+    print("max error %.2e of the peak, of the pair sum %.2e" % (err.max(), perr.max()))
+    assert np.all(err <= np.maximum(TOL, perr)), (err, perr)
+    same_search(got, pair)
+
+
+def mixed_batch(n_curves, n_lo, n_hi, seed):
+    """A batch with a constant curve (every value ties at zero) and two whose sigma_t needs more
+    harmonics than the spectrum keeps."""
+    b = synth.ragged_batch(n_curves, seed=seed, n_lo=n_lo, n_hi=n_hi, span=1500.0)
+    b.mags[b.offsets[4]:b.offsets[5]] = 17.25
+    st = np.full(n_curves, 0.3, np.float32)
+    st[[1, 7]] = 0.05
+    return b, st
+
+
+@pytest.mark.parametrize("coarse_df,top_k", [(1e-3, 10), (3e-3, 1)])
+def test_coarse_fine_curves_that_the_pair_sum_evaluates_whole(monkeypatch, coarse_df, top_k):
+    b, st = mixed_batch(64, 200, 300, 94)
+    g = synth.Grid(0.0041, 1e-4, 14501, hierarchical=True, coarse_df=coarse_df, top_k=top_k, fine_df=1.3e-5,
+                   fine_halfwidth=2e-3)
+    got, info = search(b, g, sigma_t_per_curve=st)
+    assert info["w_bytes_direct"] == 0
+    same_search(got, by_the_pair_sum(monkeypatch, b, g, sigma_t_per_curve=st))
+
+
+def test_coarse_rows_longer_than_shared_memory(monkeypatch):
+    """Coarse rows of 30,001 points (above 24,576 they are read from global memory)."""
+    b, st = mixed_batch(24, 150, 200, 95)
+    g = synth.Grid(0.01, 1e-4, 30001, hierarchical=True, coarse_df=1e-4, top_k=10, fine_df=1e-5, fine_halfwidth=1e-4)
+    got, info = search(b, g, sigma_t_per_curve=st)
+    assert info["w_bytes_direct"] == 0
+    same_search(got, by_the_pair_sum(monkeypatch, b, g, sigma_t_per_curve=st))
+
+
+def test_trial_lists_that_the_pair_sum_evaluates_whole(monkeypatch):
+    """Bands search: the constant curve's 450 trials all tie, two curves have no spectrum; their
+    trial values are the pair sum's own, the others' within the direct form's bar."""
+    b, st = mixed_batch(64, 500, 600, 96)
+    g = synth.Grid(0.00125, 1e-4, 20000, bands=True, n_bands=3, trials_per_band=150)
+    got, info = search(b, g, sigma_t_per_curve=st)
+    assert info["w_bytes_direct"] == 0
+    want = by_the_pair_sum(monkeypatch, b, g, sigma_t_per_curve=st)
+    same_search(got, want)
+    np.testing.assert_array_equal(got["trial_idx"], want["trial_idx"])
+    for c in range(b.n_curves):
+        if c in (1, 4, 7):
+            np.testing.assert_array_equal(got["trial_stat"][c], want["trial_stat"][c])
+        else:
+            np.testing.assert_allclose(got["trial_stat"][c], want["trial_stat"][c], rtol=0,
+                                       atol=TOL * np.nanmax(np.abs(want["trial_stat"][c])))
