@@ -262,14 +262,14 @@ __global__ void __launch_bounds__(kPrepThreads) k_whiten(const double* times, co
     }
     int np2 = 32;
     while (np2 < n) np2 <<= 1;
-    const double rP = 1.0 / P, rPl = recip_low(P, rP);
+    const double rP = 1.0 / P;
     // tiny, huge and non-finite quotients keep the plain division
     const bool easy = P > 1e-100 && P < 1e100;
     for (int i = tid; i < np2; i += kPrepThreads) {
         unsigned long long key = ~0ull;
         if (i < n) {
             const double t = times[off + i];
-            const double q = easy && fabs(t) < 1e100 && fabs(t) > 1e-100 ? div_by(t, P, rP, rPl) : t / P;
+            const double q = easy && fabs(t) < 1e100 && fabs(t) > 1e-100 ? div_by(t, P, rP) : t / P;
             key = (unsigned long long)__double_as_longlong(q - floor(q)) & 0x7fffffffffffffffull;
         }
         ph[i] = key;
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_whiten(const double* times, co
     for (int k = tid; k < n; k += kPrepThreads) pre[k + 1] += s_carry[k / kSeg];
     __syncthreads();
     const int w = window < n ? window : n;
-    const double total = pre[n], wd = (double)w, rw = 1.0 / wd, rwl = recip_low(wd, rw);
+    const double total = pre[n], wd = (double)w, rw = 1.0 / wd;
     for (int k = tid; k < n; k += kPrepThreads) {
         // folded positions k - w/2 .. k - w/2 + w - 1, circular
         int a = k - w / 2, b = a + w;                          // [a, b)
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_whiten(const double* times, co
         } else {
             sum = (total - pre[a]) + pre[b - n];
         }
-        out[off + idx[k]] = (float)((double)xs[k] - div_by(sum, wd, rw, rwl));
+        out[off + idx[k]] = (float)((double)xs[k] - div_by(sum, wd, rw));
     }
 }
 
