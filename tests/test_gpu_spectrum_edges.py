@@ -217,3 +217,52 @@ def test_trial_lists_that_the_pair_sum_evaluates_whole(monkeypatch):
         else:
             np.testing.assert_allclose(got["trial_stat"][c], want["trial_stat"][c], rtol=0,
                                        atol=TOL * np.nanmax(np.abs(want["trial_stat"][c])))
+
+
+SEARCHES = [dict(), dict(hierarchical=True, coarse_df=1e-3, top_k=5, fine_df=2e-5, fine_halfwidth=1e-3),
+            dict(bands=True, n_bands=3, trials_per_band=100)]
+
+
+def short_and_long(seed=98):
+    """Curves of 2 to 100 samples (one of a single time) beside 60 of 600."""
+    rng = np.random.default_rng(seed)
+    sizes = np.array([2, 2, 3, 4, 5, 7, 9, 10, 16, 31, 32, 33, 63, 64, 65, 100] + [600] * 60)
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    t = rng.uniform(0.0, 1500.0, off[-1])
+    t[off[1]:off[2]] = 40.0
+    y = 17.0 + 0.3 * np.sin(2 * np.pi * t / 2.3) + rng.normal(0, 0.1, t.shape[0])
+    z = np.zeros(len(sizes))
+    return synth.Batch(t, y.astype(np.float32), np.full(t.shape[0], 0.1, np.float32), off, z, z.astype(bool), z.astype(np.int8))
+
+
+@pytest.mark.parametrize("kw", SEARCHES)
+def test_short_curves_beside_long_ones(monkeypatch, kw):
+    b = short_and_long()
+    g = synth.Grid(0.01, 1e-4, 20000, **kw)
+    got, info = search(b, g, rows=not kw, sigma_t=0.3)
+    assert info["w_bytes_direct"] == 0
+    same_search(got, by_the_pair_sum(monkeypatch, b, g, sigma_t=0.3))
+    if not kw:
+        some = list(range(17))
+        ks = np.arange(0, g.n_freq, 97)
+        ref = oracle.batch_nckp(b.subset(some), np.full(len(some), float(np.float32(0.3))), g.freqs()[ks])
+        err = np.abs(got["rows"][some][:, ks] - ref).max(axis=1)
+        peak = np.abs(got["rows"][some]).max(axis=1)
+        peak[1] = peak[0]                  # a single time: zero at every frequency
+        print("max error %.2e of the peak" % np.max(err / peak))
+        assert np.all(err <= TOL * peak), err / peak
+
+
+@pytest.mark.parametrize("kw", SEARCHES)
+def test_waves_of_a_small_tile_budget(monkeypatch, kw):
+    """Several waves of curves (each with its chunks and its curves left to the pair sum): the results
+    of one wave."""
+    b, st = mixed_batch(64, 500, 600, 99)
+    g = synth.Grid(0.01, 1e-4, 20000, **kw)
+    got, info = search(b, g, rows=True, sigma_t_per_curve=st)
+    monkeypatch.setenv("CP_W_BUDGET_KB", str(10 * 190 * 4))
+    waves, info2 = search(b, g, rows=True, sigma_t_per_curve=st)
+    assert info["w_bytes_direct"] == info2["w_bytes_direct"] == 0
+    assert info2["launches_per_search"] > info["launches_per_search"]
+    for key in got:
+        np.testing.assert_array_equal(waves[key], got[key], err_msg=key)
