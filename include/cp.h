@@ -220,8 +220,10 @@ void cp_default_options(cp_options *opt);
  * unchanged in size until cp_destroy.  Non-finite values and a zero median
  * error are reported by the call that reads them (CP_EINVAL).
  * offsets, grid, options and sigma_t_per_curve are copied at plan time.
- * The plan owns its device memory until cp_destroy.  A plan is used by one
- * host thread at a time.
+ * The plan owns its device memory until cp_destroy; a direct-form plan through
+ * the pair spectrum up to 4 GB of workspace (an eighth of the free memory at
+ * most, or one curve's), without room for which it evaluates by the pair sum.
+ * A plan is used by one host thread at a time.
  */
 cp_status cp_plan(const double *times, const float *mags, const float *errs,
                   const int64_t *offsets, int64_t n_curves, const cp_freq_grid *grid,

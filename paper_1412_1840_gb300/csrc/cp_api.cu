@@ -4,8 +4,8 @@
 // one file of (t, magnitude, error) per star) and a trial-frequency grid to
 // device buffers, a longest-first work schedule and, optionally, a captured
 // CUDA graph of one best-period search.  All arithmetic of the method runs in
-// the kernels of cp_kernels.cu; this file only validates, schedules, allocates
-// and launches.
+// kernels (cp_kernels.cu, cp_spec.cu, cp_tensor.cu, cp_bands.cu, cp_prep.cu); this
+// file only validates, schedules, allocates and launches.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>

@@ -587,11 +587,6 @@ __device__ __forceinline__ unsigned long long cand_emit(const PairArgs& a, int c
     return a.candidates == kCandCoarse ? 0ull : make_key(v, (uint32_t)e);
 }
 
-// SEL: a launch over chosen curves (fb_slots), those that the pair-spectrum path
-// leaves to the pair sum; its own instantiation, so that the units of a plain
-// launch carry none of it.  Its w come from the magnitudes
-// instead of stored tiles (one more exponential per pair and unit), so that
-// plans whose every pass goes through the spectrum keep no tiles.
 // Butterfly reduce-scatter of 16 values: on return lane l holds the warp's sum of
 // x[l >> 1] (the same pairs in the same order as 16 separate butterflies).
 __device__ __forceinline__ float reduce_scatter16(float (&x)[16], int lane)
@@ -608,6 +603,11 @@ __device__ __forceinline__ float reduce_scatter16(float (&x)[16], int lane)
     return x[0] + __shfl_xor_sync(0xffffffffu, x[0], 1);
 }
 
+// SEL: a launch over chosen curves (fb_slots), those that the pair-spectrum path
+// leaves to the pair sum; its own instantiation, so that the units of a plain
+// launch carry none of it.  Its w come from the magnitudes
+// instead of stored tiles (one more exponential per pair and unit), so that
+// plans whose every pass goes through the spectrum keep no tiles.
 // WARPS: a unit's tiles are always summed as by kPairThreads / 32 warps (each
 // every 16th tile, then lanes, then warps); a block of fewer warps takes several
 // of these shares in turn, with the same result.
