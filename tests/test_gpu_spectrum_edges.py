@@ -266,3 +266,14 @@ def test_waves_of_a_small_tile_budget(monkeypatch, kw):
     assert info2["launches_per_search"] > info["launches_per_search"]
     for key in got:
         np.testing.assert_array_equal(waves[key], got[key], err_msg=key)
+
+
+@pytest.mark.parametrize("n", [40, 300, 448])
+def test_cos_form_pair_sum_is_the_same_on_either_block_size(monkeypatch, n):
+    """The pair sum's cos form (sigma_t 0.3 and above) on 16 warps and, with four units for every SM,
+    on blocks of 4: the same bits (the lanes are added in the same order)."""
+    b = synth.ragged_batch(1, seed=11, n_lo=n, n_hi=n, span=900.0)
+    ks = (2000, 6400, 16 * 4 * 160)         # units of 16 frequencies: fewer than 2 per SM, than 4 per SM, more
+    rows = [by_the_pair_sum(monkeypatch, b, synth.Grid(0.01, 1e-4, k), rows=True, sigma_t=0.4)["rows"][0] for k in ks]
+    for k, row in zip(ks, rows):
+        np.testing.assert_array_equal(row, rows[-1][:k])
