@@ -1068,12 +1068,14 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
 
 // Margin below which two values of a curve are not told apart by the spectrum:
 // 1e-5 of the largest magnitude in the row, admissible or not (an excluded peak
-// carries its error to the values beside it), plus 1e-6 of the scale of a noise curve, several
-// times the error of the pair sum and of the spectrum together (both below 2e-6
-// of the peak).
+// carries its error to the values beside it), plus 3e-5 of norm N, the scale of a
+// noise curve.  The second part decides where the curve covers so little of a
+// cycle that the whole row lies far below that scale: the sum cancels there, and
+// the pair sum is off by up to 1.1e-5 of norm N, the spectrum by up to 5e-6 (curves of
+// half a day at up to a cycle).
 __device__ __forceinline__ float spec_margin(float vtop, const CurveParams& P)
 {
-    return 1e-5f * vtop + 1e-6f * P.norm * (float)P.n;
+    return 1e-5f * vtop + 3e-5f * P.norm * (float)P.n;
 }
 
 // ===========================================================================

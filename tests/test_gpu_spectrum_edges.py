@@ -277,3 +277,17 @@ def test_cos_form_pair_sum_is_the_same_on_either_block_size(monkeypatch, n):
     rows = [by_the_pair_sum(monkeypatch, b, synth.Grid(0.01, 1e-4, k), rows=True, sigma_t=0.4)["rows"][0] for k in ks]
     for k, row in zip(ks, rows):
         np.testing.assert_array_equal(row, rows[-1][:k])
+
+
+@pytest.mark.parametrize("seed", range(4))
+@pytest.mark.parametrize("kw,K", [(dict(), 195), (dict(), 2500), (dict(hierarchical=True, coarse_df=1e-3, top_k=3, fine_df=1e-4,
+                                                                      fine_halfwidth=2e-3), 2500)])
+def test_curves_that_cover_little_of_a_cycle(monkeypatch, kw, K, seed):
+    """Half a day of observations on frequencies of 0 to 0.25 1/day: every value lies far below the scale
+    of a noise curve, and the rounding of both ways decides the best; it is the pair sum's."""
+    b = synth.ragged_batch(180, seed=120 + seed, n_lo=200, n_hi=480, span=0.5)
+    st = np.random.default_rng(seed).choice([0.25, 0.3, 0.5, 0.9], b.n_curves).astype(np.float32)
+    g = synth.Grid(0.0, 1e-4, K, **kw)
+    got, info = search(b, g, sigma_t_per_curve=st)
+    assert info["w_bytes_direct"] == 0
+    same_search(got, by_the_pair_sum(monkeypatch, b, g, sigma_t_per_curve=st))
