@@ -38,3 +38,12 @@ def test_roofline_peaks(bench):
     assert p["bf16_tflops_sustained"] > 0 and p["hbm_gbs"] > 0
     if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")):
         assert p["source"] == "measured"
+
+
+def test_pair_frequencies_say_what_they_are(bench):
+    """A search through the pair spectrum builds no tiles: its figure is an equivalent, and says so."""
+    by_pairs = dict(w_bytes_direct=4096.0, w_bytes_tensor=0.0, pair_freq_search=6e9)
+    assert bench.pair_freq(by_pairs, 2.0) == {"pair_freq_per_s": 3e9, "pair_freq_basis": "evaluated"}
+    assert bench.pair_freq(dict(by_pairs, w_bytes_direct=0.0, w_bytes_tensor=1.0), 2.0)["pair_freq_basis"] == "evaluated"
+    spectrum = bench.pair_freq(dict(by_pairs, w_bytes_direct=0.0), 2.0, scale=4.0)
+    assert spectrum["pair_freq_per_s"] == 12e9 and spectrum["pair_freq_basis"].startswith("equivalent")
