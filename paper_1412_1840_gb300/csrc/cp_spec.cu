@@ -1168,7 +1168,6 @@ __global__ void __launch_bounds__(kPeakThreads) k_spec_peaks(const SpecArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned int s_hist[256], s_prefix, s_need;
-    __shared__ float s_max[kPeakThreads / 32];
     __shared__ int s_n, s_m;
     __shared__ int32_t s_raw[kPeakRaw], s_k[kSpecCand];
     const int ci = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1189,13 +1188,8 @@ __global__ void __launch_bounds__(kPeakThreads) k_spec_peaks(const SpecArgs a)
         float* row = reinterpret_cast<float*>(smem);
         for (int k = tid; k < K; k += kPeakThreads) row[k] = v[k];
         v = row;
-        __syncthreads();
     }
-    float vm = 0.f;
-    for (int k = tid; k < K; k += kPeakThreads) vm = fmaxf(vm, fabsf(v[k]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) vm = fmaxf(vm, __shfl_xor_sync(0xffffffffu, vm, o));
-    if (lane == 0) s_max[warp] = vm;
+    const float vm = __uint_as_float(a.vtop[c]);         // the row's largest magnitude
     if (tid == 0) {
         s_n = 0;
         s_m = 0;
@@ -1203,8 +1197,6 @@ __global__ void __launch_bounds__(kPeakThreads) k_spec_peaks(const SpecArgs a)
         s_need = (unsigned)a.top_k;
     }
     __syncthreads();
-#pragma unroll
-    for (int w = 0; w < kPeakThreads / 32; w++) vm = fmaxf(vm, s_max[w]);
     const float m = spec_margin(vm, P);
     auto sure = [&](int k) {
         const float x = v[k];
