@@ -18,7 +18,6 @@
 #pragma once
 #include <cmath>
 #include <cstdint>
-#include <cstring>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -444,9 +443,12 @@ const char* last_error_buffer();
 __host__ __device__ __forceinline__ double div_by(double a, double b, double rb)
 {
     const double q = a * rb;
-    uint64_t bits;                                  // FP64 comparisons are slow on the device
-    memcpy(&bits, &q, sizeof bits);
-    return (bits >> 52 & 0x7ff) == 0x7ff ? q : fma(fma(-q, b, a), rb, q);
+#ifdef __CUDA_ARCH__                                // FP64 comparisons are slow on the device
+    const bool finite = (__double2hiint(q) & 0x7ff00000) != 0x7ff00000;
+#else
+    const bool finite = std::isfinite(q);
+#endif
+    return !finite ? q : fma(fma(-q, b, a), rb, q);
 }
 
 // ---------------------------------------------------------------------------
