@@ -145,6 +145,10 @@ __global__ void __launch_bounds__(kCleanThreads) k_prep_stats(const double* time
             const double sxt = utx - ut * ux / k, sxx = uxx - ux * ux / k, stt = utt - ut * ut / k;
             const double sff = a1 * a1 * stt;
             r = (sxx <= 0.0 || sff <= 0.0) ? 0.0 : a1 * sxt / sqrt(sxx * sff);
+            if (det == 0.0) {                    // one time only: no slope, no correlation
+                a0 = Sx / S + xref;
+                a1 = r = 0.0;
+            }
         }
         PrepStats p;
         p.n_out = cnt;

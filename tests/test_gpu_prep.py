@@ -134,3 +134,21 @@ def test_dropped_first_samples_have_no_part_in_the_fit(value, lead):
         np.testing.assert_allclose(d["fit"][c], [r["a0"], r["a1"], r["r"]], rtol=1e-9, atol=1e-12)
     np.testing.assert_array_equal(d["times"].cpu().numpy(), ot)
     np.testing.assert_allclose(d["mags"].cpu().numpy(), ox, rtol=0, atol=4e-6 * max(1.0, np.abs(ox).max()))
+
+
+def test_curve_of_a_single_time_has_no_trend():
+    """All samples at one time: the line is undetermined, the correlation zero
+    (its fit takes one value), the magnitudes are left alone."""
+    rng = np.random.default_rng(55)
+    n = 80
+    m = rng.normal(17.0, 0.1, 2 * n).astype(np.float32)
+    e = rng.uniform(0.03, 0.08, 2 * n).astype(np.float32)
+    t = np.concatenate([np.full(n, 2450123.25), np.zeros(n)])
+    d = cp.cp_preprocess(torch.from_numpy(t).cuda(), torch.from_numpy(m).cuda(), torch.from_numpy(e).cuda(),
+                         np.array([0, n, 2 * n], np.int64))
+    np.testing.assert_array_equal(d["flags"], [1, 1])
+    np.testing.assert_array_equal(d["mags"].cpu().numpy(), m)
+    for c in range(2):
+        w = 1.0 / e[c * n:(c + 1) * n].astype(np.float64) ** 2
+        mean = (w * m[c * n:(c + 1) * n].astype(np.float64)).sum() / w.sum()
+        np.testing.assert_allclose(d["fit"][c], [mean, 0.0, 0.0], rtol=1e-9, atol=1e-12)
