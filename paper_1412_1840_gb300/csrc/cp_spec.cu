@@ -1068,14 +1068,16 @@ __global__ void __launch_bounds__(kSumThreads) k_spec_interp(const SpecArgs a)
 
 // Margin below which two values of a curve are not told apart by the spectrum:
 // 1e-5 of the largest magnitude in the row, admissible or not (an excluded peak
-// carries its error to the values beside it), plus 3e-5 of norm N, the scale of a
-// noise curve.  The second part decides where the curve covers so little of a
-// cycle that the whole row lies far below that scale: the sum cancels there, and
-// the pair sum is off by up to 1.1e-5 of norm N, the spectrum by up to 5e-6 (curves of
-// half a day at up to a cycle).
+// carries its error to the values beside it), plus 4e-6 + 7e-7 sqrt(N) of norm N, the
+// scale of a noise curve.  The second part decides where the curve covers so little
+// of a cycle that the whole row lies below that scale: the sums cancel there, and
+// spectrum and pair sum drift apart near the top by up to 5e-6, 1.5e-5, 2.0e-5 and
+// 2.9e-5 of norm N for N up to 100, 500, 1,500 and 4,096 (198,000 rows of random
+// batches below norm N); above it by at most 0.76 of the first part alone.
 __device__ __forceinline__ float spec_margin(float vtop, const CurveParams& P)
 {
-    return 1e-5f * vtop + 3e-5f * P.norm * (float)P.n;
+    const float n = (float)P.n;
+    return 1e-5f * vtop + (4e-6f + 7e-7f * sqrtf(n)) * P.norm * n;
 }
 
 // ===========================================================================
